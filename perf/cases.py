@@ -1,0 +1,303 @@
+"""Performance cases of the CoWindow Attention library: what a training job and a serving engine ask of it.
+
+A case is one call pattern of the public binding with its sizes:
+  train         cowa_fwd then cowa_bwd on a [B,H,T,D] batch (what one attention layer does in a training step)
+  train_packed  cowa_prefill_varlen then cowa_bwd_varlen on a packed batch of documents of different lengths
+  prefill       cowa_prefill: Nq new tokens behind Nk - Nq cached ones (chunked prefill)
+  prefill_packed  cowa_prefill_varlen: a packed batch of prompts, some of them behind a cached prefix
+  decode        cowa_decode: one new token for each of B sequences over a contiguous cache
+  decode_multi  cowa_decode_multi: the Nq newest tokens of each sequence (verification of drafted tokens)
+  decode_paged  cowa_decode_paged: the same over a paged cache
+Head counts, windows and the large shapes are those of the repository's benchmark configurations
+(tiny, 8K, 32K, 128K, 128K decode, and one tensor-parallel rank of the 64-head shape).
+"""
+from __future__ import annotations
+
+import math
+import random
+
+import numpy as np
+import torch
+
+import paper_2609_32704_b200 as cowa
+
+BF16 = torch.bfloat16
+
+
+def listed():
+    heads = dict(Hq=32, Hkv=8, D=128, sink=128)
+    return [
+        # unit tests and small models: one short sequence, few heads, D = 64; launches and latency count
+        dict(name="train_tiny", kind="train", B=1, T=1024, Hq=4, Hkv=2, D=64, sink=64, local=128),
+        # ordinary pre-training length: two sequences of 8K, GQA 4
+        dict(name="train_8k", kind="train", B=2, T=8192, Hq=16, Hkv=4, D=128, sink=128, local=1024),
+        # one rank of a tensor-parallel group of eight (one KV head, eight query heads), an odd sequence length,
+        # token-major activations as a projection leaves them, reproducible gradients
+        dict(name="train_tp_rank", kind="train", B=1, T=20001, Hq=8, Hkv=1, D=128, sink=128, local=896,
+             hkv_global=8, hkv_offset=3, token_major=True, deterministic=True),
+        # long-context continued training: 32K
+        dict(name="train_32k", kind="train", B=1, T=32768, local=2048, **heads),
+        # the longest training context: 128K
+        dict(name="train_128k", kind="train", B=1, T=131072, local=4096, **heads),
+        # documents packed to one row of tokens, long-tail mix of lengths
+        dict(name="train_packed", kind="train_packed", n=24, total=40000, shortest=60, Hq=16, Hkv=4, D=128,
+             sink=128, local=1024),
+        # chunked prefill: the next 512 tokens of a prompt whose first 32K tokens are cached already
+        dict(name="prefill_chunk", kind="prefill", B=1, Nq=512, Nk=33100, local=2048, **heads),
+        # prompts of several requests in one call, half of them behind a cached prefix
+        dict(name="prefill_packed", kind="prefill_packed", n=12, total=12000, shortest=100, prefix=6000,
+             local=1024, **heads),
+        # one user, 8K of context: the smallest serving call
+        dict(name="decode_one", kind="decode", B=1, Tmax=8192, len_lo=6000, len_hi=8000, local=1024, **heads),
+        # batch of eight at 96K-128K of context
+        dict(name="decode_128k", kind="decode", B=8, Tmax=131072, len_lo=98304, len_hi=131072, local=4096, **heads),
+        # verification of drafted tokens: eight newest tokens of eight sequences
+        dict(name="decode_multi", kind="decode_multi", B=8, Nq=8, Tmax=65536, len_lo=16000, len_hi=65000,
+             local=2048, **heads),
+        # serving batch over a paged cache, contexts from short to long
+        dict(name="decode_paged", kind="decode_paged", B=32, Nq=1, Tmax=32768, page=64, len_lo=500, len_hi=32000,
+             local=1024, **heads),
+    ]
+
+
+def _log_int(rng, lo, hi):
+    return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+
+def draw(rng: random.Random):
+    kind = rng.choice(["train", "train", "train_packed", "prefill", "prefill_packed", "decode", "decode_multi",
+                       "decode_paged"])
+    Hq, Hkv = rng.choice([(4, 2), (8, 1), (8, 8), (16, 4), (16, 2), (32, 8)])
+    c = dict(kind=kind, Hq=Hq, Hkv=Hkv, D=rng.choice([64, 128, 128]), sink=rng.choice([4, 64, 128]),
+             local=_log_int(rng, 128, 4096))
+    if kind == "train":
+        T = _log_int(rng, 512, 65536)
+        if rng.random() < 0.5:
+            T = max(512, T // 256 * 256)
+        c.update(B=min(4, max(1, 32768 // T)), T=T, token_major=rng.random() < 0.5, deterministic=rng.random() < 0.3)
+        if (Hq, Hkv) == (8, 1):
+            c.update(hkv_global=8, hkv_offset=rng.randrange(8))
+    elif kind == "train_packed":
+        c.update(n=rng.randint(2, 48), total=_log_int(rng, 4000, 60000), shortest=50,
+                 deterministic=rng.random() < 0.3)
+    elif kind == "prefill":
+        Nq = _log_int(rng, 100, 4096)
+        c.update(B=rng.choice([1, 1, 2, 4]), Nq=Nq, Nk=Nq + _log_int(rng, 500, 60000))
+    elif kind == "prefill_packed":
+        c.update(n=rng.randint(2, 24), total=_log_int(rng, 2000, 30000), shortest=30,
+                 prefix=_log_int(rng, 500, 16000))
+    else:
+        hi = _log_int(rng, 2000, 120000)
+        c.update(B=rng.choice([1, 2, 4, 8, 16, 32] if hi < 40000 else [1, 2, 4, 8]), Tmax=-(-hi // 256) * 256,
+                 len_lo=rng.randint(64, hi), len_hi=hi)
+        if kind == "decode_multi":
+            c.update(Nq=rng.choice([2, 3, 4, 5, 8, 16]))
+        elif kind == "decode_paged":
+            c.update(Nq=rng.choice([1, 1, 2, 4]), page=rng.choice([16, 64, 256]))
+    return c
+
+
+# ---------------------------------------------------------------------------------------------------------------
+# sequence lengths of a case: the same multiset for every seed, in an order that follows from the seed
+
+
+def _packed_lengths(c):
+    """n document lengths from `shortest` up, geometrically spread, that add up to `total`."""
+    n, total, lo = c["n"], c["total"], c["shortest"]
+    w = [1.35 ** (0.5 * i) for i in range(n)] if n > 16 else [1.8 ** (0.7 * i) for i in range(n)]
+    rest = total - n * lo
+    lens = [lo + int(rest * x / sum(w)) for x in w]
+    lens[-1] += total - sum(lens)
+    return lens
+
+
+def _prefixes(c):
+    """Cached tokens before each prompt: every second prompt has some."""
+    return [0 if i % 2 else (c["prefix"] * (i + 1)) // c["n"] for i in range(c["n"])]
+
+
+def _decode_lengths(c):
+    B, lo, hi = c["B"], c["len_lo"], c["len_hi"]
+    return [hi if B == 1 else lo + (hi - lo) * i // (B - 1) for i in range(B)]
+
+
+# ---------------------------------------------------------------------------------------------------------------
+# inputs: values N(0,1) rounded to bf16 (activations behind a norm and a projection), scores scaled by 1/sqrt(D)
+
+
+def _normal(gen, *shape):
+    out = torch.empty(shape, dtype=BF16, device="cuda")
+    return out.normal_(generator=gen)
+
+
+def _params(c):
+    return cowa.make_params(sink=c["sink"], local=c["local"], softmax_scale=1.0 / math.sqrt(c["D"]),
+                            hkv_global=c.get("hkv_global", 0), hkv_offset=c.get("hkv_offset", 0),
+                            deterministic=bool(c.get("deterministic", False)))
+
+
+def _bytes_buffer(n):
+    return torch.empty(max(int(n), 16), dtype=torch.uint8, device="cuda")
+
+
+def prepare(case, seed):
+    c = case
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    order = random.Random(seed)
+    Hq, Hkv, D = c["Hq"], c["Hkv"], c["D"]
+    p = _params(c)
+    s = dict(kind=c["kind"], p=p)
+    dev = "cuda"
+    if c["kind"] == "train":
+        B, T = c["B"], c["T"]
+        if c.get("token_major"):
+            new = lambda H: _normal(gen, B, T, H, D).transpose(1, 2)  # noqa: E731
+        else:
+            new = lambda H: _normal(gen, B, H, T, D)  # noqa: E731
+        s.update(q=new(Hq), k=new(Hkv), v=new(Hkv), do=new(Hq))
+        s.update(o=torch.empty_like(s["q"]), dq=torch.empty_like(s["q"]), dk=torch.empty_like(s["k"]),
+                 dv=torch.empty_like(s["v"]), lse=torch.empty((B, Hq, T), dtype=torch.float32, device=dev),
+                 ws=_bytes_buffer(cowa.cowa_bwd_workspace_bytes(B, T, Hq, Hkv, D, p)))
+    elif c["kind"] == "train_packed":
+        lens = _packed_lengths(c)
+        order.shuffle(lens)
+        total = sum(lens)
+        s.update(q=_normal(gen, Hq, total, D), k=_normal(gen, Hkv, total, D), v=_normal(gen, Hkv, total, D),
+                 do=_normal(gen, Hq, total, D))
+        s.update(o=torch.empty_like(s["q"]), dq=torch.empty_like(s["q"]), dk=torch.empty_like(s["k"]),
+                 dv=torch.empty_like(s["v"]), lse=torch.empty((Hq, total), dtype=torch.float32, device=dev),
+                 ws=_bytes_buffer(cowa.cowa_bwd_varlen_workspace_bytes(len(lens), total, Hq, Hkv, D, p)),
+                 cu=torch.tensor(np.cumsum([0] + lens), dtype=torch.int32).to(dev))
+    elif c["kind"] == "prefill":
+        B, Nq, Nk = c["B"], c["Nq"], c["Nk"]
+        s.update(q=_normal(gen, B, Hq, Nq, D), k=_normal(gen, B, Hkv, Nk, D), v=_normal(gen, B, Hkv, Nk, D),
+                 lse=torch.empty((B, Hq, Nq), dtype=torch.float32, device=dev))
+        s["o"] = torch.empty_like(s["q"])
+    elif c["kind"] == "prefill_packed":
+        seqs = list(zip(_packed_lengths(c), _prefixes(c)))
+        order.shuffle(seqs)
+        nq, nk = [a for a, _ in seqs], [a + b for a, b in seqs]
+        s.update(q=_normal(gen, Hq, sum(nq), D), k=_normal(gen, Hkv, sum(nk), D), v=_normal(gen, Hkv, sum(nk), D),
+                 lse=torch.empty((Hq, sum(nq)), dtype=torch.float32, device=dev),
+                 cu_q=torch.tensor(np.cumsum([0] + nq), dtype=torch.int32).to(dev),
+                 cu_k=torch.tensor(np.cumsum([0] + nk), dtype=torch.int32).to(dev))
+        s["o"] = torch.empty_like(s["q"])
+    else:
+        B, Tmax = c["B"], c["Tmax"]
+        lens = _decode_lengths(c)
+        order.shuffle(lens)
+        s["lens"] = torch.tensor(lens, dtype=torch.int32).to(dev)
+        if c["kind"] == "decode":
+            s.update(q=_normal(gen, B, Hq, D), k=_normal(gen, B, Hkv, Tmax, D), v=_normal(gen, B, Hkv, Tmax, D),
+                     lse=torch.empty((B, Hq), dtype=torch.float32, device=dev),
+                     ws=_bytes_buffer(cowa.cowa_decode_workspace_bytes(B, Tmax, Hq, Hkv, D, p)))
+        else:
+            Nq = c["Nq"]
+            s.update(q=_normal(gen, B, Nq, Hq, D), lse=torch.empty((B, Nq, Hq), dtype=torch.float32, device=dev),
+                     ws=_bytes_buffer(cowa.cowa_decode_multi_workspace_bytes(B, Nq, Tmax, Hq, Hkv, D, p)))
+            if c["kind"] == "decode_multi":
+                s.update(k=_normal(gen, B, Hkv, Tmax, D), v=_normal(gen, B, Hkv, Tmax, D))
+            else:
+                # the pages of a sequence lie anywhere in the pool, as an allocator hands them out
+                per, page = Tmax // c["page"], c["page"]
+                s.update(k=_normal(gen, B * per, Hkv, page, D), v=_normal(gen, B * per, Hkv, page, D))
+                perm = torch.randperm(B * per, generator=gen, device=dev)
+                s["table"] = perm.to(torch.int32).view(B, per).contiguous()
+        s["o"] = torch.empty_like(s["q"])
+    return s
+
+
+def run(state):
+    s = state
+    kind, p = s["kind"], s["p"]
+    if kind == "train":
+        cowa.cowa_fwd(s["q"], s["k"], s["v"], s["o"], s["lse"], p)
+        cowa.cowa_bwd(s["q"], s["k"], s["v"], s["o"], s["lse"], s["do"], s["dq"], s["dk"], s["dv"], p, s["ws"])
+        return [s["o"], s["lse"], s["dq"], s["dk"], s["dv"]]
+    if kind == "train_packed":
+        cowa.cowa_prefill_varlen(s["q"], s["k"], s["v"], s["o"], s["lse"], s["cu"], s["cu"], p)
+        cowa.cowa_bwd_varlen(s["q"], s["k"], s["v"], s["o"], s["lse"], s["do"], s["dq"], s["dk"], s["dv"], s["cu"],
+                             p, s["ws"])
+        return [s["o"], s["lse"], s["dq"], s["dk"], s["dv"]]
+    if kind == "prefill":
+        cowa.cowa_prefill(s["q"], s["k"], s["v"], s["o"], s["lse"], p)
+    elif kind == "prefill_packed":
+        cowa.cowa_prefill_varlen(s["q"], s["k"], s["v"], s["o"], s["lse"], s["cu_q"], s["cu_k"], p)
+    elif kind == "decode":
+        cowa.cowa_decode(s["q"], s["k"], s["v"], s["lens"], s["o"], s["lse"], p, s["ws"])
+    elif kind == "decode_multi":
+        cowa.cowa_decode_multi(s["q"], s["k"], s["v"], s["lens"], s["o"], s["lse"], p, s["ws"])
+    else:
+        cowa.cowa_decode_paged(s["q"], s["k"], s["v"], s["table"], s["lens"], s["o"], s["lse"], p, s["ws"])
+    return [s["o"], s["lse"]]
+
+
+# ---------------------------------------------------------------------------------------------------------------
+# what a pass cannot do without
+
+
+def _keys_seen(win, p0, p1):
+    """Number of keys that the queries at key positions p0 .. p1 see together (numpy arrays or numbers)."""
+    sink, near, gap, length = win
+    span = lambda lo, hi: np.maximum(0, hi - np.maximum(lo, 0) + 1)  # noqa: E731
+    near_lo = np.maximum(p0 - near + 1, 0)
+    n = span(near_lo, p1)
+    long_lo = np.maximum(p0 - near - gap - length + 1, 0)
+    long_hi = np.minimum(p1 - near - gap, near_lo - 1)
+    has = (length > 0) & (long_hi >= long_lo)
+    n = n + np.where(has, span(long_lo, long_hi), 0)
+    # sink columns below the long part, and between the long part and the near one
+    sink_hi = np.minimum(sink - 1, near_lo - 1)
+    below = np.where(has, np.minimum(sink_hi, long_lo - 1), sink_hi)
+    n = n + span(0, below)
+    return n + np.where(has, span(long_hi + 1, sink_hi), 0)
+
+
+def _windows(c, Nk):
+    return cowa.cowa_default_windows(Nk, c.get("hkv_global") or c["Hkv"], c.get("hkv_offset", 0), c["Hkv"],
+                                     c["sink"], c["local"])
+
+
+def _pairs(c, Nq, Nk):
+    """Legal (query, key) pairs of one sequence, summed over the KV heads."""
+    pos = np.arange(Nk - Nq, Nk, dtype=np.int64)
+    return int(sum(_keys_seen(w, pos, pos).sum() for w in _windows(c, Nk)))
+
+
+def work(case):
+    c = case
+    Hq, Hkv, D = c["Hq"], c["Hkv"], c["D"]
+    G = Hq // Hkv
+    row = D * 2  # bytes of one bf16 row
+    if c["kind"] in ("train", "train_packed"):
+        if c["kind"] == "train":
+            pairs, tokens = c["B"] * _pairs(c, c["T"], c["T"]), c["B"] * c["T"]
+        else:
+            lens = _packed_lengths(c)
+            pairs, tokens = sum(_pairs(c, n, n) for n in lens), sum(lens)
+        # in: q, dO, k, v; out: o, dq, dk, dv, lse
+        return {"bytes": tokens * (4 * Hq * row + 4 * Hkv * row + 4 * Hq), "flops": 14 * D * G * pairs}
+    if c["kind"] in ("prefill", "prefill_packed"):
+        if c["kind"] == "prefill":
+            seqs = [(c["Nq"], c["Nk"])] * c["B"]
+        else:
+            seqs = [(a, a + b) for a, b in zip(_packed_lengths(c), _prefixes(c))]
+        seen = sum(int(_keys_seen(w, Nk - Nq, Nk - 1)) for Nq, Nk in seqs for w in _windows(c, Nk))
+        nq = sum(a for a, _ in seqs)
+        return {"bytes": 2 * row * seen + nq * Hq * (2 * row + 4),
+                "flops": 4 * D * G * sum(_pairs(c, Nq, Nk) for Nq, Nk in seqs)}
+    Nq = c.get("Nq", 1)
+    rows = pairs = 0
+    for n in _decode_lengths(c):
+        for w in _windows(c, n):
+            rows += int(_keys_seen(w, n - Nq, n - 1))
+        pairs += _pairs(c, Nq, n)
+    return {"bytes": 2 * row * rows + c["B"] * Nq * Hq * (2 * row + 4), "flops": 4 * D * G * pairs}
+
+
+def tolerance(case):
+    # bf16 inputs and outputs, fp32 sums, probabilities and dS rounded to bf16 before their second product: against
+    # a 64-bit masked attention every bf16 output of every kind is off by 2.1e-3 to 2.5e-3, the worst single value
+    # by up to 0.1 of its root mean square (dk, dq at 6000 tokens).
+    return {"rel": 1e-2, "max": 0.3}
