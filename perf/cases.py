@@ -296,6 +296,92 @@ def work(case):
     return {"bytes": 2 * row * rows + c["B"] * Nq * Hq * (2 * row + 4), "flops": 4 * D * G * pairs}
 
 
+# ---------------------------------------------------------------------------------------------------------------
+# the same outputs in 64 bits, by masked attention in plain torch
+
+
+def _exact_windows(c, Nk):
+    """(near, first distance of the long part, first distance after it) of every KV head: the keys beyond sink and
+    near window are shared out in equal bands over the heads of the whole layer."""
+    heads, off = c.get("hkv_global") or c["Hkv"], c.get("hkv_offset", 0)
+    far = max(Nk - c["sink"] - c["local"], 0)
+    return [(c["local"], c["local"] + far * (off + h) // heads, c["local"] + far * (off + h + 1) // heads)
+            for h in range(c["Hkv"])]
+
+
+def _exact_attention(c, q, k, v, do=None):
+    """One sequence: q [Hq, Nq, D], k, v [Hkv, Nk, D]; queries sit at the last Nq key positions.  Query rows are
+    taken in blocks, each with the span of keys that it can see."""
+    Hq, Nq, D = q.shape
+    Hkv, Nk = k.shape[0], k.shape[1]
+    G, sink, scale = Hq // Hkv, c["sink"], 1.0 / math.sqrt(c["D"])
+    f64 = lambda x: x.to(torch.float64)  # noqa: E731
+    o = torch.empty(q.shape, dtype=torch.float64, device=q.device)
+    lse = torch.empty((Hq, Nq), dtype=torch.float64, device=q.device)
+    grads = None if do is None else [torch.zeros(x.shape, dtype=torch.float64, device=q.device) for x in (q, k, v)]
+    key = torch.arange(Nk, device=q.device)
+    block = 1024
+    for h, (near, a, b) in enumerate(_exact_windows(c, Nk)):
+        kh, vh, hs = f64(k[h]), f64(v[h]), slice(h * G, (h + 1) * G)
+        for i0 in range(0, Nq, block):
+            i1 = min(i0 + block, Nq)
+            p0, p1 = Nk - Nq + i0, Nk - Nq + i1 - 1
+            seen = (key <= p1) & ((key < sink) | (key > p0 - near) | ((key > p0 - b) & (key <= p1 - a)))
+            idx = seen.nonzero().flatten()
+            dist = torch.arange(p0, p1 + 1, device=q.device)[:, None] - idx[None, :]
+            legal = (dist >= 0) & ((dist < near) | (idx[None, :] < sink) | ((dist >= a) & (dist < b)))
+            ks, vs = kh[idx], vh[idx]
+            x = f64(q[hs, i0:i1])
+            s = (x @ ks.T) * scale
+            s.masked_fill_(~legal, -math.inf)
+            z = torch.logsumexp(s, -1, keepdim=True)
+            s = (s - z).exp_()
+            y = s @ vs
+            o[hs, i0:i1], lse[hs, i0:i1] = y, z[..., 0]
+            if do is not None:
+                g = f64(do[hs, i0:i1])
+                grads[2][h].index_add_(0, idx, torch.einsum("gqk,gqd->kd", s, g))
+                ds = s * (g @ vs.T - (g * y).sum(-1, keepdim=True)) * scale
+                grads[0][hs, i0:i1] = ds @ ks
+                grads[1][h].index_add_(0, idx, torch.einsum("gqk,gqd->kd", ds, x))
+    return [o, lse] + (grads or [])
+
+
+def exact(case, seed):
+    c = case
+    # score pairs with every query block's whole span: above this it takes longer than it is worth
+    if c["kind"] in ("train", "train_packed") and work(c)["flops"] > 1.2e13:
+        return None
+    s = prepare(c, seed)
+    kind = c["kind"]
+    if kind in ("train", "prefill"):
+        parts = [_exact_attention(c, s["q"][b], s["k"][b], s["v"][b], s["do"][b] if kind == "train" else None)
+                 for b in range(c["B"])]
+        return [torch.stack(x) for x in zip(*parts)]
+    if kind in ("train_packed", "prefill_packed"):
+        cq = (s["cu"] if kind == "train_packed" else s["cu_q"]).tolist()
+        ck = (s["cu"] if kind == "train_packed" else s["cu_k"]).tolist()
+        parts = []
+        for b in range(len(cq) - 1):
+            rq, rk = slice(cq[b], cq[b + 1]), slice(ck[b], ck[b + 1])
+            parts.append(_exact_attention(c, s["q"][:, rq], s["k"][:, rk], s["v"][:, rk],
+                                          s["do"][:, rq] if kind == "train_packed" else None))
+        return [torch.cat(x, dim=1) for x in zip(*parts)]
+    o, lse = [], []
+    for b, n in enumerate(s["lens"].tolist()):
+        if kind == "decode_paged":
+            pages = s["table"][b].long()
+            k, v = (x[pages].transpose(0, 1).reshape(c["Hkv"], -1, c["D"])[:, :n] for x in (s["k"], s["v"]))
+        else:
+            k, v = s["k"][b, :, :n], s["v"][b, :, :n]
+        q = s["q"][b] if kind != "decode" else s["q"][b][None]  # [Nq, Hq, D]
+        y, z = _exact_attention(c, q.transpose(0, 1), k, v)
+        o.append(y.transpose(0, 1))
+        lse.append(z.T)
+    o, lse = torch.stack(o), torch.stack(lse)
+    return [o[:, 0], lse[:, 0]] if kind == "decode" else [o, lse]
+
+
 def tolerance(case):
     # bf16 inputs and outputs, fp32 sums, probabilities and dS rounded to bf16 before their second product: against
     # a 64-bit masked attention every bf16 output of every kind is off by 2.1e-3 to 2.5e-3, the worst single value
