@@ -43,6 +43,21 @@ unsigned int* device_status_word() {
   return cache[dev];
 }
 
+int sm_count() {
+  static int cached = 0;
+  if (cached == 0) {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+        n > 0)
+      cached = n;
+    else {
+      cudaGetLastError();
+      return 148;  // B200; used when no device can be queried (workspace sizing on a machine without a GPU)
+    }
+  }
+  return cached;
+}
+
 int resolve_strides(const int64_t s[3], int H, long long T, int D, CowaStrides* out) {
   if (s[0] == 0 && s[1] == 0 && s[2] == 0) {
     out->t = D; out->h = (long long)T * D; out->b = (long long)H * T * D;

@@ -820,21 +820,6 @@ __global__ void cowa_bwd_reduce_dkv_kernel(const float* __restrict__ part, __nv_
 // every query tile of every head -- the critical path when Hkv is small; in both cases the group's heads
 // are spread over `parts` blocks (a divisor of G), chosen as the smallest that gives two waves of
 // blocks and keeps the longest block under 3/4 of an even share of the work.
-int sm_count() {
-  static int cached = 0;
-  if (cached == 0) {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-        n > 0)
-      cached = n;
-    else {
-      cudaGetLastError();
-      return 148;  // B200; used when no device can be queried (workspace sizing on a machine without a GPU)
-    }
-  }
-  return cached;
-}
-
 int bwd_parts(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& hw) {
   const int nKV = (Nk + BKV - 1) / BKV;
   long long total = 0, longest = 0;
@@ -850,7 +835,7 @@ int bwd_parts(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& hw) 
   total *= (long long)B * G;
   longest *= G;
   const long long blocks = (long long)B * Hkv * nKV;
-  const int kSMs = sm_count();
+  const int kSMs = cowa::sm_count();
   for (int p = 1; p < G; ++p) {
     if (G % p) continue;
     if (blocks * p >= 2 * kSMs && longest * 4 * kSMs <= 3 * total * p) return p;

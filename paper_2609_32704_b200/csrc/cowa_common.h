@@ -29,6 +29,9 @@ int record_cuda_error(cudaError_t e);
 // Device address of the status word of the current device (nullptr on failure).
 unsigned int* device_status_word();
 
+// SMs of the current device (148 when none can be queried: workspace sizing on a machine without a GPU).
+int sm_count();
+
 // Resolves the per-head tuples of a training call (explicit, default rule or FullAttn).
 // Returns COWA_OK or an error status.
 int resolve_windows(int Nk, int Hkv, const cowa_params_t* p, CowaHeadWindows* out);

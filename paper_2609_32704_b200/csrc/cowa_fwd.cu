@@ -19,9 +19,9 @@
 // warp scan of the offset arrays and stores a sequence's last, partial tile row by row.
 #include <cuda_bf16.h>
 
-#include "cowa_common.h"
-#include "cowa_ptx.cuh"
-#include "cowa_tma.h"
+#include "cowa_fwd.h"
+
+#include <algorithm>
 
 using namespace cowa_ptx;
 
@@ -29,27 +29,6 @@ namespace {
 
 constexpr int BQ = 128, BK = 64;
 constexpr int kFwdThreads = 160;
-
-struct FwdArgs {
-  float* lse;
-  unsigned int* status;
-  int B, Nq, Nk, Hq, Hkv, G;  // packed batches: Nq, Nk unused
-  float scale_log2;
-  CowaHeadWindows wins;
-  // packed (variable-length) batches only
-  const int* cu_q;   // [B+1] row offsets of the sequences in q / o / lse
-  const int* cu_k;   // [B+1] row offsets in k / v
-  __nv_bfloat16* o;  // raw output pointer for the last, partial tile of a sequence
-  int total_q, total_k;
-  int sink, local, hkv_global, hkv_offset, full_attn, explicit_windows;
-};
-
-// bits [lo, hi] of the 32-bit word covering columns [base, base+32)
-__device__ __forceinline__ uint32_t interval_bits(int a, int b, int base) {
-  int lo = max(a - base, 0), hi = min(b - base, 31);
-  if (lo > hi) return 0u;
-  return (0xFFFFFFFFu >> (31 - (hi - lo))) << lo;
-}
 
 template <int D>
 struct FwdSmem {
@@ -455,13 +434,42 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
   a.B = B; a.Nq = Nq; a.Nk = Nk; a.Hq = Hq; a.Hkv = Hkv; a.G = Hq / Hkv;
   a.scale_log2 = p->softmax_scale * 1.4426950408889634f;
   a.wins = hw;
-  a.cu_q = cu_q; a.cu_k = cu_k; a.o = static_cast<__nv_bfloat16*>(o); a.total_q = total_q; a.total_k = total_k;
+  a.cu_q = cu_q; a.cu_k = cu_k; a.o = static_cast<__nv_bfloat16*>(o); a.total_q = total_q; a.total_k = total_k; a.so = so;
   a.sink = p->sink; a.local = p->local;
   a.hkv_global = p->hkv_global > 0 ? p->hkv_global : Hkv;
   a.hkv_offset = p->hkv_offset; a.full_attn = p->full_attn; a.explicit_windows = p->windows != nullptr;
+  const long long tiles = VARLEN ? (long long)total_q / BQ + B : (long long)((Nq + BQ - 1) / BQ) * B;
+  if (a.G % 2 == 0) {
+    // Which kernel, judged for packed batches by their average sequence, so that equal lengths give what the batched
+    // call gives, bit for bit.  Measured at D = 128, Hq 32, Hkv 8 (us, one-head kernel / pair kernel):
+    //   at most half an item per SM: the item is shared by a cluster of 2, 4 or 8 blocks, two steps each at least,
+    //     once its list is long enough to pay for the merge (B 2, Nq 137: 881 keys 20.6 / 22.6, 1784 keys 30.8 / 29.3,
+    //     3448 keys 47.7 / 39.9; Nq 512, Nk 33100, 6300 keys: 76 / 55);
+    //   fewer than three items per SM and short lists: the one-head kernel's 128-row blocks leave the smaller last
+    //     wave (T 2048, local 128: 32.2 / 35.9; local 1024: 46.2 / 40.4);
+    //   else the pair kernel (T 8192, local 128 .. 1024: 127 / 120 .. 212 / 205; T 32768, local 2048: 2100 / 1860).
+    // At D = 64 the exponentials bound both and two one-head blocks per SM keep them busier (T 22272, 4 heads, fwd and
+    // bwd 1064 / 1138), so that only the shared form is taken there.
+    const int qn = VARLEN ? std::max(total_q / B, 1) : Nq, kn = VARLEN ? std::max(total_k / B, 1) : Nk;
+    int keys = 0;  // visited by the longest list, tile remainders included
+    for (int h = 0; h < Hkv; ++h) {
+      CowaWin w = hw.w[h];
+      if (VARLEN && p->full_attn) w.n = kn;
+      else if (VARLEN && !p->windows) w = cowa_default_window(kn, a.hkv_global, a.hkv_offset + h, a.sink, a.local);
+      const long long width = (long long)std::min(w.s, kn) + std::min(w.n, kn) + std::min(w.l, kn) + 2 * BQ;
+      keys = std::max(keys, (int)std::min<long long>(width, kn));
+    }
+    const long long items = tiles * (Hq / 2), judged = (long long)((qn + BQ - 1) / BQ) * B * (Hq / 2);
+    if (items > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
+    int split = 1;
+    while (split < 8 && judged * split * 2 <= (split == 1 ? 144 : 128) && keys >= 512 * split) split *= 2;
+    const bool half_empty = judged * 2 <= 144, long_list = keys >= (D == 128 ? 1536 : 2048);
+    if (half_empty ? long_list : D == 128 && (long_list || judged >= 3 * cowa::sm_count()))
+      return cowa::launch_fwd_pair<D, VARLEN>(mq, k, v, mo, sk, sv, a, rows_k, nb, items, split, st);
+  }
   COWA_CUDA_TRY(cudaFuncSetAttribute(cowa_fwd_kernel<D, VARLEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      FwdSmem<D>::kBytes));
-  const long long nblocks = VARLEN ? ((long long)total_q / BQ + B) * Hq : (long long)((Nq + BQ - 1) / BQ) * B * Hq;
+  const long long nblocks = tiles * Hq;
   if (nblocks > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
   cowa_fwd_kernel<D, VARLEN><<<(unsigned)nblocks, kFwdThreads, FwdSmem<D>::kBytes, st>>>(mq, mk, mv, mo, a);
   COWA_CUDA_TRY(cudaGetLastError());

@@ -1,0 +1,38 @@
+// Pieces shared by the forward kernels' translation units.
+#pragma once
+#include <cuda_bf16.h>
+
+#include "cowa_common.h"
+#include "cowa_ptx.cuh"
+#include "cowa_tma.h"
+
+struct FwdArgs {
+  float* lse;
+  unsigned int* status;
+  int B, Nq, Nk, Hq, Hkv, G;  // packed batches: Nq, Nk unused
+  float scale_log2;
+  CowaHeadWindows wins;
+  // packed (variable-length) batches only
+  const int* cu_q;   // [B+1] row offsets of the sequences in q / o / lse
+  const int* cu_k;   // [B+1] row offsets in k / v
+  __nv_bfloat16* o;  // raw output pointer for the last, partial tile of a sequence
+  int total_q, total_k;
+  CowaStrides so;    // of o (batched calls)
+  int sink, local, hkv_global, hkv_offset, full_attn, explicit_windows;
+};
+
+// bits [lo, hi] of the 32-bit word covering columns [base, base+32)
+__device__ __forceinline__ uint32_t interval_bits(int a, int b, int base) {
+  int lo = max(a - base, 0), hi = min(b - base, 31);
+  if (lo > hi) return 0u;
+  return (0xFFFFFFFFu >> (31 - (hi - lo))) << lo;
+}
+
+namespace cowa {
+// Pair kernel (cowa_fwd_pair.cu): two QO heads of a group at a time, `items` = tiles x pairs of heads.  split = 1: one
+// persistent block per SM; split = 2, 4, 8: every item shared by a cluster of that many blocks.
+template <int D, bool VARLEN>
+int launch_fwd_pair(const CUtensorMap& mq, const void* k, const void* v, const CUtensorMap& mo, const CowaStrides& sk,
+                    const CowaStrides& sv, const FwdArgs& a, int rows_k, int nb, long long items, int split,
+                    cudaStream_t st);
+}  // namespace cowa

@@ -1,0 +1,713 @@
+// CoWindow Attention forward (Algorithm 1) for sm_100a: two QO heads of a GQA group per block.
+//
+// Persistent, one block per SM.  A work item is (batch, pair of QO heads that share a KV head, 128-row QO tile);
+// both heads visit the same KV tiles J_h(i), so one pass over K and V serves 256 query rows.  A step takes two
+// visited 64-key tiles (not necessarily neighbours) as one 128-key operand: S at N = 128 runs at the full tensor
+// rate (512 clocks; as two products of 64 keys 768).  Warps:
+//   warps 0-3, 4-7  softmax of head 0 / head 1: one query row per thread; then O / l and LSE
+//   warp 8          TMA producer: Q of both heads, then K and V of every step through four 32 KB slots; works out the
+//                   items' geometry one item ahead
+//   warp 9          MMA issuer, per step:  O_0 += P_0 V | S_0' = Q_0 K' | O_1 += P_1 V | S_1' = Q_1 K'
+// While the tensor pipe works for one head, the other head's warps do their softmax, so the two alternate.
+// P is handed over in two halves: O += P V starts on the first while the second is still being exponentiated.
+// P overwrites S in TMEM; S_0 (128 columns), S_1, O_0, O_1 fill all 512 columns.
+// As in the one-head kernel the running max only advances when it grows by more than 2^8; S of a step completes
+// after O += P V of the step before it (same issue order), so the rare rescale needs no further wait.
+// The next item's Q, K and V are fetched, and its first S computed, while the softmax warps still write out O.
+//
+// What bounds it: per step and pair of heads the tensor pipe needs 2048 clocks and the exponentials 2048 of the
+// special-function unit (1792 with one pair in eight on the FMA pipe); a step takes about 3150, the chain of one
+// head (S landed 900, load 100, row max 300, exponentials 1400, hand-over 150, with one warp per scheduler and
+// head to cover it) at 1.7 GHz; long calls run at the power limit below that.
+#include "cowa_fwd.h"
+
+#include <algorithm>
+
+using namespace cowa_ptx;
+
+namespace {
+
+constexpr int BQ = 128, BK = 64, BS = 2 * BK;  // query rows per tile, keys per visited tile, keys per step
+constexpr int kSplitQ = 1;  // O += P V starts once the 32-key groups 0 .. kSplitQ of P are in place
+constexpr int kPairThreads = 384;  // warps 10, 11 only make the control warpgroup whole
+constexpr int kItemReaders = 9;  // warps that read a published work item: softmax 8, MMA 1
+
+__device__ __forceinline__ uint32_t interval_bits(int a, int b, int base) {
+  int lo = max(a - base, 0), hi = min(b - base, 31);
+  if (lo > hi) return 0u;
+  return (0xFFFFFFFFu >> (31 - (hi - lo))) << lo;
+}
+
+// 2^x of a pair on the FMA and integer pipes: x = n + f with n = rint(x), |f| <= 1/2, 2^f by the polynomial of
+// degree 6 with the least largest relative error on that interval (fitted by reweighted least squares: 1.9e-9, in
+// fp32 8e-8, against 2 ulp of ex2.approx), times 2^n.  Below 2^-126 the result stays 2^-126; NaN stays NaN.
+__device__ __forceinline__ float2 exp2_fma(float2 x) {
+  auto c2 = [](float c) { return make_float2(c, c); };
+  x.x = max_nan(x.x, -126.f); x.y = max_nan(x.y, -126.f);
+  const float2 t = add2(x, c2(12582912.f));                        // 1.5 * 2^23: n in the low mantissa bits
+  const float2 f = fma2(add2(t, c2(-12582912.f)), c2(-1.f), x);
+  float2 p = fma2(c2(1.53458118e-4f), f, c2(1.33999312e-3f));
+  p = fma2(p, f, c2(9.61848896e-3f));
+  p = fma2(p, f, c2(5.55032878e-2f));
+  p = fma2(p, f, c2(2.40226469e-1f));
+  p = fma2(p, f, c2(6.93147206e-1f));
+  p = fma2(p, f, c2(1.f));
+  return mul2(p, make_float2(__uint_as_float((__float_as_uint(t.x) << 23) + 0x3F800000u),
+                             __uint_as_float((__float_as_uint(t.y) << 23) + 0x3F800000u)));
+}
+
+template <int D>
+struct PairSmem {
+  static constexpr int kQ = BQ * D * 2;    // Q tile of one head
+  static constexpr int kKV = BS * D * 2;   // K or V operand of one step
+  static constexpr int kOut = BQ * 128;    // one 64-column slab of an O tile on its way out
+  static constexpr int oQ = 0, oK = 2 * kQ, oV = oK + 2 * kKV, oOut = oV + 2 * kKV, oBar = oOut + 2 * kOut;
+  static constexpr int oItem = oBar + 256;           // two work items
+  static constexpr int kBytes = oItem + 256 + 1024;  // + alignment slack
+};
+static_assert(PairSmem<128>::kBytes <= 232448, "shared memory of a block");
+
+// One work item: where its rows lie, which KV tiles it visits and which of them need no mask.  The TMA warp works
+// it out one item ahead and leaves it in shared memory for the other warps.
+struct PairItem {
+  int b, bt, h0, hk, Nq, Nk, qbase, kbase, q0, off;
+  CowaWin w;
+  CowaRange rg[3];
+  int f_lo[3], f_hi[3];  // unmasked tiles: one interval per range (see cowa_fwd_kernel)
+  int t0, nt;            // visited 64-key tiles of this block: t0 .. t0 + nt - 1 of the list; nt = 0: no more items
+  int work;              // split items: 0 when there is nothing to write at all
+};
+static_assert(sizeof(PairItem) <= 128, "slot of a published item");
+static_assert(4 * PairSmem<128>::kKV >= 2 * BQ * 128 * 4, "fp32 O of both heads fits the K and V slots");
+
+// false: no item of this number (packed batches: the count is an upper bound) or malformed offsets
+template <bool VARLEN>
+__device__ __forceinline__ bool locate_item(const FwdArgs& a, int idx, PairItem& it) {
+  const int PG = a.G >> 1;
+  const int gp = idx % PG; idx /= PG;
+  it.hk = idx % a.Hkv; idx /= a.Hkv;
+  it.h0 = it.hk * a.G + 2 * gp;
+  int i;
+  it.w = a.wins.w[it.hk];
+  if constexpr (!VARLEN) {
+    it.b = idx % a.B; idx /= a.B;
+    i = (a.Nq + BQ - 1) / BQ - 1 - idx;  // heaviest tiles first
+    it.Nq = a.Nq; it.Nk = a.Nk; it.qbase = 0; it.kbase = 0; it.bt = it.b;
+  } else {
+    int lt, nts, pb;
+    if (!varlen_locate(a.cu_q, a.B, idx, BQ, 0, &it.b, &lt, &nts, &pb)) return false;
+    i = nts - 1 - lt;
+    it.qbase = a.cu_q[it.b]; it.Nq = a.cu_q[it.b + 1] - it.qbase;
+    it.kbase = a.cu_k[it.b]; it.Nk = a.cu_k[it.b + 1] - it.kbase;
+    it.bt = 0;
+    if (it.Nq > it.Nk || it.qbase < 0 || it.kbase < 0 || it.qbase + it.Nq > a.total_q || it.kbase + it.Nk > a.total_k) {
+      if ((threadIdx.x & 31) == 0) atomicOr(a.status, (unsigned)COWA_DEV_BAD_SEQLENS);
+      return false;
+    }
+    if (a.full_attn) { it.w.s = 0; it.w.n = it.Nk; it.w.g = 0; it.w.l = 0; }
+    else if (!a.explicit_windows) it.w = cowa_default_window(it.Nk, a.hkv_global, a.hkv_offset + it.hk, a.sink, a.local);
+  }
+  const CowaWin w = it.w;
+  it.off = it.Nk - it.Nq;
+  it.q0 = i * BQ;
+  cowa_fwd_ranges(w, it.q0, min(it.q0 + BQ, it.Nq) - 1, it.off, it.Nk, BK, it.rg);
+  it.t0 = 0;
+  it.nt = cowa_range_len(it.rg[0]) + cowa_range_len(it.rg[1]) + cowa_range_len(it.rg[2]);
+  it.work = it.nt;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) { it.f_lo[q] = 1; it.f_hi[q] = 0; }
+  if (it.q0 + BQ <= it.Nq) {
+    auto fdiv = [](long long v) -> int { return (int)(v >> 6); };  // floor of v / BK
+    static_assert(BK == 64, "shift in fdiv");
+    const long long p0 = (long long)it.q0 + it.off, p1 = p0 + BQ - 1;
+    const int causal_hi = fdiv(p0 - (BK - 1));
+    it.f_lo[0] = fdiv(p1 - w.n) + 1; it.f_hi[0] = causal_hi;
+    if (w.l > 0) {
+      it.f_lo[1] = fdiv(p1 - ((long long)w.n + w.g + w.l)) + 1;
+      it.f_hi[1] = min(causal_hi, fdiv(p0 - ((long long)w.n + w.g) - (BK - 1)));
+    }
+    it.f_lo[2] = 0; it.f_hi[2] = min(causal_hi, w.s >= BK ? (w.s - BK) / BK : -1);
+  }
+  return it.nt > 0;
+}
+
+// SPLIT: a cluster of blocks shares one item (few items, long lists): each takes a contiguous part of its steps, and
+// the partial states are merged through distributed shared memory.
+template <int D, bool VARLEN, bool SPLIT>
+__global__ void __launch_bounds__(kPairThreads, 1)
+cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
+                     const __grid_constant__ FwdArgs a, const int items) {
+  using SM = PairSmem<D>;
+  constexpr int NSLAB = D / 64;        // 64-element (128-byte) slabs along D
+  constexpr int SLAB = 128 * 128;      // bytes of one slab of a 128-row tile
+  constexpr uint32_t TMEM_COLS = 512;  // S/P of head x: [128x, 128x + 128); O of head x: [256 + 128x, ... + D)
+  constexpr uint32_t cO = 256;
+  constexpr uint32_t IDESC_S2 = idesc_bf16(128, BS, 0, 0), IDESC_S1 = idesc_bf16(128, BK, 0, 0);
+  constexpr uint32_t IDESC_O = idesc_bf16(128, D, 0, 1);
+
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sQ = smem + SM::oQ;      // [2 heads][kQ]
+  uint8_t* sK = smem + SM::oK;      // [2][kKV]
+  uint8_t* sV = smem + SM::oV;      // [2][kKV]
+  uint8_t* sOut = smem + SM::oOut;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SM::oBar);
+  uint64_t* bar_q_full = bars + 0;    //     Q of an item has landed
+  uint64_t* bar_q_empty = bars + 1;   //     every S of the item has been computed
+  uint64_t* bar_k_full = bars + 2;    // [2]
+  uint64_t* bar_k_empty = bars + 4;   // [2]
+  uint64_t* bar_v_full = bars + 6;    // [2]
+  uint64_t* bar_v_empty = bars + 8;   // [2]
+  uint64_t* bar_s = bars + 10;        // [2 heads] S of a step is in TMEM
+  uint64_t* bar_p = bars + 12;        // [2 heads][2 halves] count 4 (warps): P written over S
+  uint64_t* bar_o_full = bars + 16;   // [2 heads] O of an item is complete
+  uint64_t* bar_o_empty = bars + 18;  // [2 heads] count 4: O has been read
+  uint64_t* bar_i_full = bars + 20;   // [2] a work item has been published
+  uint64_t* bar_i_empty = bars + 22;  // [2] count kItemReaders: it has been read
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 24);
+
+  const int tid = threadIdx.x;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform by construction
+
+  if (tid == 0) {
+    for (int s = 0; s < 24; ++s)
+      mbar_init(bars + s, (s >= 12 && s < 16) || s == 18 || s == 19 ? 4 : s >= 22 ? kItemReaders : 1);
+    fence_mbar_init();
+  }
+  if (warp == 9) {
+    __syncwarp();
+    tmem_alloc(tmem_holder, TMEM_COLS);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tb = *tmem_holder;
+
+  bool ok = true;  // false once a bounded wait ran out; every role then falls through to the teardown
+  auto warp_arrive = [&](uint64_t* bar) {  // one arrival for the whole warp
+    __syncwarp();
+    if ((tid & 31) == 0) mbar_arrive(bar);
+  };
+  // Work item number ni of this block; false when a wait ran out or there is none left.  Its words pass through a
+  // shuffle so that the compiler knows them to be uniform over the warp (branches and counters on the uniform path).
+  auto next_item = [&](uint32_t ni, PairItem& it) -> bool {
+    ok = mbar_wait(bar_i_full + (ni & 1), (ni >> 1) & 1, a.status);
+    if (!ok) return false;
+    const int* src = reinterpret_cast<const int*>(smem + SM::oItem + (ni & 1) * 128);
+    int words[sizeof(PairItem) / 4];
+#pragma unroll
+    for (int i = 0; i < (int)(sizeof(PairItem) / 4); ++i) words[i] = __shfl_sync(0xFFFFFFFFu, src[i], 0);
+    __syncwarp();
+    if ((tid & 31) == 0) mbar_arrive(bar_i_empty + (ni & 1));
+    memcpy(&it, words, sizeof(PairItem));
+    return it.nt > 0;
+  };
+
+  // Registers: 168 a thread at launch; the softmax threads hold a row of S: 2 * 208 + 88 = 3 * 168.
+  if (warp >= 8) {
+   setmaxnreg_dec<88>();
+   if (warp == 8) {
+    // ======================= TMA producer =======================
+    const bool lead = elect_one();
+    if (lead) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); }
+    int c = 0;       // steps loaded so far, all items together: step c uses slot c & 1
+    uint32_t ni = 0;  // items so far
+    // Items come heaviest first; blocks take them in rounds, every second round from the other end, so that a block
+    // with a heavy item in one round has a light one in the next.
+    const int csize = SPLIT ? (int)cluster_size() : 1;
+    for (int rnd = 0; ok; ++rnd) {
+      const long long base = SPLIT ? (rnd == 0 ? 0 : items) : (long long)rnd * gridDim.x;
+      const int idx = SPLIT ? blockIdx.x / csize : (int)(base + ((rnd & 1) ? gridDim.x - 1 - blockIdx.x : blockIdx.x));
+      PairItem& it = *reinterpret_cast<PairItem*>(smem + SM::oItem + (ni & 1) * 128);
+      {
+        PairItem mine;
+        if (SPLIT) {
+          if (rnd > 0) break;
+          if (locate_item<VARLEN>(a, idx, mine)) {
+            const int n = (mine.nt + 1) >> 1, rank = (int)cluster_rank();
+            mine.t0 = 2 * (n * rank / csize);
+            mine.nt = max(min(2 * (n * (rank + 1) / csize), mine.nt) - mine.t0, 0);
+          } else {
+            mine.nt = mine.work = 0;
+          }
+        } else if (base >= items) {
+          mine.nt = 0;
+        } else if (idx >= items || !locate_item<VARLEN>(a, idx, mine)) {
+          continue;
+        }
+        if (ni >= 2) ok = mbar_wait(bar_i_empty + (ni & 1), ((ni >> 1) & 1) ^ 1, a.status);
+        if (!ok) break;
+        if (lead) {
+          it = mine;
+          mbar_arrive(bar_i_full + (ni & 1));
+        }
+        __syncwarp();
+        if (mine.nt == 0) break;
+      }
+      auto load_kv = [&](uint8_t* base, const CUtensorMap* tm, uint64_t* bar, int t) {
+        if (lead) {
+          const int nh = t + 1 < it.nt ? 2 : 1;
+          mbar_expect_tx(bar, nh * (SM::kKV / 2));
+          for (int hf = 0; hf < nh; ++hf) {
+            const int row = it.kbase + cowa_fwd_tile_at(it.rg, it.t0 + t + hf) * BK;
+            for (int s = 0; s < NSLAB; ++s) tma_load_4d(base + s * SLAB + hf * (SLAB / 2), tm, bar, s * 64, row, it.hk, it.bt);
+          }
+        }
+      };
+      for (int t = 0; t < it.nt; t += 2, ++c) {
+        const int sl = c & 1;
+        const uint32_t ph = ((c >> 1) & 1) ^ 1;
+        if (c >= 2) ok = mbar_wait(bar_k_empty + sl, ph, a.status);
+        if (!ok) break;
+        load_kv(sK + sl * SM::kKV, &tmK, bar_k_full + sl, t);
+        if (t == 0) {
+          if (ni > 0) ok = mbar_wait(bar_q_empty, (ni - 1) & 1, a.status);
+          if (!ok) break;
+          if (lead) {
+            mbar_expect_tx(bar_q_full, 2 * SM::kQ);
+            for (int x = 0; x < 2; ++x)
+              for (int s = 0; s < NSLAB; ++s)
+                tma_load_4d(sQ + x * SM::kQ + s * SLAB, &tmQ, bar_q_full, s * 64, it.qbase + it.q0, it.h0 + x, it.bt);
+          }
+        }
+        if (c >= 2) ok = mbar_wait(bar_v_empty + sl, ph, a.status);
+        if (!ok) break;
+        load_kv(sV + sl * SM::kKV, &tmV, bar_v_full + sl, t);
+      }
+      ++ni;
+    }
+   } else if (warp == 9) {
+    // ======================= MMA issuer (warp-uniform control flow, one elected lane issues) =======================
+    const bool lead = elect_one();
+    const uint64_t dQ0 = smem_desc_sw128(smem_u32(sQ), 16, 1024);    // Q, K-major (A of S)
+    const uint64_t dK0 = smem_desc_sw128(smem_u32(sK), 16, 1024);    // K, K-major (B of S)
+    const uint64_t dV0 = smem_desc_sw128(smem_u32(sV), SLAB, 1024);  // V, MN-major (B of O)
+    constexpr uint32_t kQ16 = SM::kQ >> 4, kKV16 = SM::kKV >> 4;
+    int c = 0;
+    uint32_t ni = 0;
+    PairItem it;
+    for (; ok && !(SPLIT && ni > 0) && next_item(ni, it); ++ni) {
+      const int nt = it.nt;
+      const int n = (nt + 1) >> 1;  // steps
+      auto issue_s = [&](int x, int t, int sl) {  // S_x = Q_x K^T of step t; 64 keys only in an odd last step
+        if (lead) {
+          const uint32_t id = 2 * t + 1 < nt ? IDESC_S2 : IDESC_S1;
+          const uint64_t dA = dQ0 + x * kQ16, dB = dK0 + sl * kKV16;
+#pragma unroll
+          for (int kk = 0; kk < D / 16; ++kk)
+            mma_ss(tb + x * 128, dA + (((kk / 4) * SLAB + (kk % 4) * 32) >> 4), dB + (((kk / 4) * SLAB + (kk % 4) * 32) >> 4),
+                   id, kk > 0);
+          mma_commit(bar_s + x);
+          if (x == 1) {
+            mma_commit(bar_k_empty + sl);
+            if (t == n - 1) mma_commit(bar_q_empty);
+          }
+        }
+      };
+      ok = mbar_wait(bar_k_full + (c & 1), (c >> 1) & 1, a.status) && mbar_wait(bar_q_full, ni & 1, a.status);
+      if (!ok) break;
+      tc_fence_after();
+      issue_s(0, 0, c & 1);
+      issue_s(1, 0, c & 1);
+      for (int t = 0; t < n && ok; ++t, ++c) {
+        const int sl = c & 1;
+        const uint32_t par = (c >> 1) & 1, sp = c & 1;  // slot parity; parity of this step's S and P
+        const bool two = 2 * t + 1 < nt;
+        ok = mbar_wait(bar_v_full + sl, par, a.status);
+        if (!ok) break;
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          if (t == 0 && ni > 0) {
+            ok = mbar_wait(bar_o_empty + x, (ni - 1) & 1, a.status);
+            if (!ok) break;
+          }
+          ok = mbar_wait(bar_p + 2 * x, sp, a.status);
+          if (!ok) break;
+          tc_fence_after();
+          const uint64_t dB = dV0 + sl * kKV16;
+          if (lead) {
+#pragma unroll
+            for (int kk = 0; kk < 2 * kSplitQ + 2; ++kk)
+                mma_ts(tb + cO + x * 128, tb + x * 128 + kk * 8, dB + ((kk * 2048) >> 4), IDESC_O, (t > 0 || kk > 0) ? 1u : 0u);
+          }
+          ok = mbar_wait(bar_p + 2 * x + 1, sp, a.status);
+          if (!ok) break;
+          tc_fence_after();
+          if (lead) {
+            if (two) {
+#pragma unroll
+              for (int kk = 2 * kSplitQ + 2; kk < 8; ++kk)
+                mma_ts(tb + cO + x * 128, tb + x * 128 + kk * 8, dB + ((kk * 2048) >> 4), IDESC_O, 1u);
+            }
+            if (t == n - 1) mma_commit(bar_o_full + x);
+            if (x == 1) mma_commit(bar_v_empty + sl);
+          }
+          if (t + 1 < n) {
+            if (x == 0) {
+              ok = mbar_wait(bar_k_full + (sl ^ 1), ((c + 1) >> 1) & 1, a.status);
+              if (!ok) break;
+              tc_fence_after();
+            }
+            issue_s(x, t + 1, sl ^ 1);
+          }
+        }
+      }
+    }
+   }
+  } else {
+    setmaxnreg_inc<208>();
+    // ======================= softmax: one query row per thread =======================
+    const int x = warp >> 2;                                              // head of the pair
+    const int r = tid & 127;                                              // row of the tile = TMEM lane
+    const uint32_t t_lane = tb + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t t_S = t_lane + x * 128, t_O = t_lane + cO + x * 128;
+    const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
+    uint8_t* stage = sOut + x * SM::kOut;
+    bool stored = false;  // (first thread) a bulk store from `stage` may still be reading it
+    int c = 0;
+    uint32_t ni = 0;
+    PairItem it;
+    for (; ok && !(SPLIT && ni > 0) && next_item(ni, it); ++ni) {
+      const int n = (it.nt + 1) >> 1, q0 = it.q0, off = it.off, Nk = it.Nk;
+      const int row = q0 + r;
+      const bool row_valid = row < it.Nq;
+      const int rowpos = row + off;  // position of this query on the key axis
+      float m_ref = -INFINITY, l_sum = 0.f;
+
+      // The two tiles of step t (the second one only if `two`), and whether both need no mask; straight-line code, so
+      // that it overlaps with the exponentials of the step before.
+      const int n0 = cowa_range_len(it.rg[0]), n1 = n0 + cowa_range_len(it.rg[1]);
+      struct Step { int ja, jb; bool two, full; } cur;
+      auto step_at = [&](int t) {
+        auto at = [&](int u, bool* full) {
+          const int j = u < n0 ? it.rg[0].hi - u : u < n1 ? it.rg[1].hi + n0 - u : it.rg[2].hi + n1 - u;
+          const int lo = u < n0 ? it.f_lo[0] : u < n1 ? it.f_lo[1] : it.f_lo[2];
+          const int hi = u < n0 ? it.f_hi[0] : u < n1 ? it.f_hi[1] : it.f_hi[2];
+          *full = j >= lo && j <= hi;
+          return j;
+        };
+        Step st;
+        bool fa, fb;
+        st.ja = at(it.t0 + 2 * t, &fa);
+        st.jb = at(it.t0 + 2 * t + 1, &fb);
+        st.two = 2 * t + 1 < it.nt;
+        st.full = fa && fb && st.two;
+        return st;
+      };
+      Step nxt = step_at(0);
+
+      for (int t = 0; t < n && ok; ++t, ++c) {
+        cur = nxt;
+        const int ja = cur.ja, jb = cur.jb;
+        const bool two = cur.two;
+        ok = mbar_wait(bar_s + x, c & 1, a.status);
+        if (!ok) break;
+        tc_fence_after();
+        uint32_t sr[4][32];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) tmem_ld32(t_S + q * 32, sr[q]);
+        tmem_wait_ld();
+
+        // Boundary steps: each warp looks at its 32 rows x 32 keys; most such squares are all legal.
+        if (__builtin_expect(!cur.full, 0)) {
+          const CowaWin w = it.w;
+          const int kend = row_valid ? min(rowpos, Nk - 1) : -1;  // last causal key of this row
+          const int near_lo = rowpos - w.n + 1, sink_hi = min(w.s - 1, kend);
+          const int long_hi = w.l > 0 ? min(rowpos - (w.n + w.g), kend) : -1, long_lo = rowpos - (w.n + w.g + w.l) + 1;
+          uint32_t mk[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int base = (q < 2 ? ja : jb) * BK + (q & 1) * 32;
+            mk[q] = interval_bits(near_lo, kend, base) | interval_bits(0, sink_hi, base) | interval_bits(long_lo, long_hi, base);
+            if (q >= 2 && !two) mk[q] = 0u;
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (__any_sync(0xFFFFFFFFu, mk[q] != 0xFFFFFFFFu)) {
+#pragma unroll
+              for (int e = 0; e < 32; ++e)
+                if (!((mk[q] >> e) & 1u)) sr[q][e] = 0xFF800000u;  // -inf
+            }
+        }
+        float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int e = 0; e < 32; e += 2)
+            mxa[(e >> 1) & 3] = max3(mxa[(e >> 1) & 3], __uint_as_float(sr[q][e]), __uint_as_float(sr[q][e + 1]));
+        const float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3])) * a.scale_log2;
+        // The reference moves rarely: the row sum, and the accumulator of a warp with such a row, are rescaled then.
+        const bool moved = mx > m_ref + 8.f;
+        if (__builtin_expect(__any_sync(0xFFFFFFFFu, moved), 0)) {
+          const float alpha = moved ? ex2(m_ref - mx) : 1.f;
+          if (moved) m_ref = mx;
+          l_sum *= alpha;
+          const float2 al2 = make_float2(alpha, alpha);
+#pragma unroll 1
+          for (int q = 0; q < (t > 0 ? D / 16 : 0); ++q) {
+            uint32_t ov[16];
+            tmem_ld16(t_O + q * 16, ov);
+            tmem_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 16; e += 2) {
+              const float2 y = mul2(make_float2(__uint_as_float(ov[e]), __uint_as_float(ov[e + 1])), al2);
+              ov[e] = __float_as_uint(y.x); ov[e + 1] = __float_as_uint(y.y);
+            }
+            tmem_st16(t_O + q * 16, ov);
+          }
+        }
+
+        if constexpr (VARLEN) {
+          // rows after the sequence's last key belong to the next sequence: P is exactly zero there, but
+          // 0 x (Inf or NaN) would poison this one, so those V rows are cleared before the product may start
+          // (both heads' warps write the same zeros; the slot is released only after both heads' products)
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            const int vrows = Nk - (hf ? jb : ja) * BK;
+            if (vrows < BK && (hf == 0 || two)) {
+              ok = mbar_wait(bar_v_full + (c & 1), (c >> 1) & 1, a.status);
+              if (!ok) break;
+              uint8_t* vt = sV + (c & 1) * SM::kKV + hf * (SLAB / 2);
+              const int nchunk = (BK - vrows) * 8;  // 16-byte chunks per slab
+              for (int s_ = 0; s_ < NSLAB; ++s_)
+                for (int c_ = r; c_ < nchunk; c_ += 128)
+                  *reinterpret_cast<uint4*>(vt + s_ * SLAB + vrows * 128 + c_ * 16) = make_uint4(0u, 0u, 0u, 0u);
+              fence_proxy_async_smem();
+            }
+          }
+          if (!ok) break;
+        }
+
+        // p = 2^(s * scale - m): packed fp32 pairs for the multiply-add and the row sum
+        const float sub = (m_ref == -INFINITY) ? 0.f : m_ref;
+        const float2 nsub2 = make_float2(-sub, -sub);
+        float2 rsa[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        nxt = step_at(t + 1);
+        // The exponentials of a 32-key group are issued between the sums and conversions of the group before it, so
+        // that the special-function unit does not wait for them.
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+          uint32_t pk[16];
+#pragma unroll
+          for (int e = 0; e < 32; e += 2) {
+            if (q < 4) {
+              const float2 y = fma2(make_float2(__uint_as_float(sr[q & 3][e]), __uint_as_float(sr[q & 3][e + 1])), sc2, nsub2);
+              const float2 z = e % 16 == 0 ? exp2_fma(y) : make_float2(ex2(y.x), ex2(y.y));
+              sr[q & 3][e] = __float_as_uint(z.x);
+              sr[q & 3][e + 1] = __float_as_uint(z.y);
+            }
+            if (q > 0) {
+              const float2 pp = make_float2(__uint_as_float(sr[(q - 1) & 3][e]), __uint_as_float(sr[(q - 1) & 3][e + 1]));
+              rsa[(e >> 1) & 3] = add2(rsa[(e >> 1) & 3], pp);
+              pk[e / 2] = pack_bf16(pp.x, pp.y);
+            }
+          }
+          if (q > 0) tmem_st16(t_S + (q - 1) * 16, pk);
+          if (q - 1 == kSplitQ) {  // the first half of P is in place
+            tmem_wait_st();
+            tc_fence_before();
+            warp_arrive(bar_p + 2 * x);
+          }
+        }
+        const float2 rs2 = add2(add2(rsa[0], rsa[1]), add2(rsa[2], rsa[3]));
+        l_sum += rs2.x + rs2.y;
+        tmem_wait_st();
+        tc_fence_before();
+        warp_arrive(bar_p + 2 * x + 1);
+      }
+      if (!ok) break;
+
+      // ---- epilogue: O / l, LSE ----
+      ok = mbar_wait(bar_o_full + x, ni & 1, a.status);
+      if (!ok) break;
+      if constexpr (SPLIT) {
+        // fp32 O goes where K and V were, once both heads' products have read them; the row's state where Q was
+        ok = mbar_wait(bar_o_full + (x ^ 1), ni & 1, a.status);
+        if (!ok) break;
+        tc_fence_after();
+        uint8_t* orow = sK + (x * BQ + r) * (D * 4);
+#pragma unroll
+        for (int q = 0; q < D / 32; ++q) {
+          uint32_t ov[32];
+          tmem_ld32(t_O + q * 32, ov);
+          tmem_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            *reinterpret_cast<uint4*>(orow + (((q * 8 + e) ^ (r & 7)) << 4)) =
+                make_uint4(ov[e * 4], ov[e * 4 + 1], ov[e * 4 + 2], ov[e * 4 + 3]);
+        }
+        reinterpret_cast<float2*>(sQ)[x * BQ + r] = make_float2(m_ref, l_sum);
+        continue;
+      }
+      tc_fence_after();
+      const float inv = l_sum > 0.f ? 1.f / l_sum : 0.f;
+      uint32_t ob[D / 2];
+#pragma unroll
+      for (int q = 0; q < D / 32; ++q) {
+        uint32_t ov[32];
+        tmem_ld32(t_O + q * 32, ov);
+        tmem_wait_ld();
+#pragma unroll
+        for (int e = 0; e < 32; e += 2)
+          ob[q * 16 + e / 2] = pack_bf16(__uint_as_float(ov[e]) * inv, __uint_as_float(ov[e + 1]) * inv);
+      }
+      tc_fence_before();
+      warp_arrive(bar_o_empty + x);
+      const int h = it.h0 + x;
+      if (row_valid) {
+        const size_t li = VARLEN ? (size_t)h * a.total_q + it.qbase + row : ((size_t)it.b * a.Hq + h) * it.Nq + row;
+        a.lse[li] = 0.6931471805599453f * (m_ref + log2f(l_sum));
+      }
+      if (VARLEN && q0 + BQ > it.Nq) {  // written row by row: the rows after the sequence's last belong to another one
+        if (row_valid) {
+          uint4* dst = reinterpret_cast<uint4*>(a.o + ((size_t)h * a.total_q + it.qbase + row) * D);
+#pragma unroll
+          for (int q = 0; q < D / 8; ++q) dst[q] = make_uint4(ob[q * 4], ob[q * 4 + 1], ob[q * 4 + 2], ob[q * 4 + 3]);
+        }
+      } else {
+#pragma unroll
+        for (int s = 0; s < NSLAB; ++s) {
+          if (r == 0 && stored) tma_wait_group_read<0>();
+          asm volatile("bar.sync %0, 128;" ::"r"(1 + x) : "memory");
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            *reinterpret_cast<uint4*>(stage + r * 128 + ((q ^ (r & 7)) << 4)) =
+                make_uint4(ob[s * 32 + q * 4], ob[s * 32 + q * 4 + 1], ob[s * 32 + q * 4 + 2], ob[s * 32 + q * 4 + 3]);
+          fence_proxy_async_smem();
+          asm volatile("bar.sync %0, 128;" ::"r"(1 + x) : "memory");
+          if (r == 0) {
+            tma_store_4d(&tmO, stage, s * 64, it.qbase + q0, h, it.bt);
+            tma_commit_group();
+            stored = true;
+          }
+        }
+      }
+    }
+    if (r == 0 && stored) tma_wait_group<0>();
+  }
+
+  if constexpr (SPLIT) {
+    // Merge of the cluster's partial states: block `rank` writes every csize-th part of the 256 rows, a warp a row.
+    const PairItem& it = *reinterpret_cast<const PairItem*>(smem + SM::oItem);
+    const int csize = (int)cluster_size(), rank = (int)cluster_rank(), lane = tid & 31;
+    __syncthreads();
+    if (it.nt == 0 && tid < 2 * BQ) reinterpret_cast<float2*>(sQ)[tid] = make_float2(-INFINITY, 0.f);
+    cluster_sync();
+    if (it.work > 0) {
+      const int per = 2 * BQ / csize, first = rank * per;  // this block's rows of the 2 x 128
+      const uint32_t aState = smem_u32(sQ), aO = smem_u32(sK);
+      float* wgt = reinterpret_cast<float*>(sQ + 4096);    // [per][csize]: share of every block's O in a row
+      if (tid < per) {
+        const int xr = first + tid, row = it.q0 + (xr & (BQ - 1)), h = it.h0 + (xr >> 7);
+        float2 ml[8];
+        float M = -INFINITY, L = 0.f;
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+          if (p < csize) {
+            ml[p] = ld_cluster_f2(map_cluster(aState + xr * 8, p));
+            M = fmaxf(M, ml[p].x);
+          }
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+          if (p < csize) {
+            ml[p].x = ml[p].x == -INFINITY ? 0.f : ex2(ml[p].x - M);
+            L = fmaf(ml[p].y, ml[p].x, L);
+          }
+        const float inv = L > 0.f ? 1.f / L : 0.f;
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+          if (p < csize) wgt[tid * csize + p] = ml[p].x * inv;
+        if (row < it.Nq) {
+          const size_t li = VARLEN ? (size_t)h * a.total_q + it.qbase + row : ((size_t)it.b * a.Hq + h) * it.Nq + row;
+          a.lse[li] = 0.6931471805599453f * (M + log2f(L));
+        }
+      }
+      __syncthreads();
+      constexpr int LPR = D / 4, RPW = 32 / LPR, U = 4;  // lanes per row (16 bytes of fp32 each), rows a warp takes at
+                                                         // once, such groups of rows in flight
+      const int ch = lane % LPR;
+      for (int i0 = warp * RPW * U + lane / LPR; i0 < per; i0 += (kPairThreads / 32) * RPW * U) {
+        float4 o[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) o[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int p = 0; p < csize; ++p) {
+          const uint32_t src = map_cluster(aO, p);
+          float4 v[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int xr = first + min(i0 + u * RPW, per - 1);
+            v[u] = ld_cluster_f4(src + xr * (D * 4) + ((ch ^ (xr & 7)) << 4));
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const float w = wgt[min(i0 + u * RPW, per - 1) * csize + p];
+            if (w > 0.f) {  // a block without a step left no O
+              o[u].x = fmaf(v[u].x, w, o[u].x); o[u].y = fmaf(v[u].y, w, o[u].y);
+              o[u].z = fmaf(v[u].z, w, o[u].z); o[u].w = fmaf(v[u].w, w, o[u].w);
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int i = i0 + u * RPW, xr = first + i, row = it.q0 + (xr & (BQ - 1)), h = it.h0 + (xr >> 7);
+          if (i < per && row < it.Nq) {
+            __nv_bfloat16* dst = a.o + (VARLEN ? ((size_t)h * a.total_q + it.qbase + row) * D
+                                               : (size_t)it.b * a.so.b + (size_t)h * a.so.h + (size_t)row * a.so.t);
+            *reinterpret_cast<uint2*>(dst + ch * 4) = make_uint2(pack_bf16(o[u].x, o[u].y), pack_bf16(o[u].z, o[u].w));
+          }
+        }
+      }
+    }
+    cluster_sync();  // no block leaves while another one reads its shared memory
+  }
+
+  // ---- teardown ----
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 9) {
+    __syncwarp();
+    tmem_dealloc(tb, TMEM_COLS);
+  }
+}
+
+}  // namespace
+
+namespace cowa {
+
+template <int D, bool VARLEN>
+int launch_fwd_pair(const CUtensorMap& mq, const void* k, const void* v, const CUtensorMap& mo, const CowaStrides& sk,
+                    const CowaStrides& sv, const FwdArgs& a, int rows_k, int nb, long long items, int split,
+                    cudaStream_t st) {
+  CUtensorMap mk, mv;
+  int rc;
+  if ((rc = make_tensor_map(&mk, k, MapType::BF16, D, rows_k, a.Hkv, nb, sk, 64, BK))) return rc;
+  if ((rc = make_tensor_map(&mv, v, MapType::BF16, D, rows_k, a.Hkv, nb, sv, 64, BK))) return rc;
+  auto kernel = cowa_fwd_pair_kernel<D, VARLEN, true>;
+  if constexpr (D == 128) {
+    if (split == 1) kernel = cowa_fwd_pair_kernel<D, VARLEN, false>;
+  }
+  COWA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PairSmem<D>::kBytes));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(split > 1 ? items * split : std::min<long long>(items, sm_count())));
+  cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = PairSmem<D>::kBytes; cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = split > 1 ? 1 : 0;
+  COWA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mo, a, (int)items));
+  return COWA_OK;
+}
+
+#define COWA_INSTANTIATE(D, V)                                                                                    \
+  template int launch_fwd_pair<D, V>(const CUtensorMap&, const void*, const void*, const CUtensorMap&,            \
+                                     const CowaStrides&, const CowaStrides&, const FwdArgs&, int, int, long long, \
+                                     int, cudaStream_t);
+COWA_INSTANTIATE(128, false)
+COWA_INSTANTIATE(128, true)
+COWA_INSTANTIATE(64, false)
+COWA_INSTANTIATE(64, true)
+#undef COWA_INSTANTIATE
+
+}  // namespace cowa
