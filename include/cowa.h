@@ -214,10 +214,8 @@ size_t cowa_decode_static_capacity(void);
  * tokens alike.  The paper describes no such variant; the distance rule is unchanged.
  *   q [B,Nq,Hq,D] in; o [B,Nq,Hq,D] bf16 and lse [B,Nq,Hq] fp32 (may be NULL) out;
  *   kcache, vcache [B,Hkv,Tmax,D] already hold the Nq new tokens; lens: DEVICE int32[B], Nq <= lens[b] <= Tmax.
- * 1 <= Nq <= 64; Hq/Hkv in {1,2,4,8}.  Tokens are packed into the 8 columns of the score MMA together with
- * the group's heads: 8/(Hq/Hkv) tokens share one pass over the visible rows, more tokens take more blocks
- * (their re-reads mostly hit in L2; beyond about three such passes cowa_prefill / cowa_prefill_varlen, whose
- * cost does not grow with Nq up to 128, is the faster call).  `workspace`: device, >= cowa_decode_multi_workspace_bytes, 16-byte
+ * 1 <= Nq <= 64; Hq/Hkv in {1,2,4,8}.  The tokens and heads that share a KV head are the rows of one 128-row tile
+ * (more rows take more tiles), so that every visible cache row is read once for up to 128 / (Hq/Hkv) tokens. `workspace`: device, >= cowa_decode_multi_workspace_bytes, 16-byte
  * aligned, no initialisation needed.  cowa_params_t.windows is ignored, as in cowa_decode. */
 int cowa_decode_multi(const void* q, const void* kcache, const void* vcache, const int32_t* lens,
                       void* o, float* lse, int B, int Nq, int Tmax, int Hq, int Hkv, int D,

@@ -44,6 +44,10 @@ int resolve_strides(const int64_t s[3], int H, long long T, int D, CowaStrides* 
 // True when any stride of q, k, v or o is set (for the calls that take contiguous tensors only).
 bool any_stride_set(const cowa_params_t* p);
 
+// Argument checks shared by the decode calls.
+int decode_validate(const void* q, const void* kc, const void* vc, const int32_t* lens, const void* o, int B, int Tmax,
+                    int Hq, int Hkv, int D, const cowa_params_t* p);
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace cowa

@@ -61,11 +61,6 @@ struct DecodeArgs {
   CowaStrides sk, sv;  // element strides (batch, head, token) of the contiguous-row cache
   int sink, near, hkv_global, hkv_offset, full_attn;
   float scale_log2;
-  // extended kernel only: several newest tokens per sequence and / or a paged cache
-  const int32_t* block_table;  // [B, max_pages] page of every page_size-row stretch of a sequence, or nullptr
-  int NQ;                      // query tokens per sequence, at key positions lens[b] - NQ .. lens[b] - 1
-  int tpg, ngroups;            // tokens per block (columns = tpg * Hq / Hkv <= 8), blocks per (sequence, KV head)
-  int page_size, max_pages, page_shift;  // page_shift = log2(page_size) when that is a power of two, else -1
 };
 
 // Position of the v-th visible row (v in the concatenation of the head's ranges).
@@ -93,10 +88,8 @@ __device__ __forceinline__ uint4 ldg128(const void* p) {
   return r;
 }
 
-// G = columns of the mma n-tile in use.  Plain kernel (EXT = false): the G query heads of the group, one
-// token.  Extended kernel: (token, head) pairs of up to a.tpg of the a.NQ newest tokens, token-major; every
-// column masks the keys its own token must not see; rows may come from a paged cache.
-template <int D, int G, bool EXT>
+// G = columns of the mma n-tile in use: the query heads of the group.
+template <int D, int G>
 // 5 blocks per SM (up to 102 registers, no spills) measured best: fewer, longer splits than at 7 per SM
 __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const DecodeArgs a) {
   static_assert(D == 64 || D == 128, "head dim");
@@ -110,7 +103,7 @@ __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const De
   // started, its blocks may be scheduled and wait (griddepcontrol.wait) for this grid's results.
   asm volatile("griddepcontrol.launch_dependents;");
   const int split = blockIdx.x, hk = blockIdx.y;
-  const int b = EXT ? blockIdx.z / a.ngroups : blockIdx.z;
+  const int b = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int Nk = a.lens[b];
 
@@ -119,29 +112,11 @@ __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const De
   if (a.full_attn) { w.s = 0; w.n = Nk; w.g = 0; w.l = 0; }
   else w = cowa_default_window(Nk, a.hkv_global, a.hkv_offset + hk, a.sink, a.near);
   CowaRange rg[3];
-  // extended: this block's tokens tq0 .. tq1 sit at key positions Nk - NQ + tq
-  const int gsz = EXT ? a.Hq / a.Hkv : G;
-  const int tq0 = EXT ? (blockIdx.z % a.ngroups) * a.tpg : 0;
-  const int tq1 = EXT ? min(tq0 + a.tpg, a.NQ) - 1 : 0;
-  const int pos0 = EXT ? Nk - a.NQ : Nk - 1;  // key position of token 0
-  const int nr = EXT ? cowa_decode_ranges_span(w, pos0 + tq0, pos0 + tq1, rg) : cowa_decode_ranges(w, Nk, rg);
-  // index of column c in q, o, lse and the split states ([B, NQ, Hq] order)
-  auto col = [&](int c) -> size_t {
-    if constexpr (EXT) return ((size_t)b * a.NQ + tq0 + c / gsz) * a.Hq + (size_t)hk * gsz + c % gsz;
-    else return (size_t)b * a.Hq + (size_t)hk * G + c;
-  };
-  auto col_valid = [&](int c) -> bool { return EXT ? (c < G && tq0 + c / gsz <= tq1) : (c < G); };
+  const int nr = cowa_decode_ranges(w, Nk, rg);
+  // index of column c in q, o, lse and the split states ([B, Hq] order)
+  auto col = [&](int c) -> size_t { return (size_t)b * a.Hq + (size_t)hk * G + c; };
   // address of cache row `tok` of this (sequence, KV head)
   auto row_ptr = [&](const __nv_bfloat16* base, const CowaStrides& cs, int tok) -> const __nv_bfloat16* {
-    if constexpr (EXT) {
-      if (a.block_table) {
-        // page sizes are almost always powers of two: shift and mask instead of a runtime division
-        const int pi = a.page_shift >= 0 ? tok >> a.page_shift : tok / a.page_size;
-        const int po = a.page_shift >= 0 ? tok & (a.page_size - 1) : tok % a.page_size;
-        const int pg = a.block_table[(size_t)b * a.max_pages + pi];
-        return base + (((size_t)pg * a.Hkv + hk) * a.page_size + po) * D;
-      }
-    }
     return base + (size_t)b * cs.b + (size_t)hk * cs.h + (size_t)tok * cs.t;
   };
   VisMap vm;
@@ -158,8 +133,8 @@ __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const De
 
   if (clen <= 0) {  // empty split: neutral partial state
     for (int i = tid; i < G * D; i += kThreads)
-      if (col_valid(i / D)) a.ws_o[(col(i / D) * a.S + split) * D + (i % D)] = 0.f;
-    if (tid < G && col_valid(tid)) {
+      a.ws_o[(col(i / D) * a.S + split) * D + (i % D)] = 0.f;
+    if (tid < G) {
       a.ws_m[col(tid) * a.S + split] = -INFINITY;
       a.ws_l[col(tid) * a.S + split] = 0.f;
     }
@@ -174,7 +149,7 @@ __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const De
 #pragma unroll
     for (int cc = 0; cc < KC; ++cc) {
       uint4 x = make_uint4(0, 0, 0, 0);
-      if (col_valid(g)) x = *reinterpret_cast<const uint4*>(a.q + col(g) * D + cc * 32 + t * 8);
+      if (g < G) x = *reinterpret_cast<const uint4*>(a.q + col(g) * D + cc * 32 + t * 8);
       bq[cc][0] = x.x; bq[cc][1] = x.y; bq[cc][2] = x.z; bq[cc][3] = x.w;
     }
     const int nblk = (clen + 15) >> 4;
@@ -195,13 +170,6 @@ __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const De
       }
       // c[0],c[1]: row rA, heads 2t, 2t+1;  c[2],c[3]: row rB
       const int h0 = 2 * t, h1 = 2 * t + 1;
-      if constexpr (EXT) {  // a column only sees what its own token sees (Eq. fwa_support at that token's distance)
-        const int p0_ = pos0 + tq0 + h0 / gsz, p1_ = pos0 + tq0 + h1 / gsz;
-        if (!col_valid(h0) || !cowa_visible(w, p0_ - tokA, tokA)) c[0] = -INFINITY;
-        if (!col_valid(h1) || !cowa_visible(w, p1_ - tokA, tokA)) c[1] = -INFINITY;
-        if (!col_valid(h0) || !cowa_visible(w, p0_ - tokB, tokB)) c[2] = -INFINITY;
-        if (!col_valid(h1) || !cowa_visible(w, p1_ - tokB, tokB)) c[3] = -INFINITY;
-      }
       if (rA < clen) {
         if (h0 < G) sc[h0 * kScStride + rA] = c[0] * a.scale_log2;
         if (h1 < G) sc[h1 * kScStride + rA] = c[1] * a.scale_log2;
@@ -222,9 +190,8 @@ __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const De
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     float l = 0.f;
-    const float msub = (EXT && m == -INFINITY) ? 0.f : m;  // a token that sees none of this split's rows
     for (int r = lane; r < clen; r += 32) {
-      float p = exp2f(s[r] - msub);
+      float p = exp2f(s[r] - m);
       s[r] = p;
       l += p;
     }
@@ -295,9 +262,9 @@ __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const De
     float s = 0.f;
 #pragma unroll
     for (int r = 0; r < kThreads / 32; ++r) s += sc[r * G * D + i];
-    if (col_valid(i / D)) a.ws_o[(col(i / D) * a.S + split) * D + (i % D)] = s;
+    a.ws_o[(col(i / D) * a.S + split) * D + (i % D)] = s;
   }
-  if (tid < G && col_valid(tid)) {
+  if (tid < G) {
     a.ws_m[col(tid) * a.S + split] = m_s[tid];
     a.ws_l[col(tid) * a.S + split] = l_s[tid];
   }
@@ -395,34 +362,33 @@ int max_visible(int Tmax, int hg, const cowa_params_t* p) {
 
 // Blocks of the split kernel that fit the current device at once (SM count x resident blocks per SM).
 // Falls back to 148 x 5 (B200, up to 102 registers per thread) when no device can be queried.
-template <int D, int G, bool EXT>
+template <int D, int G>
 int resident_blocks_of() {
   int dev = 0, sms = 0, occ = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cowa_decode_split_kernel<D, G, EXT>, kThreads, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cowa_decode_split_kernel<D, G>, kThreads, 0) !=
       cudaSuccess)
     return 0;
   return sms * occ;
 }
 
-template <bool EXT>
 int resident_blocks(int D, int G) {
   static int cache[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
   const int di = D == 128 ? 1 : 0, gi = G == 1 ? 0 : G == 2 ? 1 : G == 4 ? 2 : 3;
   if (cache[di][gi] == 0) {
     int r = 0;
-    if (D == 128) r = G == 1 ? resident_blocks_of<128, 1, EXT>() : G == 2 ? resident_blocks_of<128, 2, EXT>()
-                    : G == 4 ? resident_blocks_of<128, 4, EXT>() : resident_blocks_of<128, 8, EXT>();
-    else r = G == 1 ? resident_blocks_of<64, 1, EXT>() : G == 2 ? resident_blocks_of<64, 2, EXT>()
-             : G == 4 ? resident_blocks_of<64, 4, EXT>() : resident_blocks_of<64, 8, EXT>();
+    if (D == 128) r = G == 1 ? resident_blocks_of<128, 1>() : G == 2 ? resident_blocks_of<128, 2>()
+                    : G == 4 ? resident_blocks_of<128, 4>() : resident_blocks_of<128, 8>();
+    else r = G == 1 ? resident_blocks_of<64, 1>() : G == 2 ? resident_blocks_of<64, 2>()
+             : G == 4 ? resident_blocks_of<64, 4>() : resident_blocks_of<64, 8>();
     if (r <= 0) { cudaGetLastError(); return 148 * 5; }
     cache[di][gi] = r;
   }
   return cache[di][gi];
 }
 
-// Splits per (sequence, KV head[, token group]): the grid should be a whole number of waves of resident
+// Splits per (sequence, KV head): the grid should be a whole number of waves of resident
 // blocks, each split at most kChunkCap rows (its scores live in shared memory) and not much shorter than
 // 128 rows.  `vmax` bounds the visible rows of a block, `units` counts the blocks per split index.
 int splits_for(int vmax, int units, int slots) {
@@ -440,23 +406,7 @@ int splits_for(int vmax, int units, int slots) {
 
 int pick_splits(int B, int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p) {
   const int hg = p->hkv_global > 0 ? p->hkv_global : Hkv;
-  return splits_for(max_visible(Tmax, hg, p), B * Hkv, resident_blocks<false>(D, Hq / Hkv));
-}
-
-// Extended kernel: tokens per block and blocks per (sequence, KV head) for NQ tokens and group size gsz.
-void token_groups(int NQ, int gsz, int* tpg, int* ngroups, int* cols) {
-  int t = 1;
-  while (t * 2 * gsz <= 8 && t < NQ) t *= 2;
-  *tpg = t; *ngroups = (NQ + t - 1) / t; *cols = t * gsz;
-}
-
-int pick_splits_ext(int B, int NQ, int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p) {
-  const int hg = p->hkv_global > 0 ? p->hkv_global : Hkv;
-  int tpg, ngroups, cols;
-  token_groups(NQ, Hq / Hkv, &tpg, &ngroups, &cols);
-  long long vmax = (long long)max_visible(Tmax, hg, p) + 3ll * (tpg - 1);  // each range grows by the token span
-  if (vmax > Tmax) vmax = Tmax;
-  return splits_for((int)vmax, B * Hkv * ngroups, resident_blocks<true>(D, cols));
+  return splits_for(max_visible(Tmax, hg, p), B * Hkv, resident_blocks(D, Hq / Hkv));
 }
 
 // Launch of the merge kernel right behind the split kernel, allowed to start before that one has drained.
@@ -472,20 +422,20 @@ cudaError_t launch_combine(unsigned rows, const float* ws_o, const float* ws_m, 
   return cudaLaunchKernelEx(&cfg, cowa_decode_combine_kernel<D>, ws_o, ws_m, ws_l, o, lse, S);
 }
 
-template <int D, int G, bool EXT>
+template <int D, int G>
 cudaError_t launch_split(const DecodeArgs& a, cudaStream_t st) {
-  dim3 grid(a.S, a.Hkv, EXT ? a.B * a.ngroups : a.B);
-  cowa_decode_split_kernel<D, G, EXT><<<grid, kThreads, 0, st>>>(a);
+  dim3 grid(a.S, a.Hkv, a.B);
+  cowa_decode_split_kernel<D, G><<<grid, kThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
-template <int D, bool EXT>
+template <int D>
 cudaError_t dispatch_split(int G, const DecodeArgs& a, cudaStream_t st) {
   switch (G) {
-    case 1: return launch_split<D, 1, EXT>(a, st);
-    case 2: return launch_split<D, 2, EXT>(a, st);
-    case 4: return launch_split<D, 4, EXT>(a, st);
-    case 8: return launch_split<D, 8, EXT>(a, st);
+    case 1: return launch_split<D, 1>(a, st);
+    case 2: return launch_split<D, 2>(a, st);
+    case 4: return launch_split<D, 4>(a, st);
+    case 8: return launch_split<D, 8>(a, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -494,9 +444,8 @@ cudaError_t dispatch_split(int G, const DecodeArgs& a, cudaStream_t st) {
 
 namespace cowa {
 
-// Validates a decode call; on success fills S (number of splits).
-int decode_validate(const void* q, const void* kc, const void* vc, const int32_t* lens, void* o, int B,
-                    int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p, int* S) {
+int decode_validate(const void* q, const void* kc, const void* vc, const int32_t* lens, const void* o, int B,
+                    int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p) {
   if (!q || !kc || !vc || !lens || !o || !p) return COWA_ERR_INVALID_ARG;
   if (B <= 0 || Tmax <= 0 || Hq <= 0 || Hkv <= 0 || Hq % Hkv != 0) return COWA_ERR_INVALID_ARG;
   if (!p->full_attn && (p->sink < 0 || p->local < 1)) return COWA_ERR_INVALID_ARG;
@@ -510,7 +459,6 @@ int decode_validate(const void* q, const void* kc, const void* vc, const int32_t
   if (!aligned16(q) || !aligned16(kc) || !aligned16(vc) || !aligned16(o)) return COWA_ERR_MISALIGNED;
   for (int i = 0; i < 3; ++i)
     if (p->q_strides[i] || p->o_strides[i]) return COWA_ERR_UNSUPPORTED;  // q and o of a decode step are [B, Hq, D]
-  *S = pick_splits(B, Tmax, Hq, Hkv, D, p);
   return COWA_OK;
 }
 
@@ -539,9 +487,8 @@ int decode_launch(const void* q, const void* kc, const void* vc, const int32_t* 
   a.hkv_offset = p->hkv_offset;
   a.full_attn = p->full_attn;
   a.scale_log2 = p->softmax_scale * 1.4426950408889634f;
-  a.block_table = nullptr; a.NQ = 1; a.tpg = 1; a.ngroups = 1; a.page_size = 0; a.max_pages = 0; a.page_shift = -1;
   const int G = Hq / Hkv;
-  cudaError_t e = (D == 128) ? dispatch_split<128, false>(G, a, st) : dispatch_split<64, false>(G, a, st);
+  cudaError_t e = (D == 128) ? dispatch_split<128>(G, a, st) : dispatch_split<64>(G, a, st);
   if (e != cudaSuccess) return record_cuda_error(e);
   e = (D == 128) ? launch_combine<128>((unsigned)(B * Hq), a.ws_o, a.ws_m, a.ws_l, static_cast<__nv_bfloat16*>(o), lse, S, st)
                  : launch_combine<64>((unsigned)(B * Hq), a.ws_o, a.ws_m, a.ws_l, static_cast<__nv_bfloat16*>(o), lse, S, st);
@@ -549,85 +496,9 @@ int decode_launch(const void* q, const void* kc, const void* vc, const int32_t* 
   return COWA_OK;
 }
 
-// Multi-token and / or paged decode: q, o [B, NQ, Hq, D], lse [B, NQ, Hq]; block_table == nullptr means a
-// contiguous cache [B, Hkv, Tmax, D], otherwise pages [num_pages, Hkv, page_size, D] and Tmax = max_pages * page_size.
-int decode_ext_launch(const void* q, const void* kc, const void* vc, const int32_t* block_table, const int32_t* lens,
-                      void* o, float* lse, int B, int NQ, int Tmax, int page_size, int max_pages, int Hq, int Hkv,
-                      int D, const cowa_params_t* p, int S, void* ws, cudaStream_t st) {
-  DecodeArgs a;
-  a.q = static_cast<const __nv_bfloat16*>(q);
-  a.kc = static_cast<const __nv_bfloat16*>(kc);
-  a.vc = static_cast<const __nv_bfloat16*>(vc);
-  a.lens = lens;
-  const size_t rows = (size_t)B * NQ * Hq;
-  a.ws_o = static_cast<float*>(ws);
-  a.ws_m = a.ws_o + rows * S * D;
-  a.ws_l = a.ws_m + rows * S;
-  a.B = B; a.Tmax = Tmax; a.Hq = Hq; a.Hkv = Hkv; a.S = S;
-  const int64_t none[3] = {0, 0, 0};
-  resolve_strides(none, Hkv, Tmax, D, &a.sk);  // contiguous [B, Hkv, Tmax, D] (paged: rows are addressed through the table)
-  a.sv = a.sk;
-  a.sink = p->sink; a.near = p->local;
-  a.hkv_global = p->hkv_global > 0 ? p->hkv_global : Hkv;
-  a.hkv_offset = p->hkv_offset;
-  a.full_attn = p->full_attn;
-  a.scale_log2 = p->softmax_scale * 1.4426950408889634f;
-  a.block_table = block_table; a.NQ = NQ; a.page_size = page_size; a.max_pages = max_pages;
-  a.page_shift = -1;
-  if (page_size > 0 && (page_size & (page_size - 1)) == 0)
-    for (int sft = 0; sft < 31; ++sft)
-      if ((1 << sft) == page_size) a.page_shift = sft;
-  int cols;
-  token_groups(NQ, Hq / Hkv, &a.tpg, &a.ngroups, &cols);
-  cudaError_t e = (D == 128) ? dispatch_split<128, true>(cols, a, st) : dispatch_split<64, true>(cols, a, st);
-  if (e != cudaSuccess) return record_cuda_error(e);
-  e = (D == 128) ? launch_combine<128>((unsigned)rows, a.ws_o, a.ws_m, a.ws_l, static_cast<__nv_bfloat16*>(o), lse, S, st)
-                 : launch_combine<64>((unsigned)rows, a.ws_o, a.ws_m, a.ws_l, static_cast<__nv_bfloat16*>(o), lse, S, st);
-  if (e != cudaSuccess) return record_cuda_error(e);
-  return COWA_OK;
-}
-
 }  // namespace cowa
 
 extern "C" {
-
-size_t cowa_decode_multi_workspace_bytes(int B, int Nq, int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p) {
-  if (!p || B <= 0 || Nq <= 0 || Tmax <= 0 || Hq <= 0 || Hkv <= 0 || Hq % Hkv != 0 || (D != 64 && D != 128)) return 0;
-  return cowa::decode_ws_bytes(B * Nq, Hq, D, pick_splits_ext(B, Nq, Tmax, Hq, Hkv, D, p));
-}
-
-static int decode_ext(const void* q, const void* kc, const void* vc, const int32_t* block_table, const int32_t* lens,
-                      void* o, float* lse, int B, int Nq, int Tmax, int page_size, int max_pages, int Hq, int Hkv,
-                      int D, const cowa_params_t* p, void* workspace, size_t workspace_bytes, void* stream) {
-  int S = 0;
-  int st = cowa::decode_validate(q, kc, vc, lens, o, B, Tmax, Hq, Hkv, D, p, &S);
-  if (st != COWA_OK) return st;
-  if (Nq <= 0 || Nq > 64 || !workspace) return COWA_ERR_INVALID_ARG;
-  if (cowa::any_stride_set(p)) return COWA_ERR_UNSUPPORTED;
-  if ((long long)B * ((Nq + 7) / 8 * 8) > 65535) return COWA_ERR_UNSUPPORTED;
-  if (!cowa::aligned16(workspace)) return COWA_ERR_MISALIGNED;
-  S = pick_splits_ext(B, Nq, Tmax, Hq, Hkv, D, p);
-  if (workspace_bytes < cowa::decode_ws_bytes(B * Nq, Hq, D, S)) return COWA_ERR_WORKSPACE_TOO_SMALL;
-  return cowa::decode_ext_launch(q, kc, vc, block_table, lens, o, lse, B, Nq, Tmax, page_size, max_pages, Hq, Hkv, D,
-                                 p, S, workspace, static_cast<cudaStream_t>(stream));
-}
-
-int cowa_decode_multi(const void* q, const void* kcache, const void* vcache, const int32_t* lens, void* o,
-                      float* lse, int B, int Nq, int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p,
-                      void* workspace, size_t workspace_bytes, void* stream) {
-  return decode_ext(q, kcache, vcache, nullptr, lens, o, lse, B, Nq, Tmax, 0, 0, Hq, Hkv, D, p, workspace,
-                    workspace_bytes, stream);
-}
-
-int cowa_decode_paged(const void* q, const void* kpages, const void* vpages, const int32_t* block_table,
-                      const int32_t* lens, void* o, float* lse, int B, int Nq, int max_pages, int page_size,
-                      int Hq, int Hkv, int D, const cowa_params_t* p, void* workspace, size_t workspace_bytes,
-                      void* stream) {
-  if (!block_table || max_pages <= 0 || page_size <= 0 || page_size % 16 != 0) return COWA_ERR_INVALID_ARG;
-  if ((long long)max_pages * page_size > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
-  return decode_ext(q, kpages, vpages, block_table, lens, o, lse, B, Nq, max_pages * page_size, page_size, max_pages,
-                    Hq, Hkv, D, p, workspace, workspace_bytes, stream);
-}
 
 size_t cowa_decode_workspace_bytes(int B, int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p) {
   if (!p || B <= 0 || Tmax <= 0 || Hq <= 0 || Hkv <= 0 || Hq % Hkv != 0 || (D != 64 && D != 128)) return 0;
@@ -637,9 +508,9 @@ size_t cowa_decode_workspace_bytes(int B, int Tmax, int Hq, int Hkv, int D, cons
 int cowa_decode(const void* q, const void* kcache, const void* vcache, const int32_t* lens, void* o,
                 float* lse, int B, int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p,
                 void* workspace, size_t workspace_bytes, void* stream) {
-  int S = 0;
-  int st = cowa::decode_validate(q, kcache, vcache, lens, o, B, Tmax, Hq, Hkv, D, p, &S);
+  int st = cowa::decode_validate(q, kcache, vcache, lens, o, B, Tmax, Hq, Hkv, D, p);
   if (st != COWA_OK) return st;
+  const int S = pick_splits(B, Tmax, Hq, Hkv, D, p);
   if (!workspace) return COWA_ERR_INVALID_ARG;
   if (!cowa::aligned16(workspace)) return COWA_ERR_MISALIGNED;
   if (workspace_bytes < cowa::decode_ws_bytes(B, Hq, D, S)) return COWA_ERR_WORKSPACE_TOO_SMALL;
@@ -652,9 +523,9 @@ size_t cowa_decode_static_capacity(void) { return kStaticScratchBytes; }
 int cowa_decode_static(const void* q, const void* kcache, const void* vcache, const int32_t* lens, void* o,
                        float* lse, int B, int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p,
                        void* stream) {
-  int S = 0;
-  int st = cowa::decode_validate(q, kcache, vcache, lens, o, B, Tmax, Hq, Hkv, D, p, &S);
+  int st = cowa::decode_validate(q, kcache, vcache, lens, o, B, Tmax, Hq, Hkv, D, p);
   if (st != COWA_OK) return st;
+  const int S = pick_splits(B, Tmax, Hq, Hkv, D, p);
   if (cowa::decode_ws_bytes(B, Hq, D, S) > kStaticScratchBytes) return COWA_ERR_STATIC_SCRATCH_EXCEEDED;
   cudaError_t e = cudaSuccess;
   void* scratch = static_scratch_ptr(&e);

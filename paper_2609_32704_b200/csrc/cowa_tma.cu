@@ -22,7 +22,7 @@ EncodeTiledFn encode_fn() {
 }  // namespace
 
 int make_tensor_map(CUtensorMap* map, const void* base, MapType type, int D, long long T, int H, int B,
-                    const CowaStrides& st, int box_d, int box_t, bool swizzle128) {
+                    const CowaStrides& st, int box_d, int box_t, bool swizzle128, int box_h) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return record_cuda_error(cudaErrorNotSupported);
   const size_t es = type == MapType::BF16 ? 2 : 4;
@@ -32,7 +32,7 @@ int make_tensor_map(CUtensorMap* map, const void* base, MapType type, int D, lon
   cuuint64_t strides[3] = {(cuuint64_t)st.t * es, (cuuint64_t)st.h * es, (cuuint64_t)st.b * es};
   for (cuuint64_t& x : strides)
     if (x == 0) x = row;
-  cuuint32_t box[4] = {(cuuint32_t)box_d, (cuuint32_t)box_t, 1, 1};
+  cuuint32_t box[4] = {(cuuint32_t)box_d, (cuuint32_t)box_t, (cuuint32_t)box_h, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
   const CUtensorMapDataType dt = type == MapType::BF16  ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
                                  : type == MapType::F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32

@@ -1,0 +1,102 @@
+"""Sizes at which the two-head forward kernel, its cluster-shared form and the tile decode kernel can go wrong: edges of
+128-row tiles, odd numbers of 64-key tiles, the cluster sizes, several row tiles per KV head, many pieces per unit.
+Tolerances are those of the parity tests."""
+import numpy as np
+import pytest
+import torch
+
+import cowa_inputs
+import paper_2609_32704_b200 as cowa
+from oracle import cowa_oracle as orc
+from test_gpu_parity import TOL_LSE, check, multi_case, _packed_inputs, _run_varlen
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _prefill(B, Nq, Nk, Hq, Hkv, D, sink, local, token_major=False, rows=None):
+    q, _, _, _ = cowa_inputs.make_train_inputs(91, B, Nq, Hq, Hkv, D)
+    _, k, v, _ = cowa_inputs.make_train_inputs(92, B, Nk, Hq, Hkv, D)
+    scale = cowa_inputs.softmax_scale(D)
+    params = cowa.make_params(sink=sink, local=local, softmax_scale=scale)
+    put = lambda x: x.to(DEV)  # noqa: E731
+    if token_major:
+        put = lambda x: x.transpose(1, 2).contiguous().to(DEV).transpose(1, 2)  # noqa: E731
+    qd = put(q)
+    o = torch.full_like(qd, float("nan"))
+    lse = torch.full((B, Hq, Nq), float("nan"), dtype=torch.float32, device=DEV)
+    cowa.cowa_prefill(qd, put(k), put(v), o, lse, params)
+    torch.cuda.synchronize()
+    cowa.cowa_check_device_status()
+    assert torch.isfinite(o).all() and torch.isfinite(lse).all()
+    ws = orc.default_windows(Nk, Hkv, sink, local)
+    f = cowa_inputs.to_f64
+    rows = np.arange(Nq) if rows is None else np.asarray(rows)
+    for b in range(B):
+        for h in range(0, Hq, max(1, Hq // 4)):
+            o_ref, lse_ref = orc.forward_rows(f(q[b]), f(k[b]), f(v[b]), ws, scale, h, rows)
+            check(f"lse[{b},{h}]", lse[b, h].cpu().numpy()[rows], lse_ref, TOL_LSE, TOL_LSE)
+            check(f"o[{b},{h}]", o[b, h].float().cpu().numpy()[rows], o_ref)
+
+
+@pytest.mark.parametrize("B,Nq,Nk,Hq,Hkv,D,sink,local", [
+    (1, 130, 6000, 4, 2, 128, 64, 700),    # clusters of 8, last tile of two rows
+    (1, 1, 9000, 2, 1, 128, 0, 64),        # one query, one item
+    (2, 128, 3000, 8, 2, 128, 130, 333),   # clusters of 4
+    (2, 300, 2999, 32, 8, 128, 5, 1500),   # more than half an item per SM: one block per item
+    (1, 257, 7000, 8, 4, 64, 64, 500),     # the shared form at D = 64
+])
+def test_few_items(B, Nq, Nk, Hq, Hkv, D, sink, local):
+    _prefill(B, Nq, Nk, Hq, Hkv, D, sink, local)
+
+
+def test_few_items_token_major():
+    _prefill(2, 200, 4000, 8, 2, 128, 64, 500, token_major=True)
+
+
+@pytest.mark.parametrize("Nq,Nk,sink,local", [
+    (4000, 4000, 64, 64),      # short lists, odd and even numbers of key tiles, several items per block
+    (3969, 4100, 0, 1),        # near window of one key, last tile of one row
+    (2560, 2560, 200, 2000),   # every tile of the longest list visited
+])
+def test_many_items(Nq, Nk, sink, local):
+    n = Nq - 1
+    _prefill(2, Nq, Nk, 32, 8, 128, sink, local, rows=[0, 1, 63, 64, 127, 128, 129, n // 2, n - 128, n - 1, n])
+
+
+@pytest.mark.parametrize("seqs,Hq,Hkv,D", [
+    ([(300, 5000), (1, 700), (129, 9000)], 4, 2, 128),                       # clusters share the items of a packed batch
+    ([(1900, 1900), (64, 64), (2000, 2500), (1, 3000), (127, 127)], 32, 8, 128),  # one block per item
+])
+@pytest.mark.parametrize("bad", [None, float("nan"), float("inf")])
+def test_packed(seqs, Hq, Hkv, D, bad):
+    """Packed batches against the oracle; with `bad`, one sequence is filled with it and the others must not notice."""
+    q, k, v, cu_q, cu_k = _packed_inputs(93, seqs, Hq, Hkv, D)
+    scale = cowa_inputs.softmax_scale(D)
+    params = cowa.make_params(sink=20, local=900, softmax_scale=scale)
+    if bad is not None:
+        k[:, cu_k[1]:cu_k[2]] = bad
+        v[:, cu_k[1]:cu_k[2]] = bad
+    o, lse = _run_varlen(q, k, v, cu_q, cu_k, params)
+    cowa.cowa_check_device_status()
+    f = cowa_inputs.to_f64
+    for b, (nq, nk) in enumerate(seqs):
+        if bad is not None and b == 1:
+            continue
+        qs, ks = slice(cu_q[b], cu_q[b + 1]), slice(cu_k[b], cu_k[b + 1])
+        ws = orc.default_windows(nk, Hkv, 20, 900)
+        for h in (0, Hq - 1):
+            o_ref, lse_ref = orc.forward_rows(f(q[:, qs]), f(k[:, ks]), f(v[:, ks]), ws, scale, h, np.arange(nq))
+            check(f"lse[{b},{h}]", lse[h, qs].cpu().numpy(), lse_ref, TOL_LSE, TOL_LSE)
+            check(f"o[{b},{h}]", o[h, qs].float().cpu().numpy(), o_ref)
+
+
+@pytest.mark.parametrize("B,Nq,Tmax,Hq,Hkv,D,sink,local,lens,page", [
+    (1, 20, 3000, 8, 2, 128, 16, 100, [2999], None),      # 80 of 128 rows
+    (2, 40, 2500, 16, 2, 128, 64, 300, [2500, 40], 64),   # three row tiles, the last half full; len = Nq
+    (1, 64, 1500, 8, 8, 64, 0, 33, [1500], None),         # one head per group
+    (1, 1, 30000, 2, 1, 64, 4, 64, [29999], 16),          # one unit over every block: hundreds of pieces
+    (5, 3, 700, 8, 4, 128, 16, 64, [700, 3, 64, 65, 333], 80),  # lengths around one key tile, odd page size
+])
+def test_decode_tiles(B, Nq, Tmax, Hq, Hkv, D, sink, local, lens, page):
+    multi_case(B, Nq, Tmax, Hq, Hkv, D, sink, local, lens, page_size=page)
