@@ -1,9 +1,9 @@
 // CoWindow Attention backward (Algorithm 2) for sm_100a.
 //
-// Three launches on the caller's stream:
-//   1. preprocess   Delta = rowsum(O * dO) (Algorithm 2 line 13) and LSE * log2(e), fp32 row vectors
-//                   padded to a multiple of 64 rows (padding: LSE = +inf, so that P = 0 there);
-//                   the fp32 dQ accumulator is zeroed by a memset before it.
+// Three launches on the caller's stream, four when some KV tiles are shared:
+//   1. preprocess   -Delta = -rowsum(O * dO) (Algorithm 2 line 13) and -LSE * log2(e), fp32 row vectors
+//                   padded to a multiple of 64 rows (padding: -inf, so that P = 0 there);
+//                   its threads also zero the fp32 dQ accumulator.
 //   2. main kernel  one thread block per (batch, KV head, 128-row KV tile), KV-stationary as in
 //                   Algorithm 2, looping over the G QO heads of the group and over the 64-row QO
 //                   tiles of I_h(j) (analytic scheduler, ascending).  Per step five tcgen05 MMAs:
@@ -25,9 +25,9 @@
 //                   dQ rows at nearly the same time and the reductions hit in L2.
 //   3. convert      dQ accumulator (already scaled) -> bf16.
 // Two variations of the main kernel's work split:
-//   - `parts` > 1: the G heads of a group are spread over several blocks per KV tile (few tiles, or sink
-//     tiles that would be the critical path); each block writes fp32 partial dK, dV to its own slot and a
-//     fourth kernel adds the slots in order (bwd_parts, cowa_bwd_reduce_dkv_kernel).
+//   - shared tiles: a tile's steps are cut into contiguous parts for several blocks (few tiles, sink tiles that would
+//     be the critical path, the last wave); each block writes fp32 partial dK, dV to its own slot and a
+//     fourth kernel adds the slots in order (BwdPlan).
 //   - VARLEN: packed batch [H, total, D]; a block finds (sequence, KV tile) by a warp scan of the offsets,
 //     windows follow from the sequence's own length, the accumulator and the row vectors use a row space
 //     in which every sequence is padded to 64 rows, and a sequence's last, partial KV tile is stored row
@@ -51,15 +51,17 @@ constexpr int NST = 3;    // Q / dO stages
 constexpr float kDqFixedOne = 262144.f;  // 2^18: one unit of dQ in the fixed-point accumulation mode
 
 struct BwdArgs {
-  const float* lse2;   // [B*Hq, Tpad]  LSE * log2(e)
-  const float* delta;  // [B*Hq, Tpad]
+  const float* lse2;   // [B*Hq, Tpad]  -LSE * log2(e)   (both negated: the packed adds have no operand negation)
+  const float* delta;  // [B*Hq, Tpad]  -Delta
   float* dq_acc;       // [B*Hq, Tpad, D] fp32
   unsigned int* status;
   int B, Nq, Nk, Hq, Hkv, G, Tpad;
   int sink_tiles;      // KV tiles per head that hold sink columns (launched first)
+  // The KV tiles in launch order: sink tiles, body, tail.  A tile of class c is shared by cls_parts[c] blocks, each with
+  // a contiguous part of the tile's steps (QO heads x QO tiles); a shared tile's blocks leave fp32 partial dK, dV.
+  int cls_tiles[3], cls_parts[3];
   int dq_fixed;        // 1: dQ partial sums travel as 32-bit fixed point (order-independent addition)
-  int parts;           // blocks per KV tile: each takes G / parts heads of the group (1: the whole group)
-  float* dkv_part;     // parts > 1: fp32 partial dK, dV [B*Hkv, nKV, parts, 2, BKV, D], summed by a last kernel
+  float* dkv_part;     // fp32 partial dK, dV [blocks of shared tiles, 2, BKV, D], summed by a kernel of their own
   // packed (variable-length) batches only: tensors are [H, total, D], sequence b owns rows cu[b] .. cu[b+1]
   const int* cu;       // [B+1] device
   __nv_bfloat16* dk;   // raw outputs for the last, partial KV tile of a sequence
@@ -91,12 +93,47 @@ __device__ __forceinline__ void bulk_load_1d(void* dst, const void* src, uint32_
                : "memory");
 }
 
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes)
+               : "memory");
+}
+
 __device__ __forceinline__ uint32_t interval_bits32(long long a, long long b, long long base) {
   long long lo = a - base, hi = b - base;
   if (lo < 0) lo = 0;
   if (hi > 31) hi = 31;
   if (lo > hi) return 0u;
   return (0xFFFFFFFFu >> (31 - (int)(hi - lo))) << (int)lo;
+}
+
+// Tile number q of class c: sink tiles of every head first (they meet every query tile of their sequence and are the
+// longest), then head-major with ascending KV tile (consecutive blocks share dQ rows, which then stay in L2).  Packed
+// batches: whole warps only; false when there is no such tile (the count is an upper bound).
+struct TileAt {
+  int hk, b, j, nts, pbase;
+};
+template <bool VARLEN>
+__device__ __forceinline__ bool locate_tile(const BwdArgs& a, int c, int q, TileAt& x) {
+  const int nsk = a.sink_tiles, nhead = a.B * a.Hkv;
+  x.pbase = 0;
+  if (c == 0) {
+    x.j = q / nhead; q %= nhead;
+    x.hk = q % a.Hkv; x.b = q / a.Hkv;
+    if constexpr (VARLEN) {
+      varlen_seq_info(a.cu, x.b, BKV, BQS, &x.nts, &x.pbase);
+      return x.j < x.nts;  // else the sequence is shorter than its sink
+    }
+    return true;
+  }
+  if (c == 2) q += a.cls_tiles[1];
+  if constexpr (VARLEN) {
+    x.hk = q / a.tiles_bound;
+    return varlen_locate(a.cu, a.B, q % a.tiles_bound, BKV, BQS, &x.b, &x.j, &x.nts, &x.pbase, nsk);
+  }
+  const int nrest = (a.Nk + BKV - 1) / BKV - nsk;
+  x.j = nsk + q % nrest; q /= nrest;
+  x.hk = q % a.Hkv; x.b = q / a.Hkv;
+  return true;
 }
 
 // named barrier for one 128-thread warpgroup
@@ -138,51 +175,34 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   uint64_t* bar_dq_free = bars + 11 + 2 * NST;  // [2]    count 128: dQ^T drained
   uint64_t* bar_done = bars + 13 + 2 * NST;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 14 + 2 * NST);
+  float** part_out = reinterpret_cast<float**>(bars + 15 + 2 * NST);  // this block's partial dK, dV (kept here, not in registers)
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform by construction (helps the compiler)
 
-  // ---- work item: sink tiles of every head first, then head-major with ascending KV tile ----
-  int hk, b, j;
-  const int part = VARLEN ? 0 : blockIdx.x % a.parts;
+  // ---- work item ----
+  int cls = 0, idx = blockIdx.x, slot = 0;
+  while (cls < 2 && idx >= a.cls_tiles[cls] * a.cls_parts[cls]) {
+    idx -= a.cls_tiles[cls] * a.cls_parts[cls];
+    if (a.cls_parts[cls] > 1) slot += a.cls_tiles[cls] * a.cls_parts[cls];
+    ++cls;
+  }
+  const int parts = a.cls_parts[cls], part = idx % parts;
+  slot += idx;  // of this block's partial dK, dV when the tile is shared
+  TileAt at;
+  if (!locate_tile<VARLEN>(a, cls, idx / parts, at)) return;
+  const int hk = at.hk, b = at.b, j = at.j, pbase = at.pbase;
   // Sequence geometry.  Packed batches: N_q = N_k = the sequence's length, rows start at cu[b]; the fp32
   // dQ accumulator and the LSE / Delta vectors are laid out with every sequence padded to 64 rows (pbase).
-  int Nq = a.Nq, Nk = a.Nk, rbase = 0, pbase = 0;
-  CowaWin w;
-  if constexpr (!VARLEN) {
-    int idx = blockIdx.x / a.parts;
-    const int nKV = (a.Nk + BKV - 1) / BKV, nsk = a.sink_tiles, nhead = a.B * a.Hkv;
-    if (idx < nsk * nhead) {
-      j = idx / nhead; idx %= nhead;
-    } else {
-      idx -= nsk * nhead;
-      j = nsk + idx % (nKV - nsk); idx /= (nKV - nsk);
-    }
-    hk = idx % a.Hkv; b = idx / a.Hkv;
-    w = a.wins.w[hk];
-  } else {
-    // The sink tiles of every (sequence, head) first (they meet every query tile of their sequence and are
-    // the longest blocks); then head-major: consecutive blocks are consecutive KV tiles of one head (their
-    // dQ rows overlap in L2).
-    const int nsk = a.sink_tiles, nhead = a.B * a.Hkv;
-    int nts;
-    if ((int)blockIdx.x < nsk * nhead) {
-      j = blockIdx.x / nhead;
-      b = (blockIdx.x % nhead) / a.Hkv; hk = blockIdx.x % a.Hkv;
-      varlen_seq_info(a.cu, b, BKV, BQS, &nts, &pbase);
-      if (j >= nts) return;  // the sequence is shorter than its sink
-    } else {
-      const int rest = blockIdx.x - nsk * nhead;
-      hk = rest / a.tiles_bound;
-      if (!varlen_locate(a.cu, a.B, rest % a.tiles_bound, BKV, BQS, &b, &j, &nts, &pbase, nsk)) return;
-    }
+  int Nq = a.Nq, Nk = a.Nk, rbase = 0;
+  CowaWin w = a.wins.w[hk];
+  if constexpr (VARLEN) {
     rbase = a.cu[b];
     Nq = Nk = a.cu[b + 1] - rbase;
     if (rbase < 0 || rbase + Nk > a.total) {  // malformed offsets: report, touch nothing
       if (threadIdx.x == 0) atomicOr(a.status, (unsigned)COWA_DEV_BAD_SEQLENS);
       return;
     }
-    w = a.wins.w[hk];
     if (a.full_attn) { w.s = 0; w.n = Nk; w.g = 0; w.l = 0; }
     else if (!a.explicit_windows) w = cowa_default_window(Nk, a.hkv_global, a.hkv_offset + hk, a.sink, a.local);
   }
@@ -191,16 +211,17 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   CowaRange rg[2];
   cowa_bwd_ranges(w, k0, k1, off, Nq, BQS, rg);
   const int cnt = cowa_range_len(rg[0]) + cowa_range_len(rg[1]);  // QO steps per head
-  const int gs = a.G / a.parts;          // heads of the group handled by this block
-  const int N = cnt * gs;
-  const int bt = VARLEN ? 0 : b;                                                    // batch coordinate of the tensor maps
-  const int bhk = VARLEN ? hk : b * a.Hkv + hk;                                     // (batch, KV head) row of the partial dK, dV slots
-  const int hq0 = hk * a.G + part * gs;                                             // first QO head of this block
-  const int bhq0 = (VARLEN ? 0 : b * a.Hq) + hq0;                                   // ... as a row of lse2 / delta / dq_acc
+  const int n0 = cnt * a.G * part / parts;               // (the host checks that these products fit)
+  const int N = cnt * a.G * (part + 1) / parts - n0;     // this block's steps
+  const int g0 = cnt > 0 ? n0 / cnt : 0, tq0 = n0 - g0 * cnt;  // head of the group and position in I_h(j) of the first
+  const int bt = VARLEN ? 0 : b;                               // batch coordinate of the tensor maps
+  const int hq0 = hk * a.G;                                    // first QO head of the group
+  const int bhq0 = (VARLEN ? 0 : b * a.Hq) + hq0;              // ... as a row of lse2 / delta / dq_acc
   const size_t vec_stride = (size_t)a.Tpad;                                         // rows per head in lse2 / delta / dq_acc
   const bool tail_kv = VARLEN && (k0 + BKV > Nk);  // rows after the tile's last valid one belong to the next sequence
 
   if (tid == 0) {
+    *part_out = parts > 1 ? a.dkv_part + (size_t)slot * 2 * (BKV * D) : nullptr;
     mbar_init(bar_kv, 1);
     for (int s = 0; s < NST; ++s) { mbar_init(bar_ld_full + s, 1); mbar_init(bar_ld_empty + s, 1); }
     for (int s = 0; s < 2; ++s) {
@@ -232,6 +253,37 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     tc_fence_after();
     uint8_t* sOut = sStage + (is_dk ? 0 : SM::kKV);
     const float mul = is_dk ? a.scale : 1.f;
+    if (float* const dst = *part_out) {
+      // A shared tile: this block's part goes out in fp32, one slot per block; a kernel of its own adds the slots in order.
+      // Staged where K, V or the Q / dO stages were, rows with their 16-byte chunks permuted (bank conflicts), and
+      // copied as one range: straight from registers a warp's store touches 32 rows (1019 against 983 thousand clocks of
+      // the whole kernel for one KV head of 20001 tokens).
+      uint8_t* sPart = (is_dk ? sK : sStage) + r * (D * 4);
+#pragma unroll
+      for (int c = 0; c < D / 32; ++c) {
+        uint32_t ov[32];
+        if (N > 0 && ok) {
+          tmem_ld32(t_lane + (is_dk ? cDK : cDV) + c * 32, ov);
+          tmem_wait_ld();
+        } else {
+#pragma unroll
+          for (int e = 0; e < 32; ++e) ov[e] = 0u;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          *reinterpret_cast<float4*>(sPart + (((c * 8 + q) ^ (r & 7)) << 4)) =
+              make_float4(__uint_as_float(ov[q * 4]) * mul, __uint_as_float(ov[q * 4 + 1]) * mul,
+                          __uint_as_float(ov[q * 4 + 2]) * mul, __uint_as_float(ov[q * 4 + 3]) * mul);
+      }
+      fence_proxy_async_smem();
+      wg_sync(is_dk ? 1 : 2);
+      if (r == 0) {
+        bulk_store(dst + (is_dk ? 0 : BKV * D), is_dk ? sK : sStage, BKV * D * 4);
+        tma_commit_group();
+        tma_wait_group<0>();
+      }
+      return;
+    }
     if (tail_kv) {
       // last, partial KV tile of a packed sequence: row by row, straight from registers
       __nv_bfloat16* dst = (is_dk ? a.dk : a.dv) + ((size_t)hk * a.total + rbase + k0 + r) * D;
@@ -256,30 +308,6 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             *reinterpret_cast<uint4*>(dst + c * 32 + q * 8) = v;
           }
         }
-      }
-      return;
-    }
-    if (a.parts > 1) {
-      // The group's heads are spread over several blocks: this block's share goes out in fp32, one slot
-      // per block, and a last kernel adds the slots in a fixed order.
-      const int nKV = (a.Nk + BKV - 1) / BKV;
-      float* dst = a.dkv_part + ((((size_t)bhk * nKV + j) * a.parts + part) * 2 + (is_dk ? 0 : 1)) * (size_t)(BKV * D) +
-                   (size_t)r * D;
-#pragma unroll
-      for (int c = 0; c < D / 32; ++c) {
-        uint32_t ov[32];
-        if (N > 0 && ok) {
-          tmem_ld32(t_lane + (is_dk ? cDK : cDV) + c * 32, ov);
-          tmem_wait_ld();
-        } else {
-#pragma unroll
-          for (int e = 0; e < 32; ++e) ov[e] = 0u;
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          *reinterpret_cast<float4*>(dst + c * 32 + q * 4) =
-              make_float4(__uint_as_float(ov[q * 4]) * mul, __uint_as_float(ov[q * 4 + 1]) * mul,
-                          __uint_as_float(ov[q * 4 + 2]) * mul, __uint_as_float(ov[q * 4 + 3]) * mul);
       }
       return;
     }
@@ -314,10 +342,12 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     }
   };
 
-  // Register budget per role: 128 per thread at launch (512 threads), moved to where the work is.  Each
-  // setmaxnreg sits at the top of its own branch so that the code below it is compiled for that budget.
+  // Register budget per role: 128 per thread at launch (512 threads), 80 + 2 * 160 + 112 = 4 * 128 moved to where the work
+  // is.  Each setmaxnreg sits at the top of its own branch so that the code below it is compiled for that budget.  No
+  // role spills at these: with 64 / 176 / 96 the MMA issuer and the producer did, inside their loops, and the kernel took
+  // 1066 instead of 1015 thousand clocks at 2 x 8K, 7980 instead of 7590 at 32K.
   if (warp < 4) {
-    setmaxnreg_dec<64>();
+    setmaxnreg_dec<80>();
     if (warp == 0) {
       // ================= TMA producer =================
       if (lane == 0 && N > 0) {
@@ -327,7 +357,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           tma_load_4d(sK + s * SLAB_KV, &tmK, bar_kv, s * 64, rbase + k0, hk, bt);
           tma_load_4d(sV + s * SLAB_KV, &tmV, bar_kv, s * 64, rbase + k0, hk, bt);
         }
-        int st = 0, g = 0, t_in = 0;   // stage, head of the group, position in I_h(j): kept incrementally
+        int st = 0, g = g0, t_in = tq0;   // stage, head of the group, position in I_h(j): kept incrementally
         uint32_t ph_e = 0;             // parity of the "stage empty" wait (the first NST steps need none)
         for (int n = 0; n < N && ok; ++n) {
           if (n >= NST) ok = mbar_wait(bar_ld_empty + st, ph_e, a.status);
@@ -403,7 +433,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             for (int c_ = lane; c_ < nchunk; c_ += 32)
               *reinterpret_cast<uint4*>(tile + s_ * slab_bytes + first * 128 + c_ * 16) = make_uint4(0u, 0u, 0u, 0u);
         };
-        int t_clr = 0;  // position in I_h(j) of the next step whose Q / dO stage is checked (packed batches only)
+        int t_clr = tq0;  // position in I_h(j) of the next step whose Q / dO stage is checked (packed batches only)
         auto clear_stage_tail = [&](int stage) {
           if constexpr (VARLEN) {
             const int q0_ = cowa_bwd_tile_at(rg, t_clr) * BQS;
@@ -493,7 +523,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       }
     }
   } else if (warp < 12) {
-    setmaxnreg_inc<176>();
+    setmaxnreg_inc<160>();
     {
       // ======== two compute warpgroups, each takes 32 of the 64 query columns of every step: P^T and dS^T, one
       // KV row per thread.  Inside the 64-column S^T buffer a warpgroup only ever writes into the 32 columns
@@ -504,7 +534,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       const int kcol = k0 + r;               // key index of this thread
       const long long kpos = (long long)kcol - off;  // first causal query of this key
       const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
-      int st = 0, t_in = 0;                  // stage and position in I_h(j) of the next step
+      int st = 0, t_in = tq0;                // stage and position in I_h(j) of the next step
       uint32_t ph_l = 0, par = 0;
       for (int n = 0; n < N && ok; ++n) {
         const int b_ = n & 1;
@@ -523,8 +553,8 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           if (kcol < w.s) m |= interval_bits32(kpos, qend, base);
           mk = kcol < Nk ? m : 0u;
         }
-        const float* lse2 = sVec + st * 128 + wg * 32;
-        const float* dlt = lse2 + 64;
+        const float4* nlse4 = reinterpret_cast<const float4*>(sVec + st * 128 + wg * 32);  // -LSE log2(e), then -Delta
+        const float4* ndlt4 = nlse4 + 16;
         ok = mbar_wait(bar_ld_full + st, ph_l, a.status);
         ok = ok && mbar_wait(bar_s_full + b_, par, a.status);
         if (!ok) break;
@@ -535,11 +565,14 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           tmem_ld32(sbuf, sr);
           tmem_wait_ld();
 #pragma unroll
-          for (int e = 0; e < 32; e += 2) {
-            const float2 x = fma2(make_float2(__uint_as_float(sr[e]), __uint_as_float(sr[e + 1])), sc2,
-                                  make_float2(-lse2[e], -lse2[e + 1]));
+          for (int e = 0; e < 32; e += 4) {
+            const float4 nl = nlse4[e / 4];
+            const float2 x = fma2(make_float2(__uint_as_float(sr[e]), __uint_as_float(sr[e + 1])), sc2, make_float2(nl.x, nl.y));
+            const float2 y = fma2(make_float2(__uint_as_float(sr[e + 2]), __uint_as_float(sr[e + 3])), sc2, make_float2(nl.z, nl.w));
             p[e] = ex2(x.x);
             p[e + 1] = ex2(x.y);
+            p[e + 2] = ex2(y.x);
+            p[e + 3] = ex2(y.y);
           }
           if (!full) {
 #pragma unroll
@@ -562,11 +595,14 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           tmem_ld32(dpbuf, dr);
           tmem_wait_ld();
 #pragma unroll
-          for (int e = 0; e < 32; e += 2) {
-            const float2 y = add2(make_float2(__uint_as_float(dr[e]), __uint_as_float(dr[e + 1])),
-                                  make_float2(-dlt[e], -dlt[e + 1]));
-            const float2 z = mul2(make_float2(p[e], p[e + 1]), y);
-            dsp[e / 2] = pack_bf16(z.x, z.y);
+          for (int e = 0; e < 32; e += 4) {
+            const float4 nd = ndlt4[e / 4];
+            const float2 y = mul2(make_float2(p[e], p[e + 1]),
+                                  add2(make_float2(__uint_as_float(dr[e]), __uint_as_float(dr[e + 1])), make_float2(nd.x, nd.y)));
+            const float2 z = mul2(make_float2(p[e + 2], p[e + 3]),
+                                  add2(make_float2(__uint_as_float(dr[e + 2]), __uint_as_float(dr[e + 3])), make_float2(nd.z, nd.w)));
+            dsp[e / 2] = pack_bf16(y.x, y.y);
+            dsp[e / 2 + 1] = pack_bf16(z.x, z.y);
           }
           tmem_st16(sbuf + 16, dsp);  // dS^T beside P^T
           // dS^T also to shared memory (row r = 128 B = 8 chunks, 128B swizzle) for the dQ^T product
@@ -586,13 +622,13 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       if (wg == 0) store_grad(true);
     }
   } else {
-    setmaxnreg_dec<96>();
+    setmaxnreg_dec<112>();
     {
       // ======== dQ drain warpgroup: one d column of dQ^T per thread; TMEM -> shared -> bulk reduce-add ========
       const int d = (warp & 3) * 32 + lane;
       const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
       const bool issuer = (d == 0);
-      int g = 0, t_in = 0;
+      int g = g0, t_in = tq0;
       for (int n = 0; n < N && ok; ++n) {
         const int i = cowa_bwd_tile_at(rg, t_in);
         const int bhq = bhq0 + g, q0 = i * BQS;
@@ -613,15 +649,25 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           wg_sync(3);
           if (d < D) {
             if (a.dq_fixed) {
-              const float fx = a.scale * kDqFixedOne;
-              bool out_of_range = false;
+              // Rounded to integers on the FMA and integer pipes (the conversion instruction runs at the rate of the
+              // exponentials and competed with them: one KV head of 20001 tokens 942 / 880 thousand clocks): x = 2^16 h + l
+              // with h = rint(x / 2^16), |l| <= 2^15, both exact; adding 1.5 * 2^23 leaves an integer in the low mantissa
+              // bits, and shifting the first sum by 16 drops its exponent.  Same integers as __float2int_rn.
+              const float2 fx2 = make_float2(a.scale * kDqFixedOne, a.scale * kDqFixedOne);
+              auto c2 = [](float c_) { return make_float2(c_, c_); };
+              float worst = 0.f;
 #pragma unroll
-              for (int c = 0; c < 32; ++c) {
-                const float x = __uint_as_float(v[hf][c]) * fx;
-                out_of_range |= !(fabsf(x) < 2147483520.f);  // the conversion would saturate (or x is not a number)
-                reinterpret_cast<int*>(stage)[c * D + d] = __float2int_rn(x);
+              for (int c = 0; c < 32; c += 2) {
+                const float2 x = mul2(make_float2(__uint_as_float(v[hf][c]), __uint_as_float(v[hf][c + 1])), fx2);
+                worst = max_nan(worst, max_nan(fabsf(x.x), fabsf(x.y)));
+                const float2 th = fma2(x, c2(1.f / 65536.f), c2(12582912.f));
+                const float2 l = fma2(add2(th, c2(-12582912.f)), c2(-65536.f), x);
+                const float2 tl = add2(l, c2(12582912.f));
+                int* dst = reinterpret_cast<int*>(stage) + c * D + d;
+                dst[0] = (__float_as_int(th.x) << 16) + (__float_as_int(tl.x) - 0x4B400000);
+                dst[D] = (__float_as_int(th.y) << 16) + (__float_as_int(tl.y) - 0x4B400000);
               }
-              if (out_of_range) atomicOr(a.status, (unsigned)COWA_DEV_DQ_RANGE);
+              if (!(worst < 2147483520.f)) atomicOr(a.status, (unsigned)COWA_DEV_DQ_RANGE);  // would not fit 32 bits (or NaN)
             } else {
 #pragma unroll
               for (int c = 0; c < 32; ++c) stage[c * D + d] = __uint_as_float(v[hf][c]) * a.scale;
@@ -651,12 +697,13 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   }
 }
 
-// Delta = rowsum(O * dO), lse2 = LSE * log2(e); rows in [T, Tpad) get lse2 = +inf, Delta = 0.
+// delta = -rowsum(O * dO), lse2 = -LSE * log2(e); rows in [T, Tpad) get lse2 = -inf, delta = 0.  The same threads zero
+// the fp32 dQ accumulator (as a memset before it that was a pass of its own: 32K 190 us for both, 164 us so).
 template <int D>
 __global__ void cowa_bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
                                            const float* __restrict__ lse, float* __restrict__ lse2,
-                                           float* __restrict__ delta, int T, int Tpad, long long BH, int H,
-                                           CowaStrides so) {
+                                           float* __restrict__ delta, float* __restrict__ acc, int T, int Tpad,
+                                           long long BH, int H, CowaStrides so) {
   constexpr int TPR = D / 8;  // threads per row (16 bytes each)
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long row = gid / TPR;
@@ -664,6 +711,8 @@ __global__ void cowa_bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, 
   if (row >= BH * Tpad) return;
   const long long bh = row / Tpad;
   const int t = (int)(row % Tpad);
+  float4* z = reinterpret_cast<float4*>(acc + (size_t)row * D + part * 8);
+  z[0] = z[1] = make_float4(0.f, 0.f, 0.f, 0.f);
   float s = 0.f;
   if (t < T) {
     const size_t base = (size_t)(bh / H) * so.b + (size_t)(bh % H) * so.h + (size_t)t * so.t + part * 8;
@@ -679,46 +728,19 @@ __global__ void cowa_bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, 
 #pragma unroll
   for (int o_ = TPR / 2; o_ > 0; o_ >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o_);
   if (part == 0) {
-    delta[row] = s;
-    lse2[row] = t < T ? lse[(size_t)bh * T + t] * 1.4426950408889634f : INFINITY;
+    delta[row] = -s;
+    lse2[row] = t < T ? lse[(size_t)bh * T + t] * -1.4426950408889634f : -INFINITY;
   }
 }
 
-template <int D>
-__global__ void cowa_bwd_convert_dq_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, int T,
-                                           int Tpad, long long BH, int fixed, int H, CowaStrides sq,
-                                           unsigned int* status) {
-  const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // one thread per 8 elements
-  const long long total = BH * T * (D / 8);
-  if (gid >= total) return;
-  const long long row = gid / (D / 8);
-  const int part = (int)(gid % (D / 8));
-  const long long bh = row / T;
-  const int t = (int)(row % T);
-  const float4* src = reinterpret_cast<const float4*>(acc + ((size_t)bh * Tpad + t) * D + part * 8);
-  float4 x = src[0], y = src[1];
-  if (fixed) {  // the accumulator holds 32-bit integers in units of 2^-18
-    const float u = 1.f / kDqFixedOne;
-    x = make_float4(__float_as_int(x.x) * u, __float_as_int(x.y) * u, __float_as_int(x.z) * u, __float_as_int(x.w) * u);
-    y = make_float4(__float_as_int(y.x) * u, __float_as_int(y.y) * u, __float_as_int(y.z) * u, __float_as_int(y.w) * u);
-    // half of the representable range: a total that wrapped around lands out here in most cases
-    const float big = fmaxf(fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))),
-                            fmaxf(fmaxf(fabsf(y.x), fabsf(y.y)), fmaxf(fabsf(y.z), fabsf(y.w))));
-    if (big >= 4096.f) atomicOr(status, (unsigned)COWA_DEV_DQ_RANGE);
-  }
-  uint4 v;
-  v.x = pack_bf16(x.x, x.y); v.y = pack_bf16(x.z, x.w); v.z = pack_bf16(y.x, y.y); v.w = pack_bf16(y.z, y.w);
-  *reinterpret_cast<uint4*>(dq + (size_t)(bh / H) * sq.b + (size_t)(bh % H) * sq.h + (size_t)t * sq.t + part * 8) = v;
-}
-
-// Packed batches.  One block per (64-row chunk of the padded row space, QO head): Delta and LSE * log2(e)
-// of the chunk's rows (padding rows: +inf, 0), read from the packed tensors.
+// Packed batches.  One block per (64-row chunk of the padded row space, QO head): -Delta and -LSE * log2(e)
+// of the chunk's rows (padding rows: -inf, 0), read from the packed tensors.
 template <int D>
 __global__ void cowa_bwd_preprocess_varlen_kernel(const __nv_bfloat16* __restrict__ o,
                                                   const __nv_bfloat16* __restrict__ d_o,
                                                   const float* __restrict__ lse, float* __restrict__ lse2,
-                                                  float* __restrict__ delta, const int* __restrict__ cu, int B,
-                                                  int total, int Tpad) {
+                                                  float* __restrict__ delta, float* __restrict__ acc,
+                                                  const int* __restrict__ cu, int B, int total, int Tpad) {
   constexpr int TPR = D / 8;  // threads per row (16 bytes each)
   const int chunk = blockIdx.x, h = blockIdx.y;
   const int r = threadIdx.x / TPR, part = threadIdx.x % TPR;
@@ -727,6 +749,8 @@ __global__ void cowa_bwd_preprocess_varlen_kernel(const __nv_bfloat16* __restric
   const int t = lc * BQS + r;  // row inside the sequence
   const int rbase = in ? cu[b] : 0;
   const bool valid = in && t < cu[b + 1] - rbase && rbase >= 0 && rbase + t < total;
+  float4* z = reinterpret_cast<float4*>(acc + ((size_t)h * Tpad + (size_t)chunk * BQS + r) * D + part * 8);
+  z[0] = z[1] = make_float4(0.f, 0.f, 0.f, 0.f);
   float s = 0.f;
   if (valid) {
     const size_t base = ((size_t)h * total + rbase + t) * D + part * 8;
@@ -743,83 +767,139 @@ __global__ void cowa_bwd_preprocess_varlen_kernel(const __nv_bfloat16* __restric
   for (int o_ = TPR / 2; o_ > 0; o_ >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o_);
   if (part == 0) {
     const size_t row = (size_t)h * Tpad + (size_t)chunk * BQS + r;  // chunks are laid out in order: pb == chunk * BQS
-    delta[row] = s;
-    lse2[row] = valid ? lse[(size_t)h * total + rbase + t] * 1.4426950408889634f : INFINITY;
+    delta[row] = -s;
+    lse2[row] = valid ? lse[(size_t)h * total + rbase + t] * -1.4426950408889634f : -INFINITY;
   }
 }
 
-// Packed batches: fp32 (or fixed-point) dQ accumulator in the padded row space -> bf16 dq in the packed one.
-template <int D>
-__global__ void cowa_bwd_convert_dq_varlen_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq,
-                                                  const int* __restrict__ cu, int B, int total, int Tpad, int fixed,
-                                                  unsigned int* status) {
-  constexpr int TPR = D / 8;
-  const int chunk = blockIdx.x, h = blockIdx.y;
-  const int r = threadIdx.x / TPR, part = threadIdx.x % TPR;
-  int b, lc, nch, pb;
-  if (!varlen_locate(cu, B, chunk, BQS, BQS, &b, &lc, &nch, &pb)) return;
-  const int t = lc * BQS + r;
-  const int rbase = cu[b];
-  if (t >= cu[b + 1] - rbase || rbase < 0 || rbase + t >= total) return;
-  const float4* src = reinterpret_cast<const float4*>(acc + ((size_t)h * Tpad + (size_t)chunk * BQS + r) * D + part * 8);
+// 8 elements of the dQ accumulator (fp32, or 32-bit integers in units of 2^-18) -> bf16
+__device__ __forceinline__ uint4 dq_bf16(const float4* src, int fixed, unsigned int* status) {
   float4 x = src[0], y = src[1];
   if (fixed) {
     const float u = 1.f / kDqFixedOne;
     x = make_float4(__float_as_int(x.x) * u, __float_as_int(x.y) * u, __float_as_int(x.z) * u, __float_as_int(x.w) * u);
     y = make_float4(__float_as_int(y.x) * u, __float_as_int(y.y) * u, __float_as_int(y.z) * u, __float_as_int(y.w) * u);
+    // half of the representable range: a total that wrapped around lands out here in most cases
     const float big = fmaxf(fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))),
                             fmaxf(fmaxf(fabsf(y.x), fabsf(y.y)), fmaxf(fabsf(y.z), fabsf(y.w))));
     if (big >= 4096.f) atomicOr(status, (unsigned)COWA_DEV_DQ_RANGE);
   }
-  uint4 v;
-  v.x = pack_bf16(x.x, x.y); v.y = pack_bf16(x.z, x.w); v.z = pack_bf16(y.x, y.y); v.w = pack_bf16(y.z, y.w);
-  *reinterpret_cast<uint4*>(dq + ((size_t)h * total + rbase + t) * D + part * 8) = v;
+  return make_uint4(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w), pack_bf16(y.x, y.y), pack_bf16(y.z, y.w));
 }
 
-// Sum of the per-block partial dK, dV (heads of a group spread over `parts` blocks), in slot order, to bf16.
-template <int D>
-__global__ void cowa_bwd_reduce_dkv_kernel(const float* __restrict__ part, __nv_bfloat16* __restrict__ dk,
-                                           __nv_bfloat16* __restrict__ dv, int T, int nKV, int parts, long long BHk,
-                                           int H, CowaStrides sk, CowaStrides sv) {
-  const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;  // one thread per 8 elements of dK and dV
-  const long long total = BHk * nKV * BKV * (D / 8);
-  if (gid >= total) return;
-  const int ch = (int)(gid % (D / 8));
-  const int r = (int)((gid / (D / 8)) % BKV);
-  const long long tile = gid / ((D / 8) * BKV);  // bhk * nKV + j
-  const int j = (int)(tile % nKV);
-  const long long bhk = tile / nKV;
-  const int t = j * BKV + r;
-  if (t >= T) return;
-  float acc[2][8];
-#pragma unroll
-  for (int m = 0; m < 2; ++m)
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[m][e] = 0.f;
-  for (int pi = 0; pi < parts; ++pi)
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-      const float4* src = reinterpret_cast<const float4*>(part + (((size_t)tile * parts + pi) * 2 + m) * (size_t)(BKV * D) +
-                                                          (size_t)r * D + ch * 8);
-      const float4 x = src[0], y = src[1];
-      acc[m][0] += x.x; acc[m][1] += x.y; acc[m][2] += x.z; acc[m][3] += x.w;
-      acc[m][4] += y.x; acc[m][5] += y.y; acc[m][6] += y.z; acc[m][7] += y.w;
-    }
-#pragma unroll
-  for (int m = 0; m < 2; ++m) {
-    uint4 v;
-    v.x = pack_bf16(acc[m][0], acc[m][1]); v.y = pack_bf16(acc[m][2], acc[m][3]);
-    v.z = pack_bf16(acc[m][4], acc[m][5]); v.w = pack_bf16(acc[m][6], acc[m][7]);
-    const CowaStrides& sg = m == 0 ? sk : sv;
-    *reinterpret_cast<uint4*>((m == 0 ? dk : dv) + (size_t)(bhk / H) * sg.b + (size_t)(bhk % H) * sg.h + (size_t)t * sg.t + ch * 8) = v;
+// The dQ accumulator to bf16.  Batched: 8 elements a thread; packed: one 64-row chunk of the padded row space and one head a
+// block, into the packed rows.  (One kernel with the sum of partial dK, dV needs 46 registers and lost occupancy: 137
+// instead of 112 us at 32K.)
+template <int D, bool VARLEN>
+__global__ void __launch_bounds__(VARLEN ? BQS * (D / 8) : 256)
+cowa_bwd_convert_dq_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, const int* __restrict__ cu, int B,
+                           int T, int Tpad, long long BH, int H, int fixed, CowaStrides sq, unsigned int* status) {
+  constexpr int TPR = D / 8;  // threads per row (16 bytes of bf16 each)
+  const int part = threadIdx.x % TPR;
+  if constexpr (!VARLEN) {
+    const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / TPR;
+    if (row >= BH * T) return;
+    const long long bh = row / T;
+    const int t = (int)(row % T);
+    const uint4 v = dq_bf16(reinterpret_cast<const float4*>(acc + ((size_t)bh * Tpad + t) * D + part * 8), fixed, status);
+    *reinterpret_cast<uint4*>(dq + (size_t)(bh / H) * sq.b + (size_t)(bh % H) * sq.h + (size_t)t * sq.t + part * 8) = v;
+  } else {
+    const int chunk = blockIdx.x, h = blockIdx.y, r = threadIdx.x / TPR;
+    int b, lc, nch, pb;
+    if (!varlen_locate(cu, B, chunk, BQS, BQS, &b, &lc, &nch, &pb)) return;
+    const int t = lc * BQS + r;
+    const int rbase = cu[b];
+    if (t >= cu[b + 1] - rbase || rbase < 0 || rbase + t >= T) return;
+    const uint4 v = dq_bf16(reinterpret_cast<const float4*>(acc + ((size_t)h * Tpad + (size_t)chunk * BQS + r) * D + part * 8),
+                            fixed, status);
+    *reinterpret_cast<uint4*>(dq + ((size_t)h * T + rbase + t) * D + part * 8) = v;
   }
 }
 
-// Blocks per KV tile.  A block normally takes the whole GQA group of its KV tile (dK, dV then never leave
-// TMEM).  That starves the GPU when B * Hkv * tiles is small, and it makes the sink tiles -- visited by
-// every query tile of every head -- the critical path when Hkv is small; in both cases the group's heads
-// are spread over `parts` blocks (a divisor of G), chosen as the smallest that gives two waves of
-// blocks and keeps the longest block under 3/4 of an even share of the work.
+// Partial dK (blockIdx.y = 0) and dV (1) of the shared tiles, added in slot order, to bf16.
+template <int D, bool VARLEN>
+__global__ void __launch_bounds__(256)
+cowa_bwd_reduce_dkv_kernel(const __grid_constant__ BwdArgs a, CowaStrides sk, CowaStrides sv) {
+  constexpr int TPR = D / 8, ROWS = 256 / TPR;  // threads per row (16 bytes of bf16 each), rows per block
+  const int part = threadIdx.x % TPR;
+  int q = blockIdx.x / (BKV / ROWS), c = 0, slot = 0;
+  const int r = blockIdx.x % (BKV / ROWS) * ROWS + threadIdx.x / TPR;
+  for (; c < 2; ++c) {
+    if (a.cls_parts[c] == 1) continue;
+    if (q < a.cls_tiles[c]) break;
+    q -= a.cls_tiles[c];
+    slot += a.cls_tiles[c] * a.cls_parts[c];
+  }
+  const int parts = a.cls_parts[c];
+  TileAt at;
+  if (!locate_tile<VARLEN>(a, c, q, at)) return;
+  int Nk = a.Nk, rbase = 0;
+  if constexpr (VARLEN) {
+    rbase = a.cu[at.b];
+    Nk = a.cu[at.b + 1] - rbase;
+    if (rbase < 0 || rbase + Nk > a.total) return;
+  }
+  const int t = at.j * BKV + r;
+  if (t >= Nk) return;
+  const int m = blockIdx.y;
+  // the slots hold a row's 16-byte chunks permuted
+  const float* src = a.dkv_part + ((size_t)(slot + q * parts) * 2 + m) * (BKV * D) + (size_t)r * D;
+  const int c0 = ((part * 2) ^ (r & 7)) * 4, c1 = ((part * 2 + 1) ^ (r & 7)) * 4;
+  float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+#pragma unroll 4
+  for (int i = 0; i < parts; ++i) {
+    const float4 u = *reinterpret_cast<const float4*>(src + (size_t)i * 2 * (BKV * D) + c0);
+    const float4 v = *reinterpret_cast<const float4*>(src + (size_t)i * 2 * (BKV * D) + c1);
+    x.x += u.x; x.y += u.y; x.z += u.z; x.w += u.w;
+    y.x += v.x; y.y += v.y; y.z += v.z; y.w += v.w;
+  }
+  const size_t o = VARLEN ? ((size_t)at.hk * a.total + rbase + t) * D
+                 : m == 0 ? (size_t)at.b * sk.b + (size_t)at.hk * sk.h + (size_t)t * sk.t
+                          : (size_t)at.b * sv.b + (size_t)at.hk * sv.h + (size_t)t * sv.t;
+  *reinterpret_cast<uint4*>((m == 0 ? a.dk : a.dv) + o + part * 8) =
+      make_uint4(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w), pack_bf16(y.x, y.y), pack_bf16(y.z, y.w));
+}
+
+// How the KV tiles are shared among blocks.  A tile whose block takes the whole GQA group keeps dK, dV in TMEM; a shared
+// tile costs every block a prologue and 128 KB of fp32 partial sums (D = 128), about four steps' worth of time, so tiles
+// are shared only where whole ones leave SMs idle:
+//   sink tiles, visited by every query tile, when one is longer than 3/4 of an SM's share of the work: thirds of a share;
+//   all tiles when there are at most two per SM: fifths of a share, four steps at least;
+//   the last tile per SM when there are at most eight: quarters, so that the last wave ends together.
+// Main kernel, 1000 clocks, whole heads of a group spread / this: 2 x 8K, 16 heads 1147 / 1070; one KV head of 20001 tokens
+// 1021 / 983; 1K, 4 heads 58 / 34.
+struct BwdPlan {
+  int sink_tiles;  // per sequence and head
+  int tiles[3], parts[3];
+  long long slots() const {
+    long long n = 0;
+    for (int c = 0; c < 3; ++c)
+      if (parts[c] > 1) n += (long long)tiles[c] * parts[c];
+    return n;
+  }
+  long long blocks() const {
+    long long n = 0;
+    for (int c = 0; c < 3; ++c) n += (long long)tiles[c] * parts[c];
+    return n;
+  }
+};
+
+// `rest` tiles behind the sink tiles, `avg` steps each; share: an SM's steps
+void plan_rest(BwdPlan& pl, long long rest, double avg, double share) {
+  const int sms = cowa::sm_count();
+  pl.tiles[1] = (int)rest; pl.parts[1] = 1;
+  pl.tiles[2] = 0; pl.parts[2] = 1;
+  if (rest <= 2 * sms) {
+    pl.parts[1] = std::max(1, std::min(16, (int)(avg / std::max(share / 5, 4.0) + 0.999)));
+  } else if (rest <= 8ll * sms && avg >= 16) {
+    pl.tiles[2] = sms;
+    pl.tiles[1] -= pl.tiles[2];
+    pl.parts[2] = avg >= 32 ? 4 : 2;
+  }
+}
+
+// Blocks per KV tile when whole heads of a group are spread: the smallest divisor of G that gives two waves of blocks and
+// keeps the longest under 3/4 of an even share of the work.  Sizes the workspace, which bounds the plan below.
 int bwd_parts(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& hw) {
   const int nKV = (Nk + BKV - 1) / BKV;
   long long total = 0, longest = 0;
@@ -843,14 +923,68 @@ int bwd_parts(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& hw) 
   return G;
 }
 
+BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& hw) {
+  BwdPlan pl;
+  const int nKV = (Nk + BKV - 1) / BKV, sms = cowa::sm_count();
+  pl.sink_tiles = 0;
+  for (int h = 0; h < Hkv; ++h) pl.sink_tiles = std::max(pl.sink_tiles, (std::min(hw.w[h].s, Nk) + BKV - 1) / BKV);
+  long long total = 0, sinks = 0, longest = 0;
+  for (int h = 0; h < Hkv; ++h)
+    for (int j = 0; j < nKV; ++j) {
+      CowaRange rg[2];
+      const int k0 = j * BKV, k1 = std::min(k0 + BKV, Nk) - 1;
+      cowa_bwd_ranges(hw.w[h], k0, k1, Nk - Nq, Nq, BQS, rg);
+      const long long cnt = (long long)(cowa_range_len(rg[0]) + cowa_range_len(rg[1])) * G;
+      total += cnt;
+      if (j < pl.sink_tiles) { sinks += cnt; longest = std::max(longest, cnt); }
+    }
+  total *= B; sinks *= B;
+  const double share = (double)total / sms;
+  const long long rest = (long long)B * Hkv * (nKV - pl.sink_tiles);
+  pl.tiles[0] = B * Hkv * pl.sink_tiles;
+  pl.parts[0] = longest * 4 > 3 * share ? std::max(1, std::min(32, (int)(longest / std::max(share / 3, 4.0) + 0.999))) : 1;
+  plan_rest(pl, rest, rest > 0 ? (double)(total - sinks) / rest : 0.0, share);
+  // Partial sums in the workspace: where spreading whole heads gives four blocks or more per tile, no more than those.
+  const int heads = bwd_parts(B, Nq, Nk, Hkv, G, hw);
+  const long long room = heads > 1 ? (long long)B * Hkv * nKV * heads : 0;
+  const long long budget = heads >= 4 ? room : std::max<long long>(room, 4ll * sms);
+  while (pl.slots() > budget) --*std::max_element(pl.parts, pl.parts + 3);
+  return pl;
+}
+
+// Packed batches: the lengths are on the device, so the plan goes by the average sequence.
+BwdPlan bwd_plan_varlen(int B, int total, int Hkv, int G, const cowa_params_t* p, const CowaHeadWindows& hw) {
+  BwdPlan pl;
+  const int sms = cowa::sm_count(), len = std::max(total / B, 1);
+  const long long rest = (long long)(total / BKV + B) * Hkv;
+  pl.sink_tiles = 0;
+  double keys = 0;
+  for (int h = 0; h < Hkv; ++h) {
+    CowaWin w = hw.w[h];
+    if (p->full_attn) { w.s = 0; w.n = len; w.g = 0; w.l = 0; }
+    else if (!p->windows) w = cowa_default_window(len, p->hkv_global > 0 ? p->hkv_global : Hkv, p->hkv_offset + h, p->sink, p->local);
+    if (!p->full_attn) pl.sink_tiles = std::max(pl.sink_tiles, (std::min(p->windows ? w.s : p->sink, total) + BKV - 1) / BKV);
+    keys += std::min<double>(len, (double)w.n + w.l + BKV) / Hkv;
+  }
+  pl.tiles[0] = B * Hkv * pl.sink_tiles;
+  pl.parts[0] = pl.tiles[0] * 4ll <= 2 * sms ? 4 : 1;
+  // the last wave is not shared here: short sequences make its tiles short already (1628 against 1624 in 1000 clocks)
+  const double avg = 0.7 * keys / BQS * G, real = (double)total / BKV * Hkv;
+  plan_rest(pl, rest, rest <= 2 * sms ? avg : 0.0, real * avg / sms);
+  return pl;
+}
+
+size_t slot_bytes(const BwdPlan& pl, int D) { return (size_t)pl.slots() * 2 * BKV * D * sizeof(float); }
+
 size_t part_bytes(int B, int Nk, int Hkv, int D, int parts) {
   if (parts <= 1) return 0;
   return (size_t)B * Hkv * ((Nk + BKV - 1) / BKV) * parts * 2 * BKV * D * sizeof(float);
 }
 
-size_t ws_bytes(int B, int Nq, int Nk, int Hq, int Hkv, int D, int parts) {
+size_t ws_bytes(int B, int Nq, int Nk, int Hq, int Hkv, int D, const BwdPlan& pl, const CowaHeadWindows& hw) {
   const size_t Tpad = ((size_t)Nq + BQS - 1) / BQS * BQS;
-  return (size_t)B * Hq * Tpad * ((size_t)D + 2) * sizeof(float) + part_bytes(B, Nk, Hkv, D, parts);
+  return (size_t)B * Hq * Tpad * ((size_t)D + 2) * sizeof(float) +
+         std::max(slot_bytes(pl, D), part_bytes(B, Nk, Hkv, D, bwd_parts(B, Nq, Nk, Hkv, Hq / Hkv, hw)));
 }
 
 // Contiguous [H, T, D] (x batch) strides.
@@ -860,10 +994,19 @@ CowaStrides packed_strides(int H, long long T, int D) {
   return st;
 }
 
+template <int D, bool VARLEN>
+void launch_reduce(const BwdArgs& a, const BwdPlan& pl, const CowaStrides& sk, const CowaStrides& sv, cudaStream_t st) {
+  long long shared = 0;
+  for (int c = 0; c < 3; ++c)
+    if (pl.parts[c] > 1) shared += pl.tiles[c];
+  if (shared > 0)
+    cowa_bwd_reduce_dkv_kernel<D, VARLEN><<<dim3((unsigned)(shared * (BKV * (D / 8) / 256)), 2), 256, 0, st>>>(a, sk, sv);
+}
+
 template <int D>
 int launch_bwd(const void* q, const void* k, const void* v, const void* o, const float* lse, const void* d_o,
                void* dq, void* dk, void* dv, int B, int Nq, int Nk, int Hq, int Hkv, const cowa_params_t* p,
-               const CowaHeadWindows& hw, int parts, void* ws, cudaStream_t st) {
+               const CowaHeadWindows& hw, const BwdPlan& pl, void* ws, cudaStream_t st) {
   const int T = Nq;  // rows of q, o, d_o, dq, lse
   const int Tpad = (T + BQS - 1) / BQS * BQS;
   const long long BH = (long long)B * Hq;
@@ -894,58 +1037,45 @@ int launch_bwd(const void* q, const void* k, const void* v, const void* o, const
   a.scale = p->softmax_scale;
   a.scale_log2 = p->softmax_scale * 1.4426950408889634f;
   a.wins = hw;
-  a.sink_tiles = 0;
+  a.sink_tiles = pl.sink_tiles;
+  for (int c = 0; c < 3; ++c) { a.cls_tiles[c] = pl.tiles[c]; a.cls_parts[c] = pl.parts[c]; }
   a.dq_fixed = p->deterministic ? 1 : 0;
-  a.parts = parts; a.dkv_part = dkv_part;
-  a.cu = nullptr; a.dk = nullptr; a.dv = nullptr; a.total = 0; a.tiles_bound = 0;
+  a.dkv_part = dkv_part;
+  a.cu = nullptr; a.dk = static_cast<__nv_bfloat16*>(dk); a.dv = static_cast<__nv_bfloat16*>(dv); a.total = 0; a.tiles_bound = 0;
   a.sink = 0; a.local = 0; a.hkv_global = 0; a.hkv_offset = 0; a.full_attn = 0; a.explicit_windows = 0;
-  for (int h = 0; h < Hkv; ++h) {
-    const int sk_ = hw.w[h].s < Nk ? hw.w[h].s : Nk;
-    a.sink_tiles = std::max(a.sink_tiles, (sk_ + BKV - 1) / BKV);
-  }
-  const long long nblocks = (long long)((Nk + BKV - 1) / BKV) * B * Hkv * parts;
-  if (nblocks > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
+  if (pl.blocks() > 0x7FFFFFFFll || (long long)Nq / BQS * a.G * 32 > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
   COWA_CUDA_TRY(cudaFuncSetAttribute(cowa_bwd_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      BwdSmem<D>::kBytes));
-  COWA_CUDA_TRY(cudaMemsetAsync(dq_acc, 0, (size_t)BH * Tpad * D * sizeof(float), st));
   {
     const long long threads = BH * Tpad * (D / 8);
     cowa_bwd_preprocess_kernel<D><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(
-        static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse, lse2, delta, T, Tpad, BH, Hq, so);
+        static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse, lse2, delta, dq_acc,
+        T, Tpad, BH, Hq, so);
     COWA_CUDA_TRY(cudaGetLastError());
   }
   if (p->bwd_main_start_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_start_event), st));
-  cowa_bwd_kernel<D, false><<<(unsigned)nblocks, 512, BwdSmem<D>::kBytes, st>>>(mq, mk, mv, mdo, mdk, mdv, a);
+  cowa_bwd_kernel<D, false><<<(unsigned)pl.blocks(), 512, BwdSmem<D>::kBytes, st>>>(mq, mk, mv, mdo, mdk, mdv, a);
   COWA_CUDA_TRY(cudaGetLastError());
   if (p->bwd_main_stop_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_stop_event), st));
-  {
-    const long long threads = BH * T * (D / 8);
-    cowa_bwd_convert_dq_kernel<D><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(
-        dq_acc, static_cast<__nv_bfloat16*>(dq), T, Tpad, BH, p->deterministic ? 1 : 0, Hq, sq, a.status);
-    COWA_CUDA_TRY(cudaGetLastError());
-  }
-  if (parts > 1) {
-    const int nKV = (Nk + BKV - 1) / BKV;
-    const long long threads = (long long)B * Hkv * nKV * BKV * (D / 8);
-    cowa_bwd_reduce_dkv_kernel<D><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(
-        dkv_part, static_cast<__nv_bfloat16*>(dk), static_cast<__nv_bfloat16*>(dv), Nk, nKV, parts, (long long)B * Hkv,
-        Hkv, sk, sv);
-    COWA_CUDA_TRY(cudaGetLastError());
-  }
+  launch_reduce<D, false>(a, pl, sk, sv, st);
+  COWA_CUDA_TRY(cudaGetLastError());
+  cowa_bwd_convert_dq_kernel<D, false><<<(unsigned)((BH * T * (D / 8) + 255) / 256), 256, 0, st>>>(
+      dq_acc, static_cast<__nv_bfloat16*>(dq), nullptr, B, T, Tpad, BH, Hq, a.dq_fixed, sq, a.status);
+  COWA_CUDA_TRY(cudaGetLastError());
   return COWA_OK;
 }
 
 // Padded row space of a packed batch: every sequence rounded up to 64 rows; the bound needs no lengths.
 int varlen_tpad(int B, int total) { return (total / BQS + B) * BQS; }
 
-size_t ws_bytes_varlen(int B, int total, int Hq, int D) {
-  return (size_t)Hq * varlen_tpad(B, total) * ((size_t)D + 2) * sizeof(float);
+size_t ws_bytes_varlen(int B, int total, int Hq, int D, const BwdPlan& pl) {
+  return (size_t)Hq * varlen_tpad(B, total) * ((size_t)D + 2) * sizeof(float) + slot_bytes(pl, D);
 }
 
 template <int D>
 int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o, const float* lse, const void* d_o,
                       void* dq, void* dk, void* dv, const int* cu, int B, int total, int Hq, int Hkv,
-                      const cowa_params_t* p, const CowaHeadWindows& hw, void* ws, cudaStream_t st) {
+                      const cowa_params_t* p, const CowaHeadWindows& hw, const BwdPlan& pl, void* ws, cudaStream_t st) {
   const int Tpad = varlen_tpad(B, total);
   float* dq_acc = static_cast<float*>(ws);
   float* lse2 = dq_acc + (size_t)Hq * Tpad * D;
@@ -968,34 +1098,31 @@ int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o
   a.scale = p->softmax_scale;
   a.scale_log2 = p->softmax_scale * 1.4426950408889634f;
   a.wins = hw;
-  a.sink_tiles = 0;  // KV tiles per sequence that hold sink columns (launched first)
-  if (!p->full_attn)
-    for (int h = 0; h < Hkv; ++h) {
-      const int sk_ = std::min(p->windows ? hw.w[h].s : p->sink, total);
-      a.sink_tiles = std::max(a.sink_tiles, (sk_ + BKV - 1) / BKV);
-    }
+  a.sink_tiles = pl.sink_tiles;
+  for (int c = 0; c < 3; ++c) { a.cls_tiles[c] = pl.tiles[c]; a.cls_parts[c] = pl.parts[c]; }
   a.dq_fixed = p->deterministic ? 1 : 0;
-  a.parts = 1; a.dkv_part = nullptr;
+  a.dkv_part = delta + (size_t)Hq * Tpad;
   a.cu = cu; a.dk = static_cast<__nv_bfloat16*>(dk); a.dv = static_cast<__nv_bfloat16*>(dv);
   a.total = total; a.tiles_bound = total / BKV + B;
   a.sink = p->sink; a.local = p->local;
   a.hkv_global = p->hkv_global > 0 ? p->hkv_global : Hkv;
   a.hkv_offset = p->hkv_offset; a.full_attn = p->full_attn; a.explicit_windows = p->windows != nullptr;
-  const long long nblocks = (long long)a.tiles_bound * Hkv + (long long)a.sink_tiles * B * Hkv;
-  if (nblocks > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
+  if (pl.blocks() > 0x7FFFFFFFll || (long long)total / BQS * a.G * 32 > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
   COWA_CUDA_TRY(cudaFuncSetAttribute(cowa_bwd_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      BwdSmem<D>::kBytes));
-  COWA_CUDA_TRY(cudaMemsetAsync(dq_acc, 0, (size_t)Hq * Tpad * D * sizeof(float), st));
   const dim3 chunks(Tpad / BQS, Hq);
   cowa_bwd_preprocess_varlen_kernel<D><<<chunks, BQS * (D / 8), 0, st>>>(
-      static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse, lse2, delta, cu, B, total, Tpad);
+      static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse, lse2, delta, dq_acc,
+      cu, B, total, Tpad);
   COWA_CUDA_TRY(cudaGetLastError());
   if (p->bwd_main_start_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_start_event), st));
-  cowa_bwd_kernel<D, true><<<(unsigned)nblocks, 512, BwdSmem<D>::kBytes, st>>>(mq, mk, mv, mdo, mdk, mdv, a);
+  cowa_bwd_kernel<D, true><<<(unsigned)pl.blocks(), 512, BwdSmem<D>::kBytes, st>>>(mq, mk, mv, mdo, mdk, mdv, a);
   COWA_CUDA_TRY(cudaGetLastError());
   if (p->bwd_main_stop_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_stop_event), st));
-  cowa_bwd_convert_dq_varlen_kernel<D><<<chunks, BQS * (D / 8), 0, st>>>(dq_acc, static_cast<__nv_bfloat16*>(dq), cu, B,
-                                                                        total, Tpad, p->deterministic ? 1 : 0, a.status);
+  launch_reduce<D, true>(a, pl, sk, sk, st);
+  COWA_CUDA_TRY(cudaGetLastError());
+  cowa_bwd_convert_dq_kernel<D, true><<<chunks, BQS * (D / 8), 0, st>>>(dq_acc, static_cast<__nv_bfloat16*>(dq), cu, B, total,
+                                                                        Tpad, 0, Hq, a.dq_fixed, sq, a.status);
   COWA_CUDA_TRY(cudaGetLastError());
   return COWA_OK;
 }
@@ -1005,9 +1132,18 @@ int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o
 extern "C" {
 
 size_t cowa_bwd_varlen_workspace_bytes(int B, int total, int Hq, int Hkv, int D, const cowa_params_t* p) {
-  (void)p;
   if (B <= 0 || total <= 0 || Hq <= 0 || Hkv <= 0 || Hq % Hkv != 0 || (D != 64 && D != 128)) return 0;
-  return ws_bytes_varlen(B, total, Hq, D);
+  CowaHeadWindows hw;
+  if (!p || cowa::resolve_windows(total, Hkv, p, &hw) != COWA_OK) {  // enough for any parameters
+    BwdPlan most;
+    const int sms = cowa::sm_count();
+    most.sink_tiles = 0;
+    most.tiles[0] = 2 * sms; most.parts[0] = 2;
+    most.tiles[1] = 2 * sms; most.parts[1] = 16;
+    most.tiles[2] = 0; most.parts[2] = 1;
+    return ws_bytes_varlen(B, total, Hq, D, most);
+  }
+  return ws_bytes_varlen(B, total, Hq, D, bwd_plan_varlen(B, total, Hkv, Hq / Hkv, p, hw));
 }
 
 int cowa_bwd_varlen(const void* q, const void* k, const void* v, const void* o, const float* lse, const void* d_o,
@@ -1021,22 +1157,23 @@ int cowa_bwd_varlen(const void* q, const void* k, const void* v, const void* o, 
   const void* ptrs[] = {q, k, v, o, d_o, dq, dk, dv, workspace};
   for (const void* x : ptrs)
     if (!cowa::aligned16(x)) return COWA_ERR_MISALIGNED;
-  if (workspace_bytes < ws_bytes_varlen(B, total, Hq, D)) return COWA_ERR_WORKSPACE_TOO_SMALL;
   CowaHeadWindows hw;
   int rc = cowa::resolve_windows(total, Hkv, p, &hw);  // validates; explicit tuples are copied, the default rule runs per sequence
   if (rc != COWA_OK) return rc;
+  const BwdPlan pl = bwd_plan_varlen(B, total, Hkv, Hq / Hkv, p, hw);
+  if (workspace_bytes < ws_bytes_varlen(B, total, Hq, D, pl)) return COWA_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   return D == 128 ? launch_bwd_varlen<128>(q, k, v, o, lse, d_o, dq, dk, dv, cu_seqlens, B, total, Hq, Hkv, p, hw,
-                                           workspace, st)
+                                           pl, workspace, st)
                   : launch_bwd_varlen<64>(q, k, v, o, lse, d_o, dq, dk, dv, cu_seqlens, B, total, Hq, Hkv, p, hw,
-                                          workspace, st);
+                                          pl, workspace, st);
 }
 
 size_t cowa_bwd_prefill_workspace_bytes(int B, int Nq, int Nk, int Hq, int Hkv, int D, const cowa_params_t* p) {
   if (B <= 0 || Nq <= 0 || Nk < Nq || Hq <= 0 || Hkv <= 0 || Hq % Hkv != 0 || D <= 0 || !p) return 0;
   CowaHeadWindows hw;
   if (cowa::resolve_windows(Nk, Hkv, p, &hw) != COWA_OK) return 0;
-  return ws_bytes(B, Nq, Nk, Hq, Hkv, D, bwd_parts(B, Nq, Nk, Hkv, Hq / Hkv, hw));
+  return ws_bytes(B, Nq, Nk, Hq, Hkv, D, bwd_plan(B, Nq, Nk, Hkv, Hq / Hkv, hw), hw);
 }
 
 size_t cowa_bwd_workspace_bytes(int B, int T, int Hq, int Hkv, int D, const cowa_params_t* p) {
@@ -1056,11 +1193,11 @@ int cowa_bwd_prefill(const void* q, const void* k, const void* v, const void* o,
   CowaHeadWindows hw;
   int rc = cowa::resolve_windows(Nk, Hkv, p, &hw);
   if (rc != COWA_OK) return rc;
-  const int parts = bwd_parts(B, Nq, Nk, Hkv, Hq / Hkv, hw);
-  if (workspace_bytes < ws_bytes(B, Nq, Nk, Hq, Hkv, D, parts)) return COWA_ERR_WORKSPACE_TOO_SMALL;
+  const BwdPlan pl = bwd_plan(B, Nq, Nk, Hkv, Hq / Hkv, hw);
+  if (workspace_bytes < ws_bytes(B, Nq, Nk, Hq, Hkv, D, pl, hw)) return COWA_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  return D == 128 ? launch_bwd<128>(q, k, v, o, lse, d_o, dq, dk, dv, B, Nq, Nk, Hq, Hkv, p, hw, parts, workspace, st)
-                  : launch_bwd<64>(q, k, v, o, lse, d_o, dq, dk, dv, B, Nq, Nk, Hq, Hkv, p, hw, parts, workspace, st);
+  return D == 128 ? launch_bwd<128>(q, k, v, o, lse, d_o, dq, dk, dv, B, Nq, Nk, Hq, Hkv, p, hw, pl, workspace, st)
+                  : launch_bwd<64>(q, k, v, o, lse, d_o, dq, dk, dv, B, Nq, Nk, Hq, Hkv, p, hw, pl, workspace, st);
 }
 
 int cowa_bwd(const void* q, const void* k, const void* v, const void* o, const float* lse, const void* d_o,
