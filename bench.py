@@ -698,7 +698,7 @@ def run_cuda(args):
         return
 
     # ---- roofline of the dominant kernel ----
-    k_fwd, k_bwd, k_dec = f"cowa_fwd_kernel<{D}, 0>", f"cowa_bwd_kernel<{D}, 0>", f"cowa_decode_split_kernel<{cd['D']}, {cd['Hq'] // cd['Hkv']}, 0>"
+    k_fwd, k_bwd, k_dec = f"cowa_fwd_pair_kernel<{D}, 0, 0>", f"cowa_bwd_kernel<{D}, 0>", f"cowa_decode_split_kernel<{cd['D']}, {cd['Hq'] // cd['Hkv']}>"
     if bwd_ms >= fwd_ms:
         dom, dom_flops, dom_ms = k_bwd, bwd_flops, bwd_main_ms
     else:
