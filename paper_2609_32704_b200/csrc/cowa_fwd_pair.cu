@@ -615,7 +615,7 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
             ml[p].x = ml[p].x == -INFINITY ? 0.f : ex2(ml[p].x - M);
             L = fmaf(ml[p].y, ml[p].x, L);
           }
-        const float inv = L > 0.f ? 1.f / L : 0.f;
+        const float inv = L == 0.f ? 0.f : 1.f / L;  // a NaN sum has to come out as NaN
 #pragma unroll
         for (int p = 0; p < 8; ++p)
           if (p < csize) wgt[tid * csize + p] = ml[p].x * inv;
@@ -632,7 +632,9 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         float4 o[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) o[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int n = (it.work + 1) >> 1;  // steps of the item, shared out as above
         for (int p = 0; p < csize; ++p) {
+          if (n * p / csize == n * (p + 1) / csize) continue;  // a block without a step left no O
           const uint32_t src = map_cluster(aO, p);
           float4 v[U];
 #pragma unroll
@@ -643,10 +645,8 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 #pragma unroll
           for (int u = 0; u < U; ++u) {
             const float w = wgt[min(i0 + u * RPW, per - 1) * csize + p];
-            if (w > 0.f) {  // a block without a step left no O
-              o[u].x = fmaf(v[u].x, w, o[u].x); o[u].y = fmaf(v[u].y, w, o[u].y);
-              o[u].z = fmaf(v[u].z, w, o[u].z); o[u].w = fmaf(v[u].w, w, o[u].w);
-            }
+            o[u].x = fmaf(v[u].x, w, o[u].x); o[u].y = fmaf(v[u].y, w, o[u].y);
+            o[u].z = fmaf(v[u].z, w, o[u].z); o[u].w = fmaf(v[u].w, w, o[u].w);
           }
         }
 #pragma unroll
