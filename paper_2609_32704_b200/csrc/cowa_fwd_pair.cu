@@ -40,10 +40,11 @@ __device__ __forceinline__ uint32_t interval_bits(int a, int b, int base) {
 
 // 2^x of a pair on the FMA and integer pipes: x = n + f with n = rint(x), |f| <= 1/2, 2^f by the polynomial of
 // degree 6 with the least largest relative error on that interval (fitted by reweighted least squares: 1.9e-9, in
-// fp32 8e-8, against 2 ulp of ex2.approx), times 2^n.  Below 2^-126 the result stays 2^-126; NaN stays NaN.
+// fp32 8e-8, against 2 ulp of ex2.approx), times 2^n.  x is held at -127 from below, where the
+// exponent word of 2^n is 0: a masked score (-inf) weighs exactly 0, as ex2.approx gives it; NaN stays NaN.
 __device__ __forceinline__ float2 exp2_fma(float2 x) {
   auto c2 = [](float c) { return make_float2(c, c); };
-  x.x = max_nan(x.x, -126.f); x.y = max_nan(x.y, -126.f);
+  x.x = max_nan(x.x, -127.f); x.y = max_nan(x.y, -127.f);
   const float2 t = add2(x, c2(12582912.f));                        // 1.5 * 2^23: n in the low mantissa bits
   const float2 f = fma2(add2(t, c2(-12582912.f)), c2(-1.f), x);
   float2 p = fma2(c2(1.53458118e-4f), f, c2(1.33999312e-3f));

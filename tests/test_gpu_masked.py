@@ -79,3 +79,15 @@ def test_forward_inf_value_reaches_every_row_that_sees_it(shape):
     v[0, :, 3] = INF  # a sink key: every row sees it, and of a shared item one block only
     o, lse = _forward(q.to(DEV), k.to(DEV), v.to(DEV), sink, local)
     assert not torch.isfinite(o[0]).any() and torch.isfinite(lse).all()
+
+
+@pytest.mark.parametrize("shape", FORWARD)
+def test_forward_masked_keys_weigh_exactly_nothing(shape):
+    B, Nq, Nk, Hq, Hkv, D, sink, local = shape
+    q, k, v = _forward_inputs(B, Nq, Nk, Hq, Hkv, D)
+    clean_o, clean_lse = _forward(q.to(DEV), k.to(DEV), v.to(DEV), sink, local)
+    first = Nq // 2 - (Nk - Nq + Nq // 2) % 64 + 8  # the rows before it see none of the keys from here on: column 8 of a tile
+    assert first > 0 and (Nk - Nq + first) % 64 == 8
+    v[:, :, Nk - Nq + first:] = 3e38
+    o, lse = _forward(q.to(DEV), k.to(DEV), v.to(DEV), sink, local)
+    assert torch.equal(o[:, :, :first], clean_o[:, :, :first]) and torch.equal(lse, clean_lse)
