@@ -215,16 +215,19 @@ size_t cowa_decode_static_capacity(void);
  *   q [B,Nq,Hq,D] in; o [B,Nq,Hq,D] bf16 and lse [B,Nq,Hq] fp32 (may be NULL) out;
  *   kcache, vcache [B,Hkv,Tmax,D] already hold the Nq new tokens; lens: DEVICE int32[B], Nq <= lens[b] <= Tmax.
  * 1 <= Nq <= 64; Hq/Hkv in {1,2,4,8}.  The tokens and heads that share a KV head are the rows of one 128-row tile
- * (more rows take more tiles), so that every visible cache row is read once for up to 128 / (Hq/Hkv) tokens. `workspace`: device, >= cowa_decode_multi_workspace_bytes, 16-byte
- * aligned, no initialisation needed.  cowa_params_t.windows is ignored, as in cowa_decode. */
+ * (more rows take more tiles), so that every visible cache row is read once for up to 128 / (Hq/Hkv) tokens.
+ * Whole tiles of 64 cache rows are loaded, but a row reaches only the tokens that see it, whatever it holds (Inf
+ * and NaN included).  `workspace`: device, >= cowa_decode_multi_workspace_bytes, 16-byte aligned, no initialisation
+ * needed.  cowa_params_t.windows is ignored, as in cowa_decode. */
 int cowa_decode_multi(const void* q, const void* kcache, const void* vcache, const int32_t* lens,
                       void* o, float* lse, int B, int Nq, int Tmax, int Hq, int Hkv, int D,
                       const cowa_params_t* p, void* workspace, size_t workspace_bytes, void* stream);
 
 /* The same over a paged KV cache (not in the paper: a serving-side memory layout).
  *   kpages, vpages [num_pages, Hkv, page_size, D] bf16; block_table: DEVICE int32 [B, max_pages], entry
- *   [b, i] = page holding tokens [i*page_size, (i+1)*page_size) of sequence b (entries past the sequence's
- *   last page are not read); page_size a multiple of 16; lens[b] <= max_pages * page_size.
+ *   [b, i] = page holding tokens [i*page_size, (i+1)*page_size) of sequence b (entries of pages without a key
+ *   that a token of the call sees in one of its heads are not read: past the sequence's last page, or between the
+ *   windows); page_size a multiple of 16; lens[b] <= max_pages * page_size.
  * Other arguments, Nq included (Nq = 1 is plain paged decode), as for cowa_decode_multi; workspace size from
  * cowa_decode_multi_workspace_bytes with Tmax = max_pages * page_size.  Page indices are not range-checked. */
 int cowa_decode_paged(const void* q, const void* kpages, const void* vpages, const int32_t* block_table,

@@ -8,7 +8,9 @@
 // row states (reference max, sum, un-normalised O, fp32) in the workspace and a second kernel merges a unit's pieces.
 // Bound by HBM: 32 KB per step; two blocks per SM take a step in about 1600 clocks each, twice the rate at which HBM
 // feeds them.
-// Warps 0-3: softmax, one row per thread (only as many warps as there are rows); warp 4: TMA; warp 5: MMA issue.
+// Warps 0-3: softmax, one row per thread (only as many warps as there are rows); warp 4: TMA; warp 5: MMA issue.  V rows
+// that no token sees are cleared by warp 3 beside the softmax, by all four warps when a tile has rows for each of them
+// (a warp of its own would leave the threads 128 registers, and they spill).
 #include <cuda_bf16.h>
 #include <string.h>
 
@@ -70,10 +72,41 @@ struct Piece {
 };
 static_assert(sizeof(Piece) <= 128, "slot of a published piece");
 
+// Key tile of step t of a piece, and whether every token sees all of it.
+__device__ __forceinline__ int tile_of(const Piece& pc, int t, bool* full) {
+  const int i = pc.t0 + t, n0 = cowa_range_len(pc.u.rg[0]), n1 = n0 + cowa_range_len(pc.u.rg[1]);
+  const int j = i < n0 ? pc.u.rg[0].hi - i : i < n1 ? pc.u.rg[1].hi + n0 - i : pc.u.rg[2].hi + n1 - i;
+  const int lo = i < n0 ? pc.f_lo[0] : i < n1 ? pc.f_lo[1] : pc.f_lo[2];
+  const int hi = i < n0 ? pc.f_hi[0] : i < n1 ? pc.f_hi[1] : pc.f_hi[2];
+  *full = j >= lo && j <= hi;
+  return j;
+}
+
 __device__ __forceinline__ uint32_t interval_bits(int a, int b, int base) {
   int lo = max(a - base, 0), hi = min(b - base, 31);
   if (lo > hi) return 0u;
   return (0xFFFFFFFFu >> (31 - (hi - lo))) << lo;
+}
+
+// The keys that tokens at key positions p0 .. p1 (p0 >= 0) see, some of them (first = p0, last = p1) or each of them by
+// the same window (first = p1, last = p0), in the 64 keys from `row0` on: one bit per key.
+__device__ __forceinline__ unsigned long long seen_bits(const CowaWin& w, int first, int last, int row0) {
+  uint32_t m[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int base = row0 + q * 32;
+    m[q] = interval_bits(max(first - w.n + 1, 0), last, base) | interval_bits(0, min(w.s - 1, last), base);
+    if (w.l > 0) m[q] |= interval_bits(first - (w.n + w.g + w.l) + 1, last - (w.n + w.g), base);
+  }
+  return (unsigned long long)m[1] << 32 | m[0];
+}
+// Keys of a unit that some token sees.  Other rows of the cache are nobody's: they may be stale, non-finite, or lie in pages
+// that were handed to somebody else.
+__device__ __forceinline__ unsigned long long seen_by_some(const Unit& u, int row0) {
+  return seen_bits(u.w, max(u.off + u.tok0, 0), u.off + u.tok1 - 1, row0);
+}
+__device__ __forceinline__ unsigned long long seen_by_all(const Unit& u, int row0) {
+  return seen_bits(u.w, u.off + u.tok1 - 1, max(u.off + u.tok0, 0), row0);
 }
 
 // QR rows of Q and NS slots each for K and V: 128 and 2, or, when a tile has at most 32 rows (S and O of the other rows
@@ -84,6 +117,40 @@ struct TileSmem {
   static constexpr int oQ = 0, oK = kQ, oV = oK + NS * kKV, oBar = oV + NS * kKV, oPiece = oBar + 256, oScan = oPiece + 256;
   static constexpr int kBytes = oScan + 64 + 1024;  // + alignment slack
 };
+
+// a pair of bf16 holds an Inf or a NaN
+__device__ __forceinline__ bool nonfinite(uint32_t x) { return (x & 0x7F80u) == 0x7F80u || (x & 0x7F800000u) == 0x7F800000u; }
+
+// O += P V of one step on the FMA pipe, each row over the keys it sees (mk): for tiles whose V holds an Inf or a NaN.
+template <int D>
+__device__ __forceinline__ void add_seen(const uint8_t* vt, uint32_t t_P, uint32_t t_O, unsigned long long mk) {
+#pragma unroll 1
+  for (int q = 0; q < D / 16; ++q) {
+    uint32_t ov[16], pw;
+    tmem_ld16(t_O + q * 16, ov);
+#pragma unroll 1
+    for (int r = 0; r < BK; ++r) {
+      tmem_ld1(t_P + (r >> 1), pw);
+      tmem_wait_ld();
+      const float p = __uint_as_float(r & 1 ? pw & 0xFFFF0000u : pw << 16);
+      const uint8_t* row = vt + (q >> 2) * (BK * 128) + r * 128;
+      const bool sees = (mk >> r) & 1ull;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint4 x = *reinterpret_cast<const uint4*>(row + ((((q & 3) * 2 + h) ^ (r & 7)) << 4));
+        const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const float y = __uint_as_float(e & 1 ? xs[e >> 1] & 0xFFFF0000u : xs[e >> 1] << 16);
+          const float o = __uint_as_float(ov[h * 8 + e]);
+          ov[h * 8 + e] = __float_as_uint(sees ? fmaf(p, y, o) : o);
+        }
+      }
+    }
+    tmem_st16(t_O + q * 16, ov);
+  }
+  tmem_wait_st();
+}
 
 template <int D, int QR, int NS>
 __global__ void __launch_bounds__(kThreads, 2)
@@ -106,15 +173,17 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   uint64_t* bar_pv = bars + 2;        //     O += P V of a step has completed
   uint64_t* bar_s = bars + 3;         // [2] S of a step is in TMEM buffer b
   uint64_t* bar_i_full = bars + 5;    // [2] a piece has been published
-  uint64_t* bar_i_empty = bars + 7;   // [2] count nw + 1: it has been read
+  uint64_t* bar_i_empty = bars + 7;   // [2] count nw + 1, + 1 with a warp 3 that clears: it has been read
   uint64_t* bar_p = bars + 9;         // [2] count nw: P written over S
-  uint64_t* bar_o_empty = bars + 11;  //     count nw: O of a piece has been read
+  uint64_t* bar_v_read = bars + 11;   //     count nw: add_seen has read a V tile
   uint64_t* bar_k_full = bars + 12;             // [NS]
   uint64_t* bar_k_empty = bar_k_full + NS;      // [NS]
   uint64_t* bar_v_full = bar_k_full + 2 * NS;   // [NS]
   uint64_t* bar_v_empty = bar_k_full + 3 * NS;  // [NS]
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bar_k_full + 4 * NS);
-  int* scan = reinterpret_cast<int*>(smem + SM::oScan);  // 6 warp totals, then first unit and its list position
+  uint64_t* bar_v_seen = bar_k_full + 4 * NS;   // [NS] count 1, or 4: V rows that no token sees are cleared
+  uint64_t* bar_v_go = bar_k_full + 5 * NS;     // [NS] V of a boundary tile is on its way (warp 3 passes other steps by)
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bar_k_full + 6 * NS);
+  int* scan = reinterpret_cast<int*>(smem + SM::oScan);  // 6 warp totals; [8], [9] first unit and its list position; [10 ..] per slot: step whose V is not finite
 
   // the merge kernel may start as soon as every block of this grid has (it waits for this grid's results itself)
   asm volatile("griddepcontrol.launch_dependents;");
@@ -124,8 +193,11 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 
   if (tid == 128) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); }
   if (tid == 0) {
-    for (int s = 0; s < 12 + 4 * NS; ++s)
-      mbar_init(bars + s, s == 7 || s == 8 ? nw + 1 : s >= 9 && s < 12 ? nw : 1);
+    for (int s = 0; s < 12 + 6 * NS; ++s) {
+      const bool v_seen = bars + s >= bar_v_seen && bars + s < bar_v_go;
+      mbar_init(bars + s, s == 7 || s == 8 ? min(nw + 2, 5) : s >= 9 && s < 12 ? nw : v_seen && nw == 4 ? 4 : 1);
+    }
+    for (int s = 0; s < NS; ++s) scan[10 + s] = 0;
     fence_mbar_init();
   }
   if (warp == 5) {
@@ -195,6 +267,29 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     return pc.n > 0;
   };
 
+  // Boundary tiles, once V is in `slot`: clears the rows that no token sees and looks through those that not every token
+  // sees; scan[10 + slot] becomes c + 1 (of step c) when one of these holds an Inf or a NaN.  Warp wi of n.
+  auto clear_unseen = [&](const Unit& u, int j, int slot, int c, int wi, int n) {
+    constexpr int CPR = D / 8, RPI = 32 / CPR;  // 16-byte chunks per row, rows per pass of a warp
+    const int ch = lane % CPR;
+    const unsigned long long some = seen_by_some(u, j * BK), all = seen_by_all(u, j * BK);
+    uint8_t* vt = sV + slot * SM::kKV + (ch >> 3) * SLAB_K;
+    bool bad = false;
+#pragma unroll 4
+    for (int r = wi * RPI + lane / CPR; r < BK; r += n * RPI) {
+      uint4* x = reinterpret_cast<uint4*>(vt + r * 128 + (((ch & 7) ^ (r & 7)) << 4));
+      if (!((some >> r) & 1ull)) {
+        *x = make_uint4(0u, 0u, 0u, 0u);
+      } else if (!((all >> r) & 1ull)) {
+        const uint4 y = *x;
+        bad = bad || nonfinite(y.x) || nonfinite(y.y) || nonfinite(y.z) || nonfinite(y.w);
+      }
+    }
+    fence_proxy_async_smem();
+    if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) *(volatile int*)(scan + 10 + slot) = c + 1;
+    warp_arrive(bar_v_seen + slot);
+  };
+
   if (warp == 4) {
     // ======================= TMA producer =======================
     const bool lead = elect_one();
@@ -236,12 +331,14 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       __syncwarp();
       if (pc.n == 0) break;
 
-      // One 64-row tile.  Paged cache: every lane looks up the page of its box (box rows of one page) and loads it;
-      // boxes past the sequence's last key are left out (their table entries may be anything).
+      // One 64-row tile.  Paged cache: every lane looks up the page of its box (box rows of one page) and loads it; boxes
+      // without a key that a token sees are left out (their table entries may be anything): page -1.
       const int boxes = a.block_table ? BK / a.box : 1;
       auto page_of = [&](int t) -> int {
-        const int row = cowa_fwd_tile_at(pc.u.rg, pc.t0 + t) * BK + lane * a.box;
-        return lane < boxes && row < pc.u.Nk ? a.block_table[(size_t)pc.u.b * a.max_pages + row / a.page_size] : 0;
+        const int row0 = cowa_fwd_tile_at(pc.u.rg, pc.t0 + t) * BK, row = row0 + lane * a.box;
+        const unsigned long long box_mask = (a.box == 64 ? ~0ull : (1ull << a.box) - 1) << (lane * a.box & 63);
+        if (lane >= boxes || !(seen_by_some(pc.u, row0) & box_mask)) return -1;
+        return max(a.block_table[(size_t)pc.u.b * a.max_pages + row / a.page_size], 0);
       };
       auto load = [&](uint8_t* dst, const CUtensorMap* tm, uint64_t* bar, int t, int page) {
         const int row0 = cowa_fwd_tile_at(pc.u.rg, pc.t0 + t) * BK;
@@ -251,16 +348,16 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             for (int s = 0; s < NSLAB; ++s) tma_load_4d(dst + s * SLAB_K, tm, bar, s * 64, row0, pc.u.hk, pc.u.b);
           }
         } else {
-          const int live = min(boxes, (pc.u.Nk - row0 + a.box - 1) / a.box);
-          if (lead) mbar_expect_tx(bar, live * a.box * D * 2);
+          const unsigned live = __ballot_sync(0xFFFFFFFFu, page >= 0);
+          if (lead) mbar_expect_tx(bar, __popc(live) * a.box * D * 2);
           __syncwarp();
-          if (lane < live)
+          if (page >= 0)
             for (int s = 0; s < NSLAB; ++s)
               tma_load_4d(dst + s * SLAB_K + lane * a.box * 128, tm, bar, s * 64, (row0 + lane * a.box) % a.page_size, pc.u.hk,
                           page);
         }
       };
-      int page = a.block_table ? page_of(0) : 0;
+      int page = a.block_table ? page_of(0) : 0;  // this lane's page of the next tile
       for (int t = 0; t < pc.n; ++t) {
         if (rnd > 0) ok = mbar_wait(bar_k_empty + sl, (rnd - 1) & 1, a.status);
         if (!ok) break;
@@ -279,6 +376,9 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         if (rnd > 0) ok = mbar_wait(bar_v_empty + sl, (rnd - 1) & 1, a.status);
         if (!ok) break;
         load(sV + sl * SM::kKV, &tmV, bar_v_full + sl, t, page);
+        bool full;
+        tile_of(pc, t, &full);
+        if (lead && !full) mbar_arrive(bar_v_go + sl);
         page = next;
         if (++sl == NS) { sl = 0; ++rnd; }
       }
@@ -323,7 +423,6 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       for (int t = 0; t < n && ok; ++t, ++c) {
         const int b_ = c & 1;
         if (t + 1 < n) issue_s(b_ ^ 1, t + 2 == n);  // its buffer last held P(c - 1), whose product was issued before
-        if (t == 0 && ni > 0) ok = ok && mbar_wait(bar_o_empty, (ni - 1) & 1, a.status);
         ok = ok && mbar_wait(bar_v_full + vs, vr, a.status) && mbar_wait(bar_p + b_, (c >> 1) & 1, a.status);
         if (!ok) break;
         tc_fence_after();
@@ -331,7 +430,7 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           const uint64_t dB = dV0 + vs * kKV16;
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk)
-            mma_ts(tb + cO, tb + b_ * 64 + kk * 8, dB + ((kk * 2048) >> 4), IDESC_O, (t > 0 || kk > 0) ? 1u : 0u);
+            mma_ts(tb + cO, tb + b_ * 64 + kk * 8, dB + ((kk * 2048) >> 4), IDESC_O, 1u);
           mma_commit(bar_pv);
           mma_commit(bar_v_empty + vs);
         }
@@ -345,6 +444,7 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
     int c = 0, vs = 0;    // steps so far; slot of this step's V
     uint32_t vr = 0;      // parity of its load
+    uint32_t zr = 0;      // parities of bar_v_seen (bit per slot) and bar_v_read (bit 31)
     uint32_t ni = 0;
     Piece pc;
     for (; ok && next_piece(ni, pc); ++ni) {
@@ -354,13 +454,18 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       const int rowpos = pc.u.off + tok;  // position of this query on the key axis
       const CowaWin w = pc.u.w;
       float m_ref = -INFINITY, l_sum = 0.f;
-      const int n0 = cowa_range_len(pc.u.rg[0]), n1 = n0 + cowa_range_len(pc.u.rg[1]);
+      {  // every product of the piece adds to O (the first one waits for this warp's P)
+        uint32_t zero[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) zero[e] = 0u;
+#pragma unroll
+        for (int q = 0; q < D / 16; ++q) tmem_st16(t_O + q * 16, zero);
+      }
 
       for (int t = 0; t < n && ok; ++t, ++c) {
-        const int b_ = c & 1, i = pc.t0 + t;
-        const int j = i < n0 ? pc.u.rg[0].hi - i : i < n1 ? pc.u.rg[1].hi + n0 - i : pc.u.rg[2].hi + n1 - i;
-        const int fl = i < n0 ? pc.f_lo[0] : i < n1 ? pc.f_lo[1] : pc.f_lo[2];
-        const int fh = i < n0 ? pc.f_hi[0] : i < n1 ? pc.f_hi[1] : pc.f_hi[2];
+        const int b_ = c & 1;
+        bool full;
+        const int j = tile_of(pc, t, &full);
         const uint32_t t_S = t_lane + b_ * 64;
 
         ok = mbar_wait(bar_s + b_, (c >> 1) & 1, a.status);
@@ -370,18 +475,19 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         tmem_ld32(t_S, sr[0]);
         tmem_ld32(t_S + 32, sr[1]);
         tmem_wait_ld();
-        if (__builtin_expect(!(j >= fl && j <= fh), 0)) {
+        uint32_t mk[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};  // keys this row sees
+        if (__builtin_expect(!full, 0)) {
           const int kend = row_valid ? min(rowpos, Nk - 1) : -1;  // last causal key of this row
           const int near_lo = rowpos - w.n + 1, sink_hi = min(w.s - 1, kend);
           const int long_hi = w.l > 0 ? min(rowpos - (w.n + w.g), kend) : -1, long_lo = rowpos - (w.n + w.g + w.l) + 1;
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
             const int base_ = j * BK + q * 32;
-            const uint32_t mk =
+            mk[q] =
                 interval_bits(near_lo, kend, base_) | interval_bits(0, sink_hi, base_) | interval_bits(long_lo, long_hi, base_);
 #pragma unroll
             for (int e = 0; e < 32; ++e)
-              if (!((mk >> e) & 1u)) sr[q][e] = 0xFF800000u;  // -inf
+              if (!((mk[q] >> e) & 1u)) sr[q][e] = 0xFF800000u;  // -inf
           }
         }
         float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
@@ -433,18 +539,30 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         }
         tmem_st32(t_S, pk);  // P over the first 32 columns of this S buffer
         tmem_wait_st();
-        // Rows of the tile after the sequence's last key hold whatever the cache or an earlier tile left there.  P is
-        // exactly zero there, but 0 x (Inf or NaN) in the product would not be, so they are cleared first.
-        const int vrows = Nk - j * BK;
-        if (__builtin_expect(vrows < BK, 0)) {
-          ok = mbar_wait(bar_v_full + vs, vr, a.status);
+        // P is exactly zero where a row does not see a key, but 0 x (Inf or NaN) in the product would not be: V rows that
+        // no token sees have been cleared; where a row that some see holds such a value, every row takes the
+        // keys it sees in add_seen, and the product gets zeros.
+        if (__builtin_expect(!full, 0)) {
+          if (nw == 4) {
+            ok = mbar_wait(bar_v_full + vs, vr, a.status);
+            if (!ok) break;
+            clear_unseen(pc.u, j, vs, c, warp, 4);
+          }
+          ok = mbar_wait(bar_v_seen + vs, (zr >> vs) & 1, a.status);
           if (!ok) break;
-          uint8_t* vt = sV + vs * SM::kKV;
-          const int nchunk = (BK - vrows) * 8;  // 16-byte chunks per slab
-          for (int s_ = 0; s_ < NSLAB; ++s_)
-            for (int c_ = tid; c_ < nchunk; c_ += nw * 32)
-              *reinterpret_cast<uint4*>(vt + s_ * SLAB_K + vrows * 128 + c_ * 16) = make_uint4(0u, 0u, 0u, 0u);
-          fence_proxy_async_smem();
+          zr ^= 1u << vs;
+          if (__builtin_expect(*(volatile int*)(scan + 10 + vs) == c + 1, 0)) {
+            uint8_t* vt = sV + vs * SM::kKV;
+            __syncwarp();
+            add_seen<D>(vt, t_S, t_O, (unsigned long long)mk[1] << 32 | mk[0]);
+            warp_arrive(bar_v_read);
+            ok = mbar_wait(bar_v_read, zr >> 31, a.status);
+            if (!ok) break;
+            zr ^= 1u << 31;
+            for (int c_ = tid; c_ < SM::kKV / 16; c_ += nw * 32)
+              *reinterpret_cast<uint4*>(vt + c_ * 16) = make_uint4(0u, 0u, 0u, 0u);
+            fence_proxy_async_smem();
+          }
         }
         tc_fence_before();
         warp_arrive(bar_p + b_);
@@ -468,9 +586,27 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           for (int e = 0; e < 4; ++e) dst[e] = make_uint4(ov[e * 4], ov[e * 4 + 1], ov[e * 4 + 2], ov[e * 4 + 3]);
         }
       }
-      tc_fence_before();
-      warp_arrive(bar_o_empty);
       if (row_valid) a.ws_ml[srow] = make_float2(m_ref, l_sum);
+    }
+  } else if (warp == 3) {
+    // ======================= boundary tiles, beside fewer than four softmax warps =======================
+    // The TMA warp says when a tile of its kind is on its way: this warp passes the other steps by, and a wait for V alone
+    // could meet the slot's load of two rounds before, which has the same parity.
+    int c = 0, vs = 0;
+    uint32_t vr = 0, gr = 0;  // parity of the slot's load; parities of bar_v_go, a bit per slot
+    Piece pc;
+    for (uint32_t ni = 0; ok && next_piece(ni, pc); ++ni) {
+      for (int t = 0; t < pc.n; ++t, ++c) {
+        bool full;
+        const int j = tile_of(pc, t, &full);
+        if (!full) {
+          ok = mbar_wait(bar_v_go + vs, (gr >> vs) & 1, a.status) && mbar_wait(bar_v_full + vs, vr, a.status);
+          if (!ok) break;
+          gr ^= 1u << vs;
+          clear_unseen(pc.u, j, vs, c, 0, 1);
+        }
+        if (++vs == NS) { vs = 0; vr ^= 1; }
+      }
     }
   }
 

@@ -1,5 +1,6 @@
 """What a row sees must reach it, and what it does not see must not: NaN, Inf and huge values in q, k and v through every
-kernel of the forward.  A row that sees a NaN is NaN; a row that does not is the row computed without it."""
+kernel of the forward and of the multi-token / paged decode.  A row that sees a NaN is NaN; a row that does not is the
+row computed without it."""
 import numpy as np
 import pytest
 import torch
@@ -7,6 +8,7 @@ import torch
 import cowa_inputs
 import paper_2609_32704_b200 as cowa
 from oracle import cowa_oracle as orc
+from test_gpu_parity import TOL_LSE, check
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -91,3 +93,112 @@ def test_forward_masked_keys_weigh_exactly_nothing(shape):
     v[:, :, Nk - Nq + first:] = 3e38
     o, lse = _forward(q.to(DEV), k.to(DEV), v.to(DEV), sink, local)
     assert torch.equal(o[:, :, :first], clean_o[:, :, :first]) and torch.equal(lse, clean_lse)
+
+
+# ------------------------------------------------------------------ decode of several tokens, contiguous and paged
+
+def _decode(q, kc, vc, lens, params, page=None, hide=None):
+    """o, lse of the call; with `page`, the cache goes through a pool of pages, and hide(i) says that page i of a sequence
+    is handed out to another request (a page of NaN)."""
+    B, Nq, Hq, D = q.shape
+    Hkv, Tmax = kc.shape[1], kc.shape[2]
+    o = torch.full_like(q, 7.0).to(DEV)
+    lse = torch.full((B, Nq, Hq), 7.0, dtype=torch.float32, device=DEV)
+    lens_d = torch.tensor(lens, dtype=torch.int32, device=DEV)
+    if page is None:
+        nbytes = cowa.cowa_decode_multi_workspace_bytes(B, Nq, Tmax, Hq, Hkv, D, params)
+        ws = torch.full((nbytes,), 0xFF, dtype=torch.uint8, device=DEV)
+        cowa.cowa_decode_multi(q.to(DEV), kc.to(DEV), vc.to(DEV), lens_d, o, lse, params, ws)
+    else:
+        assert Tmax % page == 0
+        npg = Tmax // page
+        other = B * npg  # the other request's page
+        table = torch.arange(B * npg, dtype=torch.int32).reshape(B, npg)
+        kp = torch.full((B * npg + 1, Hkv, page, D), NAN, dtype=torch.bfloat16)
+        vp = torch.full_like(kp, NAN)
+        for b in range(B):
+            for i in range(npg):
+                if hide is not None and hide(b, i):
+                    table[b, i] = other
+                else:
+                    kp[b * npg + i], vp[b * npg + i] = kc[b, :, i * page:(i + 1) * page], vc[b, :, i * page:(i + 1) * page]
+        nbytes = cowa.cowa_decode_multi_workspace_bytes(B, Nq, Tmax, Hq, Hkv, D, params)
+        ws = torch.full((nbytes,), 0xFF, dtype=torch.uint8, device=DEV)
+        cowa.cowa_decode_paged(q.to(DEV), kp.to(DEV), vp.to(DEV), table.to(DEV), lens_d, o, lse, params, ws)
+    torch.cuda.synchronize()
+    cowa.cowa_check_device_status()
+    return o.float().cpu(), lse.cpu()
+
+
+def _decode_inputs(B, Nq, Tmax, Hq, Hkv, D):
+    q = cowa_inputs.make_train_inputs(103, B, Nq, Hq, Hkv, D)[0].permute(0, 2, 1, 3).contiguous()
+    _, kc, vc, _ = cowa_inputs.make_decode_inputs(104, B, Tmax, Hq, Hkv, D, Tmax, Tmax)
+    return q, kc, vc
+
+
+DECODE = [  # B, Nq, Tmax, Hq, Hkv, D, sink, local, lens, global heads, offset
+    (2, 3, 4096, 16, 2, 128, 20, 100, [4001, 2222], 16, 5),  # eight heads per group
+    (1, 5, 3072, 8, 2, 128, 7, 70, [3000], 2, 0),            # four
+    (2, 8, 2048, 4, 4, 64, 4, 33, [2048, 130], 8, 4),        # one head, D = 64
+    (1, 20, 4096, 8, 1, 128, 100, 300, [3777], 8, 6),        # two row tiles
+    (6, 2, 8192, 16, 8, 64, 16, 5000, [8192, 8000, 7777, 6500, 8100, 7001], 8, 0),  # many steps between boundary tiles
+]
+
+
+@pytest.mark.parametrize("case", DECODE)
+@pytest.mark.parametrize("bad", [NAN, INF])
+@pytest.mark.parametrize("page", [None, 16, 64])
+def test_decode_keys_that_no_token_sees(case, bad, page):
+    """Rows that no token of the call sees hold non-finite values, and pages that no head sees belong to somebody else."""
+    B, Nq, Tmax, Hq, Hkv, D, sink, local, lens, hg, off = case
+    q, kc, vc = _decode_inputs(B, Nq, Tmax, Hq, Hkv, D)
+    scale = cowa_inputs.softmax_scale(D)
+    params = cowa.make_params(sink=sink, local=local, softmax_scale=scale, hkv_global=hg, hkv_offset=off)
+    kb, vb, used = kc.clone(), vc.clone(), {}
+    for b in range(B):
+        ws = orc.default_windows(lens[b], hg, sink, local)[off:off + Hkv]
+        for h in range(Hkv):
+            seen = _sees(ws[h], np.arange(Nq), lens[b] - Nq, np.arange(Tmax)).any(0)
+            assert not seen[:lens[b]].all()
+            kb[b, h, ~seen], vb[b, h, ~seen] = bad, bad
+            used[b] = used.get(b, False) | seen
+    o, lse = _decode(q, kb, vb, lens, params, page, lambda b, i: not used[b][i * page:(i + 1) * page].any())
+    f = cowa_inputs.to_f64
+    for b in range(B):
+        n = lens[b]
+        ws = orc.default_windows(n, hg, sink, local)[off:off + Hkv]
+        o_ref, lse_ref = orc.forward(f(q[b].permute(1, 0, 2)), f(kc[b, :, :n]), f(vc[b, :, :n]), ws, scale)
+        check(f"lse[b={b}]", lse[b].permute(1, 0).numpy(), lse_ref, TOL_LSE, TOL_LSE)
+        check(f"o[b={b}]", o[b].permute(1, 0, 2).numpy(), o_ref)
+
+
+@pytest.mark.parametrize("case", DECODE)
+@pytest.mark.parametrize("where", ["q", "k", "v"])
+@pytest.mark.parametrize("page", [None, 16])
+def test_decode_nan_reaches_the_tokens_that_see_it_and_no_other(case, where, page):
+    B, Nq, Tmax, Hq, Hkv, D, sink, local, lens, hg, off = case
+    q, kc, vc = _decode_inputs(B, Nq, Tmax, Hq, Hkv, D)
+    params = cowa.make_params(sink=sink, local=local, softmax_scale=cowa_inputs.softmax_scale(D), hkv_global=hg, hkv_offset=off)
+    clean_o, clean_lse = _decode(q, kc, vc, lens, params, page)
+    t = Nq // 2
+    # the key of token t, and one at the far edge of the near window: the later tokens do not see it any more
+    for key in (lens[0] - Nq + t, lens[0] - Nq + t - local + 1):
+        qb, kb, vb = q.clone(), kc.clone(), vc.clone()
+        if where == "q":
+            qb[0, t] = NAN
+        else:
+            (kb if where == "k" else vb)[0, :, key] = NAN
+        o, lse = _decode(qb, kb, vb, lens, params, page)
+        for h in range(Hq):
+            w = orc.default_windows(lens[0], hg, sink, local)[off + h * Hkv // Hq]
+            hit = np.arange(Nq) == t if where == "q" else _sees(w, np.arange(Nq), lens[0] - Nq, [key])[:, 0]
+            assert hit[t]
+            assert torch.isnan(o[0, hit, h]).all(), f"head {h}: a NaN in {where} came out as a number"
+            # the masked weights are exactly zero, so the other tokens differ by the order of their sums at most
+            assert torch.isfinite(o[0, ~hit, h]).all()
+            assert torch.allclose(o[0, ~hit, h], clean_o[0, ~hit, h], rtol=2.0 ** -7, atol=2.0 ** -8)
+            if where != "v":
+                assert torch.isnan(lse[0, hit, h]).all()
+            assert torch.equal(lse[0, ~hit, h], clean_lse[0, ~hit, h])
+        for b in range(1, B):
+            assert torch.equal(o[b], clean_o[b]) and torch.equal(lse[b], clean_lse[b])
