@@ -100,3 +100,48 @@ def test_packed(seqs, Hq, Hkv, D, bad):
 ])
 def test_decode_tiles(B, Nq, Tmax, Hq, Hkv, D, sink, local, lens, page):
     multi_case(B, Nq, Tmax, Hq, Hkv, D, sink, local, lens, page_size=page)
+
+
+@pytest.mark.parametrize("Nq,page", [(4, None), (1, 64)])
+def test_decode_tiles_round_weights_below_an_exact_maximum(Nq, page):
+    """The error against 64 bits is no larger than that of exact arithmetic whose weights are rounded to bf16 below the
+    exact maximum of every 256 visible keys, as the single-token kernel rounds them (2 % for the fp32 sums and for which
+    keys share a maximum; a reference that lags by up to 2^8 is off by 6 % more)."""
+    B, Tmax, Hq, Hkv, D, sink, local = 6, 8192, 16, 8, 64, 64, 6000  # about twenty steps per block
+    lens = [8192, 8000, 7777, 8100, 8191, 7900]
+    q = cowa_inputs.make_train_inputs(95, B, Nq, Hq, Hkv, D)[0].permute(0, 2, 1, 3).contiguous()
+    _, kc, vc, _ = cowa_inputs.make_decode_inputs(96, B, Tmax, Hq, Hkv, D, Tmax, Tmax)
+    scale = cowa_inputs.softmax_scale(D)
+    params = cowa.make_params(sink=sink, local=local, softmax_scale=scale)
+    o = torch.full_like(q, float("nan")).to(DEV)
+    ws = torch.empty(cowa.cowa_decode_multi_workspace_bytes(B, Nq, Tmax, Hq, Hkv, D, params), dtype=torch.uint8, device=DEV)
+    lens_d = torch.tensor(lens, dtype=torch.int32, device=DEV)
+    if page is None:
+        cowa.cowa_decode_multi(q.to(DEV), kc.to(DEV), vc.to(DEV), lens_d, o, None, params, ws)
+    else:
+        n = Tmax // page
+        table = torch.arange(B * n, dtype=torch.int32, device=DEV).reshape(B, n)
+        pages = lambda x: x.reshape(B, Hkv, n, page, D).transpose(1, 2).reshape(B * n, Hkv, page, D).to(DEV)  # noqa: E731
+        cowa.cowa_decode_paged(q.to(DEV), pages(kc), pages(vc), table, lens_d, o, None, params, ws)
+    torch.cuda.synchronize()
+    cowa.cowa_check_device_status()
+    f = cowa_inputs.to_f64
+    bf16 = lambda x: torch.from_numpy(x).to(torch.bfloat16).double().numpy()  # noqa: E731
+    err = bound = 0.0
+    for b in range(B):
+        n, ws_ = lens[b], orc.default_windows(lens[b], Hkv, sink, local)
+        want, _ = orc.forward(f(q[b].permute(1, 0, 2)), f(kc[b, :, :n]), f(vc[b, :, :n]), ws_, scale)
+        err += np.sum((f(o[b].permute(1, 0, 2)) - want) ** 2)
+        for h in range(Hq):
+            k, v, (s, near, gap, width) = f(kc[b, h * Hkv // Hq, :n]), f(vc[b, h * Hkv // Hq, :n]), ws_[h * Hkv // Hq]
+            for t in range(Nq):
+                d = n - Nq + t - np.arange(n)
+                seen = (d >= 0) & ((d < near) | (np.arange(n) < s) | ((d >= near + gap) & (d < near + gap + width)))
+                x, vs = k[seen] @ f(q[b, t, h]) * scale, v[seen]
+                acc, total = 0.0, 0.0
+                for i in range(0, len(x), 256):
+                    w = np.exp(x[i:i + 256] - x[i:i + 256].max())
+                    up = np.exp(x[i:i + 256].max() - x.max())
+                    acc, total = acc + up * (bf16(w) @ vs[i:i + 256]), total + up * w.sum()
+                bound += np.sum((bf16(acc / total) - want[h, t]) ** 2)
+    assert err <= 1.02 ** 2 * bound
