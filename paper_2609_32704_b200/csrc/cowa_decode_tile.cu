@@ -807,6 +807,7 @@ extern "C" {
 
 size_t cowa_decode_multi_workspace_bytes(int B, int Nq, int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p) {
   if (!p || B <= 0 || Nq <= 0 || Tmax <= 0 || Hq <= 0 || Hkv <= 0 || Hq % Hkv != 0 || (D != 64 && D != 128)) return 0;
+  if (Hq / Hkv > BQ) return 0;  // a group that does not fit a row tile (the calls take groups of up to 8)
   return plan_of(B, Nq, Tmax, Hq, Hkv, D, p).bytes;
 }
 

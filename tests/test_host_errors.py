@@ -85,6 +85,14 @@ def test_decode_calls_refuse_misaligned_or_small_workspace():
                                None) == TOO_SMALL
 
 
+def test_workspace_query_of_groups_the_decode_calls_do_not_take():
+    p = _p()
+    for D_ in (64, 128):
+        assert cowa.cowa_decode_multi_workspace_bytes(1, 1, 512, 256, 1, D_, p) == 0
+        assert cowa.cowa_decode_multi_workspace_bytes(2, 4, 512, 129, 1, D_, p) == 0
+        assert cowa.cowa_decode_multi_workspace_bytes(1, 1, 512, 128, 1, D_, p) > 0
+
+
 def test_scale_and_window_arguments():
     L = cowa.lib()
     a = _ptrs(6)
