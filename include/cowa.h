@@ -91,7 +91,7 @@ typedef struct {
   int64_t q_strides[3], k_strides[3], v_strides[3], o_strides[3];
   /* cowa_bwd / cowa_bwd_prefill / cowa_bwd_varlen only: optional CUDA events (cudaEvent_t handles owned by the
    * caller, or NULL) recorded on the call's stream just before and just after the main backward kernel
-   * (Algorithm 2's loops), so that a profiler can time that kernel apart from the preprocess, memset and
+   * (Algorithm 2's loops), so that a profiler can time that kernel apart from the preprocess and
    * conversion launches of the same call. */
   void* bwd_main_start_event;
   void* bwd_main_stop_event;
@@ -137,7 +137,8 @@ int cowa_prefill_varlen(const void* q, const void* k, const void* v, void* o, fl
  * bitwise reproducible; for dq see cowa_params_t.deterministic.
  * `workspace` (device, >= cowa_bwd_workspace_bytes for the same B, T, Hq, Hkv, D and params, 16-byte
  * aligned) holds the fp32 dq accumulator, the row vector rowsum(o*d_o) (Algorithm 2 line 13) and those
- * partial sums; it needs no initialisation. */
+ * partial sums (up to seven slots of 256 D floats per SM, nine in the packed call: 136 and 175 MB at D = 128; up to 14
+ * where the packed call's size is asked for without parameters); it needs no initialisation. */
 int cowa_bwd(const void* q, const void* k, const void* v, const void* o, const float* lse,
              const void* d_o, void* dq, void* dk, void* dv,
              int B, int T, int Hq, int Hkv, int D, const cowa_params_t* p,

@@ -898,37 +898,12 @@ void plan_rest(BwdPlan& pl, long long rest, double avg, double share) {
   }
 }
 
-// Blocks per KV tile when whole heads of a group are spread: the smallest divisor of G that gives two waves of blocks and
-// keeps the longest under 3/4 of an even share of the work.  Sizes the workspace, which bounds the plan below.
-int bwd_parts(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& hw) {
-  const int nKV = (Nk + BKV - 1) / BKV;
-  long long total = 0, longest = 0;
-  for (int h = 0; h < Hkv; ++h)
-    for (int j = 0; j < nKV; ++j) {
-      CowaRange rg[2];
-      const int k0 = j * BKV, k1 = std::min(k0 + BKV, Nk) - 1;
-      cowa_bwd_ranges(hw.w[h], k0, k1, Nk - Nq, Nq, BQS, rg);
-      const long long cnt = cowa_range_len(rg[0]) + cowa_range_len(rg[1]);
-      total += cnt;
-      longest = std::max(longest, cnt);
-    }
-  total *= (long long)B * G;
-  longest *= G;
-  const long long blocks = (long long)B * Hkv * nKV;
-  const int kSMs = cowa::sm_count();
-  for (int p = 1; p < G; ++p) {
-    if (G % p) continue;
-    if (blocks * p >= 2 * kSMs && longest * 4 * kSMs <= 3 * total * p) return p;
-  }
-  return G;
-}
-
 BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& hw) {
   BwdPlan pl;
   const int nKV = (Nk + BKV - 1) / BKV, sms = cowa::sm_count();
   pl.sink_tiles = 0;
   for (int h = 0; h < Hkv; ++h) pl.sink_tiles = std::max(pl.sink_tiles, (std::min(hw.w[h].s, Nk) + BKV - 1) / BKV);
-  long long total = 0, sinks = 0, longest = 0;
+  long long total = 0, sinks = 0, longest = 0, longest_sink = 0;
   for (int h = 0; h < Hkv; ++h)
     for (int j = 0; j < nKV; ++j) {
       CowaRange rg[2];
@@ -936,17 +911,21 @@ BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& h
       cowa_bwd_ranges(hw.w[h], k0, k1, Nk - Nq, Nq, BQS, rg);
       const long long cnt = (long long)(cowa_range_len(rg[0]) + cowa_range_len(rg[1])) * G;
       total += cnt;
-      if (j < pl.sink_tiles) { sinks += cnt; longest = std::max(longest, cnt); }
+      longest = std::max(longest, cnt);
+      if (j < pl.sink_tiles) { sinks += cnt; longest_sink = std::max(longest_sink, cnt); }
     }
   total *= B; sinks *= B;
   const double share = (double)total / sms;
   const long long rest = (long long)B * Hkv * (nKV - pl.sink_tiles);
   pl.tiles[0] = B * Hkv * pl.sink_tiles;
-  pl.parts[0] = longest * 4 > 3 * share ? std::max(1, std::min(32, (int)(longest / std::max(share / 3, 4.0) + 0.999))) : 1;
+  pl.parts[0] = longest_sink * 4 > 3 * share ? std::max(1, std::min(32, (int)(longest_sink / std::max(share / 3, 4.0) + 0.999))) : 1;
   plan_rest(pl, rest, rest > 0 ? (double)(total - sinks) / rest : 0.0, share);
-  // Partial sums in the workspace: where spreading whole heads gives four blocks or more per tile, no more than those.
-  const int heads = bwd_parts(B, Nq, Nk, Hkv, G, hw);
-  const long long room = heads > 1 ? (long long)B * Hkv * nKV * heads : 0;
+  // Memory for partial sums: `heads` slots per tile, the smallest divisor of G that gives two waves of blocks and keeps the
+  // longest tile under 3/4 of a share, where that is at least four; else four slots per SM (75 MB at D = 128) or that.
+  const long long ntiles = (long long)B * Hkv * nKV;
+  int heads = 1;
+  while (heads < G && (G % heads != 0 || ntiles * heads < 2 * sms || longest * 4 * sms > 3 * total * heads)) ++heads;
+  const long long room = heads > 1 ? ntiles * heads : 0;
   const long long budget = heads >= 4 ? room : std::max<long long>(room, 4ll * sms);
   while (pl.slots() > budget) --*std::max_element(pl.parts, pl.parts + 3);
   return pl;
@@ -976,15 +955,9 @@ BwdPlan bwd_plan_varlen(int B, int total, int Hkv, int G, const cowa_params_t* p
 
 size_t slot_bytes(const BwdPlan& pl, int D) { return (size_t)pl.slots() * 2 * BKV * D * sizeof(float); }
 
-size_t part_bytes(int B, int Nk, int Hkv, int D, int parts) {
-  if (parts <= 1) return 0;
-  return (size_t)B * Hkv * ((Nk + BKV - 1) / BKV) * parts * 2 * BKV * D * sizeof(float);
-}
-
-size_t ws_bytes(int B, int Nq, int Nk, int Hq, int Hkv, int D, const BwdPlan& pl, const CowaHeadWindows& hw) {
+size_t ws_bytes(int B, int Nq, int Hq, int D, const BwdPlan& pl) {
   const size_t Tpad = ((size_t)Nq + BQS - 1) / BQS * BQS;
-  return (size_t)B * Hq * Tpad * ((size_t)D + 2) * sizeof(float) +
-         std::max(slot_bytes(pl, D), part_bytes(B, Nk, Hkv, D, bwd_parts(B, Nq, Nk, Hkv, Hq / Hkv, hw)));
+  return (size_t)B * Hq * Tpad * ((size_t)D + 2) * sizeof(float) + slot_bytes(pl, D);
 }
 
 // Contiguous [H, T, D] (x batch) strides.
@@ -1134,13 +1107,14 @@ extern "C" {
 size_t cowa_bwd_varlen_workspace_bytes(int B, int total, int Hq, int Hkv, int D, const cowa_params_t* p) {
   if (B <= 0 || total <= 0 || Hq <= 0 || Hkv <= 0 || Hq % Hkv != 0 || (D != 64 && D != 128)) return 0;
   CowaHeadWindows hw;
-  if (!p || cowa::resolve_windows(total, Hkv, p, &hw) != COWA_OK) {  // enough for any parameters
-    BwdPlan most;
-    const int sms = cowa::sm_count();
-    most.sink_tiles = 0;
-    most.tiles[0] = 2 * sms; most.parts[0] = 2;
-    most.tiles[1] = 2 * sms; most.parts[1] = 16;
-    most.tiles[2] = 0; most.parts[2] = 1;
+  if (!p || cowa::resolve_windows(total, Hkv, p, &hw) != COWA_OK) {
+    // Enough for any parameters: full attention has the most steps per tile, hence parts; and as many sink tiles as are
+    // shared at all (bwd_plan_varlen).
+    cowa_params_t full = {};
+    full.full_attn = 1;
+    BwdPlan most = bwd_plan_varlen(B, total, Hkv, Hq / Hkv, &full, hw);
+    most.tiles[0] = std::min(cowa::sm_count() / 2, (int)std::min<long long>((long long)B * Hkv * ((total + BKV - 1) / BKV), 1 << 20));
+    most.parts[0] = 4;
     return ws_bytes_varlen(B, total, Hq, D, most);
   }
   return ws_bytes_varlen(B, total, Hq, D, bwd_plan_varlen(B, total, Hkv, Hq / Hkv, p, hw));
@@ -1173,7 +1147,7 @@ size_t cowa_bwd_prefill_workspace_bytes(int B, int Nq, int Nk, int Hq, int Hkv, 
   if (B <= 0 || Nq <= 0 || Nk < Nq || Hq <= 0 || Hkv <= 0 || Hq % Hkv != 0 || D <= 0 || !p) return 0;
   CowaHeadWindows hw;
   if (cowa::resolve_windows(Nk, Hkv, p, &hw) != COWA_OK) return 0;
-  return ws_bytes(B, Nq, Nk, Hq, Hkv, D, bwd_plan(B, Nq, Nk, Hkv, Hq / Hkv, hw), hw);
+  return ws_bytes(B, Nq, Hq, D, bwd_plan(B, Nq, Nk, Hkv, Hq / Hkv, hw));
 }
 
 size_t cowa_bwd_workspace_bytes(int B, int T, int Hq, int Hkv, int D, const cowa_params_t* p) {
@@ -1194,7 +1168,7 @@ int cowa_bwd_prefill(const void* q, const void* k, const void* v, const void* o,
   int rc = cowa::resolve_windows(Nk, Hkv, p, &hw);
   if (rc != COWA_OK) return rc;
   const BwdPlan pl = bwd_plan(B, Nq, Nk, Hkv, Hq / Hkv, hw);
-  if (workspace_bytes < ws_bytes(B, Nq, Nk, Hq, Hkv, D, pl, hw)) return COWA_ERR_WORKSPACE_TOO_SMALL;
+  if (workspace_bytes < ws_bytes(B, Nq, Hq, D, pl)) return COWA_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   return D == 128 ? launch_bwd<128>(q, k, v, o, lse, d_o, dq, dk, dv, B, Nq, Nk, Hq, Hkv, p, hw, pl, workspace, st)
                   : launch_bwd<64>(q, k, v, o, lse, d_o, dq, dk, dv, B, Nq, Nk, Hq, Hkv, p, hw, pl, workspace, st);

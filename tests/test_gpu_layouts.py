@@ -70,7 +70,7 @@ def test_fwd_bwd_token_major_layout(B, T, Hq, Hkv, D, sink, local):
 
 
 def test_bwd_token_major_layout_with_split_groups():
-    """Few KV tiles: the group's heads are spread over several blocks and a last kernel adds their partial
+    """Few KV tiles: every tile's steps are spread over several blocks and a last kernel adds their partial
     dK, dV; that kernel writes through the strides too."""
     B, T, Hq, Hkv, D, sink, local = 1, 1500, 8, 1, 128, 40, 200
     q, k, v, d_o = cowa_inputs.make_train_inputs(96, B, T, Hq, Hkv, D)

@@ -15,6 +15,7 @@ import torch
 import cowa_inputs
 import paper_2609_32704_b200 as cowa
 from oracle import cowa_oracle as orc
+from test_bwd_plan import bwd_plan, slots, slots_asked_for
 
 pytestmark = pytest.mark.gpu
 
@@ -319,24 +320,16 @@ def test_bwd_full_attn_and_explicit_windows():
     bwd_case(1, 700, 2, 2, 128, 0, 1, windows=[(0, 50, 100, 200), (20, 10, 0, 0)])
 
 
-def _bwd_blocks_per_tile(B, T, Hq, Hkv, D, params):
-    """How many blocks share a KV tile's GQA group, read off the workspace size."""
-    tpad = (T + 63) // 64 * 64
-    extra = cowa.cowa_bwd_workspace_bytes(B, T, Hq, Hkv, D, params) - B * Hq * tpad * (D + 2) * 4
-    per = B * Hkv * ((T + 127) // 128) * 2 * 128 * D * 4
-    assert extra % per == 0
-    return max(extra // per, 1)
-
-
 def test_bwd_tensor_parallel_shard():
-    # One KV head of eight and its 8 QO heads, as a TP=8 rank holds them: windows of the global head, and
-    # (few blocks, long sink tiles) the group's heads spread over several blocks per KV tile.
+    # One KV head of eight and its 8 QO heads, as a TP=8 rank holds them: windows of the global head, and (few tiles, a long
+    # sink tile) every tile's steps cut into parts for several blocks.
     T, Hq, D, sink, local = 3000, 8, 128, 40, 200
     scale = cowa_inputs.softmax_scale(D)
     for r in (0, 5):
         q, k, v, d_o = cowa_inputs.make_train_inputs(56 + r, 1, T, Hq, 1, D)
         params = cowa.make_params(sink=sink, local=local, softmax_scale=scale, hkv_global=8, hkv_offset=r)
-        assert _bwd_blocks_per_tile(1, T, Hq, 1, D, params) == 8
+        cls, _ = bwd_plan(1, T, T, 1, Hq, orc.default_windows(T, 8, sink, local)[r:r + 1])
+        assert slots_asked_for(1, T, Hq, 1, D, params) == slots(cls) and cls[0][1] > 1 and cls[1][1] > 1
         dq, dk, dv = run_fwd_bwd(q.to(DEV), k.to(DEV), v.to(DEV), d_o.to(DEV), params)
         ws = orc.default_windows(T, 8, sink, local)[r:r + 1]
         f = cowa_inputs.to_f64
@@ -347,16 +340,48 @@ def test_bwd_tensor_parallel_shard():
 
 
 def test_bwd_group_split_over_some_blocks():
-    # A shape where the group of 8 heads is split over 4 blocks of 2 heads each; dK, dV stay bitwise
-    # repeatable because the partial sums are added in slot order.
+    # A shape where sink tiles and the rest are shared by several blocks each; dK, dV stay bitwise repeatable because the
+    # partial sums are added in slot order.
     B, T, Hq, Hkv, D, sink, local = 4, 2048, 16, 2, 64, 16, 256
     params = cowa.make_params(sink=sink, local=local, softmax_scale=cowa_inputs.softmax_scale(D))
-    assert _bwd_blocks_per_tile(B, T, Hq, Hkv, D, params) == 4
+    cls, _ = bwd_plan(B, T, T, Hkv, Hq // Hkv, orc.default_windows(T, Hkv, sink, local))
+    assert slots_asked_for(B, T, Hq, Hkv, D, params) == slots(cls) and cls[0][1] > 1 and cls[1][1] > 1
     bwd_case(B, T, Hq, Hkv, D, sink, local, seed=58)
     q, k, v, d_o = cowa_inputs.make_train_inputs(58, B, T, Hq, Hkv, D, device=DEV)
     _, dk1, dv1 = run_fwd_bwd(q, k, v, d_o, params)
     _, dk2, dv2 = run_fwd_bwd(q, k, v, d_o, params)
     assert torch.equal(dk1, dk2) and torch.equal(dv1, dv2)
+
+
+def test_bwd_parts_cut_inside_a_head():
+    # Three QO heads per KV head, five parts per tile: a part begins in the middle of a head's steps.
+    B, T, Hq, D, local = 2, 700, 3, 128, 64
+    ws = orc.default_windows(T, 1, 0, local)
+    (_, (_, parts), _), steps = bwd_plan(B, T, T, 1, Hq, ws)
+    assert parts == 5 and any(n * i // parts % (n // Hq) for _, n in steps[0] for i in range(1, parts))
+    params = cowa.make_params(sink=0, local=local, softmax_scale=cowa_inputs.softmax_scale(D))
+    assert slots_asked_for(B, T, Hq, 1, D, params) == 5 * len(steps[0]) * B
+    bwd_case(B, T, Hq, 1, D, 0, local, seed=76)
+
+
+def test_bwd_shared_last_wave():
+    # More than two tiles per SM: only the sink tiles and the last tile of every SM are shared.  dK, dV of tiles of all
+    # three kinds, those at the line between the whole and the shared tiles among them.
+    B, T, Hq, Hkv, D, sink, local = 1, 8192, 8, 8, 64, 100, 1024
+    params = cowa.make_params(sink=sink, local=local, softmax_scale=cowa_inputs.softmax_scale(D))
+    ws = orc.default_windows(T, Hkv, sink, local)
+    (nsink, p0), (body, p1), (tail, p2) = bwd_plan(B, T, T, Hkv, 1, ws)[0]
+    assert p0 > 1 and p1 == 1 and p2 > 1 and (nsink, body, tail) == (8, 356, 148)
+    assert slots_asked_for(B, T, Hq, Hkv, D, params) == slots([(nsink, p0), (body, p1), (tail, p2)])
+    q, k, v, d_o = cowa_inputs.make_train_inputs(75, B, T, Hq, Hkv, D)
+    dq, dk, dv = run_fwd_bwd(q.to(DEV), k.to(DEV), v.to(DEV), d_o.to(DEV), params)
+    f = cowa_inputs.to_f64
+    line = [(1 + x % 63, x // 63) for x in (body - 1, body)]  # (tile, head) in launch order, 63 tiles per head behind the sink
+    for tile, hk in [(0, 0), (0, 7), (1, 0), (63, 4), *line, (1, 7), (63, 7)]:
+        cols = np.arange(tile * 128, tile * 128 + 128)
+        dk_r, dv_r = orc.backward_dkdv_cols(f(q[0]), f(k[0]), f(v[0]), f(d_o[0]), ws, params.softmax_scale, hk, cols)
+        check_grad(f"dk[{hk},{tile}]", dk[0, hk, cols].float().cpu().numpy(), dk_r)
+        check_grad(f"dv[{hk},{tile}]", dv[0, hk, cols].float().cpu().numpy(), dv_r)
 
 
 def test_fwd_bwd_equal_area_windows():
@@ -537,6 +562,7 @@ def test_bwd_prefill_shapes(B, Nq, Nk, Hq, Hkv, D, sink, local):
     ([64, 65, 2048, 5], 8, 2, 64, 5, 60, "default"),
     ([900, 333], 4, 4, 128, 8, 50, "full"),
     ([1500, 2000, 77], 4, 2, 128, 0, 0, "explicit"),
+    ([5, 64, 1, 700, 2000], 2, 2, 128, 100, 300, "default"),  # shared sink tiles with fewer steps than blocks
 ])
 def test_bwd_varlen(lens, Hq, Hkv, D, sink, local, mode):
     seqs = [(n, n) for n in lens]
