@@ -215,7 +215,8 @@ size_t cowa_decode_static_capacity(void);
  * tokens alike.  The paper describes no such variant; the distance rule is unchanged.
  *   q [B,Nq,Hq,D] in; o [B,Nq,Hq,D] bf16 and lse [B,Nq,Hq] fp32 (may be NULL) out;
  *   kcache, vcache [B,Hkv,Tmax,D] already hold the Nq new tokens; lens: DEVICE int32[B], Nq <= lens[b] <= Tmax.
- * 1 <= Nq <= 64; Hq/Hkv in {1,2,4,8}.  The tokens and heads that share a KV head are the rows of one 128-row tile
+ * 1 <= Nq <= 64; Hq/Hkv in {1,2,4,8}; B <= 65535, and row tiles x their 64-key steps, and B Nq Hq, below 2^31.
+ * The tokens and heads that share a KV head are the rows of one 128-row tile
  * (more rows take more tiles), so that every visible cache row is read once for up to 128 / (Hq/Hkv) tokens.
  * Whole tiles of 64 cache rows are loaded, but a row reaches only the tokens that see it, whatever it holds (Inf
  * and NaN included).  `workspace`: device, >= cowa_decode_multi_workspace_bytes, 16-byte aligned, no initialisation

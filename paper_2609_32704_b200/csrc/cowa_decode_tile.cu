@@ -713,7 +713,8 @@ __global__ void __launch_bounds__(WPR == 1 ? 128 : WPR * 32) cowa_decode_tile_me
 
 // Shape of a call: row tiles, units, blocks and the workspace they need.
 struct TilePlan {
-  int tpt, ntiles, rows, units, blocks;
+  int tpt, ntiles, rows, blocks;
+  long long units, steps;  // steps: of the longest possible list
   size_t bytes;
 };
 
@@ -723,7 +724,7 @@ TilePlan plan_of(int B, int Nq, int Tmax, int Hq, int Hkv, int D, const cowa_par
   t.tpt = std::min(BQ / G, Nq);
   t.ntiles = (Nq + t.tpt - 1) / t.tpt;
   t.rows = t.tpt * G;
-  t.units = B * Hkv * t.ntiles;
+  t.units = (long long)B * Hkv * t.ntiles;
   // one wave of two blocks per SM, fewer when the longest possible list leaves a block less than two steps
   const int hg = p->hkv_global > 0 ? p->hkv_global : Hkv;
   long long vis = Tmax;
@@ -731,8 +732,8 @@ TilePlan plan_of(int B, int Nq, int Tmax, int Hq, int Hkv, int D, const cowa_par
     const long long shared = (long long)p->sink + p->local, band = (std::max((long long)Tmax - shared, 0ll) + hg - 1) / hg;
     vis = std::min<long long>(vis, shared + band + 3 * (BK + t.tpt));
   }
-  const long long steps = (vis + BK - 1) / BK * t.units;
-  t.blocks = (int)std::max(1ll, std::min<long long>(2ll * cowa::sm_count(), (steps + 1) / 2));
+  t.steps = (vis + BK - 1) / BK * t.units;
+  t.blocks = (int)std::max(1ll, std::min<long long>(2ll * cowa::sm_count(), (t.steps + 1) / 2));
   t.bytes = (size_t)(t.blocks + t.units) * t.rows * (D + 2) * sizeof(float) + (size_t)t.units * sizeof(int2);
   return t;
 }
@@ -780,16 +781,17 @@ int decode_ext(const void* q, const void* kc, const void* vc, const int32_t* blo
   if (rc != COWA_OK) return rc;
   if (Nq <= 0 || Nq > 64 || !workspace) return COWA_ERR_INVALID_ARG;
   if (cowa::any_stride_set(p)) return COWA_ERR_UNSUPPORTED;
-  if ((long long)B * ((Nq + 7) / 8 * 8) > 65535) return COWA_ERR_UNSUPPORTED;
   if (!cowa::aligned16(workspace)) return COWA_ERR_MISALIGNED;
   const TilePlan t = plan_of(B, Nq, Tmax, Hq, Hkv, D, p);
+  // units, the list of all their steps (t.steps leaves out partial tiles) and the merged rows are counted in 32 bits
+  if (t.steps + 3 * t.units > 0x7FFFFFFFll || (long long)B * Nq * Hq > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
   if (workspace_bytes < t.bytes) return COWA_ERR_WORKSPACE_TOO_SMALL;
   TileArgs a;
   a.lens = lens; a.block_table = block_table;
   a.status = cowa::device_status_word();
   if (!a.status) return COWA_ERR_CUDA;
   a.B = B; a.Nq = Nq; a.Hq = Hq; a.Hkv = Hkv; a.G = Hq / Hkv;
-  a.tpt = t.tpt; a.ntiles = t.ntiles; a.rows = t.rows; a.units = t.units;
+  a.tpt = t.tpt; a.ntiles = t.ntiles; a.rows = t.rows; a.units = (int)t.units;
   a.page_size = page_size; a.max_pages = max_pages;
   a.box = !block_table ? BK : page_size % 64 == 0 ? 64 : page_size % 32 == 0 ? 32 : 16;
   a.sink = p->sink; a.local = p->local;

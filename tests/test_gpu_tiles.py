@@ -102,6 +102,11 @@ def test_decode_tiles(B, Nq, Tmax, Hq, Hkv, D, sink, local, lens, page):
     multi_case(B, Nq, Tmax, Hq, Hkv, D, sink, local, lens, page_size=page)
 
 
+def test_decode_of_many_sequences():
+    B = 8200  # dozens of units per thread of the share-out
+    multi_case(B, 1, 64, 2, 1, 64, 4, 16, [1 + i % 64 for i in range(B)], page_size=16)
+
+
 @pytest.mark.parametrize("Nq,page", [(4, None), (1, 64)])
 def test_decode_tiles_round_weights_below_an_exact_maximum(Nq, page):
     """The error against 64 bits is no larger than that of exact arithmetic whose weights are rounded to bf16 below the

@@ -9,7 +9,7 @@ import paper_2609_32704_b200 as cowa
 
 OK_PTR = 0x7F0000001000        # 16-byte aligned, never dereferenced
 BAD_PTR = OK_PTR + 8           # not 16-byte aligned
-MISALIGNED, TOO_SMALL, INVALID = -3, -4, -1
+MISALIGNED, TOO_SMALL, INVALID, UNSUPPORTED = -3, -4, -1, -2
 B, T, HQ, HKV, D = 2, 4096, 8, 2, 128
 
 
@@ -91,6 +91,20 @@ def test_workspace_query_of_groups_the_decode_calls_do_not_take():
         assert cowa.cowa_decode_multi_workspace_bytes(1, 1, 512, 256, 1, D_, p) == 0
         assert cowa.cowa_decode_multi_workspace_bytes(2, 4, 512, 129, 1, D_, p) == 0
         assert cowa.cowa_decode_multi_workspace_bytes(1, 1, 512, 128, 1, D_, p) > 0
+
+
+def test_decode_of_many_sequences_is_bounded_by_what_the_kernel_counts():
+    L, p = cowa.lib(), _p()
+    a = _ptrs(6)
+    a7 = a[:3] + [C.c_void_p(OK_PTR)] + a[3:]
+    ws = C.c_void_p(OK_PTR)
+    for B_, Nq in ((8191, 1), (8192, 1), (65535, 1), (1024, 64)):  # taken: only the workspace is too small
+        assert L.cowa_decode_multi(*a, B_, Nq, T, HQ, HKV, D, C.byref(p), ws, 16, None) == TOO_SMALL
+        assert L.cowa_decode_paged(*a7, B_, Nq, T // 64, 64, HQ, HKV, D, C.byref(p), ws, 16, None) == TOO_SMALL
+    # more units, steps or rows than 32 bits count
+    assert L.cowa_decode_multi(*a, 65535, 1, T, 65535, 65535, D, C.byref(p), ws, 16, None) == UNSUPPORTED
+    assert L.cowa_decode_paged(*a7, 65535, 1, 1 << 24, 64, HQ, HKV, D, C.byref(p), ws, 16, None) == UNSUPPORTED
+    assert L.cowa_decode_multi(*a, 65535, 64, T, 1024, 128, D, C.byref(p), ws, 16, None) == UNSUPPORTED
 
 
 def test_scale_and_window_arguments():
