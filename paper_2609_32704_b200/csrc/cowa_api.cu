@@ -3,6 +3,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <vector>
 #include "cowa_common.h"
 #include "cowa_ptx.cuh"
@@ -44,18 +45,18 @@ unsigned int* device_status_word() {
 }
 
 int sm_count() {
-  static int cached = 0;
-  if (cached == 0) {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-        n > 0)
-      cached = n;
-    else {
-      cudaGetLastError();
-      return 148;  // B200; used when no device can be queried (workspace sizing on a machine without a GPU)
+  static std::atomic<int> cache[64];  // per device
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
+    n = cache[dev].load(std::memory_order_relaxed);
+    if (n > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) {
+      cache[dev].store(n, std::memory_order_relaxed);
+      return n;
     }
   }
-  return cached;
+  cudaGetLastError();
+  return 148;
 }
 
 int resolve_strides(const int64_t s[3], int H, long long T, int D, CowaStrides* out) {

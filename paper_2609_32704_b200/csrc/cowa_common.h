@@ -29,7 +29,8 @@ int record_cuda_error(cudaError_t e);
 // Device address of the status word of the current device (nullptr on failure).
 unsigned int* device_status_word();
 
-// SMs of the current device (148 when none can be queried: workspace sizing on a machine without a GPU).
+// SMs of the current device.  148, a B200's, when none can be queried: a workspace sized on a machine without a GPU fits
+// devices with that many, and a call on any other checks its size against its own count.
 int sm_count();
 
 // Resolves the per-head tuples of a training call (explicit, default rule or FullAttn).
