@@ -441,13 +441,17 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
   const long long tiles = VARLEN ? (long long)total_q / BQ + B : (long long)((Nq + BQ - 1) / BQ) * B;
   if (a.G % 2 == 0) {
     // Which kernel, judged for packed batches by their average sequence, so that equal lengths give what the batched
-    // call gives, bit for bit.  Measured at D = 128, Hq 32, Hkv 8 (us, one-head kernel / pair kernel):
-    //   at most half an item per SM: the item is shared by a cluster of 2, 4 or 8 blocks, two steps each at least,
-    //     once its list is long enough to pay for the merge (B 2, Nq 137: 881 keys 20.6 / 22.6, 1784 keys 30.8 / 29.3,
-    //     3448 keys 47.7 / 39.9; Nq 512, Nk 33100, 6300 keys: 76 / 55);
-    //   fewer than three items per SM and short lists: the one-head kernel's 128-row blocks leave the smaller last
-    //     wave (T 2048, local 128: 32.2 / 35.9; local 1024: 46.2 / 40.4);
-    //   else the pair kernel (T 8192, local 128 .. 1024: 127 / 120 .. 212 / 205; T 32768, local 2048: 2100 / 1860).
+    // call gives, bit for bit.  At D = 128 (us, one-head / pair kernel):
+    //   No more items than clusters of two that the device holds, and a list long enough to pay for the merge: the item is
+    //     shared by a cluster of 2, 4 or 8 blocks, two steps each at least, as long as all clusters are resident.  Hq 32,
+    //     Hkv 8, Nq 128: 1816 keys 37.9 / 25.6, 4941 keys 85 / 36 with clusters of four; of eight, two waves, 54.
+    //   Else the pair kernel's persistent blocks pay when their rounds come out even:
+    //     every tile's list is about as long (a chunk behind a cache of its own length or more) and not short: Hq 32,
+    //     Nq 1024, 1129 keys 1.00, 1816 keys 1.09, 4941 keys 1.13 times the one-head kernel's rate;
+    //     causal lists from nothing up: three items per SM, or half of that and lists of 1280 keys.  T 2048, Hq 16, local
+    //     1024 (0.9 items per SM) 0.88 times; Hq 32 (1.7) local 128 0.87, local 1024 1.13; T 3072 (2.6) local 128 0.91,
+    //     local 2048 1.10; T 8192 (6.9) local 1024 1.03; T 32768, local 2048 1.13.  In between the last round decides, by
+    //     up to a tenth either way (T 6000, Hq 16, 2.5 items per SM: 0.90; T 2048, Hq 32, 1.7: 1.13).
     // At D = 64 the exponentials bound both and two one-head blocks per SM keep them busier (T 22272, 4 heads, fwd and
     // bwd 1064 / 1138), so that only the shared form is taken there.
     const int qn = VARLEN ? std::max(total_q / B, 1) : Nq, kn = VARLEN ? std::max(total_k / B, 1) : Nk;
@@ -461,10 +465,11 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
     }
     const long long items = tiles * (Hq / 2), judged = (long long)((qn + BQ - 1) / BQ) * B * (Hq / 2);
     if (items > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
+    const bool shared = judged <= cowa::resident_clusters(2), even = kn >= 2ll * qn;
     int split = 1;
-    while (split < 8 && judged * split * 2 <= (split == 1 ? 144 : 128) && keys >= 512 * split) split *= 2;
-    const bool half_empty = judged * 2 <= 144, long_list = keys >= (D == 128 ? 1536 : 2048);
-    if (half_empty ? long_list : D == 128 && (long_list || judged >= 3 * cowa::sm_count()))
+    while (split < 8 && judged <= cowa::resident_clusters(split * 2) && keys >= 512 * split) split *= 2;
+    const bool rounds = judged >= 3 * cowa::sm_count() || (even ? keys >= 1536 : keys >= 1280 && 2 * judged >= 3 * cowa::sm_count());
+    if (shared ? keys >= (D == 128 ? 1536 : 2048) : D == 128 && rounds)
       return cowa::launch_fwd_pair<D, VARLEN>(mq, k, v, mo, sk, sv, a, rows_k, nb, items, split, st);
   }
   COWA_CUDA_TRY(cudaFuncSetAttribute(cowa_fwd_kernel<D, VARLEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -29,6 +29,10 @@ __device__ __forceinline__ uint32_t interval_bits(int a, int b, int base) {
 }
 
 namespace cowa {
+// Clusters of `size` (2, 4, 8) blocks of the pair kernel that the current device holds at once: a block takes an SM, and a
+// cluster lies within one GPC, so that large ones leave SMs out (74, 33 and 15 on the B200 measured).
+int resident_clusters(int size);
+
 // Pair kernel (cowa_fwd_pair.cu): two QO heads of a group at a time, `items` = tiles x pairs of heads.  split = 1: one
 // persistent block per SM; split = 2, 4, 8: every item shared by a cluster of that many blocks.
 template <int D, bool VARLEN>

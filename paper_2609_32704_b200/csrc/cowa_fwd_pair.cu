@@ -22,6 +22,7 @@
 #include "cowa_fwd.h"
 
 #include <algorithm>
+#include <atomic>
 
 using namespace cowa_ptx;
 
@@ -676,6 +677,30 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 }  // namespace
 
 namespace cowa {
+
+int resident_clusters(int size) {
+  static std::atomic<int> cache[64][3];  // per device
+  const int i = size == 2 ? 0 : size == 4 ? 1 : 2;
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
+    n = cache[dev][i].load(std::memory_order_relaxed);
+    if (n > 0) return n;
+    const auto kernel = cowa_fwd_pair_kernel<128, false, true>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)size); cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = PairSmem<128>::kBytes;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PairSmem<128>::kBytes) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0) {
+      cache[dev][i].store(n, std::memory_order_relaxed);
+      return n;
+    }
+  }
+  cudaGetLastError();
+  return size == 2 ? 72 : size == 4 ? 32 : 15;
+}
 
 template <int D, bool VARLEN>
 int launch_fwd_pair(const CUtensorMap& mq, const void* k, const void* v, const CUtensorMap& mo, const CowaStrides& sk,
