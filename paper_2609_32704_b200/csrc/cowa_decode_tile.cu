@@ -82,12 +82,6 @@ __device__ __forceinline__ int tile_of(const Piece& pc, int t, bool* full) {
   return j;
 }
 
-__device__ __forceinline__ uint32_t interval_bits(int a, int b, int base) {
-  int lo = max(a - base, 0), hi = min(b - base, 31);
-  if (lo > hi) return 0u;
-  return (0xFFFFFFFFu >> (31 - (hi - lo))) << lo;
-}
-
 // The keys that tokens at key positions p0 .. p1 (p0 >= 0) see, some of them (first = p0, last = p1) or each of them by
 // the same window (first = p1, last = p0), in the 64 keys from `row0` on: one bit per key.
 __device__ __forceinline__ unsigned long long seen_bits(const CowaWin& w, int first, int last, int row0) {

@@ -470,7 +470,7 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
     while (split < 8 && judged <= cowa::resident_clusters(split * 2) && keys >= 512 * split) split *= 2;
     const bool rounds = judged >= 3 * cowa::sm_count() || (even ? keys >= 1536 : keys >= 1280 && 2 * judged >= 3 * cowa::sm_count());
     if (shared ? keys >= (D == 128 ? 1536 : 2048) : D == 128 && rounds)
-      return cowa::launch_fwd_pair<D, VARLEN>(mq, k, v, mo, sk, sv, a, rows_k, nb, items, split, st);
+      return cowa::launch_fwd_pair<D, VARLEN>(mq, mk, mv, mo, a, items, split, st);
   }
   COWA_CUDA_TRY(cudaFuncSetAttribute(cowa_fwd_kernel<D, VARLEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      FwdSmem<D>::kBytes));

@@ -21,22 +21,15 @@ struct FwdArgs {
   int sink, local, hkv_global, hkv_offset, full_attn, explicit_windows;
 };
 
-// bits [lo, hi] of the 32-bit word covering columns [base, base+32)
-__device__ __forceinline__ uint32_t interval_bits(int a, int b, int base) {
-  int lo = max(a - base, 0), hi = min(b - base, 31);
-  if (lo > hi) return 0u;
-  return (0xFFFFFFFFu >> (31 - (hi - lo))) << lo;
-}
-
 namespace cowa {
 // Clusters of `size` (2, 4, 8) blocks of the pair kernel that the current device holds at once: a block takes an SM, and a
 // cluster lies within one GPC, so that large ones leave SMs out (74, 33 and 15 on the B200 measured).
 int resident_clusters(int size);
 
-// Pair kernel (cowa_fwd_pair.cu): two QO heads of a group at a time, `items` = tiles x pairs of heads.  split = 1: one
-// persistent block per SM; split = 2, 4, 8: every item shared by a cluster of that many blocks.
+// Pair kernel (cowa_fwd_pair.cu; the tensor maps of the one-head kernel, 64-row boxes of K and V): two QO heads of a
+// group at a time, `items` = tiles x pairs of heads.  split = 1: one persistent block per SM; split = 2, 4, 8: every item
+// shared by a cluster of that many blocks.
 template <int D, bool VARLEN>
-int launch_fwd_pair(const CUtensorMap& mq, const void* k, const void* v, const CUtensorMap& mo, const CowaStrides& sk,
-                    const CowaStrides& sv, const FwdArgs& a, int rows_k, int nb, long long items, int split,
-                    cudaStream_t st);
+int launch_fwd_pair(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mo,
+                    const FwdArgs& a, long long items, int split, cudaStream_t st);
 }  // namespace cowa

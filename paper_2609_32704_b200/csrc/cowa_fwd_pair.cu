@@ -33,12 +33,6 @@ constexpr int kSplitQ = 1;  // O += P V starts once the 32-key groups 0 .. kSpli
 constexpr int kPairThreads = 384;  // warps 10, 11 only make the control warpgroup whole
 constexpr int kItemReaders = 9;  // warps that read a published work item: softmax 8, MMA 1
 
-__device__ __forceinline__ uint32_t interval_bits(int a, int b, int base) {
-  int lo = max(a - base, 0), hi = min(b - base, 31);
-  if (lo > hi) return 0u;
-  return (0xFFFFFFFFu >> (31 - (hi - lo))) << lo;
-}
-
 // 2^x of a pair on the FMA and integer pipes: x = n + f with n = rint(x), |f| <= 1/2, 2^f by the polynomial of
 // degree 6 with the least largest relative error on that interval (fitted by reweighted least squares: 1.9e-9, in
 // fp32 8e-8, against 2 ulp of ex2.approx), times 2^n.  x is held at -127 from below, where the
@@ -703,13 +697,8 @@ int resident_clusters(int size) {
 }
 
 template <int D, bool VARLEN>
-int launch_fwd_pair(const CUtensorMap& mq, const void* k, const void* v, const CUtensorMap& mo, const CowaStrides& sk,
-                    const CowaStrides& sv, const FwdArgs& a, int rows_k, int nb, long long items, int split,
-                    cudaStream_t st) {
-  CUtensorMap mk, mv;
-  int rc;
-  if ((rc = make_tensor_map(&mk, k, MapType::BF16, D, rows_k, a.Hkv, nb, sk, 64, BK))) return rc;
-  if ((rc = make_tensor_map(&mv, v, MapType::BF16, D, rows_k, a.Hkv, nb, sv, 64, BK))) return rc;
+int launch_fwd_pair(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mo,
+                    const FwdArgs& a, long long items, int split, cudaStream_t st) {
   auto kernel = cowa_fwd_pair_kernel<D, VARLEN, true>;
   if constexpr (D == 128) {
     if (split == 1) kernel = cowa_fwd_pair_kernel<D, VARLEN, false>;
@@ -726,10 +715,9 @@ int launch_fwd_pair(const CUtensorMap& mq, const void* k, const void* v, const C
   return COWA_OK;
 }
 
-#define COWA_INSTANTIATE(D, V)                                                                                    \
-  template int launch_fwd_pair<D, V>(const CUtensorMap&, const void*, const void*, const CUtensorMap&,            \
-                                     const CowaStrides&, const CowaStrides&, const FwdArgs&, int, int, long long, \
-                                     int, cudaStream_t);
+#define COWA_INSTANTIATE(D, V)                                                                                          \
+  template int launch_fwd_pair<D, V>(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const CUtensorMap&,    \
+                                     const FwdArgs&, long long, int, cudaStream_t);
 COWA_INSTANTIATE(128, false)
 COWA_INSTANTIATE(128, true)
 COWA_INSTANTIATE(64, false)

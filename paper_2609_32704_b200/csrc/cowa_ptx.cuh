@@ -308,6 +308,13 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   return d;
 }
 
+// bits of the 32 columns [base, base + 32) that lie in [a, b]
+__device__ __forceinline__ uint32_t interval_bits(int a, int b, int base) {
+  int lo = max(a - base, 0), hi = min(b - base, 31);
+  if (lo > hi) return 0u;
+  return (0xFFFFFFFFu >> (31 - (hi - lo))) << lo;
+}
+
 // two fp32 -> packed bf16x2 (lo in the low half), round to nearest even
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   uint32_t r;
