@@ -14,11 +14,25 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda"
 
 
-def _prefill(B, Nq, Nk, Hq, Hkv, D, sink, local, token_major=False, rows=None):
+# What a call may ask for besides the default rule: (parameters, the windows of an Nk-token sequence)
+MODES = {
+    "default": lambda Hkv, sink, local: (dict(sink=sink, local=local), lambda Nk: orc.default_windows(Nk, Hkv, sink, local)),
+    "full": lambda Hkv, sink, local: (dict(sink=sink, local=local, full_attn=True), lambda Nk: [(0, Nk, 0, 0)] * Hkv),
+    # the local heads are some of three times as many
+    "rank": lambda Hkv, sink, local: (dict(sink=sink, local=local, hkv_global=3 * Hkv, hkv_offset=Hkv + 1),
+                                      lambda Nk: orc.default_windows(Nk, 3 * Hkv, sink, local)[Hkv + 1:2 * Hkv + 1]),
+    # tuples of their own for every head: gap or none, wide sink or none, no long window at all
+    "tuples": lambda Hkv, sink, local: (lambda ws: (dict(windows=ws), lambda Nk: ws))(
+        [[(0, 1500, 300, 1100), (200, 70, 0, 2000), (130, 1700, 0, 0), (1, 1, 65, 1800)][h % 4] for h in range(Hkv)]),
+}
+
+
+def _prefill(B, Nq, Nk, Hq, Hkv, D, sink, local, token_major=False, rows=None, mode="default"):
     q, _, _, _ = cowa_inputs.make_train_inputs(91, B, Nq, Hq, Hkv, D)
     _, k, v, _ = cowa_inputs.make_train_inputs(92, B, Nk, Hq, Hkv, D)
     scale = cowa_inputs.softmax_scale(D)
-    params = cowa.make_params(sink=sink, local=local, softmax_scale=scale)
+    kw, windows = MODES[mode](Hkv, sink, local)
+    params = cowa.make_params(softmax_scale=scale, **kw)
     put = lambda x: x.to(DEV)  # noqa: E731
     if token_major:
         put = lambda x: x.transpose(1, 2).contiguous().to(DEV).transpose(1, 2)  # noqa: E731
@@ -29,7 +43,7 @@ def _prefill(B, Nq, Nk, Hq, Hkv, D, sink, local, token_major=False, rows=None):
     torch.cuda.synchronize()
     cowa.cowa_check_device_status()
     assert torch.isfinite(o).all() and torch.isfinite(lse).all()
-    ws = orc.default_windows(Nk, Hkv, sink, local)
+    ws = windows(Nk)
     f = cowa_inputs.to_f64
     rows = np.arange(Nq) if rows is None else np.asarray(rows)
     for b in range(B):
@@ -50,6 +64,17 @@ def test_few_items(B, Nq, Nk, Hq, Hkv, D, sink, local):
     _prefill(B, Nq, Nk, Hq, Hkv, D, sink, local)
 
 
+@pytest.mark.parametrize("mode", ["full", "rank", "tuples"])
+@pytest.mark.parametrize("B,Nq,Nk,Hq,Hkv,D", [
+    (1, 130, 6000, 8, 4, 128),    # an item shared by a cluster
+    (1, 200, 5000, 8, 4, 64),     # the same at D = 64
+    (2, 1100, 3000, 32, 4, 128),  # persistent blocks
+])
+def test_window_modes(B, Nq, Nk, Hq, Hkv, D, mode):
+    n = Nq - 1
+    _prefill(B, Nq, Nk, Hq, Hkv, D, 64, 1500, mode=mode, rows=[0, 1, 63, 127, 128, 129, n - 1, n])
+
+
 def test_few_items_token_major():
     _prefill(2, 200, 4000, 8, 2, 128, 64, 500, token_major=True)
 
@@ -67,6 +92,7 @@ def test_many_items(Nq, Nk, sink, local):
 @pytest.mark.parametrize("seqs,Hq,Hkv,D", [
     ([(300, 5000), (1, 700), (129, 9000)], 4, 2, 128),                       # clusters share the items of a packed batch
     ([(1900, 1900), (64, 64), (2000, 2500), (1, 3000), (127, 127)], 32, 8, 128),  # one block per item
+    ([(200, 9000), (1, 5000), (130, 7000)], 4, 2, 64),                       # clusters at D = 64
 ])
 @pytest.mark.parametrize("bad", [None, float("nan"), float("inf")])
 def test_packed(seqs, Hq, Hkv, D, bad):
@@ -89,6 +115,28 @@ def test_packed(seqs, Hq, Hkv, D, bad):
             o_ref, lse_ref = orc.forward_rows(f(q[:, qs]), f(k[:, ks]), f(v[:, ks]), ws, scale, h, np.arange(nq))
             check(f"lse[{b},{h}]", lse[h, qs].cpu().numpy(), lse_ref, TOL_LSE, TOL_LSE)
             check(f"o[{b},{h}]", o[h, qs].float().cpu().numpy(), o_ref)
+
+
+@pytest.mark.parametrize("mode", ["full", "rank", "tuples"])
+@pytest.mark.parametrize("seqs,Hq,Hkv,D", [
+    ([(300, 5000), (1, 1700), (129, 6000)], 8, 4, 128),
+    ([(200, 6000), (130, 4000)], 8, 4, 64),
+    ([(1900, 1900), (64, 64), (1500, 2500), (127, 127)], 32, 4, 128),
+])
+def test_packed_window_modes(seqs, Hq, Hkv, D, mode):
+    q, k, v, cu_q, cu_k = _packed_inputs(97, seqs, Hq, Hkv, D)
+    scale = cowa_inputs.softmax_scale(D)
+    kw, windows = MODES[mode](Hkv, 64, 1500)
+    o, lse = _run_varlen(q, k, v, cu_q, cu_k, cowa.make_params(softmax_scale=scale, **kw))
+    cowa.cowa_check_device_status()
+    f = cowa_inputs.to_f64
+    for b, (nq, nk) in enumerate(seqs):
+        qs, ks = slice(cu_q[b], cu_q[b + 1]), slice(cu_k[b], cu_k[b + 1])
+        rows = np.unique(np.clip([0, 1, 63, 126, 127, 128, nq - 2, nq - 1], 0, nq - 1))
+        for h in range(0, Hq, Hq // 4):
+            o_ref, lse_ref = orc.forward_rows(f(q[:, qs]), f(k[:, ks]), f(v[:, ks]), windows(nk), scale, h, rows)
+            check(f"lse[{b},{h}]", lse[h, qs].cpu().numpy()[rows], lse_ref, TOL_LSE, TOL_LSE)
+            check(f"o[{b},{h}]", o[h, qs].float().cpu().numpy()[rows], o_ref)
 
 
 @pytest.mark.parametrize("B,Nq,Tmax,Hq,Hkv,D,sink,local,lens,page", [
