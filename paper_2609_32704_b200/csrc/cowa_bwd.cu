@@ -199,7 +199,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   if constexpr (VARLEN) {
     rbase = a.cu[b];
     Nq = Nk = a.cu[b + 1] - rbase;
-    if (rbase < 0 || rbase + Nk > a.total) {  // malformed offsets: report, touch nothing
+    if (rbase < 0 || rbase + Nk > a.total || pbase < 0 || pbase > a.Tpad - Nk) {  // malformed offsets: report, touch nothing
       if (threadIdx.x == 0) atomicOr(a.status, (unsigned)COWA_DEV_BAD_SEQLENS);
       return;
     }
@@ -473,7 +473,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             commit(bar_s_full + 1);
           }
         }
-        // Step n uses TMEM buffer b = n & 1 (the two compute warpgroups alternate steps).  Issue order:
+        // Step n uses TMEM buffer b = n & 1.  Issue order:
         //   dV(n) | dP^T(n+1) | dK(n) | S^T(n+2) | dQ^T(n)
         // so that every wait below is for something produced about one step earlier.
         int st = 0, st1 = (N > 1) ? 1 : 0, st2 = 2 % NST;    // stages of steps n, n+1, n+2
@@ -837,7 +837,7 @@ cowa_bwd_reduce_dkv_kernel(const __grid_constant__ BwdArgs a, CowaStrides sk, Co
   if constexpr (VARLEN) {
     rbase = a.cu[at.b];
     Nk = a.cu[at.b + 1] - rbase;
-    if (rbase < 0 || rbase + Nk > a.total) return;
+    if (rbase < 0 || rbase + Nk > a.total || at.pbase < 0 || at.pbase > a.Tpad - Nk) return;
   }
   const int t = at.j * BKV + r;
   if (t >= Nk) return;

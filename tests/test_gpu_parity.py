@@ -601,6 +601,26 @@ def test_bwd_varlen(lens, Hq, Hkv, D, sink, local, mode):
         check_grad(f"varlen dv[seq {b}]", dv[:, sl].float().cpu().numpy(), dv_r)
 
 
+def test_bwd_varlen_overlapping_offsets_reported():
+    """Offsets that step back make sequences overlap and their padded rows outgrow the workspace's row space: the ones
+    that do not fit are skipped and reported, nothing is written past the workspace, the library stays usable."""
+    Hq, Hkv, D, total = 2, 1, 64, 700
+    q, k, v, d_o = (x[0].to(DEV) for x in cowa_inputs.make_train_inputs(77, 1, total, Hq, Hkv, D))
+    params = cowa.make_params(sink=4, local=100, softmax_scale=0.125)
+    cu = torch.tensor([0, 600, 100, 700], dtype=torch.int32, device=DEV)  # 640 + 640 padded rows of 832
+    dq, dk, dv = (torch.empty_like(x) for x in (q, k, v))
+    o, lse = torch.zeros_like(q), torch.zeros((Hq, total), dtype=torch.float32, device=DEV)
+    nbytes = cowa.cowa_bwd_varlen_workspace_bytes(3, total, Hq, Hkv, D, params)
+    ws = torch.full((nbytes + 4 * 2 ** 20,), 0xFF, dtype=torch.uint8, device=DEV)
+    cowa.cowa_bwd_varlen(q, k, v, o, lse, d_o, dq, dk, dv, cu, params, ws[:nbytes])
+    torch.cuda.synchronize()
+    with pytest.raises(cowa.CowaError) as e:
+        cowa.cowa_check_device_status()
+    assert e.value.status == -8
+    assert (ws[nbytes:] == 0xFF).all()
+    cowa.cowa_check_device_status()
+
+
 @pytest.mark.parametrize("bad", [float("nan"), float("inf")])
 def test_packed_batch_nonfinite_neighbour_does_not_leak(bad):
     """Rows past the end of a sequence share its last tiles in shared memory.  They are multiplied by exact
