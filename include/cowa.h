@@ -24,6 +24,10 @@
  *     device memory and keeps no state between calls except cached kernel
  *     attributes and the per-thread error code behind cowa_last_cuda_error().
  *     All work is enqueued on `stream`; no call synchronises.
+ *   - Results do not depend on the contents of other sequences of a batch, but their last bits may depend on its
+ *     sizes: the forward calls choose a kernel and a split by B, Nq, Nk, the head counts and, packed, the average
+ *     length, the multi-token and paged calls cut a sequence's keys at places that follow from all lengths.  The
+ *     same call on the same sizes and lengths gives the same bits (dq: see cowa_params_t.deterministic).
  *   - Return value: COWA_OK (0) or a negative cowa_status_t.  Arguments are validated
  *     before anything is launched.  There is no CPU fallback.
  *   - Preconditions not checked on the device: near >= 1 for every head (so each
@@ -265,7 +269,8 @@ int cowa_equal_area_windows(int Nq, int Nk, int Hkv_global, int hkv_offset, int 
  *   COWA_SCHED_BWD    for each head h, KV tile j:  h, j, n, then n pairs (i, full) with i ascending
  *   COWA_SCHED_DECODE for each head h: h, r, then r pairs (start, end) of visible key ranges [start,end)
  *                     ascending, then m, then m visited block_k-block indices; Nq = 1 is the decode step,
- *                     Nq > 1 the union over the Nq newest tokens (what cowa_decode_multi streams)
+ *                     Nq > 1 the union over the Nq newest tokens (cowa_decode_multi streams the 64-row tiles
+ *                     that hold it)
  * full = 1 when every pair of the nominal block_q x block_k tile is legal, else 0 (boundary tile).
  * *out_len receives the number of int32 needed; COWA_ERR_WORKSPACE_TOO_SMALL if out_cap is less
  * (nothing beyond out_cap is written). */
