@@ -112,6 +112,11 @@ __device__ __forceinline__ uint32_t interval_bits32(long long a, long long b, lo
 struct TileAt {
   int hk, b, j, nts, pbase;
 };
+// Packed batches: offsets that step back make sequences overlap, and their padded rows may outgrow the row space; such a
+// sequence has no tiles here, the preprocess kernel reports it.  (With the report in this kernel it spilled, 332 bytes.)
+__device__ __forceinline__ bool fits(const BwdArgs& a, const TileAt& x) {
+  return (unsigned)x.pbase <= (unsigned)(a.Tpad - (a.cu[x.b + 1] - a.cu[x.b]));
+}
 template <bool VARLEN>
 __device__ __forceinline__ bool locate_tile(const BwdArgs& a, int c, int q, TileAt& x) {
   const int nsk = a.sink_tiles, nhead = a.B * a.Hkv;
@@ -121,14 +126,14 @@ __device__ __forceinline__ bool locate_tile(const BwdArgs& a, int c, int q, Tile
     x.hk = q % a.Hkv; x.b = q / a.Hkv;
     if constexpr (VARLEN) {
       varlen_seq_info(a.cu, x.b, BKV, BQS, &x.nts, &x.pbase);
-      return x.j < x.nts;  // else the sequence is shorter than its sink
+      return x.j < x.nts && fits(a, x);  // else the sequence is shorter than its sink
     }
     return true;
   }
   if (c == 2) q += a.cls_tiles[1];
   if constexpr (VARLEN) {
     x.hk = q / a.tiles_bound;
-    return varlen_locate(a.cu, a.B, q % a.tiles_bound, BKV, BQS, &x.b, &x.j, &x.nts, &x.pbase, nsk);
+    return varlen_locate(a.cu, a.B, q % a.tiles_bound, BKV, BQS, &x.b, &x.j, &x.nts, &x.pbase, nsk) && fits(a, x);
   }
   const int nrest = (a.Nk + BKV - 1) / BKV - nsk;
   x.j = nsk + q % nrest; q /= nrest;
@@ -199,7 +204,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   if constexpr (VARLEN) {
     rbase = a.cu[b];
     Nq = Nk = a.cu[b + 1] - rbase;
-    if (rbase < 0 || rbase + Nk > a.total || pbase < 0 || pbase > a.Tpad - Nk) {  // malformed offsets: report, touch nothing
+    if (rbase < 0 || rbase + Nk > a.total) {  // malformed offsets: report, touch nothing
       if (threadIdx.x == 0) atomicOr(a.status, (unsigned)COWA_DEV_BAD_SEQLENS);
       return;
     }
@@ -740,11 +745,15 @@ __global__ void cowa_bwd_preprocess_varlen_kernel(const __nv_bfloat16* __restric
                                                   const __nv_bfloat16* __restrict__ d_o,
                                                   const float* __restrict__ lse, float* __restrict__ lse2,
                                                   float* __restrict__ delta, float* __restrict__ acc,
-                                                  const int* __restrict__ cu, int B, int total, int Tpad) {
+                                                  const int* __restrict__ cu, int B, int total, int Tpad,
+                                                  unsigned int* status) {
   constexpr int TPR = D / 8;  // threads per row (16 bytes each)
   const int chunk = blockIdx.x, h = blockIdx.y;
   const int r = threadIdx.x / TPR, part = threadIdx.x % TPR;
   int b, lc, nch, pb;
+  if (chunk == 0 && h == 0 && threadIdx.x < 32 && varlen_locate(cu, B, Tpad / BQS, BQS, BQS, &b, &lc, &nch, &pb) &&
+      threadIdx.x == 0)
+    atomicOr(status, (unsigned)COWA_DEV_BAD_SEQLENS);  // more chunks than the row space holds: see fits
   const bool in = varlen_locate(cu, B, chunk, BQS, BQS, &b, &lc, &nch, &pb);
   const int t = lc * BQS + r;  // row inside the sequence
   const int rbase = in ? cu[b] : 0;
@@ -837,7 +846,7 @@ cowa_bwd_reduce_dkv_kernel(const __grid_constant__ BwdArgs a, CowaStrides sk, Co
   if constexpr (VARLEN) {
     rbase = a.cu[at.b];
     Nk = a.cu[at.b + 1] - rbase;
-    if (rbase < 0 || rbase + Nk > a.total || at.pbase < 0 || at.pbase > a.Tpad - Nk) return;
+    if (rbase < 0 || rbase + Nk > a.total) return;
   }
   const int t = at.j * BKV + r;
   if (t >= Nk) return;
@@ -1086,7 +1095,7 @@ int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o
   const dim3 chunks(Tpad / BQS, Hq);
   cowa_bwd_preprocess_varlen_kernel<D><<<chunks, BQS * (D / 8), 0, st>>>(
       static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse, lse2, delta, dq_acc,
-      cu, B, total, Tpad);
+      cu, B, total, Tpad, a.status);
   COWA_CUDA_TRY(cudaGetLastError());
   if (p->bwd_main_start_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_start_event), st));
   cowa_bwd_kernel<D, true><<<(unsigned)pl.blocks(), 512, BwdSmem<D>::kBytes, st>>>(mq, mk, mv, mdo, mdk, mdv, a);
