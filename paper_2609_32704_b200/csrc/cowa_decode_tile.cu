@@ -9,7 +9,7 @@
 // Bound by HBM: 32 KB per step; two blocks per SM take a step in about 1600 clocks each, twice the rate at which HBM
 // feeds them.
 // Warps 0-3: softmax, one row per thread (only as many warps as there are rows); warp 4: TMA; warp 5: MMA issue.  V rows
-// that no token sees are cleared by warp 3 beside the softmax, by all four warps when a tile has rows for each of them
+// that no token sees are cleared by the warps without rows beside the softmax, by all four when each of them has rows
 // (a warp of its own would leave the threads 128 registers, and they spill).
 #include <cuda_bf16.h>
 #include <string.h>
@@ -167,15 +167,15 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   uint64_t* bar_pv = bars + 2;        //     O += P V of a step has completed
   uint64_t* bar_s = bars + 3;         // [2] S of a step is in TMEM buffer b
   uint64_t* bar_i_full = bars + 5;    // [2] a piece has been published
-  uint64_t* bar_i_empty = bars + 7;   // [2] count nw + 1, + 1 with a warp 3 that clears: it has been read
+  uint64_t* bar_i_empty = bars + 7;   // [2] count 5 (warps 0-3, MMA): it has been read
   uint64_t* bar_p = bars + 9;         // [2] count nw: P written over S
   uint64_t* bar_v_read = bars + 11;   //     count nw: add_seen has read a V tile
   uint64_t* bar_k_full = bars + 12;             // [NS]
   uint64_t* bar_k_empty = bar_k_full + NS;      // [NS]
   uint64_t* bar_v_full = bar_k_full + 2 * NS;   // [NS]
   uint64_t* bar_v_empty = bar_k_full + 3 * NS;  // [NS]
-  uint64_t* bar_v_seen = bar_k_full + 4 * NS;   // [NS] count 1, or 4: V rows that no token sees are cleared
-  uint64_t* bar_v_go = bar_k_full + 5 * NS;     // [NS] V of a boundary tile is on its way (warp 3 passes other steps by)
+  uint64_t* bar_v_seen = bar_k_full + 4 * NS;   // [NS] count 4 - nw, or 4: V rows that no token sees are cleared
+  uint64_t* bar_v_go = bar_k_full + 5 * NS;     // [NS] V of a boundary tile is on its way (the clearing warps pass other steps by)
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bar_k_full + 6 * NS);
   int* scan = reinterpret_cast<int*>(smem + SM::oScan);  // 6 warp totals; [8], [9] first unit and its list position; [10 ..] per slot: step whose V is not finite
 
@@ -189,7 +189,7 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   if (tid == 0) {
     for (int s = 0; s < 12 + 6 * NS; ++s) {
       const bool v_seen = bars + s >= bar_v_seen && bars + s < bar_v_go;
-      mbar_init(bars + s, s == 7 || s == 8 ? min(nw + 2, 5) : s >= 9 && s < 12 ? nw : v_seen && nw == 4 ? 4 : 1);
+      mbar_init(bars + s, s == 7 || s == 8 ? 5 : s >= 9 && s < 12 ? nw : !v_seen ? 1 : nw < 4 ? 4 - nw : 4);
     }
     for (int s = 0; s < NS; ++s) scan[10 + s] = 0;
     fence_mbar_init();
@@ -269,14 +269,20 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     const unsigned long long some = seen_by_some(u, j * BK), all = seen_by_all(u, j * BK);
     uint8_t* vt = sV + slot * SM::kKV + (ch >> 3) * SLAB_K;
     bool bad = false;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint32_t look = ~(uint32_t)(all >> (32 * h)), keep = (uint32_t)(some >> (32 * h));
+      if (look == 0u) continue;
 #pragma unroll 4
-    for (int r = wi * RPI + lane / CPR; r < BK; r += n * RPI) {
-      uint4* x = reinterpret_cast<uint4*>(vt + r * 128 + (((ch & 7) ^ (r & 7)) << 4));
-      if (!((some >> r) & 1ull)) {
-        *x = make_uint4(0u, 0u, 0u, 0u);
-      } else if (!((all >> r) & 1ull)) {
-        const uint4 y = *x;
-        bad = bad || nonfinite(y.x) || nonfinite(y.y) || nonfinite(y.z) || nonfinite(y.w);
+      for (int r = wi * RPI + lane / CPR; r < 32; r += n * RPI) {
+        if (!((look >> r) & 1u)) continue;
+        uint4* x = reinterpret_cast<uint4*>(vt + (h * 32 + r) * 128 + (((ch & 7) ^ (r & 7)) << 4));
+        if (!((keep >> r) & 1u)) {
+          *x = make_uint4(0u, 0u, 0u, 0u);
+        } else {
+          const uint4 y = *x;
+          bad = bad || nonfinite(y.x) || nonfinite(y.y) || nonfinite(y.z) || nonfinite(y.w);
+        }
       }
     }
     fence_proxy_async_smem();
@@ -586,9 +592,9 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       }
       if (row_valid) a.ws_ml[srow] = make_float2(m_ref, l_sum);
     }
-  } else if (warp == 3) {
+  } else if (warp < 4) {
     // ======================= boundary tiles, beside fewer than four softmax warps =======================
-    // The TMA warp says when a tile of its kind is on its way: this warp passes the other steps by, and a wait for V alone
+    // The TMA warp says when a tile of its kind is on its way: these warps pass the other steps by, and a wait for V alone
     // could meet the slot's load of two rounds before, which has the same parity.
     int c = 0, vs = 0;
     uint32_t vr = 0, gr = 0;  // parity of the slot's load; parities of bar_v_go, a bit per slot
@@ -601,7 +607,7 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           ok = mbar_wait(bar_v_go + vs, (gr >> vs) & 1, a.status) && mbar_wait(bar_v_full + vs, vr, a.status);
           if (!ok) break;
           gr ^= 1u << vs;
-          clear_unseen(pc.u, j, vs, c, 0, 1);
+          clear_unseen(pc.u, j, vs, c, warp - nw, 4 - nw);
         }
         if (++vs == NS) { vs = 0; vr ^= 1; }
       }
