@@ -5,22 +5,30 @@
 //                   padded to a multiple of 64 rows (padding: -inf, so that P = 0 there);
 //                   its threads also zero the fp32 dQ accumulator.
 //   2. main kernel  one thread block per (batch, KV head, 128-row KV tile), KV-stationary as in
-//                   Algorithm 2, looping over the G QO heads of the group and over the 64-row QO
+//                   Algorithm 2, looping over the G QO heads of the group and over the 128-row QO
 //                   tiles of I_h(j) (analytic scheduler, ascending).  Per step five tcgen05 MMAs:
-//                     S^T  = K Q^T            (TMEM, 128 kv x 64 q)
+//                     S^T  = K Q^T            (TMEM, 128 kv x 128 q)
 //                     dP^T = V dO^T           (TMEM)
 //                     dV  += P^T dO           (P^T as the TMEM operand)
 //                     dK  += dS^T Q           (dS^T as the TMEM operand)
-//                     dQ^T = K^T dS^T         (dS^T from shared memory; 128 d x 64 q in TMEM)
+//                     dQ^T = K^T dS^T         (dS^T from shared memory; 128 d x 128 q in TMEM)
 //                   dK and dV stay in TMEM for the whole loop, all G heads included, so they need no
 //                   atomics (Algorithm 2 line 17 needs them only because it gives each QO head its
 //                   own program).  dQ^T is drained by a separate warpgroup through shared memory and
-//                   added to the fp32 accumulator with bulk add-reductions of contiguous 32-row ranges (Algorithm 2 line 15).
-//                   Warp roles: TMA producer / MMA issuer / two compute warpgroups (P, dS; each takes 32
-//                   of the 64 query columns of every step, which halves the latency between S^T and
-//                   dS^T) / dQ drain warpgroup, connected by mbarriers; S^T is double buffered so that the
-//                   MMAs of steps n+1, n+2 overlap the element-wise work of
-//                   step n.  Blocks are ordered sink tiles first (they meet every query tile), then
+//                   added to the fp32 accumulator with bulk add-reductions (Algorithm 2 line 15).
+//                   Warp roles: TMA producer / MMA issuer / two compute warpgroups (P, dS; each takes 64
+//                   of the 128 query columns of every step) / dQ drain warpgroup, connected by mbarriers.
+//                   What bounds it: shared memory.  Of a step's ~4150 clocks the products' operands take
+//                   2048 (128 bytes a clock), the Q and dO loads 512, dS^T 256, the dQ staging 1024 written
+//                   and read; the tensor pipe needs 2560, the exponentials 1024.  With steps of 64 queries
+//                   K and V were read twice as often (2816), and a row constant per column and thread came
+//                   out of shared memory as a broadcast (1024 more): 32K, 32 heads 4840 -> 4650 us.  The
+//                   512 columns of TMEM hold S^T, dP^T, dK, dV; P^T and dS^T take the outer halves of S^T
+//                   and dP^T, dQ^T the 128 columns between them, so that the next S^T and dP^T only wait
+//                   until dQ^T is in registers.  Per step n the MMAs run in the order
+//                     dK(n-1) | dQ^T(n-1) | dP^T(n)   beside the exponentials of step n
+//                     dV(n)   | S^T(n+1)              beside dS^T(n)
+//                   Blocks are ordered sink tiles first (they meet every query tile), then
 //                   head by head with ascending KV tile, so that the blocks in flight sweep the same
 //                   dQ rows at nearly the same time and the reductions hit in L2.
 //   3. convert      dQ accumulator (already scaled) -> bf16.
@@ -46,14 +54,15 @@ using namespace cowa_ptx;
 namespace {
 
 constexpr int BKV = 128;  // KV rows per block (MMA M)
-constexpr int BQS = 64;   // QO rows per step (MMA N of S^T / dP^T)
-constexpr int NST = 3;    // Q / dO stages
+constexpr int BQT = 128;  // QO rows per step (MMA N of S^T / dP^T)
+constexpr int BQS = 64;   // unit of the padded row space (half a step) and of the plan's step counts
+constexpr int NST = 2;    // Q stages (Q(n) is read again by dK(n) after S^T(n+1)); dO has one
 constexpr float kDqFixedOne = 262144.f;  // 2^18: one unit of dQ in the fixed-point accumulation mode
 
 struct BwdArgs {
   const float* lse2;   // [B*Hq, Tpad]  -LSE * log2(e)   (both negated: the packed adds have no operand negation)
   const float* delta;  // [B*Hq, Tpad]  -Delta
-  float* dq_acc;       // [B*Hq, Tpad, D] fp32
+  float* dq_acc;       // fp32 [B*Hq, Tpad / 64, D / 32, 16, 32, 4]: 64 rows, 32 d, then four rows of one d (a drain warp's tile)
   unsigned int* status;
   int B, Nq, Nk, Hq, Hkv, G, Tpad;
   int sink_tiles;      // KV tiles per head that hold sink columns (launched first)
@@ -75,15 +84,13 @@ struct BwdArgs {
 template <int D>
 struct BwdSmem {
   static constexpr int kKV = BKV * D * 2;      // K or V tile
-  static constexpr int kQS = BQS * D * 2;      // Q or dO step tile
-  static constexpr int kStage = 2 * kQS;       // Q + dO
-  static constexpr int kDS = BKV * BQS * 2;    // dS^T tile (bf16)
-  static constexpr int oK = 0, oV = kKV, oStage = 2 * kKV, oDS = oStage + NST * kStage;
-  static constexpr int oVec = oDS + 2 * kDS;   // per stage: 64 floats lse2, 64 floats delta
-  static constexpr int oDQ = oVec + NST * 512;  // dQ staging: two tiles of 32 query rows x D fp32
-  static constexpr int kDQ = 32 * D * 4;
-  static constexpr int oBar = oDQ + 2 * kDQ;
-  static constexpr int kBytes = oBar + 256 + 1024;  // barriers + alignment slack; 232192 B at D = 128 (limit 232448)
+  static constexpr int kQ = BQT * D * 2;       // Q or dO tile of a step
+  static constexpr int kDS = BKV * BQS * 2;    // dS^T of half a step (bf16)
+  static constexpr int oK = 0, oV = kKV, oQ = 2 * kKV, oDO = oQ + NST * kQ, oDS = oDO + kQ;
+  static constexpr int oVec = oDS + 2 * kDS;   // per stage: 128 floats lse2, 128 floats delta
+  static constexpr int oDQ = oVec + NST * 1024;  // dQ staging: per drain warp two tiles of 32 query rows x 32 d, fp32
+  static constexpr int oBar = oDQ + 8 * 4096;
+  static constexpr int kBytes = oBar + 256;    // 231680 B at D = 128 (limit 232448)
 };
 
 __device__ __forceinline__ void bulk_load_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -96,14 +103,6 @@ __device__ __forceinline__ void bulk_load_1d(void* dst, const void* src, uint32_
 __device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
   asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes)
                : "memory");
-}
-
-__device__ __forceinline__ uint32_t interval_bits32(long long a, long long b, long long base) {
-  long long lo = a - base, hi = b - base;
-  if (lo < 0) lo = 0;
-  if (hi > 31) hi = 31;
-  if (lo > hi) return 0u;
-  return (0xFFFFFFFFu >> (31 - (int)(hi - lo))) << (int)lo;
 }
 
 // Tile number q of class c: sink tiles of every head first (they meet every query tile of their sequence and are the
@@ -153,34 +152,41 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   using SM = BwdSmem<D>;
   constexpr int NSLAB = D / 64;
   constexpr int SLAB_KV = BKV * 128;  // bytes of one 64-wide slab of a 128-row tile
-  constexpr int SLAB_QS = BQS * 128;  // ... of a 64-row tile
+  constexpr int SLAB_Q = BQT * 128;   // ... of a Q or dO tile
   // TMEM columns
-  constexpr uint32_t cS0 = 0, cDP0 = 128, cDK = 256, cDV = 384, TMEM_COLS = 512;  // S^T x2, dP^T/dQ^T x2, dK, dV
-  constexpr uint32_t ID_ST = idesc_bf16(128, BQS, 0, 0);   // S^T, dP^T
+  constexpr uint32_t cS = 0, cDP = 128, cDK = 256, cDV = 384, TMEM_COLS = 512;
+  constexpr uint32_t cDS = cDP + 64, cDQ = cS + 64;  // P^T over the first half of S^T, dS^T over the second of dP^T, dQ^T between
+  constexpr uint32_t ID_ST = idesc_bf16(128, BQT, 0, 0);   // S^T, dP^T
   constexpr uint32_t ID_ACC = idesc_bf16(128, D, 0, 1);    // dV, dK (B = dO / Q, MN-major)
-  constexpr uint32_t ID_DQ = idesc_bf16(128, BQS, 1, 1);   // dQ^T (A = K^T, B = dS^T, both MN-major)
+  constexpr uint32_t ID_DQ = idesc_bf16(128, BQT, 1, 1);   // dQ^T (A = K^T, B = dS^T, both MN-major)
 
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* sK = smem + SM::oK;
   uint8_t* sV = smem + SM::oV;
-  uint8_t* sStage = smem + SM::oStage;
+  uint8_t* sQ = smem + SM::oQ;
+  uint8_t* sDO = smem + SM::oDO;
   uint8_t* sDS = smem + SM::oDS;
   float* sVec = reinterpret_cast<float*>(smem + SM::oVec);
-  float* sDQ = reinterpret_cast<float*>(smem + SM::oDQ);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SM::oBar);
   uint64_t* bar_kv = bars + 0;
-  uint64_t* bar_ld_full = bars + 1;             // [NST]  Q/dO/LSE/Delta of a step have landed
-  uint64_t* bar_ld_empty = bars + 1 + NST;      // [NST]  the step's products have consumed the stage
-  uint64_t* bar_s_full = bars + 1 + 2 * NST;    // [2]    S^T of a step is in TMEM buffer b
-  uint64_t* bar_dp_full = bars + 3 + 2 * NST;   // [2]    dP^T ...
-  uint64_t* bar_p_ready = bars + 5 + 2 * NST;   // [2]    count 256: P^T written over S^T
-  uint64_t* bar_ds_ready = bars + 7 + 2 * NST;  // [2]    count 256: dS^T in TMEM and shared memory, dP^T consumed
-  uint64_t* bar_dq_full = bars + 9 + 2 * NST;   // [2]    dQ^T is in the columns dP^T left
-  uint64_t* bar_dq_free = bars + 11 + 2 * NST;  // [2]    count 128: dQ^T drained
-  uint64_t* bar_done = bars + 13 + 2 * NST;
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 14 + 2 * NST);
-  float** part_out = reinterpret_cast<float**>(bars + 15 + 2 * NST);  // this block's partial dK, dV (kept here, not in registers)
+  uint64_t* bar_q_full = bars + 1;    // [2] Q, LSE, Delta of a step have landed
+  uint64_t* bar_q_empty = bars + 3;   // [2] ... are consumed
+  uint64_t* bar_o_full = bars + 5;    // dO ...
+  uint64_t* bar_o_empty = bars + 6;
+  uint64_t* bar_s_full = bars + 7;    // S^T is in TMEM
+  uint64_t* bar_s_read = bars + 8;    // count 256: S^T is in registers
+  uint64_t* bar_p_ready = bars + 9;   // count 256: P^T written over the first half of S^T
+  uint64_t* bar_dp_full = bars + 10;  // dP^T is in TMEM
+  uint64_t* bar_ds_ready = bars + 11; // count 256: dS^T in TMEM (over the second half of dP^T) and shared memory
+  uint64_t* bar_dq_full = bars + 12;  // dQ^T is in TMEM
+  uint64_t* bar_dq_free = bars + 13;  // [2] count 128: ... has left the columns of dP^T, of S^T
+  uint64_t* bar_done = bars + 15;
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 16);
+  float** part_out = reinterpret_cast<float**>(bars + 17);  // this block's partial dK, dV (kept here, not in registers)
+  // What the roles would otherwise each hold or compute (registers: nothing spills in the batched form)
+  int* step_info = reinterpret_cast<int*>(bars + 18);          // [2] by stage: first query of the step, bit 0: none of its pairs is masked
+  long long* dq_at = reinterpret_cast<long long*>(bars + 19);  // [4] by step: first element of its dQ rows, bit 0: no second half
+  int* geo = reinterpret_cast<int*>(bars + 23);                // window, off, Nq, Nk, steps of this block
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform by construction (helps the compiler)
@@ -214,10 +220,10 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const int off = Nk - Nq;
   const int k0 = j * BKV, k1 = min(k0 + BKV, Nk) - 1;
   CowaRange rg[2];
-  cowa_bwd_ranges(w, k0, k1, off, Nq, BQS, rg);
+  cowa_bwd_ranges(w, k0, k1, off, Nq, BQT, rg);
   const int cnt = cowa_range_len(rg[0]) + cowa_range_len(rg[1]);  // QO steps per head
   const int n0 = cnt * a.G * part / parts;               // (the host checks that these products fit)
-  const int N = cnt * a.G * (part + 1) / parts - n0;     // this block's steps
+  const int steps = cnt * a.G * (part + 1) / parts - n0; // this block's steps
   const int g0 = cnt > 0 ? n0 / cnt : 0, tq0 = n0 - g0 * cnt;  // head of the group and position in I_h(j) of the first
   const int bt = VARLEN ? 0 : b;                               // batch coordinate of the tensor maps
   const int hq0 = hk * a.G;                                    // first QO head of the group
@@ -226,14 +232,16 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const bool tail_kv = VARLEN && (k0 + BKV > Nk);  // rows after the tile's last valid one belong to the next sequence
 
   if (tid == 0) {
+    geo[0] = w.s; geo[1] = w.n; geo[2] = w.g; geo[3] = w.l; geo[4] = off; geo[5] = Nq; geo[6] = Nk; geo[7] = steps;
     *part_out = parts > 1 ? a.dkv_part + (size_t)slot * 2 * (BKV * D) : nullptr;
     mbar_init(bar_kv, 1);
-    for (int s = 0; s < NST; ++s) { mbar_init(bar_ld_full + s, 1); mbar_init(bar_ld_empty + s, 1); }
     for (int s = 0; s < 2; ++s) {
-      mbar_init(bar_s_full + s, 1); mbar_init(bar_dp_full + s, 1);
-      mbar_init(bar_p_ready + s, 256); mbar_init(bar_ds_ready + s, 256);
-      mbar_init(bar_dq_full + s, 1); mbar_init(bar_dq_free + s, 128);
+      mbar_init(bar_q_full + s, 1); mbar_init(bar_q_empty + s, 1);
+      mbar_init(bar_dq_free + s, 128);
     }
+    mbar_init(bar_dq_full, 1); mbar_init(bar_o_full, 1); mbar_init(bar_o_empty, 1);
+    mbar_init(bar_s_full, 1); mbar_init(bar_s_read, 256); mbar_init(bar_p_ready, 256);
+    mbar_init(bar_dp_full, 1); mbar_init(bar_ds_ready, 256);
     mbar_init(bar_done, 1);
     fence_mbar_init();
   }
@@ -245,25 +253,26 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_holder;
+  constexpr uint32_t tmem_base = 0;  // the allocation is all of TMEM
 
   bool ok = true;
+  auto step_count = [&]() { return static_cast<const volatile int*>(geo)[7]; };  // (each role reads it for itself)
 
   // dK (first compute warpgroup) and dV (drain warpgroup): TMEM -> bf16 -> shared -> TMA store.  Called from
   // inside the role branches so that it is compiled under that role's register budget.
   auto store_grad = [&](bool is_dk) {
-    const int r = (warp & 3) * 32 + lane;
+    const int N = step_count(), r = (warp & 3) * 32 + lane;
     const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
     if (N > 0) ok = mbar_wait(bar_done, 0, a.status) && ok;
     tc_fence_after();
-    uint8_t* sOut = sStage + (is_dk ? 0 : SM::kKV);
+    uint8_t* sOut = sQ + (is_dk ? 0 : SM::kKV);
     const float mul = is_dk ? a.scale : 1.f;
     if (float* const dst = *part_out) {
       // A shared tile: this block's part goes out in fp32, one slot per block; a kernel of its own adds the slots in order.
       // Staged where K, V or the Q / dO stages were, rows with their 16-byte chunks permuted (bank conflicts), and
       // copied as one range: straight from registers a warp's store touches 32 rows (1019 against 983 thousand clocks of
       // the whole kernel for one KV head of 20001 tokens).
-      uint8_t* sPart = (is_dk ? sK : sStage) + r * (D * 4);
+      uint8_t* sPart = (is_dk ? sK : sQ) + r * (D * 4);
 #pragma unroll
       for (int c = 0; c < D / 32; ++c) {
         uint32_t ov[32];
@@ -283,7 +292,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       fence_proxy_async_smem();
       wg_sync(is_dk ? 1 : 2);
       if (r == 0) {
-        bulk_store(dst + (is_dk ? 0 : BKV * D), is_dk ? sK : sStage, BKV * D * 4);
+        bulk_store(dst + (is_dk ? 0 : BKV * D), is_dk ? sK : sQ, BKV * D * 4);
         tma_commit_group();
         tma_wait_group<0>();
       }
@@ -347,12 +356,11 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     }
   };
 
-  // Register budget per role: 128 per thread at launch (512 threads), 80 + 2 * 160 + 112 = 4 * 128 moved to where the work
-  // is.  Each setmaxnreg sits at the top of its own branch so that the code below it is compiled for that budget.  No
-  // role spills at these: with 64 / 176 / 96 the MMA issuer and the producer did, inside their loops, and the kernel took
-  // 1066 instead of 1015 thousand clocks at 2 x 8K, 7980 instead of 7590 at 32K.
+  // Register budget per role: 128 per thread at launch (512 threads), 80 + 2 * 152 + 128 = 4 * 128 moved to where the work
+  // is.  Each setmaxnreg sits at the top of its own branch so that the code below it is compiled for that budget.
   if (warp < 4) {
     setmaxnreg_dec<80>();
+    const int N = step_count();
     if (warp == 0) {
       // ================= TMA producer =================
       if (lane == 0 && N > 0) {
@@ -362,24 +370,31 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           tma_load_4d(sK + s * SLAB_KV, &tmK, bar_kv, s * 64, rbase + k0, hk, bt);
           tma_load_4d(sV + s * SLAB_KV, &tmV, bar_kv, s * 64, rbase + k0, hk, bt);
         }
-        int st = 0, g = g0, t_in = tq0;   // stage, head of the group, position in I_h(j): kept incrementally
-        uint32_t ph_e = 0;             // parity of the "stage empty" wait (the first NST steps need none)
+        int g = g0, t_in = tq0;   // head of the group, position in I_h(j): kept incrementally
         for (int n = 0; n < N && ok; ++n) {
-          if (n >= NST) ok = mbar_wait(bar_ld_empty + st, ph_e, a.status);
-          if (!ok) break;
+          const int st = n & 1;
+          const uint32_t ph_e = ((n >> 1) & 1) ^ 1;  // parity of the "stage empty" waits (the first two steps need none)
           const int i = cowa_bwd_tile_at(rg, t_in);
-          const int bhq = bhq0 + g, q0 = i * BQS;
-          uint8_t* sQ = sStage + st * SM::kStage;
-          uint8_t* sdO = sQ + SM::kQS;
-          mbar_expect_tx(bar_ld_full + st, SM::kStage + 512);
-          for (int s = 0; s < NSLAB; ++s) {
-            tma_load_4d(sQ + s * SLAB_QS, &tmQ, bar_ld_full + st, s * 64, rbase + q0, hq0 + g, bt);
-            tma_load_4d(sdO + s * SLAB_QS, &tmdO, bar_ld_full + st, s * 64, rbase + q0, hq0 + g, bt);
-          }
-          bulk_load_1d(sVec + st * 128, a.lse2 + (size_t)bhq * vec_stride + pbase + q0, 256, bar_ld_full + st);
-          bulk_load_1d(sVec + st * 128 + 64, a.delta + (size_t)bhq * vec_stride + pbase + q0, 256, bar_ld_full + st);
+          const int bhq = bhq0 + g, q0 = i * BQT;
+          auto load_do = [&]() {
+            mbar_expect_tx(bar_o_full, SM::kQ);
+            for (int s = 0; s < NSLAB; ++s)
+              tma_load_4d(sDO + s * SLAB_Q, &tmdO, bar_o_full, s * 64, rbase + q0, hq0 + g, bt);
+          };
+          if (n >= 2) ok = mbar_wait(bar_q_empty + st, ph_e, a.status);
+          if (!ok) break;
+          const uint32_t vb = q0 + BQS < Nq ? BQT * 4 : BQS * 4;  // the row space is padded to 64 rows only
+          step_info[st] = q0 + (cowa_tile_full(w, q0, BQT, k0, BKV, off, Nq, Nk) ? 1 : 0);
+          dq_at[n & 3] = (long long)((size_t)bhq * vec_stride + pbase + q0) * D + (q0 + BQS < Nq ? 0 : 1);
+          mbar_expect_tx(bar_q_full + st, SM::kQ + 2 * vb);
+          for (int s = 0; s < NSLAB; ++s)
+            tma_load_4d(sQ + st * SM::kQ + s * SLAB_Q, &tmQ, bar_q_full + st, s * 64, rbase + q0, hq0 + g, bt);
+          bulk_load_1d(sVec + st * 256, a.lse2 + (size_t)bhq * vec_stride + pbase + q0, vb, bar_q_full + st);
+          bulk_load_1d(sVec + st * 256 + 128, a.delta + (size_t)bhq * vec_stride + pbase + q0, vb, bar_q_full + st);
+          if (n >= 1) ok = mbar_wait(bar_o_empty, (n - 1) & 1, a.status);
+          if (!ok) break;
+          load_do();
           if (++t_in == cnt) { t_in = 0; ++g; }
-          if (++st == NST) { st = 0; if (n >= NST) ph_e ^= 1; }
         }
       }
     } else if (warp == 1) {
@@ -396,33 +411,33 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         const uint64_t dK_k = smem_desc_sw128(smem_u32(sK), 16, 1024);                       // K, K-major (A of S^T)
         const uint64_t dV_k = smem_desc_sw128(smem_u32(sV), 16, 1024);                       // V, K-major (A of dP^T)
         const uint64_t dK_mn = smem_desc_sw128(smem_u32(sK), D == 128 ? SLAB_KV : 0, 1024);  // K^T, MN-major (A of dQ^T)
-        const uint64_t dQ_k0 = smem_desc_sw128(smem_u32(sStage), 16, 1024);                  // Q of stage 0, K-major (B of S^T)
-        const uint64_t dO_k0 = smem_desc_sw128(smem_u32(sStage) + SM::kQS, 16, 1024);        // dO of stage 0, K-major (B of dP^T)
-        const uint64_t dQ_mn0 = smem_desc_sw128(smem_u32(sStage), SLAB_QS, 1024);            // Q, MN-major (B of dK)
-        const uint64_t dO_mn0 = smem_desc_sw128(smem_u32(sStage) + SM::kQS, SLAB_QS, 1024);  // dO, MN-major (B of dV)
-        const uint64_t dDS0 = smem_desc_sw128(smem_u32(sDS), 0, 1024);                       // dS^T, MN-major (B of dQ^T)
-        constexpr uint32_t kStage16 = SM::kStage >> 4, kDS16 = SM::kDS >> 4;
+        const uint64_t dQ_k0 = smem_desc_sw128(smem_u32(sQ), 16, 1024);        // Q of stage 0, K-major (B of S^T)
+        const uint64_t dO_k0 = smem_desc_sw128(smem_u32(sDO), 16, 1024);       // dO of stage 0, K-major (B of dP^T)
+        const uint64_t dQ_mn0 = smem_desc_sw128(smem_u32(sQ), SLAB_Q, 1024);   // Q, MN-major (B of dK)
+        const uint64_t dO_mn0 = smem_desc_sw128(smem_u32(sDO), SLAB_Q, 1024);  // dO, MN-major (B of dV)
+        const uint64_t dDS = smem_desc_sw128(smem_u32(sDS), SM::kDS, 1024);    // dS^T, MN-major (B of dQ^T)
+        constexpr uint32_t kQ16 = SM::kQ >> 4;
 
-        auto gemm_st = [&](uint32_t d_col, uint64_t dA, uint64_t dB) {  // [128 x 64] = A[128 x D] B[64 x D]^T
+        auto gemm_st = [&](uint32_t d_col, uint64_t dA, uint64_t dB) {  // [128 x 128] = A[128 x D] B[128 x D]^T
           if (lead) {
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk)
               mma_ss(tb + d_col, dA + (((kk / 4) * SLAB_KV + (kk % 4) * 32) >> 4),
-                     dB + (((kk / 4) * SLAB_QS + (kk % 4) * 32) >> 4), ID_ST, kk > 0);
+                     dB + (((kk / 4) * SLAB_Q + (kk % 4) * 32) >> 4), ID_ST, kk > 0);
           }
         };
-        auto gemm_acc = [&](uint32_t d_col, uint32_t a_col, uint64_t dB, uint32_t acc_first) {  // [128 x D] += A(TMEM) B
+        auto gemm_acc = [&](uint32_t d_col, uint32_t a_col, uint64_t dB, uint32_t acc_first, int k0_, int k1_) {  // [128 x D] += A(TMEM) B
           if (lead) {
 #pragma unroll
-            for (int kk = 0; kk < BQS / 16; ++kk)
-              mma_ts(tb + d_col, tb + a_col + (kk >> 1) * 32 + (kk & 1) * 8, dB + ((kk * 2048) >> 4), ID_ACC, kk > 0 ? 1u : acc_first);
+            for (int kk = k0_; kk < k1_; ++kk)  // 32-query blocks 0, 2 from one warpgroup's columns, 1, 3 from the other's
+              mma_ts(tb + d_col, tb + a_col + ((kk >> 1) & 1) * 32 + (kk >> 2) * 16 + (kk & 1) * 8, dB + ((kk * 2048) >> 4), ID_ACC, kk > 0 ? 1u : acc_first);
           }
         };
-        auto gemm_dq = [&](uint32_t d_col, uint64_t dB) {  // dQ^T[D x 64] = K^T dS^T
+        auto gemm_dq = [&]() {  // dQ^T[D x 128] = K^T dS^T
           if (lead) {
 #pragma unroll
             for (int kk = 0; kk < BKV / 16; ++kk)
-              mma_ss(tb + d_col, dK_mn + ((kk * 2048) >> 4), dB + ((kk * 2048) >> 4), ID_DQ, kk > 0);
+              mma_ss(tb + cDQ, dK_mn + ((kk * 2048) >> 4), dDS + ((kk * 2048) >> 4), ID_DQ, kk > 0);
           }
         };
         auto commit = [&](uint64_t* bar) {
@@ -438,15 +453,11 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             for (int c_ = lane; c_ < nchunk; c_ += 32)
               *reinterpret_cast<uint4*>(tile + s_ * slab_bytes + first * 128 + c_ * 16) = make_uint4(0u, 0u, 0u, 0u);
         };
-        int t_clr = tq0;  // position in I_h(j) of the next step whose Q / dO stage is checked (packed batches only)
-        auto clear_stage_tail = [&](int stage) {
+        auto clear_tail = [&](uint8_t* tile, int stage) {  // Q or dO tile of the step whose Q is in this stage
           if constexpr (VARLEN) {
-            const int q0_ = cowa_bwd_tile_at(rg, t_clr) * BQS;
-            if (++t_clr == cnt) t_clr = 0;
-            if (q0_ + BQS > Nq) {
-              uint8_t* sQ_ = sStage + stage * SM::kStage;
-              clear_rows(sQ_, Nq - q0_, BQS, SLAB_QS);
-              clear_rows(sQ_ + SM::kQS, Nq - q0_, BQS, SLAB_QS);
+            const int q0_ = step_info[stage], nq = static_cast<const volatile int*>(geo)[5];
+            if (!(q0_ & 1) && q0_ + BQT > nq) {
+              clear_rows(tile, nq - q0_, BQT, SLAB_Q);
               fence_proxy_async_smem();
               __syncwarp();
             }
@@ -459,237 +470,292 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           fence_proxy_async_smem();
           __syncwarp();
         }
-        // prologue: S^T(0), dP^T(0), S^T(1)
-        ok = ok && mbar_wait(bar_ld_full + 0, 0, a.status);
+        ok = ok && mbar_wait(bar_q_full, 0, a.status);
         if (ok) {
-          clear_stage_tail(0);
+          clear_tail(sQ, 0);
           tc_fence_after();
-          gemm_st(cS0, dK_k, dQ_k0);
-          commit(bar_s_full + 0);
-          gemm_st(cDP0, dV_k, dO_k0);
-          commit(bar_dp_full + 0);
+          gemm_st(cS, dK_k, dQ_k0);
+          commit(bar_s_full);
         }
-        if (ok && N > 1) {
-          ok = mbar_wait(bar_ld_full + 1, 0, a.status);
-          if (ok) {
-            clear_stage_tail(1);
-            tc_fence_after();
-            gemm_st(cS0 + 64, dK_k, dQ_k0 + kStage16);
-            commit(bar_s_full + 1);
-          }
-        }
-        // Step n uses TMEM buffer b = n & 1.  Issue order:
-        //   dV(n) | dP^T(n+1) | dK(n) | S^T(n+2) | dQ^T(n)
-        // so that every wait below is for something produced about one step earlier.
-        int st = 0, st1 = (N > 1) ? 1 : 0, st2 = 2 % NST;    // stages of steps n, n+1, n+2
-        uint32_t ph2 = (2 / NST) & 1;                        // parity of the load that fills stage st2 for step n+2
-        uint32_t par = 0;                                    // (n >> 1) & 1
         auto body = [&](int n, auto B_) {
-          constexpr int b_ = decltype(B_)::value;
-          constexpr uint32_t sbuf = cS0 + b_ * 64, dpbuf = cDP0 + b_ * 64, dpother = cDP0 + (b_ ^ 1) * 64;
-          ok = mbar_wait(bar_p_ready + b_, par, a.status);
-          if (!ok) return;
-          tc_fence_after();
-          gemm_acc(cDV, sbuf, dO_mn0 + st * kStage16, n > 0 ? 1u : 0u);     // dV += P^T dO
-          if (n + 1 < N) {                                                  // dP^T(n+1), once dQ^T(n-1) has left its buffer
-            if (n >= 1) {
-              ok = mbar_wait(bar_dq_free + (b_ ^ 1), ((n - 1) >> 1) & 1, a.status);
-              if (!ok) return;
-              tc_fence_after();
-            }
-            gemm_st(dpother, dV_k, dO_k0 + st1 * kStage16);
-            commit(bar_dp_full + (b_ ^ 1));
-          }
-          ok = mbar_wait(bar_ds_ready + b_, par, a.status);
-          if (!ok) return;
-          tc_fence_after();
-          gemm_acc(cDK, sbuf + 16, dQ_mn0 + st * kStage16, n > 0 ? 1u : 0u);  // dK += dS^T Q
-          commit(bar_ld_empty + st);
-          if (n + 2 < N) {                                                  // S^T(n+2) into the buffer P^T(n), dS^T(n) just left:
-            ok = mbar_wait(bar_ld_full + st2, ph2, a.status);               // it heads the next step's dependency chain, so it
-            if (!ok) return;                                                // goes ahead of dQ^T(n), which only feeds the drain
-            clear_stage_tail(st2);
+          constexpr int st = decltype(B_)::value;
+          const uint32_t par = n & 1;
+          if (n > 0) {
+            ok = mbar_wait(bar_ds_ready, par ^ 1, a.status);
+            if (!ok) return;
             tc_fence_after();
-            gemm_st(sbuf, dK_k, dQ_k0 + st2 * kStage16);
-            commit(bar_s_full + b_);
+            gemm_acc(cDK, cDS, dQ_mn0 + (st ^ 1) * kQ16, n > 1 ? 1u : 0u, 0, 8);
+            commit(bar_q_empty + (st ^ 1));
+            ok = mbar_wait(bar_s_read, par, a.status);
+            if (!ok) return;
+            tc_fence_after();
+            gemm_dq();
+            commit(bar_dq_full);
           }
-          gemm_dq(dpbuf, dDS0 + b_ * kDS16);                                // dQ^T = K^T dS^T over the consumed dP^T(n)
-          commit(bar_dq_full + b_);
-          // advance the bookkeeping to step n+1
-          st = st1; st1 = st2;
-          if (++st2 == NST) { st2 = 0; ph2 ^= 1; }
-          if (b_ == 1) par ^= 1;
+          ok = mbar_wait(bar_o_full, par, a.status);
+          if (ok && n > 0) ok = mbar_wait(bar_dq_free, par ^ 1, a.status);
+          if (!ok) return;
+          clear_tail(sDO, st);
+          tc_fence_after();
+          gemm_st(cDP, dV_k, dO_k0);
+          commit(bar_dp_full);
+          ok = mbar_wait(bar_p_ready, par, a.status);
+          if (!ok) return;
+          tc_fence_after();
+          gemm_acc(cDV, cS, dO_mn0, n > 0 ? 1u : 0u, 0, 8);
+          commit(bar_o_empty);
+          if (n + 1 < N) {
+            ok = mbar_wait(bar_q_full + (st ^ 1), ((n + 1) >> 1) & 1, a.status);
+            if (ok && n > 0) ok = mbar_wait(bar_dq_free + 1, par ^ 1, a.status);
+            if (!ok) return;
+            clear_tail(sQ + (st ^ 1) * SM::kQ, st ^ 1);
+            tc_fence_after();
+            gemm_st(cS, dK_k, dQ_k0 + (st ^ 1) * kQ16);
+            commit(bar_s_full);
+          }
         };
         for (int n = 0; n < N && ok; n += 2) {
           body(n, std::integral_constant<int, 0>{});
           if (n + 1 < N && ok) body(n + 1, std::integral_constant<int, 1>{});
         }
+        if (ok) {
+          ok = mbar_wait(bar_ds_ready, (N - 1) & 1, a.status);
+          if (ok && N > 1) ok = mbar_wait(bar_dq_free + 1, N & 1, a.status);
+          if (ok) {
+            tc_fence_after();
+            gemm_dq();
+            commit(bar_dq_full);
+            gemm_acc(cDK, cDS, dQ_mn0 + ((N - 1) & 1) * kQ16, N > 1 ? 1u : 0u, 0, 8);
+          }
+        }
         commit(bar_done);
       }
     }
   } else if (warp < 12) {
-    setmaxnreg_inc<160>();
+    setmaxnreg_inc<152>();
     {
-      // ======== two compute warpgroups, each takes 32 of the 64 query columns of every step: P^T and dS^T, one
-      // KV row per thread.  Inside the 64-column S^T buffer a warpgroup only ever writes into the 32 columns
-      // it reads: P^T (bf16 pairs) into the first 16 of them, dS^T into the last 16.
-      const int wg = (warp - 4) >> 2;        // query columns [32 wg, 32 wg + 32) of every step
-      const int r = (warp & 3) * 32 + lane;  // KV row = TMEM lane
+      const int N = step_count();
+      // ======== two compute warpgroups: P^T and dS^T of two blocks of 32 queries each.  A warpgroup only writes into
+      // columns that it has read: P^T (bf16 pairs) into its first block of S^T, dS^T into its second of dP^T.
+      const int wg = (warp - 4) >> 2;  // queries [32 wg, 32 wg + 32) of both halves of every step
+      // A thread holds the fragments of the 16-lane TMEM accesses: keys row0 + {0, 8, 16, 24}, query pairs 8 j + 2 (lane % 4)
+      // of every 32-query block: eight row constants a block instead of 32 broadcast ones.
+      const int lane4 = lane >> 2, pair = (lane & 3) * 2;
       const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-      const int kcol = k0 + r;               // key index of this thread
-      const long long kpos = (long long)kcol - off;  // first causal query of this key
+      const uint32_t ds_st = smem_u32(sDS) + ((warp & 3) * 32 + (lane & 15)) * 128;  // this lane's row for stmatrix
+      const uint32_t ds_ch = wg * 4 + (lane >> 4);                                   // ... and 16-byte chunk
       const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
-      int st = 0, t_in = tq0;                // stage and position in I_h(j) of the next step
-      uint32_t ph_l = 0, par = 0;
-      for (int n = 0; n < N && ok; ++n) {
-        const int b_ = n & 1;
-        const uint32_t sbuf = t_lane + cS0 + b_ * 64 + wg * 32, dpbuf = t_lane + cDP0 + b_ * 64 + wg * 32;
-        uint8_t* ds_row = sDS + b_ * SM::kDS + r * 128;
-        const int i = cowa_bwd_tile_at(rg, t_in);
-        const int q0 = i * BQS;
-        const bool full = cowa_tile_full(w, q0, BQS, k0, BKV, off, Nq, Nk);
-        uint32_t mk = 0xFFFFFFFFu;
-        if (!full) {
-          const long long qend = Nq - 1;
-          const long long base = q0 + wg * 32;
-          uint32_t m = interval_bits32(kpos, min(kpos + w.n - 1, qend), base);
-          if (w.l > 0)
-            m |= interval_bits32(kpos + w.n + w.g, min(kpos + (long long)w.n + w.g + w.l - 1, qend), base);
-          if (kcol < w.s) m |= interval_bits32(kpos, qend, base);
-          mk = kcol < Nk ? m : 0u;
+      // queries that see this lane's key: [near_lo, near_hi] and [far_lo, far_hi]
+      int near_lo = 0, near_hi = -1, far_lo = 0, far_hi = -1;
+      {
+        const volatile int* g_ = geo;
+        const int kcol = k0 + (warp & 3) * 32 + lane;
+        const long long kpos = (long long)kcol - g_[4], qend = g_[5] - 1, far = kpos + g_[1] + g_[2];
+        if (kcol < g_[6]) {
+          near_lo = (int)max(min(kpos, qend + 1), 0ll);
+          near_hi = (int)max(kcol < g_[0] ? qend : min(kpos + g_[1] - 1, qend), -1ll);
+          far_lo = (int)max(min(far, qend + 1), 0ll);
+          far_hi = (int)max(g_[3] > 0 ? min(far + g_[3] - 1, qend) : -1ll, -1ll);
         }
-        const float4* nlse4 = reinterpret_cast<const float4*>(sVec + st * 128 + wg * 32);  // -LSE log2(e), then -Delta
-        const float4* ndlt4 = nlse4 + 16;
-        ok = mbar_wait(bar_ld_full + st, ph_l, a.status);
-        ok = ok && mbar_wait(bar_s_full + b_, par, a.status);
+      }
+      for (int n = 0; n < N && ok; ++n) {
+        const int st = n & 1;
+        const uint32_t par = n & 1;
+        const uint32_t sbuf = t_lane + cS + wg * 32, dpbuf = t_lane + cDP + wg * 32;
+        const float2* nlse2 = reinterpret_cast<const float2*>(sVec + st * 256 + wg * 32 + pair);  // -LSE log2(e), then -Delta
+        ok = mbar_wait(bar_q_full + st, (n >> 1) & 1, a.status);
+        float2 rc[8];  // row constants, read ahead of the wait for the product: shared memory is busy with its operands
+#pragma unroll
+        for (int j = 0; j < 8; ++j) rc[j] = nlse2[(j >> 2) * 32 + (j & 3) * 4];
+        const int info = step_info[st];
+        const bool full = info & 1;
+        uint32_t mk[2], all[2] = {0xFFFFFFFFu, 0xFFFFFFFFu}, seen[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};
+        if (!full) {
+#pragma unroll
+          for (int cb = 0; cb < 2; ++cb) {
+            const int base = info + cb * 64 + wg * 32;
+            mk[cb] = interval_bits(near_lo, near_hi, base) | interval_bits(far_lo, far_hi, base);
+            all[cb] = __ballot_sync(0xffffffffu, mk[cb] == 0xFFFFFFFFu);
+            seen[cb] = __ballot_sync(0xffffffffu, mk[cb] != 0u);
+          }
+        }
+        ok = ok && mbar_wait(bar_s_full, par, a.status);
         if (!ok) break;
         tc_fence_after();
-        float p[32];
-        {
-          uint32_t sr[32], pk[16];
-          tmem_ld32(sbuf, sr);
-          tmem_wait_ld();
+        float p[2][2][16];  // [query block][16-key half]
 #pragma unroll
-          for (int e = 0; e < 32; e += 4) {
-            const float4 nl = nlse4[e / 4];
-            const float2 x = fma2(make_float2(__uint_as_float(sr[e]), __uint_as_float(sr[e + 1])), sc2, make_float2(nl.x, nl.y));
-            const float2 y = fma2(make_float2(__uint_as_float(sr[e + 2]), __uint_as_float(sr[e + 3])), sc2, make_float2(nl.z, nl.w));
-            p[e] = ex2(x.x);
-            p[e + 1] = ex2(x.y);
-            p[e + 2] = ex2(y.x);
-            p[e + 3] = ex2(y.y);
+        for (int cb = 1; cb >= 0; --cb)
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            tmem_ld_frag(sbuf + cb * 64 + ((uint32_t)(h * 16) << 16), p[cb][h]);
+        tmem_wait_ld();
+        tc_fence_before();
+        mbar_arrive(bar_s_read);
+#pragma unroll
+        for (int cb = 0; cb < 2; ++cb) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            float* x = p[cb][h];
+            // of a boundary step only the 16 keys x 32 queries that the boundary crosses are masked, and those beyond it zeroed
+            if ((seen[cb] >> (h * 16)) & 0xFFFFu) {
+#pragma unroll
+              for (int e = 0; e < 16; e += 2) {
+                const float2 y = fma2(make_float2(x[e], x[e + 1]), sc2, rc[cb * 4 + e / 4]);
+                x[e] = ex2(y.x);
+                x[e + 1] = ex2(y.y);
+              }
+              if (((all[cb] >> (h * 16)) & 0xFFFFu) != 0xFFFFu) {
+                const uint32_t m0 = __shfl_sync(0xffffffffu, mk[cb], h * 16 + lane4) >> pair;
+                const uint32_t m1 = __shfl_sync(0xffffffffu, mk[cb], h * 16 + 8 + lane4) >> pair;
+#pragma unroll
+                for (int e = 0; e < 16; ++e)
+                  if (!((((e & 2) ? m1 : m0) >> ((e >> 2) * 8 + (e & 1))) & 1u)) x[e] = 0.f;
+              }
+            } else {
+#pragma unroll
+              for (int e = 0; e < 16; ++e) x[e] = 0.f;
+            }
+            uint32_t pk[8];
+#pragma unroll
+            for (int e = 0; e < 16; e += 2) pk[e / 2] = pack_bf16(x[e], x[e + 1]);
+            tmem_st_frag(sbuf + cb * 16 + ((uint32_t)(h * 16) << 16), pk);  // P^T: 32 queries as 16 bf16 pairs
           }
-          if (!full) {
-#pragma unroll
-            for (int e = 0; e < 32; ++e)
-              if (!((mk >> e) & 1u)) p[e] = 0.f;
-          }
-#pragma unroll
-          for (int e = 0; e < 32; e += 2) pk[e / 2] = pack_bf16(p[e], p[e + 1]);
-          tmem_st16(sbuf, pk);  // P^T: this warpgroup's 32 queries as 16 bf16 pairs
         }
         tmem_wait_st();
         tc_fence_before();
-        mbar_arrive(bar_p_ready + b_);
+        mbar_arrive(bar_p_ready);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) rc[j] = nlse2[64 + (j >> 2) * 32 + (j & 3) * 4];
 
-        ok = mbar_wait(bar_dp_full + b_, par, a.status);
+        ok = mbar_wait(bar_dp_full, par, a.status);
         if (!ok) break;
         tc_fence_after();
-        {
-          uint32_t dr[32], dsp[16];
-          tmem_ld32(dpbuf, dr);
+#pragma unroll
+        for (int cb = 1; cb >= 0; --cb) {  // (dS^T goes where the second block was)
+          float dr[2][16];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) tmem_ld_frag(dpbuf + cb * 64 + ((uint32_t)(h * 16) << 16), dr[h]);
+          // rows past the padded row space: what lies in their Delta is anything
+          const bool none = cb == 1 && !full && info + BQS >= static_cast<const volatile int*>(geo)[5];
           tmem_wait_ld();
 #pragma unroll
-          for (int e = 0; e < 32; e += 4) {
-            const float4 nd = ndlt4[e / 4];
-            const float2 y = mul2(make_float2(p[e], p[e + 1]),
-                                  add2(make_float2(__uint_as_float(dr[e]), __uint_as_float(dr[e + 1])), make_float2(nd.x, nd.y)));
-            const float2 z = mul2(make_float2(p[e + 2], p[e + 3]),
-                                  add2(make_float2(__uint_as_float(dr[e + 2]), __uint_as_float(dr[e + 3])), make_float2(nd.z, nd.w)));
-            dsp[e / 2] = pack_bf16(y.x, y.y);
-            dsp[e / 2 + 1] = pack_bf16(z.x, z.y);
-          }
-          tmem_st16(sbuf + 16, dsp);  // dS^T beside P^T
-          // dS^T also to shared memory (row r = 128 B = 8 chunks, 128B swizzle) for the dQ^T product
+          for (int h = 0; h < 2; ++h) {
+            uint32_t dsp[8];
 #pragma unroll
-          for (int ch = 0; ch < 4; ++ch)
-            *reinterpret_cast<uint4*>(ds_row + (((wg * 4 + ch) ^ (r & 7)) << 4)) =
-                make_uint4(dsp[ch * 4], dsp[ch * 4 + 1], dsp[ch * 4 + 2], dsp[ch * 4 + 3]);
+            for (int e = 0; e < 16; e += 2) {
+              const float2 y = mul2(make_float2(p[cb][h][e], p[cb][h][e + 1]), add2(make_float2(dr[h][e], dr[h][e + 1]), rc[cb * 4 + e / 4]));
+              dsp[e / 2] = pack_bf16(y.x, y.y);
+            }
+            if (none) {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) dsp[e] = 0u;
+            }
+            tmem_st_frag(dpbuf + 64 + cb * 16 + ((uint32_t)(h * 16) << 16), dsp);
+            // dS^T also to shared memory (a key's row = 128 B = 8 chunks, 128B swizzle) for the dQ^T product, whose last
+            // reading of the tile is complete: it was issued ahead of dP^T
+#pragma unroll
+            for (int j = 0; j < 4; j += 2)
+              stmatrix4(ds_st + cb * SM::kDS + h * 2048 + (((ds_ch + j) ^ (lane & 7)) << 4), dsp + 2 * j);
+          }
         }
         tmem_wait_st();
         tc_fence_before();
         fence_proxy_async_smem();
-        mbar_arrive(bar_ds_ready + b_);
-        if (b_) par ^= 1;
-        if (++st == NST) { st = 0; ph_l ^= 1; }
-        if (++t_in == cnt) t_in = 0;
+        mbar_arrive(bar_ds_ready);
       }
       if (wg == 0) store_grad(true);
     }
   } else {
-    setmaxnreg_dec<112>();
     {
+      const int N = step_count();
       // ======== dQ drain warpgroup: one d column of dQ^T per thread; TMEM -> shared -> bulk reduce-add ========
-      const int d = (warp & 3) * 32 + lane;
+      float* sDQ = reinterpret_cast<float*>(smem + SM::oDQ) + (warp & 3) * 2048;
       const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-      const bool issuer = (d == 0);
-      int g = g0, t_in = tq0;
+      const bool mine = (warp & 3) * 32 < D;
       for (int n = 0; n < N && ok; ++n) {
-        const int i = cowa_bwd_tile_at(rg, t_in);
-        const int bhq = bhq0 + g, q0 = i * BQS;
-        if (++t_in == cnt) { t_in = 0; ++g; }
-        ok = mbar_wait(bar_dq_full + (n & 1), (n >> 1) & 1, a.status);
+        ok = mbar_wait(bar_dq_full, n & 1, a.status);
         if (!ok) break;
         tc_fence_after();
-        uint32_t v[2][32];
-        tmem_ld32(t_lane + cDP0 + (n & 1) * 64, v[0]);
-        tmem_ld32(t_lane + cDP0 + (n & 1) * 64 + 32, v[1]);
-        tmem_wait_ld();
-        tc_fence_before();
-        mbar_arrive(bar_dq_free + (n & 1));
+        // 32 query rows of this warp's 32 d: staged in one of two tiles and added to the accumulator as one range
+        const long long at_ = dq_at[n & 3];
+        float* gdst = a.dq_acc + (at_ & ~1ll) + (warp & 3) * (BQS * 32);
+        auto add_rows = [&](const uint32_t (&v)[32], int quarter) {
+          if (!mine || (quarter >= 2 && (at_ & 1))) return;
+          float* stage = sDQ + (quarter & 1) * 1024;
+          if (lane == 0) tma_wait_group_read<1>();  // the reduction issued from this tile before has read it
+          __syncwarp();
+          if (a.dq_fixed) {
+            // Rounded to integers on the FMA and integer pipes (the conversion instruction runs at the rate of the
+            // exponentials and competes with them): below 2^22, x + 1.5 * 2^23 has rint(x) in its low mantissa bits.  Larger
+            // ones go in two parts, x = 2^16 h + l with h = rint(x / 2^16), |l| <= 2^15, both exact; shifting the first
+            // sum by 16 drops its exponent.  Both give what __float2int_rn gives.
+            const float2 fx2 = make_float2(a.scale * kDqFixedOne, a.scale * kDqFixedOne);
+            auto c2 = [](float c_) { return make_float2(c_, c_); };
+            float worst = 0.f;
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          float* stage = sDQ + hf * (SM::kDQ / 4);
-          if (issuer) tma_wait_group_read<1>();  // the reduction issued from this tile one step ago has read it
-          wg_sync(3);
-          if (d < D) {
-            if (a.dq_fixed) {
-              // Rounded to integers on the FMA and integer pipes (the conversion instruction runs at the rate of the
-              // exponentials and competed with them: one KV head of 20001 tokens 942 / 880 thousand clocks): x = 2^16 h + l
-              // with h = rint(x / 2^16), |l| <= 2^15, both exact; adding 1.5 * 2^23 leaves an integer in the low mantissa
-              // bits, and shifting the first sum by 16 drops its exponent.  Same integers as __float2int_rn.
-              const float2 fx2 = make_float2(a.scale * kDqFixedOne, a.scale * kDqFixedOne);
-              auto c2 = [](float c_) { return make_float2(c_, c_); };
-              float worst = 0.f;
+            for (int c = 0; c < 32; c += 2)
+              worst = max_nan(worst, max_nan(fabsf(__uint_as_float(v[c])), fabsf(__uint_as_float(v[c + 1]))));
+            worst *= fabsf(fx2.x);
+            if (__all_sync(0xffffffffu, worst < 4194303.f)) {
 #pragma unroll
-              for (int c = 0; c < 32; c += 2) {
-                const float2 x = mul2(make_float2(__uint_as_float(v[hf][c]), __uint_as_float(v[hf][c + 1])), fx2);
-                worst = max_nan(worst, max_nan(fabsf(x.x), fabsf(x.y)));
-                const float2 th = fma2(x, c2(1.f / 65536.f), c2(12582912.f));
-                const float2 l = fma2(add2(th, c2(-12582912.f)), c2(-65536.f), x);
-                const float2 tl = add2(l, c2(12582912.f));
-                int* dst = reinterpret_cast<int*>(stage) + c * D + d;
-                dst[0] = (__float_as_int(th.x) << 16) + (__float_as_int(tl.x) - 0x4B400000);
-                dst[D] = (__float_as_int(th.y) << 16) + (__float_as_int(tl.y) - 0x4B400000);
+              for (int c = 0; c < 32; c += 4) {
+                const float2 x = fma2(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), fx2, c2(12582912.f));
+                const float2 y = fma2(make_float2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), fx2, c2(12582912.f));
+                *reinterpret_cast<int4*>(stage + c * 32 + lane * 4) =
+                    make_int4(__float_as_int(x.x) - 0x4B400000, __float_as_int(x.y) - 0x4B400000,
+                              __float_as_int(y.x) - 0x4B400000, __float_as_int(y.y) - 0x4B400000);
               }
-              if (!(worst < 2147483520.f)) atomicOr(a.status, (unsigned)COWA_DEV_DQ_RANGE);  // would not fit 32 bits (or NaN)
             } else {
 #pragma unroll
-              for (int c = 0; c < 32; ++c) stage[c * D + d] = __uint_as_float(v[hf][c]) * a.scale;
+              for (int c = 0; c < 32; c += 4) {
+                int o[4];
+#pragma unroll
+                for (int e = 0; e < 4; e += 2) {
+                  const float2 x = mul2(make_float2(__uint_as_float(v[c + e]), __uint_as_float(v[c + e + 1])), fx2);
+                  const float2 th = fma2(x, c2(1.f / 65536.f), c2(12582912.f));
+                  const float2 l = fma2(add2(th, c2(-12582912.f)), c2(-65536.f), x);
+                  const float2 tl = add2(l, c2(12582912.f));
+                  o[e] = (__float_as_int(th.x) << 16) + (__float_as_int(tl.x) - 0x4B400000);
+                  o[e + 1] = (__float_as_int(th.y) << 16) + (__float_as_int(tl.y) - 0x4B400000);
+                }
+                *reinterpret_cast<int4*>(stage + c * 32 + lane * 4) = make_int4(o[0], o[1], o[2], o[3]);
+              }
+              if (!(worst < 2147483520.f)) atomicOr(a.status, (unsigned)COWA_DEV_DQ_RANGE);  // would not fit 32 bits (or NaN)
             }
+          } else {
+#pragma unroll
+            for (int c = 0; c < 32; c += 4)
+              *reinterpret_cast<float4*>(stage + c * 32 + lane * 4) =
+                  make_float4(__uint_as_float(v[c]) * a.scale, __uint_as_float(v[c + 1]) * a.scale,
+                              __uint_as_float(v[c + 2]) * a.scale, __uint_as_float(v[c + 3]) * a.scale);
           }
           fence_proxy_async_smem();
-          wg_sync(3);
-          if (issuer) {
-            // 32 query rows of the accumulator are one contiguous range (rows are D floats, padded row space)
-            void* gdst = a.dq_acc + (((size_t)bhq * vec_stride + pbase + q0 + hf * 32) * D);
-            if (a.dq_fixed) bulk_reduce_add_s32(gdst, stage, 32 * D * 4);
-            else bulk_reduce_add_f32(gdst, stage, 32 * D * 4);
+          __syncwarp();
+          if (lane == 0) {
+            float* dst = gdst + (quarter >> 1) * (BQS * D) + (quarter & 1) * 1024;
+            if (a.dq_fixed) bulk_reduce_add_s32(dst, stage, 4096);
+            else bulk_reduce_add_f32(dst, stage, 4096);
             tma_commit_group();
           }
-        }
+        };
+        // first the columns that dP^T waits for, then those of S^T, as registers allow
+        uint32_t v0[32], v1[32], v2[32];
+        tmem_ld32(t_lane + cDQ + 64, v0);
+        tmem_ld32(t_lane + cDQ + 96, v1);
+        tmem_wait_ld();
+        tc_fence_before();
+        mbar_arrive(bar_dq_free);
+        add_rows(v0, 2);
+        tmem_ld32(t_lane + cDQ, v2);
+        tmem_ld32(t_lane + cDQ + 32, v0);
+        tmem_wait_ld();
+        tc_fence_before();
+        mbar_arrive(bar_dq_free + 1);
+        add_rows(v1, 3);
+        add_rows(v2, 0);
+        add_rows(v0, 1);
       }
-      if (issuer) tma_wait_group<0>();
+      if (lane == 0) tma_wait_group<0>();
       store_grad(false);
     }
   }
@@ -781,47 +847,46 @@ __global__ void cowa_bwd_preprocess_varlen_kernel(const __nv_bfloat16* __restric
   }
 }
 
-// 8 elements of the dQ accumulator (fp32, or 32-bit integers in units of 2^-18) -> bf16
-__device__ __forceinline__ uint4 dq_bf16(const float4* src, int fixed, unsigned int* status) {
-  float4 x = src[0], y = src[1];
-  if (fixed) {
-    const float u = 1.f / kDqFixedOne;
-    x = make_float4(__float_as_int(x.x) * u, __float_as_int(x.y) * u, __float_as_int(x.z) * u, __float_as_int(x.w) * u);
-    y = make_float4(__float_as_int(y.x) * u, __float_as_int(y.y) * u, __float_as_int(y.z) * u, __float_as_int(y.w) * u);
-    // half of the representable range: a total that wrapped around lands out here in most cases
-    const float big = fmaxf(fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))),
-                            fmaxf(fmaxf(fabsf(y.x), fabsf(y.y)), fmaxf(fabsf(y.z), fabsf(y.w))));
-    if (big >= 4096.f) atomicOr(status, (unsigned)COWA_DEV_DQ_RANGE);
-  }
-  return make_uint4(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w), pack_bf16(y.x, y.y), pack_bf16(y.z, y.w));
-}
-
-// The dQ accumulator to bf16.  Batched: 8 elements a thread; packed: one 64-row chunk of the padded row space and one head a
-// block, into the packed rows.  (One kernel with the sum of partial dK, dV needs 46 registers and lost occupancy: 137
-// instead of 112 us at 32K.)
+// The dQ accumulator to bf16: one 64-row chunk of the row space and one head a block, every row's 16-byte pieces of four
+// rows and one d (see the drain); a thread takes four rows of two d, so that a warp reads 1 KB ranges and writes whole
+// sectors.  (One kernel with the sum of partial dK, dV needs 46 registers and lost occupancy: 137 instead of 112 us at 32K.)
 template <int D, bool VARLEN>
-__global__ void __launch_bounds__(VARLEN ? BQS * (D / 8) : 256)
+__global__ void __launch_bounds__(256)
 cowa_bwd_convert_dq_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, const int* __restrict__ cu, int B,
-                           int T, int Tpad, long long BH, int H, int fixed, CowaStrides sq, unsigned int* status) {
-  constexpr int TPR = D / 8;  // threads per row (16 bytes of bf16 each)
-  const int part = threadIdx.x % TPR;
+                           int T, int Tpad, int H, int fixed, CowaStrides sq, unsigned int* status) {
+  const int nchunk = Tpad / BQS, chunk = VARLEN ? blockIdx.x : blockIdx.x % nchunk, bh = VARLEN ? blockIdx.y : blockIdx.x / nchunk;
+  int rows, first;  // rows of this chunk, and the first one's place among the rows of dq
+  __nv_bfloat16* out;
   if constexpr (!VARLEN) {
-    const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / TPR;
-    if (row >= BH * T) return;
-    const long long bh = row / T;
-    const int t = (int)(row % T);
-    const uint4 v = dq_bf16(reinterpret_cast<const float4*>(acc + ((size_t)bh * Tpad + t) * D + part * 8), fixed, status);
-    *reinterpret_cast<uint4*>(dq + (size_t)(bh / H) * sq.b + (size_t)(bh % H) * sq.h + (size_t)t * sq.t + part * 8) = v;
+    first = chunk * BQS;
+    rows = T - first;
+    out = dq + (size_t)(bh / H) * sq.b + (size_t)(bh % H) * sq.h;
   } else {
-    const int chunk = blockIdx.x, h = blockIdx.y, r = threadIdx.x / TPR;
     int b, lc, nch, pb;
     if (!varlen_locate(cu, B, chunk, BQS, BQS, &b, &lc, &nch, &pb)) return;
-    const int t = lc * BQS + r;
     const int rbase = cu[b];
-    if (t >= cu[b + 1] - rbase || rbase < 0 || rbase + t >= T) return;
-    const uint4 v = dq_bf16(reinterpret_cast<const float4*>(acc + ((size_t)h * Tpad + (size_t)chunk * BQS + r) * D + part * 8),
-                            fixed, status);
-    *reinterpret_cast<uint4*>(dq + ((size_t)h * T + rbase + t) * D + part * 8) = v;
+    first = rbase + lc * BQS;
+    rows = rbase < 0 ? 0 : min(cu[b + 1], T) - first;
+    out = dq + (size_t)bh * sq.h;
+  }
+  const float4* src = reinterpret_cast<const float4*>(acc + ((size_t)bh * Tpad + (size_t)chunk * BQS) * D);
+#pragma unroll
+  for (int i = 0; i < D / 32; ++i) {
+    const int item = i * 256 + threadIdx.x, r = item / 16 % 16 * 4, d = item / 256 * 32 + item % 16 * 2;
+    float4 x = src[item * 2], y = src[item * 2 + 1];
+    if (fixed) {
+      const float u = 1.f / kDqFixedOne;
+      x = make_float4(__float_as_int(x.x) * u, __float_as_int(x.y) * u, __float_as_int(x.z) * u, __float_as_int(x.w) * u);
+      y = make_float4(__float_as_int(y.x) * u, __float_as_int(y.y) * u, __float_as_int(y.z) * u, __float_as_int(y.w) * u);
+      // half of the representable range: a total that wrapped around lands out here in most cases
+      const float big = fmaxf(fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))),
+                              fmaxf(fmaxf(fabsf(y.x), fabsf(y.y)), fmaxf(fabsf(y.z), fabsf(y.w))));
+      if (big >= 4096.f) atomicOr(status, (unsigned)COWA_DEV_DQ_RANGE);
+    }
+    const uint32_t v[4] = {pack_bf16(x.x, y.x), pack_bf16(x.y, y.y), pack_bf16(x.z, y.z), pack_bf16(x.w, y.w)};
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (r + e < rows) *reinterpret_cast<uint32_t*>(out + (size_t)(first + r + e) * sq.t + d) = v[e];
   }
 }
 
@@ -1005,8 +1070,8 @@ int launch_bwd(const void* q, const void* k, const void* v, const void* o, const
   if ((rc = cowa::resolve_strides(p->o_strides, Hq, Nq, D, &so))) return rc;
   if (BH > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
   CUtensorMap mq, mk, mv, mdo, mdk, mdv;
-  if ((rc = cowa::make_tensor_map(&mq, q, cowa::MapType::BF16, D, T, Hq, B, sq, 64, BQS))) return rc;
-  if ((rc = cowa::make_tensor_map(&mdo, d_o, cowa::MapType::BF16, D, T, Hq, B, so, 64, BQS))) return rc;
+  if ((rc = cowa::make_tensor_map(&mq, q, cowa::MapType::BF16, D, T, Hq, B, sq, 64, BQT))) return rc;
+  if ((rc = cowa::make_tensor_map(&mdo, d_o, cowa::MapType::BF16, D, T, Hq, B, so, 64, BQT))) return rc;
   if ((rc = cowa::make_tensor_map(&mk, k, cowa::MapType::BF16, D, Nk, Hkv, B, sk, 64, BKV))) return rc;
   if ((rc = cowa::make_tensor_map(&mv, v, cowa::MapType::BF16, D, Nk, Hkv, B, sv, 64, BKV))) return rc;
   if ((rc = cowa::make_tensor_map(&mdk, dk, cowa::MapType::BF16, D, Nk, Hkv, B, sk, 64, BKV))) return rc;
@@ -1041,8 +1106,8 @@ int launch_bwd(const void* q, const void* k, const void* v, const void* o, const
   if (p->bwd_main_stop_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_stop_event), st));
   launch_reduce<D, false>(a, pl, sk, sv, st);
   COWA_CUDA_TRY(cudaGetLastError());
-  cowa_bwd_convert_dq_kernel<D, false><<<(unsigned)((BH * T * (D / 8) + 255) / 256), 256, 0, st>>>(
-      dq_acc, static_cast<__nv_bfloat16*>(dq), nullptr, B, T, Tpad, BH, Hq, a.dq_fixed, sq, a.status);
+  cowa_bwd_convert_dq_kernel<D, false><<<(unsigned)(Tpad / BQS * BH), 256, 0, st>>>(
+      dq_acc, static_cast<__nv_bfloat16*>(dq), nullptr, B, T, Tpad, Hq, a.dq_fixed, sq, a.status);
   COWA_CUDA_TRY(cudaGetLastError());
   return COWA_OK;
 }
@@ -1066,8 +1131,8 @@ int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o
   CUtensorMap mq, mk, mv, mdo, mdk, mdv;
   int rc;
   const CowaStrides sq = packed_strides(Hq, total, D), sk = packed_strides(Hkv, total, D);
-  if ((rc = cowa::make_tensor_map(&mq, q, cowa::MapType::BF16, D, total, Hq, 1, sq, 64, BQS))) return rc;
-  if ((rc = cowa::make_tensor_map(&mdo, d_o, cowa::MapType::BF16, D, total, Hq, 1, sq, 64, BQS))) return rc;
+  if ((rc = cowa::make_tensor_map(&mq, q, cowa::MapType::BF16, D, total, Hq, 1, sq, 64, BQT))) return rc;
+  if ((rc = cowa::make_tensor_map(&mdo, d_o, cowa::MapType::BF16, D, total, Hq, 1, sq, 64, BQT))) return rc;
   if ((rc = cowa::make_tensor_map(&mk, k, cowa::MapType::BF16, D, total, Hkv, 1, sk, 64, BKV))) return rc;
   if ((rc = cowa::make_tensor_map(&mv, v, cowa::MapType::BF16, D, total, Hkv, 1, sk, 64, BKV))) return rc;
   if ((rc = cowa::make_tensor_map(&mdk, dk, cowa::MapType::BF16, D, total, Hkv, 1, sk, 64, BKV))) return rc;
@@ -1103,8 +1168,8 @@ int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o
   if (p->bwd_main_stop_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_stop_event), st));
   launch_reduce<D, true>(a, pl, sk, sk, st);
   COWA_CUDA_TRY(cudaGetLastError());
-  cowa_bwd_convert_dq_kernel<D, true><<<chunks, BQS * (D / 8), 0, st>>>(dq_acc, static_cast<__nv_bfloat16*>(dq), cu, B, total,
-                                                                        Tpad, 0, Hq, a.dq_fixed, sq, a.status);
+  cowa_bwd_convert_dq_kernel<D, true><<<chunks, 256, 0, st>>>(dq_acc, static_cast<__nv_bfloat16*>(dq), cu, B, total, Tpad, Hq,
+                                                              a.dq_fixed, sq, a.status);
   COWA_CUDA_TRY(cudaGetLastError());
   return COWA_OK;
 }
