@@ -1,6 +1,6 @@
 // CoWindow Attention forward (Algorithm 1) for sm_100a: two QO heads of a GQA group per block.
 //
-// Persistent, one block per SM.  A work item is (batch, pair of QO heads that share a KV head, 128-row QO tile);
+// One block per SM at a time, each taking over further blocks of the grid (cluster launch control).  A work item is (batch, pair of QO heads that share a KV head, 128-row QO tile);
 // both heads visit the same KV tiles J_h(i), so one pass over K and V serves 256 query rows.  A step takes two
 // visited 64-key tiles (not necessarily neighbours) as one 128-key operand: S at N = 128 runs at the full tensor
 // rate (512 clocks; as two products of 64 keys 768).  Warps:
@@ -58,6 +58,7 @@ struct PairSmem {
   static constexpr int kKV = BS * D * 2;   // K or V operand of one step
   static constexpr int kOut = BQ * 128;    // one 64-column slab of an O tile on its way out
   static constexpr int oQ = 0, oK = 2 * kQ, oV = oK + 2 * kKV, oOut = oV + 2 * kKV, oBar = oOut + 2 * kOut;
+  static constexpr int oNext = oBar + 240;           // the next item's number, as the hardware answers
   static constexpr int oItem = oBar + 256;           // two work items
   static constexpr int kBytes = oItem + 256 + 1024;  // + alignment slack
 };
@@ -133,7 +134,7 @@ template <int D, bool VARLEN, bool SPLIT>
 __global__ void __launch_bounds__(kPairThreads, 1)
 cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                      const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
-                     const __grid_constant__ FwdArgs a, const int items) {
+                     const __grid_constant__ FwdArgs a) {
   using SM = PairSmem<D>;
   constexpr int NSLAB = D / 64;        // 64-element (128-byte) slabs along D
   constexpr int SLAB = 128 * 128;      // bytes of one slab of a 128-row tile
@@ -161,14 +162,15 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   uint64_t* bar_o_empty = bars + 18;  // [2 heads] count 4: O has been read
   uint64_t* bar_i_full = bars + 20;   // [2] a work item has been published
   uint64_t* bar_i_empty = bars + 22;  // [2] count kItemReaders: it has been read
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 24);
+  uint64_t* bar_next = bars + 24;     //     the next item's number is here
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 25);
 
   const int tid = threadIdx.x;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform by construction
 
   if (tid == 0) {
-    for (int s = 0; s < 24; ++s)
-      mbar_init(bars + s, (s >= 12 && s < 16) || s == 18 || s == 19 ? 4 : s >= 22 ? kItemReaders : 1);
+    for (int s = 0; s < 25; ++s)
+      mbar_init(bars + s, (s >= 12 && s < 16) || s == 18 || s == 19 ? 4 : s == 22 || s == 23 ? kItemReaders : 1);
     fence_mbar_init();
   }
   if (warp == 9) {
@@ -210,17 +212,33 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     if (lead) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); }
     int c = 0;       // steps loaded so far, all items together: step c uses slot c & 1
     uint32_t ni = 0;  // items so far
-    // Items come heaviest first; blocks take them in rounds, every second round from the other end, so that a block
-    // with a heavy item in one round has a light one in the next.
+    // The grid has a block per item, heaviest items first.  A block starts with its own and, towards the end of an item,
+    // takes over the next one whose block has not started: lists differ in length, and with a fixed share of the items per
+    // block the last SM was busy 20 % longer than the average one (one KV head of 20001 tokens), 25 % for packed prompts.
     const int csize = SPLIT ? (int)cluster_size() : 1;
-    for (int rnd = 0; ok; ++rnd) {
-      const long long base = SPLIT ? (rnd == 0 ? 0 : items) : (long long)rnd * gridDim.x;
-      const int idx = SPLIT ? blockIdx.x / csize : (int)(base + ((rnd & 1) ? gridDim.x - 1 - blockIdx.x : blockIdx.x));
+    uint32_t asked = 0, answered = 0;  // requests
+    auto ask = [&]() {
+      if (lead) {
+        mbar_expect_tx(bar_next, 16);
+        clc_request(smem + SM::oNext, bar_next);
+      }
+      ++asked;
+    };
+    auto next_index = [&]() -> int {
+      answered = asked;
+      if (!mbar_wait(bar_next, (asked - 1) & 1, a.status)) { ok = false; return -1; }
+      const int x = __shfl_sync(0xFFFFFFFFu, clc_block(smem + SM::oNext), 0);
+      fence_proxy_async_smem();  // read before the next answer is written
+      __syncwarp();
+      return x;
+    };
+    int idx = SPLIT ? blockIdx.x / csize : blockIdx.x;
+    while (ok) {
       PairItem& it = *reinterpret_cast<PairItem*>(smem + SM::oItem + (ni & 1) * 128);
       {
         PairItem mine;
         if (SPLIT) {
-          if (rnd > 0) break;
+          if (ni > 0) break;
           if (locate_item<VARLEN>(a, idx, mine)) {
             const int n = (mine.nt + 1) >> 1, rank = (int)cluster_rank();
             mine.t0 = 2 * (n * rank / csize);
@@ -228,9 +246,11 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
           } else {
             mine.nt = mine.work = 0;
           }
-        } else if (base >= items) {
+        } else if (idx < 0) {
           mine.nt = 0;
-        } else if (idx >= items || !locate_item<VARLEN>(a, idx, mine)) {
+        } else if (!locate_item<VARLEN>(a, idx, mine)) {
+          ask();
+          idx = next_index();
           continue;
         }
         if (ni >= 2) ok = mbar_wait(bar_i_empty + (ni & 1), ((ni >> 1) & 1) ^ 1, a.status);
@@ -252,11 +272,13 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
           }
         }
       };
+      const int ask_at = max((it.nt - 1) / 2 - 2, 0) * 2;  // two steps before the last
       for (int t = 0; t < it.nt; t += 2, ++c) {
         const int sl = c & 1;
         const uint32_t ph = ((c >> 1) & 1) ^ 1;
         if (c >= 2) ok = mbar_wait(bar_k_empty + sl, ph, a.status);
         if (!ok) break;
+        if (!SPLIT && t == ask_at) ask();  // a microsecond or more before the answer is needed
         load_kv(sK + sl * SM::kKV, &tmK, bar_k_full + sl, t);
         if (t == 0) {
           if (ni > 0) ok = mbar_wait(bar_q_empty, (ni - 1) & 1, a.status);
@@ -273,7 +295,9 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         load_kv(sV + sl * SM::kKV, &tmV, bar_v_full + sl, t);
       }
       ++ni;
+      if (!SPLIT && ok) idx = next_index();
     }
+    if (asked != answered) mbar_wait(bar_next, (asked - 1) & 1, a.status);  // (a wait ran out) no answer may come later
    } else if (warp == 9) {
     // ======================= MMA issuer (warp-uniform control flow, one elected lane issues) =======================
     const bool lead = elect_one();
@@ -705,13 +729,13 @@ int launch_fwd_pair(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensor
   }
   COWA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PairSmem<D>::kBytes));
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(split > 1 ? items * split : std::min<long long>(items, sm_count())));
+  cfg.gridDim = dim3((unsigned)(items * split));
   cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = PairSmem<D>::kBytes; cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr; cfg.numAttrs = split > 1 ? 1 : 0;
-  COWA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mo, a, (int)items));
+  COWA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mo, a));
   return COWA_OK;
 }
 
