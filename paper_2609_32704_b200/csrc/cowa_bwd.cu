@@ -107,7 +107,7 @@ __device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t 
 
 // Tile number q of class c: sink tiles of every head first (they meet every query tile of their sequence and are the
 // longest), then head-major with ascending KV tile (consecutive blocks share dQ rows, which then stay in L2).  Packed
-// batches: whole warps only; false when there is no such tile (the count is an upper bound).
+// batches: the same sequence by sequence, longest first; whole warps only; false when there is no such tile (the count is an upper bound).
 struct TileAt {
   int hk, b, j, nts, pbase;
 };
@@ -131,6 +131,13 @@ __device__ __forceinline__ bool locate_tile(const BwdArgs& a, int c, int q, Tile
   }
   if (c == 2) q += a.cls_tiles[1];
   if constexpr (VARLEN) {
+    if (a.B <= kLongestFirst) {
+      if (!varlen_locate_longest(a.cu, a.cu, a.B, q, BKV, a.Hkv, nsk, &x.b, &x.j, &x.nts)) return false;
+      const int n = x.nts - nsk;
+      x.hk = x.j / n; x.j = nsk + x.j % n;
+      varlen_seq_info(a.cu, x.b, BKV, BQS, &x.nts, &x.pbase);
+      return fits(a, x);
+    }
     x.hk = q / a.tiles_bound;
     return varlen_locate(a.cu, a.B, q % a.tiles_bound, BKV, BQS, &x.b, &x.j, &x.nts, &x.pbase, nsk) && fits(a, x);
   }

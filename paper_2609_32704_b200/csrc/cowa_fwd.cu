@@ -78,10 +78,12 @@ cowa_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     b = idx % a.B; idx /= a.B;
     i = (a.Nq + BQ - 1) / BQ - 1 - idx;
   } else {
-    // idx counts the QO tiles of the packed batch, sequence after sequence, each sequence's heaviest
-    // (last) tile first.  Every warp finds its (sequence, tile) by a cooperative scan of the offsets.
+    // idx counts the QO tiles of the packed batch, longest sequence first, each sequence's heaviest (last) tile first.
+    // Every warp finds its (sequence, tile) by a cooperative scan of the offsets.  The grid is an upper bound.
     int lt, nts, pb;
-    if (!varlen_locate(a.cu_q, a.B, idx, BQ, 0, &b, &lt, &nts, &pb)) return;  // the grid is an upper bound
+    if (a.B <= kLongestFirst ? !varlen_locate_longest(a.cu_q, a.cu_k, a.B, idx, BQ, 1, 0, &b, &lt, &nts)
+                             : !varlen_locate(a.cu_q, a.B, idx, BQ, 0, &b, &lt, &nts, &pb))
+      return;
     i = nts - 1 - lt;
   }
   const int h = hk * a.G + g;

@@ -404,6 +404,43 @@ __device__ __forceinline__ bool varlen_locate(const int* __restrict__ cu, int B,
   return false;
 }
 
+// The same with the sequences taken longest first (by their length in cu_len; equal ones in order), `mult` work items per
+// tile: the sequence that work item idx belongs to, the item's number in it and the sequence's tile count.  The last items
+// of a batch are then its shortest lists, whatever the order in the batch.  Up to kLongestFirst sequences: every lane
+// compares its two with all others, which is a few hundred instructions; for more the order of the batch stays.
+constexpr int kLongestFirst = 64;
+__device__ __forceinline__ bool varlen_locate_longest(const int* __restrict__ cu, const int* __restrict__ cu_len, int B,
+                                                      int idx, int tile, int mult, int skip, int* b_out, int* item,
+                                                      int* tiles_in_seq) {
+  const int lane = threadIdx.x & 31;
+  int len[2], n[2], ahead[2] = {0, 0};
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int b = i * 32 + lane;
+    len[i] = b < B ? cu_len[b + 1] - cu_len[b] : -1;
+    n[i] = b < B ? max((max(cu[b + 1] - cu[b], 0) + tile - 1) / tile - skip, 0) * mult : 0;
+  }
+  for (int j = 0; j < B; ++j) {
+    const int lj = __shfl_sync(0xFFFFFFFFu, j < 32 ? len[0] : len[1], j & 31);
+    const int nj = __shfl_sync(0xFFFFFFFFu, j < 32 ? n[0] : n[1], j & 31);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (lj > len[i] || (lj == len[i] && j < i * 32 + lane)) ahead[i] += nj;
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, idx >= ahead[i] && idx < ahead[i] + n[i]);
+    if (m) {
+      const int src = __ffs(m) - 1;
+      *b_out = i * 32 + src;
+      *item = idx - __shfl_sync(0xFFFFFFFFu, ahead[i], src);
+      *tiles_in_seq = __shfl_sync(0xFFFFFFFFu, n[i], src) / mult + skip;
+      return true;
+    }
+  }
+  return false;
+}
+
 // Companion of varlen_locate for a known sequence b: its tile count and its padded row base (warp-cooperative).
 __device__ __forceinline__ void varlen_seq_info(const int* __restrict__ cu, int b, int tile, int pad, int* tiles_in_seq,
                                                 int* pad_base) {
