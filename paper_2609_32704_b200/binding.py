@@ -101,6 +101,41 @@ def lib():
     return _lib
 
 
+class _PythonPath:
+    """Stands in for the native argument path where it cannot be loaded: every call takes the Python path."""
+    fwd = prefill = prefill_varlen = bwd = bwd_varlen = decode = decode_multi = decode_paged = staticmethod(lambda *a: None)
+
+
+_native = None
+
+
+def _call():
+    """The native argument path (csrc_py/cowa_call.cpp).  Its functions return the entry point's status, or None when the
+    call is left to the code below them."""
+    global _native
+    if _native is None:
+        import torch
+        L = lib()
+        try:
+            from . import _cowa_call as m
+            if m.torch_version != torch.__version__.split("+")[0]:
+                raise ImportError("built against another torch")
+            m.bind(Params, [C.cast(getattr(L, n), C.c_void_p).value for n in (
+                "cowa_fwd", "cowa_prefill", "cowa_prefill_varlen", "cowa_bwd", "cowa_bwd_varlen", "cowa_decode",
+                "cowa_decode_multi", "cowa_decode_paged")])
+            _native = m
+        except ImportError:
+            _native = _PythonPath
+    return _native
+
+
+def _done(status, where):
+    if status is None:
+        return False
+    _check(status, where)
+    return True
+
+
 def make_params(sink=0, local=1, block=128, softmax_scale=1.0, windows=None, full_attn=False,
                 hkv_global=0, hkv_offset=0, block_q=None, block_k=None, deterministic=False):
     """Fills a cowa_params_t.  `windows`: optional list of (sink, near, gap, len) per KV head."""
@@ -181,6 +216,8 @@ def _same_layout(a, b, na, nb):
 def cowa_fwd(q, k, v, o, lse, params):
     """q [B,Hq,T,D], k/v [B,Hkv,T,D] bf16 -> o (bf16), lse (fp32 [B,Hq,T]); all preallocated.  q, k, v, o may
     be strided views with that shape (e.g. x.transpose(1, 2) of a [B,T,H,D] tensor)."""
+    if _done(_call().fwd(q, k, v, o, lse, params), "cowa_fwd"):
+        return
     import torch
     for t, n in ((q, "q"), (k, "k"), (v, "v"), (o, "o")):
         _need(t, torch.bfloat16, n, strided=True)
@@ -194,6 +231,8 @@ def cowa_fwd(q, k, v, o, lse, params):
 
 def cowa_prefill(q, k, v, o, lse, params):
     """Forward with N_q <= N_k (bottom-right aligned): q [B,Hq,Nq,D], k/v [B,Hkv,Nk,D] -> o, lse [B,Hq,Nq]."""
+    if _done(_call().prefill(q, k, v, o, lse, params), "cowa_prefill"):
+        return
     import torch
     for t, n in ((q, "q"), (k, "k"), (v, "v"), (o, "o")):
         _need(t, torch.bfloat16, n, strided=True)
@@ -208,6 +247,8 @@ def cowa_prefill(q, k, v, o, lse, params):
 def cowa_prefill_varlen(q, k, v, o, lse, cu_seqlens_q, cu_seqlens_k, params):
     """Packed batch: q [Hq,total_q,D], k/v [Hkv,total_k,D] -> o, lse [Hq,total_q]; cu_seqlens_* are CUDA int32
     tensors of B+1 row offsets."""
+    if _done(_call().prefill_varlen(q, k, v, o, lse, cu_seqlens_q, cu_seqlens_k, params), "cowa_prefill_varlen"):
+        return
     import torch
     for t, n in ((q, "q"), (k, "k"), (v, "v"), (o, "o")):
         _need(t, torch.bfloat16, n)
@@ -231,6 +272,8 @@ def cowa_bwd_workspace_bytes(B, T, Hq, Hkv, D, params):
 def cowa_bwd(q, k, v, o, lse, d_o, dq, dk, dv, params, workspace):
     """Gradients dq, dk, dv (bf16, preallocated) of cowa_fwd; workspace: uint8 CUDA tensor.  Strided views are
     accepted when d_o is laid out like o, dq like q, dk like k and dv like v."""
+    if _done(_call().bwd(q, k, v, o, lse, d_o, dq, dk, dv, params, workspace), "cowa_bwd"):
+        return
     import torch
     for t, n in ((q, "q"), (k, "k"), (v, "v"), (o, "o"), (d_o, "d_o"), (dq, "dq"), (dk, "dk"), (dv, "dv")):
         _need(t, torch.bfloat16, n, strided=True)
@@ -272,6 +315,8 @@ def cowa_bwd_varlen_workspace_bytes(B, total, Hq, Hkv, D, params):
 def cowa_bwd_varlen(q, k, v, o, lse, d_o, dq, dk, dv, cu_seqlens, params, workspace):
     """Packed batch (N_q = N_k per sequence): q/o/d_o/dq [Hq,total,D], k/v/dk/dv [Hkv,total,D], lse [Hq,total];
     cu_seqlens CUDA int32 [B+1]."""
+    if _done(_call().bwd_varlen(q, k, v, o, lse, d_o, dq, dk, dv, cu_seqlens, params, workspace), "cowa_bwd_varlen"):
+        return
     import torch
     for t, n in ((q, "q"), (k, "k"), (v, "v"), (o, "o"), (d_o, "d_o"), (dq, "dq"), (dk, "dk"), (dv, "dv")):
         _need(t, torch.bfloat16, n)
@@ -292,6 +337,8 @@ def cowa_decode_workspace_bytes(B, Tmax, Hq, Hkv, D, params):
 def cowa_decode(q, kcache, vcache, lens, o, lse, params, workspace):
     """q [B,Hq,D], caches [B,Hkv,Tmax,D] bf16 (strided views with that shape are accepted, e.g. a
     [B,Tmax,Hkv,D] cache transposed), lens int32 [B] (device) -> o [B,Hq,D], lse [B,Hq] or None."""
+    if _done(_call().decode(q, kcache, vcache, lens, o, lse, params, workspace), "cowa_decode"):
+        return
     import torch
     for t, n in ((q, "q"), (o, "o")):
         _need(t, torch.bfloat16, n)
@@ -318,6 +365,8 @@ def cowa_decode_multi_workspace_bytes(B, Nq, Tmax, Hq, Hkv, D, params):
 
 def cowa_decode_multi(q, kcache, vcache, lens, o, lse, params, workspace):
     """q, o [B,Nq,Hq,D]; kcache/vcache [B,Hkv,Tmax,D]; lens int32 [B] (device); lse [B,Nq,Hq] or None."""
+    if _done(_call().decode_multi(q, kcache, vcache, lens, o, lse, params, workspace), "cowa_decode_multi"):
+        return
     import torch
     for t, n in ((q, "q"), (kcache, "kcache"), (vcache, "vcache"), (o, "o")):
         _need(t, torch.bfloat16, n)
@@ -334,6 +383,8 @@ def cowa_decode_multi(q, kcache, vcache, lens, o, lse, params, workspace):
 
 def cowa_decode_paged(q, kpages, vpages, block_table, lens, o, lse, params, workspace):
     """q, o [B,Nq,Hq,D]; kpages/vpages [num_pages,Hkv,page_size,D]; block_table int32 [B,max_pages] (device)."""
+    if _done(_call().decode_paged(q, kpages, vpages, block_table, lens, o, lse, params, workspace), "cowa_decode_paged"):
+        return
     import torch
     for t, n in ((q, "q"), (kpages, "kpages"), (vpages, "vpages"), (o, "o")):
         _need(t, torch.bfloat16, n)

@@ -1,4 +1,4 @@
-"""Builds libcowa.so (all CUDA translation units, sm_100a) in-tree with nvcc."""
+"""Builds libcowa.so (all CUDA translation units, sm_100a) in-tree with nvcc, and the binding's argument path with g++."""
 from __future__ import annotations
 
 import os
@@ -11,6 +11,8 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 OBJ_DIR = os.path.join(HERE, "build")
 LIB_PATH = os.path.join(HERE, "libcowa.so")
+CALL_SRC = os.path.join(HERE, "csrc_py", "cowa_call.cpp")
+CALL_PATH = os.path.join(HERE, "_cowa_call.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -47,15 +49,40 @@ def _compile(src, verbose):
     return obj, True
 
 
+def _build_call_module(verbose):
+    """The binding's native argument path: a Python extension over torch's headers (no CUDA code)."""
+    if os.path.exists(CALL_PATH) and os.path.getmtime(CALL_PATH) >= max(os.path.getmtime(CALL_SRC), _headers_mtime()):
+        return
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) or "/usr/local/cuda"
+    inc = [INCLUDE, os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    cmd += [f"-I{d}" for d in inc] + [CALL_SRC, "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu",
+                                      "-ltorch_python", "-o", CALL_PATH]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or r.returncode != 0:
+        sys.stderr.write(r.stdout + r.stderr)
+    if r.returncode != 0:
+        raise RuntimeError("g++ failed on cowa_call.cpp")
+
+
 def build_library(verbose=False, force=False):
-    """Compiles every .cu under csrc/ and links libcowa.so.  Returns its path."""
+    """Compiles every .cu under csrc/ and links libcowa.so, beside it _cowa_call.so.  Returns libcowa.so's path."""
     os.makedirs(OBJ_DIR, exist_ok=True)
     if force:
         for f in os.listdir(OBJ_DIR):
             if f.endswith(".o"):
                 os.remove(os.path.join(OBJ_DIR, f))
+        if os.path.exists(CALL_PATH):
+            os.remove(CALL_PATH)
     with ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 1)) as ex:
+        call = ex.submit(_build_call_module, verbose)
         res = list(ex.map(lambda s: _compile(s, verbose), _sources()))
+        call.result()
     objs = [o for o, _ in res]
     rebuilt = any(ch for _, ch in res)
     if rebuilt or not os.path.exists(LIB_PATH):
