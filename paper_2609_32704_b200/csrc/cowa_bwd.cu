@@ -167,6 +167,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   constexpr uint32_t ID_ACC = idesc_bf16(128, D, 0, 1);    // dV, dK (B = dO / Q, MN-major)
   constexpr uint32_t ID_DQ = idesc_bf16(128, BQT, 1, 1);   // dQ^T (A = K^T, B = dS^T, both MN-major)
 
+  grid_enter();
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* sK = smem + SM::oK;
   uint8_t* sV = smem + SM::oV;
@@ -782,6 +783,7 @@ __global__ void cowa_bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, 
                                            const float* __restrict__ lse, float* __restrict__ lse2,
                                            float* __restrict__ delta, float* __restrict__ acc, int T, int Tpad,
                                            long long BH, int H, CowaStrides so) {
+  grid_enter();
   constexpr int TPR = D / 8;  // threads per row (16 bytes each)
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long row = gid / TPR;
@@ -820,6 +822,7 @@ __global__ void cowa_bwd_preprocess_varlen_kernel(const __nv_bfloat16* __restric
                                                   float* __restrict__ delta, float* __restrict__ acc,
                                                   const int* __restrict__ cu, int B, int total, int Tpad,
                                                   unsigned int* status) {
+  grid_enter();
   constexpr int TPR = D / 8;  // threads per row (16 bytes each)
   const int chunk = blockIdx.x, h = blockIdx.y;
   const int r = threadIdx.x / TPR, part = threadIdx.x % TPR;
@@ -861,6 +864,7 @@ template <int D, bool VARLEN>
 __global__ void __launch_bounds__(256)
 cowa_bwd_convert_dq_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, const int* __restrict__ cu, int B,
                            int T, int Tpad, int H, int fixed, CowaStrides sq, unsigned int* status) {
+  grid_enter();
   const int nchunk = Tpad / BQS, chunk = VARLEN ? blockIdx.x : blockIdx.x % nchunk, bh = VARLEN ? blockIdx.y : blockIdx.x / nchunk;
   int rows, first;  // rows of this chunk, and the first one's place among the rows of dq
   __nv_bfloat16* out;
@@ -901,6 +905,7 @@ cowa_bwd_convert_dq_kernel(const float* __restrict__ acc, __nv_bfloat16* __restr
 template <int D, bool VARLEN>
 __global__ void __launch_bounds__(256)
 cowa_bwd_reduce_dkv_kernel(const __grid_constant__ BwdArgs a, CowaStrides sk, CowaStrides sv) {
+  grid_enter();
   constexpr int TPR = D / 8, ROWS = 256 / TPR;  // threads per row (16 bytes of bf16 each), rows per block
   const int part = threadIdx.x % TPR;
   int q = blockIdx.x / (BKV / ROWS), c = 0, slot = 0;
@@ -1049,12 +1054,12 @@ CowaStrides packed_strides(int H, long long T, int D) {
 }
 
 template <int D, bool VARLEN>
-void launch_reduce(const BwdArgs& a, const BwdPlan& pl, const CowaStrides& sk, const CowaStrides& sv, cudaStream_t st) {
+cudaError_t launch_reduce(const BwdArgs& a, const BwdPlan& pl, const CowaStrides& sk, const CowaStrides& sv, cudaStream_t st) {
   long long shared = 0;
   for (int c = 0; c < 3; ++c)
     if (pl.parts[c] > 1) shared += pl.tiles[c];
-  if (shared > 0)
-    cowa_bwd_reduce_dkv_kernel<D, VARLEN><<<dim3((unsigned)(shared * (BKV * (D / 8) / 256)), 2), 256, 0, st>>>(a, sk, sv);
+  if (shared == 0) return cudaSuccess;
+  return cowa::launch_chained(cowa_bwd_reduce_dkv_kernel<D, VARLEN>, dim3((unsigned)(shared * (BKV * (D / 8) / 256)), 2), 256, 0, st, a, sk, sv);
 }
 
 template <int D>
@@ -1102,20 +1107,16 @@ int launch_bwd(const void* q, const void* k, const void* v, const void* o, const
                                      BwdSmem<D>::kBytes));
   {
     const long long threads = BH * Tpad * (D / 8);
-    cowa_bwd_preprocess_kernel<D><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(
-        static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse, lse2, delta, dq_acc,
-        T, Tpad, BH, Hq, so);
-    COWA_CUDA_TRY(cudaGetLastError());
+    COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_preprocess_kernel<D>, dim3((unsigned)((threads + 255) / 256)), 256, 0, st,
+                                       static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse,
+                                       lse2, delta, dq_acc, T, Tpad, BH, Hq, so));
   }
   if (p->bwd_main_start_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_start_event), st));
-  cowa_bwd_kernel<D, false><<<(unsigned)pl.blocks(), 512, BwdSmem<D>::kBytes, st>>>(mq, mk, mv, mdo, mdk, mdv, a);
-  COWA_CUDA_TRY(cudaGetLastError());
+  COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_kernel<D, false>, dim3((unsigned)pl.blocks()), 512, BwdSmem<D>::kBytes, st, mq, mk, mv, mdo, mdk, mdv, a));
   if (p->bwd_main_stop_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_stop_event), st));
-  launch_reduce<D, false>(a, pl, sk, sv, st);
-  COWA_CUDA_TRY(cudaGetLastError());
-  cowa_bwd_convert_dq_kernel<D, false><<<(unsigned)(Tpad / BQS * BH), 256, 0, st>>>(
-      dq_acc, static_cast<__nv_bfloat16*>(dq), nullptr, B, T, Tpad, Hq, a.dq_fixed, sq, a.status);
-  COWA_CUDA_TRY(cudaGetLastError());
+  COWA_CUDA_TRY((launch_reduce<D, false>(a, pl, sk, sv, st)));
+  COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_convert_dq_kernel<D, false>, dim3((unsigned)(Tpad / BQS * BH)), 256, 0, st, dq_acc,
+                                     static_cast<__nv_bfloat16*>(dq), nullptr, B, T, Tpad, Hq, a.dq_fixed, sq, a.status));
   return COWA_OK;
 }
 
@@ -1165,19 +1166,15 @@ int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o
   COWA_CUDA_TRY(cudaFuncSetAttribute(cowa_bwd_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      BwdSmem<D>::kBytes));
   const dim3 chunks(Tpad / BQS, Hq);
-  cowa_bwd_preprocess_varlen_kernel<D><<<chunks, BQS * (D / 8), 0, st>>>(
-      static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse, lse2, delta, dq_acc,
-      cu, B, total, Tpad, a.status);
-  COWA_CUDA_TRY(cudaGetLastError());
+  COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_preprocess_varlen_kernel<D>, chunks, BQS * (D / 8), 0, st,
+                                     static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse, lse2,
+                                     delta, dq_acc, cu, B, total, Tpad, a.status));
   if (p->bwd_main_start_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_start_event), st));
-  cowa_bwd_kernel<D, true><<<(unsigned)pl.blocks(), 512, BwdSmem<D>::kBytes, st>>>(mq, mk, mv, mdo, mdk, mdv, a);
-  COWA_CUDA_TRY(cudaGetLastError());
+  COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_kernel<D, true>, dim3((unsigned)pl.blocks()), 512, BwdSmem<D>::kBytes, st, mq, mk, mv, mdo, mdk, mdv, a));
   if (p->bwd_main_stop_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_stop_event), st));
-  launch_reduce<D, true>(a, pl, sk, sk, st);
-  COWA_CUDA_TRY(cudaGetLastError());
-  cowa_bwd_convert_dq_kernel<D, true><<<chunks, 256, 0, st>>>(dq_acc, static_cast<__nv_bfloat16*>(dq), cu, B, total, Tpad, Hq,
-                                                              a.dq_fixed, sq, a.status);
-  COWA_CUDA_TRY(cudaGetLastError());
+  COWA_CUDA_TRY((launch_reduce<D, true>(a, pl, sk, sk, st)));
+  COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_convert_dq_kernel<D, true>, chunks, 256, 0, st, dq_acc, static_cast<__nv_bfloat16*>(dq), cu,
+                                     B, total, Tpad, Hq, a.dq_fixed, sq, a.status));
   return COWA_OK;
 }
 

@@ -49,6 +49,19 @@ bool any_stride_set(const cowa_params_t* p);
 int decode_validate(const void* q, const void* kc, const void* vc, const int32_t* lens, const void* o, int B, int Tmax,
                     int Hq, int Hkv, int D, const cowa_params_t* p);
 
+// Launches a kernel that starts with grid_wait or grid_enter: its launch overlaps the end of the kernel before it in the
+// stream, whichever that is (1 to 2 us a kernel; forward and backward at 1K are five).
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace cowa

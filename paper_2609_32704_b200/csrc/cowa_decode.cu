@@ -19,6 +19,7 @@
 #include <cuda_bf16.h>
 
 #include "cowa_common.h"
+#include "cowa_ptx.cuh"
 
 namespace {
 
@@ -99,9 +100,7 @@ __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const De
   __shared__ __align__(16) float sc[G * kScStride];  // scores, later the value-phase reduction buffer
   __shared__ float m_s[G], l_s[G];
 
-  // The merge kernel is launched with programmatic stream serialisation: once every block of this grid has
-  // started, its blocks may be scheduled and wait (griddepcontrol.wait) for this grid's results.
-  asm volatile("griddepcontrol.launch_dependents;");
+  cowa_ptx::grid_enter();  // the merge kernel's blocks may be scheduled beside this one's; they wait for its results
   const int split = blockIdx.x, hk = blockIdx.y;
   const int b = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -284,7 +283,7 @@ __global__ void __launch_bounds__(128) cowa_decode_combine_kernel(const float* _
   __shared__ float part[4][D];
   const size_t bh = blockIdx.x;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // the split kernel's states are complete and visible
+  cowa_ptx::grid_enter();  // the split kernel's states are complete and visible
   const float* m = ws_m + bh * S;
   const float* l = ws_l + bh * S;
   const float* po = ws_o + bh * S * D + lane * V;
@@ -409,24 +408,16 @@ int pick_splits(int B, int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p)
   return splits_for(max_visible(Tmax, hg, p), B * Hkv, resident_blocks(D, Hq / Hkv));
 }
 
-// Launch of the merge kernel right behind the split kernel, allowed to start before that one has drained.
 template <int D>
 cudaError_t launch_combine(unsigned rows, const float* ws_o, const float* ws_m, const float* ws_l, __nv_bfloat16* o,
                            float* lse, int S, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(rows); cfg.blockDim = dim3(128); cfg.dynamicSmemBytes = 0; cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, cowa_decode_combine_kernel<D>, ws_o, ws_m, ws_l, o, lse, S);
+  return cowa::launch_chained(cowa_decode_combine_kernel<D>, dim3(rows), 128, 0, st, ws_o, ws_m, ws_l, o, lse, S);
 }
 
 template <int D, int G>
 cudaError_t launch_split(const DecodeArgs& a, cudaStream_t st) {
   dim3 grid(a.S, a.Hkv, a.B);
-  cowa_decode_split_kernel<D, G><<<grid, kThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  return cowa::launch_chained(cowa_decode_split_kernel<D, G>, grid, kThreads, 0, st, a);
 }
 
 template <int D>

@@ -179,8 +179,7 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bar_k_full + 6 * NS);
   int* scan = reinterpret_cast<int*>(smem + SM::oScan);  // 6 warp totals; [8], [9] first unit and its list position; [10 ..] per slot: step whose V is not finite
 
-  // the merge kernel may start as soon as every block of this grid has (it waits for this grid's results itself)
-  asm volatile("griddepcontrol.launch_dependents;");
+  grid_enter();  // the merge kernel's blocks may be scheduled beside this one's; they wait for its results
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform by construction
   const int nw = (a.rows + 31) >> 5;                       // softmax warps with rows
@@ -639,7 +638,7 @@ __global__ void __launch_bounds__(WPR == 1 ? 128 : WPR * 32) cowa_decode_tile_me
   const int u = (b * a.Hkv + h / a.G) * a.ntiles + tile;
   Unit x;
   unit_of(a, u, x);
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // the row states are complete and visible
+  grid_enter();  // the row states are complete and visible
   const int2 info = x.nt > 0 ? a.ws_unit[u] : make_int2(0, 0);  // no visible key: 0 / 0
   const size_t first = (size_t)(info.x + u) * a.rows + row;  // piece i lies a.rows rows further
   const int S = info.y;
@@ -758,19 +757,13 @@ int launch_tile(const void* q, const void* kc, const void* vc, void* o, float* l
   const auto kernel = few ? cowa_decode_tile_kernel<D, 32, 3> : cowa_decode_tile_kernel<D, 128, 2>;
   const int smem = few ? TileSmem<D, 32, 3>::kBytes : TileSmem<D, 128, 2>::kBytes;
   COWA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  kernel<<<t.blocks, kThreads, smem, st>>>(mq, mk, mv, a);
-  COWA_CUDA_TRY(cudaGetLastError());
-  cudaLaunchConfig_t cfg = {};
+  COWA_CUDA_TRY(cowa::launch_chained(kernel, dim3((unsigned)t.blocks), kThreads, smem, st, mq, mk, mv, a));
   // one warp per row while a unit has a few pieces on average, eight warps when it has many (one long sequence)
   const bool many = t.blocks > 16 * t.units;
   const int nrows = a.B * a.Nq * a.Hq;
-  cfg.gridDim = dim3((unsigned)(many ? nrows : (nrows + 3) / 4)); cfg.blockDim = dim3(many ? 256 : 128); cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
   const auto merge = many ? cowa_decode_tile_merge_kernel<D, 8> : cowa_decode_tile_merge_kernel<D, 1>;
-  COWA_CUDA_TRY(cudaLaunchKernelEx(&cfg, merge, (const TileArgs)a, static_cast<__nv_bfloat16*>(o), lse));
+  COWA_CUDA_TRY(cowa::launch_chained(merge, dim3((unsigned)(many ? nrows : (nrows + 3) / 4)), many ? 256 : 128, 0, st, a,
+                                     static_cast<__nv_bfloat16*>(o), lse));
   return COWA_OK;
 }
 

@@ -52,6 +52,7 @@ cowa_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   constexpr uint32_t IDESC_S = idesc_bf16(128, BK, 0, 0);
   constexpr uint32_t IDESC_O = idesc_bf16(128, D, 0, 1);
 
+  grid_enter();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sQ = smem + SM::oQ;
@@ -478,8 +479,7 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
                                      FwdSmem<D>::kBytes));
   const long long nblocks = tiles * Hq;
   if (nblocks > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
-  cowa_fwd_kernel<D, VARLEN><<<(unsigned)nblocks, kFwdThreads, FwdSmem<D>::kBytes, st>>>(mq, mk, mv, mo, a);
-  COWA_CUDA_TRY(cudaGetLastError());
+  COWA_CUDA_TRY(cowa::launch_chained(cowa_fwd_kernel<D, VARLEN>, dim3((unsigned)nblocks), kFwdThreads, FwdSmem<D>::kBytes, st, mq, mk, mv, mo, a));
   return COWA_OK;
 }
 

@@ -145,6 +145,8 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   constexpr uint32_t IDESC_S2 = idesc_bf16(128, BS, 0, 0), IDESC_S1 = idesc_bf16(128, BK, 0, 0);
   constexpr uint32_t IDESC_O = idesc_bf16(128, D, 0, 1);
 
+  if constexpr (SPLIT) grid_enter();
+  else grid_wait();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sQ = smem + SM::oQ;      // [2 heads][kQ]
@@ -733,10 +735,12 @@ int launch_fwd_pair(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensor
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(items * split));
   cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = PairSmem<D>::kBytes; cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = split > 1 ? 1 : 0;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)split; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = split > 1 ? 2 : 1;
   COWA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mo, a));
   return COWA_OK;
 }

@@ -96,6 +96,16 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
   return v;
 }
 
+// ------------------------------------------------------------------ kernels in a row (see cowa::launch_chained)
+// Top of a kernel, ahead of every access to global memory and of its TMEM allocation: the kernel before it in the stream is
+// complete and its results are visible.  The next kernel may have its blocks scheduled from here on (not earlier: it would
+// then run beside the kernel before this one).
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_enter() {
+  grid_wait();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ------------------------------------------------------------------ taking over blocks of the grid that have not started
 // Asks for the next block of this grid that has not started; the 16-byte answer comes through the mbarrier (expect_tx 16).
 __device__ __forceinline__ void clc_request(void* answer, uint64_t* bar) {
