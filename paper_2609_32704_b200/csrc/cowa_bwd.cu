@@ -176,11 +176,12 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   uint8_t* sDS = smem + SM::oDS;
   float* sVec = reinterpret_cast<float*>(smem + SM::oVec);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SM::oBar);
-  uint64_t* bar_kv = bars + 0;
+  uint64_t* bar_k = bars + 0;
+  uint64_t* bar_v = bars + 6;
   uint64_t* bar_q_full = bars + 1;    // [2] Q, LSE, Delta of a step have landed
   uint64_t* bar_q_empty = bars + 3;   // [2] ... are consumed
   uint64_t* bar_o_full = bars + 5;    // dO ...
-  uint64_t* bar_o_empty = bars + 6;
+  uint64_t* bar_o_empty = bars + 30;
   uint64_t* bar_s_full = bars + 7;    // S^T is in TMEM
   uint64_t* bar_s_read = bars + 8;    // count 256: S^T is in registers
   uint64_t* bar_p_ready = bars + 9;   // count 256: P^T written over the first half of S^T
@@ -242,7 +243,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   if (tid == 0) {
     geo[0] = w.s; geo[1] = w.n; geo[2] = w.g; geo[3] = w.l; geo[4] = off; geo[5] = Nq; geo[6] = Nk; geo[7] = steps;
     *part_out = parts > 1 ? a.dkv_part + (size_t)slot * 2 * (BKV * D) : nullptr;
-    mbar_init(bar_kv, 1);
+    mbar_init(bar_k, 1); mbar_init(bar_v, 1);
     for (int s = 0; s < 2; ++s) {
       mbar_init(bar_q_full + s, 1); mbar_init(bar_q_empty + s, 1);
       mbar_init(bar_dq_free + s, 128);
@@ -266,21 +267,21 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   bool ok = true;
   auto step_count = [&]() { return static_cast<const volatile int*>(geo)[7]; };  // (each role reads it for itself)
 
-  // dK (first compute warpgroup) and dV (drain warpgroup): TMEM -> bf16 -> shared -> TMA store.  Called from
-  // inside the role branches so that it is compiled under that role's register budget.
+  // dK (first compute warpgroup) and dV (second, while the last dQ^T and dK are still being computed): TMEM -> bf16 ->
+  // shared -> TMA store.  With dV behind the last dQ^T in the drain warpgroup a block of nine steps took 2000 clocks longer.
   auto store_grad = [&](bool is_dk) {
     const int N = step_count(), r = (warp & 3) * 32 + lane;
     const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-    if (N > 0) ok = mbar_wait(bar_done, 0, a.status) && ok;
+    if (N > 0) ok = (is_dk ? mbar_wait(bar_done, 0, a.status) : mbar_wait(bar_o_empty, (N - 1) & 1, a.status)) && ok;
     tc_fence_after();
-    uint8_t* sOut = sQ + (is_dk ? 0 : SM::kKV);
+    uint8_t* sOut = is_dk ? sQ : sDO;  // free by then, like V for partial sums
     const float mul = is_dk ? a.scale : 1.f;
     if (float* const dst = *part_out) {
       // A shared tile: this block's part goes out in fp32, one slot per block; a kernel of its own adds the slots in order.
-      // Staged where K, V or the Q / dO stages were, rows with their 16-byte chunks permuted (bank conflicts), and
+      // Staged where Q, or V and dO were, rows with their 16-byte chunks permuted (bank conflicts), and
       // copied as one range: straight from registers a warp's store touches 32 rows (1019 against 983 thousand clocks of
       // the whole kernel for one KV head of 20001 tokens).
-      uint8_t* sPart = (is_dk ? sK : sQ) + r * (D * 4);
+      uint8_t* sPart = (is_dk ? sQ : r < BKV / 2 ? sV : sDO - SM::kQ) + r * (D * 4);
 #pragma unroll
       for (int c = 0; c < D / 32; ++c) {
         uint32_t ov[32];
@@ -300,9 +301,10 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       fence_proxy_async_smem();
       wg_sync(is_dk ? 1 : 2);
       if (r == 0) {
-        bulk_store(dst + (is_dk ? 0 : BKV * D), is_dk ? sK : sQ, BKV * D * 4);
+        for (int half = 0; half < 2; ++half)
+          bulk_store(dst + (is_dk ? 0 : BKV * D) + half * (BKV * D / 2), is_dk ? sQ + half * SM::kQ : half ? sDO : sV, BKV * D * 2);
         tma_commit_group();
-        tma_wait_group<0>();
+        tma_wait_group_read<0>();
       }
       return;
     }
@@ -360,7 +362,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     if (r == 0 && ok) {
       for (int s = 0; s < NSLAB; ++s) tma_store_4d(is_dk ? &tmdK : &tmdV, sOut + s * SLAB_KV, s * 64, rbase + k0, hk, bt);
       tma_commit_group();
-      tma_wait_group<0>();
+      tma_wait_group_read<0>();
     }
   };
 
@@ -373,11 +375,11 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       // ================= TMA producer =================
       if (lane == 0 && N > 0) {
         prefetch_tmap(&tmQ); prefetch_tmap(&tmdO); prefetch_tmap(&tmK); prefetch_tmap(&tmV);
-        mbar_expect_tx(bar_kv, 2 * SM::kKV);
-        for (int s = 0; s < NSLAB; ++s) {
-          tma_load_4d(sK + s * SLAB_KV, &tmK, bar_kv, s * 64, rbase + k0, hk, bt);
-          tma_load_4d(sV + s * SLAB_KV, &tmV, bar_kv, s * 64, rbase + k0, hk, bt);
-        }
+        auto load_kv = [&](uint8_t* tile, const CUtensorMap* tm, uint64_t* bar) {
+          mbar_expect_tx(bar, SM::kKV);
+          for (int s = 0; s < NSLAB; ++s) tma_load_4d(tile + s * SLAB_KV, tm, bar, s * 64, rbase + k0, hk, bt);
+        };
+        load_kv(sK, &tmK, bar_k);  // S^T(0) waits for K and Q only
         int g = g0, t_in = tq0;   // head of the group, position in I_h(j): kept incrementally
         for (int n = 0; n < N && ok; ++n) {
           const int st = n & 1;
@@ -399,7 +401,8 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             tma_load_4d(sQ + st * SM::kQ + s * SLAB_Q, &tmQ, bar_q_full + st, s * 64, rbase + q0, hq0 + g, bt);
           bulk_load_1d(sVec + st * 256, a.lse2 + (size_t)bhq * vec_stride + pbase + q0, vb, bar_q_full + st);
           bulk_load_1d(sVec + st * 256 + 128, a.delta + (size_t)bhq * vec_stride + pbase + q0, vb, bar_q_full + st);
-          if (n >= 1) ok = mbar_wait(bar_o_empty, (n - 1) & 1, a.status);
+          if (n == 0) load_kv(sV, &tmV, bar_v);
+          else ok = mbar_wait(bar_o_empty, (n - 1) & 1, a.status);
           if (!ok) break;
           load_do();
           if (++t_in == cnt) { t_in = 0; ++g; }
@@ -471,13 +474,14 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             }
           }
         };
-        ok = mbar_wait(bar_kv, 0, a.status);
-        if (ok && tail_kv) {
-          clear_rows(sK, Nk - k0, BKV, SLAB_KV);
-          clear_rows(sV, Nk - k0, BKV, SLAB_KV);
+        auto clear_kv_tail = [&](uint8_t* tile) {
+          if (!tail_kv) return;
+          clear_rows(tile, Nk - k0, BKV, SLAB_KV);
           fence_proxy_async_smem();
           __syncwarp();
-        }
+        };
+        ok = mbar_wait(bar_k, 0, a.status);
+        if (ok) clear_kv_tail(sK);
         ok = ok && mbar_wait(bar_q_full, 0, a.status);
         if (ok) {
           clear_tail(sQ, 0);
@@ -503,6 +507,11 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           ok = mbar_wait(bar_o_full, par, a.status);
           if (ok && n > 0) ok = mbar_wait(bar_dq_free, par ^ 1, a.status);
           if (!ok) return;
+          if (n == 0) {
+            ok = mbar_wait(bar_v, 0, a.status);
+            if (!ok) return;
+            clear_kv_tail(sV);
+          }
           clear_tail(sDO, st);
           tc_fence_after();
           gemm_st(cDP, dV_k, dO_k0);
@@ -671,7 +680,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         fence_proxy_async_smem();
         mbar_arrive(bar_ds_ready);
       }
-      if (wg == 0) store_grad(true);
+      store_grad(wg == 0);
     }
   } else {
     {
@@ -763,8 +772,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         add_rows(v2, 0);
         add_rows(v0, 1);
       }
-      if (lane == 0) tma_wait_group<0>();
-      store_grad(false);
+      if (lane == 0) tma_wait_group_read<0>();
     }
   }
 
@@ -956,7 +964,8 @@ cowa_bwd_reduce_dkv_kernel(const __grid_constant__ BwdArgs a, CowaStrides sk, Co
 // 1021 / 983; 1K, 4 heads 58 / 34.
 struct BwdPlan {
   int sink_tiles;  // per sequence and head
-  int tiles[3], parts[3];
+  int tiles[3], parts[3];  // parts: what the workspace has room for
+  int run[3];              // what the blocks take
   long long slots() const {
     long long n = 0;
     for (int c = 0; c < 3; ++c)
@@ -965,8 +974,22 @@ struct BwdPlan {
   }
   long long blocks() const {
     long long n = 0;
-    for (int c = 0; c < 3; ++c) n += (long long)tiles[c] * parts[c];
+    for (int c = 0; c < 3; ++c) n += (long long)tiles[c] * run[c];
     return n;
+  }
+  // How many of the parts of body tiles are worth a block: a block costs about four steps (128 queries each) besides its own
+  // and 0.02 for its partial sums, and half a block is lost at the end.  Forward and backward, us, all parts / these: 821
+  // tokens x 4 (2 KV heads) 113 / 107, 2048 tokens 103 / 99, 6000 tokens 165 / 145, 20001 tokens 785 / 766; 1024 tokens, less
+  // than a block per SM, 31 with four parts and 36 with two.
+  void choose_run(double steps) {
+    for (int c = 0; c < 3; ++c) run[c] = parts[c];
+    const int sms = cowa::sm_count();
+    double best = 0;
+    for (int p = 1; p <= parts[1]; ++p) {
+      const long long n = (long long)tiles[0] * parts[0] + (long long)tiles[1] * p + (long long)tiles[2] * parts[2];
+      const double t = (4 + steps / p) * (std::max((double)n / sms, 1.0) + 0.5) + (p > 1 ? 0.02 * tiles[1] * p : 0);
+      if (p == 1 || t < best) { best = t; run[1] = p; }
+    }
   }
 };
 
@@ -1014,6 +1037,7 @@ BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& h
   const long long room = heads > 1 ? ntiles * heads : 0;
   const long long budget = heads >= 4 ? room : std::max<long long>(room, 4ll * sms);
   while (pl.slots() > budget) --*std::max_element(pl.parts, pl.parts + 3);
+  pl.choose_run(rest > 0 ? (double)(total - sinks) / rest * BQS / BQT : 0.0);
   return pl;
 }
 
@@ -1036,6 +1060,7 @@ BwdPlan bwd_plan_varlen(int B, int total, int Hkv, int G, const cowa_params_t* p
   // the last wave is not shared here: short sequences make its tiles short already (1628 against 1624 in 1000 clocks)
   const double avg = 0.7 * keys / BQS * G, real = (double)total / BKV * Hkv;
   plan_rest(pl, rest, rest <= 2 * sms ? avg : 0.0, real * avg / sms);
+  pl.choose_run(avg * BQS / BQT);
   return pl;
 }
 
@@ -1057,7 +1082,7 @@ template <int D, bool VARLEN>
 cudaError_t launch_reduce(const BwdArgs& a, const BwdPlan& pl, const CowaStrides& sk, const CowaStrides& sv, cudaStream_t st) {
   long long shared = 0;
   for (int c = 0; c < 3; ++c)
-    if (pl.parts[c] > 1) shared += pl.tiles[c];
+    if (pl.run[c] > 1) shared += pl.tiles[c];
   if (shared == 0) return cudaSuccess;
   return cowa::launch_chained(cowa_bwd_reduce_dkv_kernel<D, VARLEN>, dim3((unsigned)(shared * (BKV * (D / 8) / 256)), 2), 256, 0, st, a, sk, sv);
 }
@@ -1097,7 +1122,7 @@ int launch_bwd(const void* q, const void* k, const void* v, const void* o, const
   a.scale_log2 = p->softmax_scale * 1.4426950408889634f;
   a.wins = hw;
   a.sink_tiles = pl.sink_tiles;
-  for (int c = 0; c < 3; ++c) { a.cls_tiles[c] = pl.tiles[c]; a.cls_parts[c] = pl.parts[c]; }
+  for (int c = 0; c < 3; ++c) { a.cls_tiles[c] = pl.tiles[c]; a.cls_parts[c] = pl.run[c]; }
   a.dq_fixed = p->deterministic ? 1 : 0;
   a.dkv_part = dkv_part;
   a.cu = nullptr; a.dk = static_cast<__nv_bfloat16*>(dk); a.dv = static_cast<__nv_bfloat16*>(dv); a.total = 0; a.tiles_bound = 0;
@@ -1154,7 +1179,7 @@ int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o
   a.scale_log2 = p->softmax_scale * 1.4426950408889634f;
   a.wins = hw;
   a.sink_tiles = pl.sink_tiles;
-  for (int c = 0; c < 3; ++c) { a.cls_tiles[c] = pl.tiles[c]; a.cls_parts[c] = pl.parts[c]; }
+  for (int c = 0; c < 3; ++c) { a.cls_tiles[c] = pl.tiles[c]; a.cls_parts[c] = pl.run[c]; }
   a.dq_fixed = p->deterministic ? 1 : 0;
   a.dkv_part = delta + (size_t)Hq * Tpad;
   a.cu = cu; a.dk = static_cast<__nv_bfloat16*>(dk); a.dv = static_cast<__nv_bfloat16*>(dv);

@@ -397,7 +397,7 @@ cowa_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     if (tid == 0 && ok && nt > 0 && !tail_rows) {
       for (int s = 0; s < NSLAB; ++s) tma_store_4d(&tmO, sQ + s * SLAB_Q, s * 64, qbase + q0, h, bt);
       tma_commit_group();
-      tma_wait_group<0>();
+      tma_wait_group_read<0>();
     }
   }
 

@@ -609,7 +609,7 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         }
       }
     }
-    if (r == 0 && stored) tma_wait_group<0>();
+    if (r == 0 && stored) tma_wait_group_read<0>();
   }
 
   if constexpr (SPLIT) {
