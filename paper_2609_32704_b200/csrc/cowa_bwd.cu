@@ -413,7 +413,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       // The whole warp runs this loop (uniform control flow, so that descriptors and counters stay in
       // uniform registers); only the elected lane executes the tcgen05 instructions.  Everything that
       // can be computed once is: descriptor of every operand base, stage and parity bookkeeping is
-      // incremental, and the loop body is instantiated for both TMEM buffers.
+      // incremental.
       if (N > 0) {
         const bool lead = elect_one();
         const uint32_t tb = tmem_base;
@@ -489,8 +489,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           gemm_st(cS, dK_k, dQ_k0);
           commit(bar_s_full);
         }
-        auto body = [&](int n, auto B_) {
-          constexpr int st = decltype(B_)::value;
+        auto body = [&](int n, int st) {
           const uint32_t par = n & 1;
           if (n > 0) {
             ok = mbar_wait(bar_ds_ready, par ^ 1, a.status);
@@ -531,10 +530,8 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             commit(bar_s_full);
           }
         };
-        for (int n = 0; n < N && ok; n += 2) {
-          body(n, std::integral_constant<int, 0>{});
-          if (n + 1 < N && ok) body(n + 1, std::integral_constant<int, 1>{});
-        }
+#pragma unroll 1
+        for (int n = 0; n < N && ok; ++n) body(n, n & 1);
         if (ok) {
           ok = mbar_wait(bar_ds_ready, (N - 1) & 1, a.status);
           if (ok && N > 1) ok = mbar_wait(bar_dq_free + 1, N & 1, a.status);
@@ -696,9 +693,9 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // 32 query rows of this warp's 32 d: staged in one of two tiles and added to the accumulator as one range
         const long long at_ = dq_at[n & 3];
         float* gdst = a.dq_acc + (at_ & ~1ll) + (warp & 3) * (BQS * 32);
-        auto add_rows = [&](const uint32_t (&v)[32], int quarter) {
-          if (!mine || (quarter >= 2 && (at_ & 1))) return;
-          float* stage = sDQ + (quarter & 1) * 1024;
+        auto add_rows = [&](const uint32_t (&v)[32], int half, int odd) {
+          if (!mine || (half && (at_ & 1))) return;
+          float* stage = sDQ + odd * 1024;
           if (lane == 0) tma_wait_group_read<1>();  // the reduction issued from this tile before has read it
           __syncwarp();
           if (a.dq_fixed) {
@@ -749,28 +746,25 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
-            float* dst = gdst + (quarter >> 1) * (BQS * D) + (quarter & 1) * 1024;
+            float* dst = gdst + half * (BQS * D) + odd * 1024;
             if (a.dq_fixed) bulk_reduce_add_s32(dst, stage, 4096);
             else bulk_reduce_add_f32(dst, stage, 4096);
             tma_commit_group();
           }
         };
-        // first the columns that dP^T waits for, then those of S^T, as registers allow
-        uint32_t v0[32], v1[32], v2[32];
-        tmem_ld32(t_lane + cDQ + 64, v0);
-        tmem_ld32(t_lane + cDQ + 96, v1);
-        tmem_wait_ld();
-        tc_fence_before();
-        mbar_arrive(bar_dq_free);
-        add_rows(v0, 2);
-        tmem_ld32(t_lane + cDQ, v2);
-        tmem_ld32(t_lane + cDQ + 32, v0);
-        tmem_wait_ld();
-        tc_fence_before();
-        mbar_arrive(bar_dq_free + 1);
-        add_rows(v1, 3);
-        add_rows(v2, 0);
-        add_rows(v0, 1);
+        // First the columns that dP^T waits for, then those of S^T.  One loop body, like the MMA warp's: the roles' loops
+        // together outgrow the instruction cache (two and four copies: 32K 7660 us forward and backward, this 7410).
+#pragma unroll 1
+        for (int half = 1; half >= 0; --half) {
+          uint32_t v0[32], v1[32];
+          tmem_ld32(t_lane + cDQ + half * 64, v0);
+          tmem_ld32(t_lane + cDQ + half * 64 + 32, v1);
+          tmem_wait_ld();
+          tc_fence_before();
+          mbar_arrive(bar_dq_free + (half ^ 1));
+          add_rows(v0, half, 0);
+          add_rows(v1, half, 1);
+        }
       }
       if (lane == 0) tma_wait_group_read<0>();
     }
