@@ -5,8 +5,10 @@
 //                   padded to a multiple of 64 rows (padding: -inf, so that P = 0 there);
 //                   its threads also zero the fp32 dQ accumulator.
 //   2. main kernel  one thread block per (batch, KV head, 128-row KV tile), KV-stationary as in
-//                   Algorithm 2, looping over the G QO heads of the group and over the 128-row QO
-//                   tiles of I_h(j) (analytic scheduler, ascending).  Per step five tcgen05 MMAs:
+//                   Algorithm 2, looping over the G QO heads of the group and over the 64-row QO
+//                   tiles of I_h(j) (analytic scheduler, ascending).  A step takes two entries of that list, one
+//                   head's after the other's, not necessarily neighbours (with 128-row tiles instead up to a
+//                   tenth more rows were visited: windows of 300 and 466 keys).  Per step five tcgen05 MMAs:
 //                     S^T  = K Q^T            (TMEM, 128 kv x 128 q)
 //                     dP^T = V dO^T           (TMEM)
 //                     dV  += P^T dO           (P^T as the TMEM operand)
@@ -54,9 +56,10 @@ using namespace cowa_ptx;
 namespace {
 
 constexpr int BKV = 128;  // KV rows per block (MMA M)
-constexpr int BQT = 128;  // QO rows per step (MMA N of S^T / dP^T)
-constexpr int BQS = 64;   // unit of the padded row space (half a step) and of the plan's step counts
+constexpr int BQT = 128;  // QO rows per step (MMA N of S^T / dP^T): two tiles
+constexpr int BQS = 64;   // rows of a QO tile, unit of the padded row space and of the plan's step counts
 constexpr int NST = 2;    // Q stages (Q(n) is read again by dK(n) after S^T(n+1)); dO has one
+constexpr int kNoTile = 0x7FFFFF00;  // in place of a step's second tile: no query of it sees anything
 constexpr float kDqFixedOne = 262144.f;  // 2^18: one unit of dQ in the fixed-point accumulation mode
 
 struct BwdArgs {
@@ -90,7 +93,7 @@ struct BwdSmem {
   static constexpr int oVec = oDS + 2 * kDS;   // per stage: 128 floats lse2, 128 floats delta
   static constexpr int oDQ = oVec + NST * 1024;  // dQ staging: per drain warp two tiles of 32 query rows x 32 d, fp32
   static constexpr int oBar = oDQ + 8 * 4096;
-  static constexpr int kBytes = oBar + 256;    // 231680 B at D = 128 (limit 232448)
+  static constexpr int kBytes = oBar + 320;    // 231744 B at D = 128 (limit 232448)
 };
 
 __device__ __forceinline__ void bulk_load_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -155,6 +158,7 @@ __global__ void __launch_bounds__(512, 1)
 cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmdO,
                 const __grid_constant__ CUtensorMap tmdK, const __grid_constant__ CUtensorMap tmdV,
+                const __grid_constant__ CUtensorMap tmQ2, const __grid_constant__ CUtensorMap tmdO2,  // boxes of 128 rows
                 const __grid_constant__ BwdArgs a) {
   using SM = BwdSmem<D>;
   constexpr int NSLAB = D / 64;
@@ -181,7 +185,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   uint64_t* bar_q_full = bars + 1;    // [2] Q, LSE, Delta of a step have landed
   uint64_t* bar_q_empty = bars + 3;   // [2] ... are consumed
   uint64_t* bar_o_full = bars + 5;    // dO ...
-  uint64_t* bar_o_empty = bars + 30;
+  uint64_t* bar_o_empty = bars + 28;
   uint64_t* bar_s_full = bars + 7;    // S^T is in TMEM
   uint64_t* bar_s_read = bars + 8;    // count 256: S^T is in registers
   uint64_t* bar_p_ready = bars + 9;   // count 256: P^T written over the first half of S^T
@@ -193,9 +197,9 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 16);
   float** part_out = reinterpret_cast<float**>(bars + 17);  // this block's partial dK, dV (kept here, not in registers)
   // What the roles would otherwise each hold or compute (registers: nothing spills in the batched form)
-  int* step_info = reinterpret_cast<int*>(bars + 18);          // [2] by stage: first query of the step, bit 0: none of its pairs is masked
-  long long* dq_at = reinterpret_cast<long long*>(bars + 19);  // [4] by step: first element of its dQ rows, bit 0: no second half
-  int* geo = reinterpret_cast<int*>(bars + 23);                // window, off, Nq, Nk, steps of this block
+  int2* step_info = reinterpret_cast<int2*>(bars + 18);        // [2] by stage: first queries of the step's tiles; bit 0: no pair is masked, bit 1: rows past the sequence's end
+  longlong2* dq_at = reinterpret_cast<longlong2*>(bars + 20);  // [4] by step: first elements of its tiles' dQ rows, -1: no second tile
+  int* geo = reinterpret_cast<int*>(bars + 32);                // window, off, Nq, Nk, steps of this block
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform by construction (helps the compiler)
@@ -229,10 +233,11 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const int off = Nk - Nq;
   const int k0 = j * BKV, k1 = min(k0 + BKV, Nk) - 1;
   CowaRange rg[2];
-  cowa_bwd_ranges(w, k0, k1, off, Nq, BQT, rg);
-  const int cnt = cowa_range_len(rg[0]) + cowa_range_len(rg[1]);  // QO steps per head
+  cowa_bwd_ranges(w, k0, k1, off, Nq, BQS, rg);
+  const int cnt = cowa_range_len(rg[0]) + cowa_range_len(rg[1]);  // QO tiles per head
   const int n0 = cnt * a.G * part / parts;               // (the host checks that these products fit)
-  const int steps = cnt * a.G * (part + 1) / parts - n0; // this block's steps
+  const int tiles = cnt * a.G * (part + 1) / parts - n0; // this block's QO tiles
+  const int steps = (tiles + 1) >> 1;
   const int g0 = cnt > 0 ? n0 / cnt : 0, tq0 = n0 - g0 * cnt;  // head of the group and position in I_h(j) of the first
   const int bt = VARLEN ? 0 : b;                               // batch coordinate of the tensor maps
   const int hq0 = hk * a.G;                                    // first QO head of the group
@@ -384,28 +389,38 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         for (int n = 0; n < N && ok; ++n) {
           const int st = n & 1;
           const uint32_t ph_e = ((n >> 1) & 1) ^ 1;  // parity of the "stage empty" waits (the first two steps need none)
-          const int i = cowa_bwd_tile_at(rg, t_in);
-          const int bhq = bhq0 + g, q0 = i * BQT;
-          auto load_do = [&]() {
-            mbar_expect_tx(bar_o_full, SM::kQ);
-            for (int s = 0; s < NSLAB; ++s)
-              tma_load_4d(sDO + s * SLAB_Q, &tmdO, bar_o_full, s * 64, rbase + q0, hq0 + g, bt);
-          };
+          int q0[2], gh[2];
+          q0[0] = cowa_bwd_tile_at(rg, t_in) * BQS; gh[0] = g;
+          if (++t_in == cnt) { t_in = 0; ++g; }
+          const bool two = 2 * n + 1 < tiles;  // else the first tile again, every pair of it masked
+          q0[1] = two ? cowa_bwd_tile_at(rg, t_in) * BQS : q0[0]; gh[1] = two ? g : gh[0];
+          if (two && ++t_in == cnt) { t_in = 0; ++g; }
           if (n >= 2) ok = mbar_wait(bar_q_empty + st, ph_e, a.status);
           if (!ok) break;
-          const uint32_t vb = q0 + BQS < Nq ? BQT * 4 : BQS * 4;  // the row space is padded to 64 rows only
-          step_info[st] = q0 + (cowa_tile_full(w, q0, BQT, k0, BKV, off, Nq, Nk) ? 1 : 0);
-          dq_at[n & 3] = (long long)((size_t)bhq * vec_stride + pbase + q0) * D + (q0 + BQS < Nq ? 0 : 1);
-          mbar_expect_tx(bar_q_full + st, SM::kQ + 2 * vb);
-          for (int s = 0; s < NSLAB; ++s)
-            tma_load_4d(sQ + st * SM::kQ + s * SLAB_Q, &tmQ, bar_q_full + st, s * 64, rbase + q0, hq0 + g, bt);
-          bulk_load_1d(sVec + st * 256, a.lse2 + (size_t)bhq * vec_stride + pbase + q0, vb, bar_q_full + st);
-          bulk_load_1d(sVec + st * 256 + 128, a.delta + (size_t)bhq * vec_stride + pbase + q0, vb, bar_q_full + st);
+          auto info = [&](int x) {
+            return q0[x] + (cowa_tile_full(w, q0[x], BQS, k0, BKV, off, Nq, Nk) ? 1 : 0) + (q0[x] + BQS > Nq ? 2 : 0);
+          };
+          step_info[st] = make_int2(info(0), two ? info(1) : kNoTile);
+          auto rows = [&](int x) -> size_t { return (size_t)(bhq0 + gh[x]) * vec_stride + pbase + q0[x]; };  // in lse2, delta, dq_acc
+          dq_at[n & 3] = make_longlong2((long long)rows(0) * D, two ? (long long)rows(1) * D : -1ll);
+          // neighbours of one head, as nearly always, come in one piece
+          const int pieces = two && gh[1] == gh[0] && q0[1] == q0[0] + BQS ? 1 : 2;
+          auto load_rows = [&](uint8_t* tile, const CUtensorMap* tm, const CUtensorMap* tm2, uint64_t* bar) {
+            for (int x = 0; x < pieces; ++x)
+              for (int s = 0; s < NSLAB; ++s)
+                tma_load_4d(tile + s * SLAB_Q + x * (SLAB_Q / 2), pieces == 1 ? tm2 : tm, bar, s * 64, rbase + q0[x], hq0 + gh[x], bt);
+          };
+          mbar_expect_tx(bar_q_full + st, SM::kQ + 2 * BQT * 4);
+          load_rows(sQ + st * SM::kQ, &tmQ, &tmQ2, bar_q_full + st);
+          for (int x = 0; x < pieces; ++x) {
+            bulk_load_1d(sVec + st * 256 + x * BQS, a.lse2 + rows(x), BQT * 4 / pieces, bar_q_full + st);
+            bulk_load_1d(sVec + st * 256 + 128 + x * BQS, a.delta + rows(x), BQT * 4 / pieces, bar_q_full + st);
+          }
           if (n == 0) load_kv(sV, &tmV, bar_v);
           else ok = mbar_wait(bar_o_empty, (n - 1) & 1, a.status);
           if (!ok) break;
-          load_do();
-          if (++t_in == cnt) { t_in = 0; ++g; }
+          mbar_expect_tx(bar_o_full, SM::kQ);
+          load_rows(sDO, &tmdO, &tmdO2, bar_o_full);
         }
       }
     } else if (warp == 1) {
@@ -464,14 +479,18 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             for (int c_ = lane; c_ < nchunk; c_ += 32)
               *reinterpret_cast<uint4*>(tile + s_ * slab_bytes + first * 128 + c_ * 16) = make_uint4(0u, 0u, 0u, 0u);
         };
-        auto clear_tail = [&](uint8_t* tile, int stage) {  // Q or dO tile of the step whose Q is in this stage
+        auto clear_tail = [&](uint8_t* tile, int stage) {  // Q or dO of the step whose Q is in this stage
           if constexpr (VARLEN) {
-            const int q0_ = step_info[stage], nq = static_cast<const volatile int*>(geo)[5];
-            if (!(q0_ & 1) && q0_ + BQT > nq) {
-              clear_rows(tile, nq - q0_, BQT, SLAB_Q);
-              fence_proxy_async_smem();
-              __syncwarp();
+            const int2 q0_ = step_info[stage];
+            if (!((q0_.x | q0_.y) & 2)) return;
+            const int nq = static_cast<const volatile int*>(geo)[5];
+#pragma unroll 1
+            for (int x = 0; x < 2; ++x) {
+              const int q = x && q0_.y != kNoTile ? q0_.y : q0_.x;  // (without a second tile the first lies there again)
+              if (q & 2) clear_rows(tile + x * (SLAB_Q / 2), nq - (q & ~63), BQS, SLAB_Q);
             }
+            fence_proxy_async_smem();
+            __syncwarp();
           }
         };
         auto clear_kv_tail = [&](uint8_t* tile) {
@@ -581,13 +600,13 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         float2 rc[8];  // row constants, read ahead of the wait for the product: shared memory is busy with its operands
 #pragma unroll
         for (int j = 0; j < 8; ++j) rc[j] = nlse2[(j >> 2) * 32 + (j & 3) * 4];
-        const int info = step_info[st];
-        const bool full = info & 1;
+        const int2 info = step_info[st];
+        const bool full = info.x & info.y & 1;
         uint32_t mk[2], all[2] = {0xFFFFFFFFu, 0xFFFFFFFFu}, seen[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};
         if (!full) {
 #pragma unroll
           for (int cb = 0; cb < 2; ++cb) {
-            const int base = info + cb * 64 + wg * 32;
+            const int base = ((cb ? info.y : info.x) & ~63) + wg * 32;
             mk[cb] = interval_bits(near_lo, near_hi, base) | interval_bits(far_lo, far_hi, base);
             all[cb] = __ballot_sync(0xffffffffu, mk[cb] == 0xFFFFFFFFu);
             seen[cb] = __ballot_sync(0xffffffffu, mk[cb] != 0u);
@@ -649,8 +668,6 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           float dr[2][16];
 #pragma unroll
           for (int h = 0; h < 2; ++h) tmem_ld_frag(dpbuf + cb * 64 + ((uint32_t)(h * 16) << 16), dr[h]);
-          // rows past the padded row space: what lies in their Delta is anything
-          const bool none = cb == 1 && !full && info + BQS >= static_cast<const volatile int*>(geo)[5];
           tmem_wait_ld();
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
@@ -659,10 +676,6 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             for (int e = 0; e < 16; e += 2) {
               const float2 y = mul2(make_float2(p[cb][h][e], p[cb][h][e + 1]), add2(make_float2(dr[h][e], dr[h][e + 1]), rc[cb * 4 + e / 4]));
               dsp[e / 2] = pack_bf16(y.x, y.y);
-            }
-            if (none) {
-#pragma unroll
-              for (int e = 0; e < 8; ++e) dsp[e] = 0u;
             }
             tmem_st_frag(dpbuf + 64 + cb * 16 + ((uint32_t)(h * 16) << 16), dsp);
             // dS^T also to shared memory (a key's row = 128 B = 8 chunks, 128B swizzle) for the dQ^T product, whose last
@@ -691,10 +704,10 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         if (!ok) break;
         tc_fence_after();
         // 32 query rows of this warp's 32 d: staged in one of two tiles and added to the accumulator as one range
-        const long long at_ = dq_at[n & 3];
-        float* gdst = a.dq_acc + (at_ & ~1ll) + (warp & 3) * (BQS * 32);
+        const longlong2 at_ = dq_at[n & 3];
         auto add_rows = [&](const uint32_t (&v)[32], int half, int odd) {
-          if (!mine || (half && (at_ & 1))) return;
+          const long long at = half ? at_.y : at_.x;
+          if (!mine || at < 0) return;
           float* stage = sDQ + odd * 1024;
           if (lane == 0) tma_wait_group_read<1>();  // the reduction issued from this tile before has read it
           __syncwarp();
@@ -746,7 +759,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
-            float* dst = gdst + half * (BQS * D) + odd * 1024;
+            float* dst = a.dq_acc + at + (warp & 3) * (BQS * 32) + odd * 1024;
             if (a.dq_fixed) bulk_reduce_add_s32(dst, stage, 4096);
             else bulk_reduce_add_f32(dst, stage, 4096);
             tma_commit_group();
@@ -1114,9 +1127,11 @@ int launch_bwd(const void* q, const void* k, const void* v, const void* o, const
   if ((rc = cowa::resolve_strides(p->v_strides, Hkv, Nk, D, &sv))) return rc;
   if ((rc = cowa::resolve_strides(p->o_strides, Hq, Nq, D, &so))) return rc;
   if (BH > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
-  CUtensorMap mq, mk, mv, mdo, mdk, mdv;
-  if ((rc = cowa::make_tensor_map(&mq, q, cowa::MapType::BF16, D, T, Hq, B, sq, 64, BQT))) return rc;
-  if ((rc = cowa::make_tensor_map(&mdo, d_o, cowa::MapType::BF16, D, T, Hq, B, so, 64, BQT))) return rc;
+  CUtensorMap mq, mk, mv, mdo, mdk, mdv, mq2, mdo2;
+  if ((rc = cowa::make_tensor_map(&mq, q, cowa::MapType::BF16, D, T, Hq, B, sq, 64, BQS))) return rc;
+  if ((rc = cowa::make_tensor_map(&mq2, q, cowa::MapType::BF16, D, T, Hq, B, sq, 64, BQT))) return rc;
+  if ((rc = cowa::make_tensor_map(&mdo, d_o, cowa::MapType::BF16, D, T, Hq, B, so, 64, BQS))) return rc;
+  if ((rc = cowa::make_tensor_map(&mdo2, d_o, cowa::MapType::BF16, D, T, Hq, B, so, 64, BQT))) return rc;
   if ((rc = cowa::make_tensor_map(&mk, k, cowa::MapType::BF16, D, Nk, Hkv, B, sk, 64, BKV))) return rc;
   if ((rc = cowa::make_tensor_map(&mv, v, cowa::MapType::BF16, D, Nk, Hkv, B, sv, 64, BKV))) return rc;
   if ((rc = cowa::make_tensor_map(&mdk, dk, cowa::MapType::BF16, D, Nk, Hkv, B, sk, 64, BKV))) return rc;
@@ -1145,7 +1160,7 @@ int launch_bwd(const void* q, const void* k, const void* v, const void* o, const
                                        lse2, delta, dq_acc, T, Tpad, BH, Hq, so));
   }
   if (p->bwd_main_start_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_start_event), st));
-  COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_kernel<D, false>, dim3((unsigned)pl.blocks()), 512, BwdSmem<D>::kBytes, st, mq, mk, mv, mdo, mdk, mdv, a));
+  COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_kernel<D, false>, dim3((unsigned)pl.blocks()), 512, BwdSmem<D>::kBytes, st, mq, mk, mv, mdo, mdk, mdv, mq2, mdo2, a));
   if (p->bwd_main_stop_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_stop_event), st));
   COWA_CUDA_TRY((launch_reduce<D, false>(a, pl, sk, sv, st)));
   COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_convert_dq_kernel<D, false>, dim3((unsigned)(Tpad / BQS * BH)), 256, 0, st, dq_acc,
@@ -1169,11 +1184,13 @@ int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o
   float* lse2 = dq_acc + (size_t)Hq * Tpad * D;
   float* delta = lse2 + (size_t)Hq * Tpad;
   if (cowa::any_stride_set(p)) return COWA_ERR_UNSUPPORTED;  // packed tensors are contiguous [H, total, D]
-  CUtensorMap mq, mk, mv, mdo, mdk, mdv;
+  CUtensorMap mq, mk, mv, mdo, mdk, mdv, mq2, mdo2;
   int rc;
   const CowaStrides sq = packed_strides(Hq, total, D), sk = packed_strides(Hkv, total, D);
-  if ((rc = cowa::make_tensor_map(&mq, q, cowa::MapType::BF16, D, total, Hq, 1, sq, 64, BQT))) return rc;
-  if ((rc = cowa::make_tensor_map(&mdo, d_o, cowa::MapType::BF16, D, total, Hq, 1, sq, 64, BQT))) return rc;
+  if ((rc = cowa::make_tensor_map(&mq, q, cowa::MapType::BF16, D, total, Hq, 1, sq, 64, BQS))) return rc;
+  if ((rc = cowa::make_tensor_map(&mq2, q, cowa::MapType::BF16, D, total, Hq, 1, sq, 64, BQT))) return rc;
+  if ((rc = cowa::make_tensor_map(&mdo, d_o, cowa::MapType::BF16, D, total, Hq, 1, sq, 64, BQS))) return rc;
+  if ((rc = cowa::make_tensor_map(&mdo2, d_o, cowa::MapType::BF16, D, total, Hq, 1, sq, 64, BQT))) return rc;
   if ((rc = cowa::make_tensor_map(&mk, k, cowa::MapType::BF16, D, total, Hkv, 1, sk, 64, BKV))) return rc;
   if ((rc = cowa::make_tensor_map(&mv, v, cowa::MapType::BF16, D, total, Hkv, 1, sk, 64, BKV))) return rc;
   if ((rc = cowa::make_tensor_map(&mdk, dk, cowa::MapType::BF16, D, total, Hkv, 1, sk, 64, BKV))) return rc;
@@ -1203,7 +1220,7 @@ int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o
                                      static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse, lse2,
                                      delta, dq_acc, cu, B, total, Tpad, a.status));
   if (p->bwd_main_start_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_start_event), st));
-  COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_kernel<D, true>, dim3((unsigned)pl.blocks()), 512, BwdSmem<D>::kBytes, st, mq, mk, mv, mdo, mdk, mdv, a));
+  COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_kernel<D, true>, dim3((unsigned)pl.blocks()), 512, BwdSmem<D>::kBytes, st, mq, mk, mv, mdo, mdk, mdv, mq2, mdo2, a));
   if (p->bwd_main_stop_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_stop_event), st));
   COWA_CUDA_TRY((launch_reduce<D, true>(a, pl, sk, sk, st)));
   COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_convert_dq_kernel<D, true>, chunks, 256, 0, st, dq_acc, static_cast<__nv_bfloat16*>(dq), cu,
