@@ -20,11 +20,11 @@
 //                   added to the fp32 accumulator with bulk add-reductions (Algorithm 2 line 15).
 //                   Warp roles: TMA producer / MMA issuer / two compute warpgroups (P, dS; each takes 64
 //                   of the 128 query columns of every step) / dQ drain warpgroup, connected by mbarriers.
-//                   What bounds it: shared memory.  Of a step's ~4150 clocks the products' operands take
+//                   What bounds it: shared memory.  Of a step's ~3920 clocks the products' operands take
 //                   2048 (128 bytes a clock), the Q and dO loads 512, dS^T 256, the dQ staging 1024 written
 //                   and read; the tensor pipe needs 2560, the exponentials 1024.  With steps of 64 queries
 //                   K and V were read twice as often (2816), and a row constant per column and thread came
-//                   out of shared memory as a broadcast (1024 more): 32K, 32 heads 4840 -> 4650 us.  The
+//                   out of shared memory as a broadcast (1024 more): 32K, 32 heads 7.83 -> 6.92 M cycles.  The
 //                   512 columns of TMEM hold S^T, dP^T, dK, dV; P^T and dS^T take the outer halves of S^T
 //                   and dP^T, dQ^T the 128 columns between them, so that the next S^T and dP^T only wait
 //                   until dQ^T is in registers.  Per step n the MMAs run in the order
