@@ -448,7 +448,9 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
     //   No more items than clusters of two that the device holds, and a list long enough to pay for the merge: the item is
     //     shared by a cluster of 2, 4 or 8 blocks, two steps each at least, as long as all clusters are resident.  Hq 32,
     //     Hkv 8, Nq 128: 1816 keys 37.9 / 25.6, 4941 keys 85 / 36 with clusters of four; of eight, two waves, 54.
-    //   Else the pair kernel's persistent blocks pay when their rounds come out even:
+    //   Else the pair kernel pays when its larger items still share out evenly (the figures are from a fixed share of the
+    //   items per block; now that blocks take items as they come free it has gained up to a fifth where the rule takes it,
+    //   and the lines have been left where they are):
     //     every tile's list is about as long (a chunk behind a cache of its own length or more) and not short: Hq 32,
     //     Nq 1024, 1129 keys 1.00, 1816 keys 1.09, 4941 keys 1.13 times the one-head kernel's rate;
     //     causal lists from nothing up: three items per SM, or half of that and lists of 1280 keys.  T 2048, Hq 16, local
