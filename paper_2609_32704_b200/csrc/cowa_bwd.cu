@@ -715,7 +715,8 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             // Rounded to integers on the FMA and integer pipes (the conversion instruction runs at the rate of the
             // exponentials and competes with them): below 2^22, x + 1.5 * 2^23 has rint(x) in its low mantissa bits.  Larger
             // ones go in two parts, x = 2^16 h + l with h = rint(x / 2^16), |l| <= 2^15, both exact; shifting the first
-            // sum by 16 drops its exponent.  Both give what __float2int_rn gives.
+            // sum by 16 drops its exponent.  Both give what __float2int_rn gives for the product x rounded to fp32 (in one
+            // FMA with the addition it would not be rounded, and an element's bits would depend on its neighbours' size).
             const float2 fx2 = make_float2(a.scale * kDqFixedOne, a.scale * kDqFixedOne);
             auto c2 = [](float c_) { return make_float2(c_, c_); };
             float worst = 0.f;
@@ -726,11 +727,10 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             if (__all_sync(0xffffffffu, worst < 4194303.f)) {
 #pragma unroll
               for (int c = 0; c < 32; c += 4) {
-                const float2 x = fma2(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), fx2, c2(12582912.f));
-                const float2 y = fma2(make_float2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), fx2, c2(12582912.f));
-                *reinterpret_cast<int4*>(stage + c * 32 + lane * 4) =
-                    make_int4(__float_as_int(x.x) - 0x4B400000, __float_as_int(x.y) - 0x4B400000,
-                              __float_as_int(y.x) - 0x4B400000, __float_as_int(y.y) - 0x4B400000);
+                const float2 x = mul2(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), fx2);
+                const float2 y = mul2(make_float2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), fx2);
+                auto low = [](float t) { return __float_as_int(__fadd_rn(t, 12582912.f)) - 0x4B400000; };  // (a packed addition is merged)
+                *reinterpret_cast<int4*>(stage + c * 32 + lane * 4) = make_int4(low(x.x), low(x.y), low(y.x), low(y.y));
               }
             } else {
 #pragma unroll
