@@ -1001,9 +1001,11 @@ struct BwdPlan {
   // How many of the parts of body tiles are worth a block: a block costs about four steps (128 queries each) besides its own
   // and 0.02 for its partial sums, and half a block is lost at the end.  Forward and backward, us, all parts / these: 821
   // tokens x 4 (2 KV heads) 113 / 107, 2048 tokens 103 / 99, 6000 tokens 165 / 145, 20001 tokens 785 / 766; 1024 tokens, less
-  // than a block per SM, 31 with four parts and 36 with two.
-  void choose_run(double steps) {
+  // than a block per SM, 31 with four parts and 36 with two.  Reproducible gradients take all parts: other groups of steps
+  // would give dK and dV other bits (20001 tokens 782 / 803).
+  void choose_run(double steps, bool reproducible) {
     for (int c = 0; c < 3; ++c) run[c] = parts[c];
+    if (reproducible) return;
     const int sms = cowa::sm_count();
     double best = 0;
     for (int p = 1; p <= parts[1]; ++p) {
@@ -1028,7 +1030,7 @@ void plan_rest(BwdPlan& pl, long long rest, double avg, double share) {
   }
 }
 
-BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& hw) {
+BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& hw, bool reproducible) {
   BwdPlan pl;
   const int nKV = (Nk + BKV - 1) / BKV, sms = cowa::sm_count();
   pl.sink_tiles = 0;
@@ -1058,7 +1060,7 @@ BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& h
   const long long room = heads > 1 ? ntiles * heads : 0;
   const long long budget = heads >= 4 ? room : std::max<long long>(room, 4ll * sms);
   while (pl.slots() > budget) --*std::max_element(pl.parts, pl.parts + 3);
-  pl.choose_run(rest > 0 ? (double)(total - sinks) / rest * BQS / BQT : 0.0);
+  pl.choose_run(rest > 0 ? (double)(total - sinks) / rest * BQS / BQT : 0.0, reproducible);
   return pl;
 }
 
@@ -1081,7 +1083,7 @@ BwdPlan bwd_plan_varlen(int B, int total, int Hkv, int G, const cowa_params_t* p
   // the last wave is not shared here: short sequences make its tiles short already (1628 against 1624 in 1000 clocks)
   const double avg = 0.7 * keys / BQS * G, real = (double)total / BKV * Hkv;
   plan_rest(pl, rest, rest <= 2 * sms ? avg : 0.0, real * avg / sms);
-  pl.choose_run(avg * BQS / BQT);
+  pl.choose_run(avg * BQS / BQT, p->deterministic != 0);
   return pl;
 }
 
@@ -1275,7 +1277,7 @@ size_t cowa_bwd_prefill_workspace_bytes(int B, int Nq, int Nk, int Hq, int Hkv, 
   if (B <= 0 || Nq <= 0 || Nk < Nq || Hq <= 0 || Hkv <= 0 || Hq % Hkv != 0 || D <= 0 || !p) return 0;
   CowaHeadWindows hw;
   if (cowa::resolve_windows(Nk, Hkv, p, &hw) != COWA_OK) return 0;
-  return ws_bytes(B, Nq, Hq, D, bwd_plan(B, Nq, Nk, Hkv, Hq / Hkv, hw));
+  return ws_bytes(B, Nq, Hq, D, bwd_plan(B, Nq, Nk, Hkv, Hq / Hkv, hw, p->deterministic != 0));
 }
 
 size_t cowa_bwd_workspace_bytes(int B, int T, int Hq, int Hkv, int D, const cowa_params_t* p) {
@@ -1295,7 +1297,7 @@ int cowa_bwd_prefill(const void* q, const void* k, const void* v, const void* o,
   CowaHeadWindows hw;
   int rc = cowa::resolve_windows(Nk, Hkv, p, &hw);
   if (rc != COWA_OK) return rc;
-  const BwdPlan pl = bwd_plan(B, Nq, Nk, Hkv, Hq / Hkv, hw);
+  const BwdPlan pl = bwd_plan(B, Nq, Nk, Hkv, Hq / Hkv, hw, p->deterministic != 0);
   if (workspace_bytes < ws_bytes(B, Nq, Hq, D, pl)) return COWA_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   return D == 128 ? launch_bwd<128>(q, k, v, o, lse, d_o, dq, dk, dv, B, Nq, Nk, Hq, Hkv, p, hw, pl, workspace, st)

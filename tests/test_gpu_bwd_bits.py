@@ -1,5 +1,7 @@
 """GPU tests of the reproducible mode's bits: gradients that repeat from run to run also have to repeat from version to version
 of the kernels, so that a resumed training run goes on as it would have."""
+import zlib
+
 import numpy as np
 import pytest
 import torch
@@ -35,3 +37,43 @@ def test_partial_dq_is_the_rounded_product_rounded_to_an_integer():
     assert raw.dtype == np.float32 and np.abs(raw * unit).max() < 2.0 ** 22
     assert not torch.equal(want, bf16(np.rint(raw.astype(np.float64) * unit))), "these inputs do not tell the two apart"
     assert torch.equal(dev[6].cpu(), want)
+
+
+# CRC-32 of dq, dk, dv on 148 SMs, from the kernels with steps of 64 queries and fixed parts of a tile.
+BITS = {
+    "2 x 1500": (dict(B=2, T=1500, Hq=8, Hkv=2, D=128, sink=64, local=300), ["db333b91", "b37dcb24", "765d4edd"]),
+    "4 x 821, D = 64": (dict(B=4, T=821, Hq=8, Hkv=2, D=64, sink=4, local=466), ["efb22a5b", "d994e355", "f2a96f23"]),
+    "one rank of eight": (dict(B=1, T=5001, Hq=8, Hkv=1, D=128, sink=128, local=896, hkv_global=8, hkv_offset=3),
+                          ["3097b9f1", "fc1a6e69", "48a9bbe7"]),
+    "packed": (dict(lens=[300, 1, 64, 777, 0, 129, 400], Hq=8, Hkv=2, D=128, sink=16, local=200),
+               ["cccbda80", "7c4f115f", "b6063426"]),
+}
+
+
+def gradient_bits(B=1, T=0, Hq=0, Hkv=0, D=0, lens=None, **window):
+    """Gradients of random tensors: o and lse need not be the forward's, whose bits are not the subject here."""
+    q, k, v, d_o = cowa_inputs.make_train_inputs(370, B, sum(lens) if lens else T, Hq, Hkv, D)
+    o = cowa_inputs.make_train_inputs(371, *d_o.shape[:1], d_o.shape[2], Hq, Hkv, D)[0]
+    lse = torch.randn(d_o.shape[:-1], generator=torch.Generator().manual_seed(372)) + 4
+    if lens:
+        q, k, v, d_o, o, lse = (x[0] for x in (q, k, v, d_o, o, lse))
+    q, k, v, d_o, o, lse = (x.to(DEV) for x in (q, k, v, d_o, o, lse))
+    params = cowa.make_params(softmax_scale=cowa_inputs.softmax_scale(D), deterministic=True, **window)
+    grads = [torch.full_like(x, float("nan")) for x in (q, k, v)]
+    if lens:
+        n = cowa.cowa_bwd_varlen_workspace_bytes(len(lens), sum(lens), Hq, Hkv, D, params)
+        cu = torch.tensor(np.cumsum([0] + lens), dtype=torch.int32, device=DEV)
+        ws = torch.empty(n, dtype=torch.uint8, device=DEV)
+        cowa.cowa_bwd_varlen(q, k, v, o, lse, d_o, *grads, cu, params, ws)
+    else:
+        ws = torch.empty(cowa.cowa_bwd_workspace_bytes(B, T, Hq, Hkv, D, params), dtype=torch.uint8, device=DEV)
+        cowa.cowa_bwd(q, k, v, o, lse, d_o, *grads, params, ws)
+    torch.cuda.synchronize()
+    cowa.cowa_check_device_status()
+    return ["%08x" % zlib.crc32(x.cpu().view(torch.int16).numpy().tobytes()) for x in grads]
+
+
+@pytest.mark.parametrize("name", BITS)
+def test_gradients_have_the_bits_that_they_always_had(name):
+    case, want = BITS[name]
+    assert gradient_bits(**case) == want
