@@ -794,10 +794,8 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 // delta = -rowsum(O * dO), lse2 = -LSE * log2(e); rows in [T, Tpad) get lse2 = -inf, delta = 0.  The same threads zero
 // the fp32 dQ accumulator (as a memset before it that was a pass of its own: 32K 190 us for both, 164 us so).
 template <int D>
-__global__ void cowa_bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
-                                           const float* __restrict__ lse, float* __restrict__ lse2,
-                                           float* __restrict__ delta, float* __restrict__ acc, int T, int Tpad,
-                                           long long BH, int H, CowaStrides so) {
+__global__ void cowa_bwd_preprocess_kernel(const __nv_bfloat16* o, const __nv_bfloat16* d_o, const float* lse, float* lse2,
+                                           float* delta, float* acc, int T, int Tpad, long long BH, int H, CowaStrides so) {
   grid_enter();
   constexpr int TPR = D / 8;  // threads per row (16 bytes each)
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -834,10 +832,8 @@ __global__ void cowa_bwd_preprocess_kernel(const __nv_bfloat16* __restrict__ o, 
 // tokens, 16 heads: one row a thread 142 us, this 102; 680 MB).
 template <int D>
 __global__ void __launch_bounds__(256)
-cowa_bwd_preprocess_varlen_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
-                                  const float* __restrict__ lse, float* __restrict__ lse2, float* __restrict__ delta,
-                                  float* __restrict__ acc, const int* __restrict__ cu, int B, int total, int Tpad,
-                                  unsigned int* status) {
+cowa_bwd_preprocess_varlen_kernel(const __nv_bfloat16* o, const __nv_bfloat16* d_o, const float* lse, float* lse2, float* delta,
+                                  float* acc, const int* cu, int B, int total, int Tpad, unsigned int* status) {
   grid_enter();
   constexpr int TPR = D / 8;                          // threads per row (16 bytes each)
   constexpr int ROWS = 256 / TPR, PASS = BQS / ROWS;  // rows at a time
@@ -891,8 +887,8 @@ cowa_bwd_preprocess_varlen_kernel(const __nv_bfloat16* __restrict__ o, const __n
 // sectors.  (One kernel with the sum of partial dK, dV needs 46 registers and lost occupancy: 137 instead of 112 us at 32K.)
 template <int D, bool VARLEN>
 __global__ void __launch_bounds__(256)
-cowa_bwd_convert_dq_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, const int* __restrict__ cu, int B,
-                           int T, int Tpad, int H, int fixed, CowaStrides sq, unsigned int* status) {
+cowa_bwd_convert_dq_kernel(const float* acc, __nv_bfloat16* dq, const int* cu, int B, int T, int Tpad, int H, int fixed,
+                           CowaStrides sq, unsigned int* status) {
   grid_enter();
   const int nchunk = Tpad / BQS, chunk = VARLEN ? blockIdx.x : blockIdx.x % nchunk, bh = VARLEN ? blockIdx.y : blockIdx.x / nchunk;
   int rows, first;  // rows of this chunk, and the first one's place among the rows of dq

@@ -83,7 +83,7 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint3
 
 __device__ __forceinline__ uint4 ldg128(const void* p) {
   uint4 r;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];\n"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];\n"
                : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
                : "l"(p));
   return r;
@@ -274,11 +274,8 @@ __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const De
 // with shuffles, takes every fourth split with D/32 columns per lane (several loads in flight), and the
 // four partial sums meet in shared memory.
 template <int D>
-__global__ void __launch_bounds__(128) cowa_decode_combine_kernel(const float* __restrict__ ws_o,
-                                                                  const float* __restrict__ ws_m,
-                                                                  const float* __restrict__ ws_l,
-                                                                  __nv_bfloat16* __restrict__ o,
-                                                                  float* __restrict__ lse, int S) {
+__global__ void __launch_bounds__(128) cowa_decode_combine_kernel(const float* ws_o, const float* ws_m, const float* ws_l,
+                                                                  __nv_bfloat16* o, float* lse, int S) {
   constexpr int V = D / 32;  // columns per lane
   __shared__ float part[4][D];
   const size_t bh = blockIdx.x;

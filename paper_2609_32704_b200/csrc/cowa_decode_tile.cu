@@ -627,8 +627,7 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 // takes every WPR-th group of eight and the partial results meet in shared memory.
 template <int D, int WPR>
 __global__ void __launch_bounds__(WPR == 1 ? 128 : WPR * 32) cowa_decode_tile_merge_kernel(const __grid_constant__ TileArgs a,
-                                                                                         __nv_bfloat16* __restrict__ o,
-                                                                                         float* __restrict__ lse) {
+                                                                                         __nv_bfloat16* o, float* lse) {
   constexpr int V = D / 32, U = 8;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int r = WPR == 1 ? blockIdx.x * 4 + warp : blockIdx.x;

@@ -99,7 +99,9 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
 // ------------------------------------------------------------------ kernels in a row (see cowa::launch_chained)
 // Top of a kernel, ahead of every access to global memory and of its TMEM allocation: the kernel before it in the stream is
 // complete and its results are visible.  The next kernel may have its blocks scheduled from here on (not earlier: it would
-// then run beside the kernel before this one).
+// then run beside the kernel before this one).  A kernel's life thus begins while the one before it still writes, so that
+// nothing it reads is read-only for its whole life: no loads through the non-coherent path (ld.global.nc, __ldg, pointers to
+// const declared __restrict__), which the compiler might even move over the wait.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_enter() {
   grid_wait();
@@ -380,7 +382,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // the last tile.  *pad_base is the number of rows before the sequence when every sequence is padded to a
 // multiple of `pad` rows (pad > 0).  With skip > 0 the first `skip` tiles of every sequence are left out of
 // the count (they are handed out separately); *local_tile still counts from the sequence's first tile.
-__device__ __forceinline__ bool varlen_locate(const int* __restrict__ cu, int B, int idx, int tile, int pad, int* b_out,
+__device__ __forceinline__ bool varlen_locate(const int* cu, int B, int idx, int tile, int pad, int* b_out,
                                               int* local_tile, int* tiles_in_seq, int* pad_base, int skip = 0) {
   const int lane = threadIdx.x & 31;
   int base = 0, pbase = 0;
@@ -419,7 +421,7 @@ __device__ __forceinline__ bool varlen_locate(const int* __restrict__ cu, int B,
 // of a batch are then its shortest lists, whatever the order in the batch.  Up to kLongestFirst sequences: every lane
 // compares its two with all others, which is a few hundred instructions; for more the order of the batch stays.
 constexpr int kLongestFirst = 64;
-__device__ __forceinline__ bool varlen_locate_longest(const int* __restrict__ cu, const int* __restrict__ cu_len, int B,
+__device__ __forceinline__ bool varlen_locate_longest(const int* cu, const int* cu_len, int B,
                                                       int idx, int tile, int mult, int skip, int* b_out, int* item,
                                                       int* tiles_in_seq) {
   const int lane = threadIdx.x & 31;
@@ -452,7 +454,7 @@ __device__ __forceinline__ bool varlen_locate_longest(const int* __restrict__ cu
 }
 
 // Companion of varlen_locate for a known sequence b: its tile count and its padded row base (warp-cooperative).
-__device__ __forceinline__ void varlen_seq_info(const int* __restrict__ cu, int b, int tile, int pad, int* tiles_in_seq,
+__device__ __forceinline__ void varlen_seq_info(const int* cu, int b, int tile, int pad, int* tiles_in_seq,
                                                 int* pad_base) {
   const int lane = threadIdx.x & 31;
   int sum = 0;
