@@ -79,11 +79,11 @@ cowa_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     b = idx % a.B; idx /= a.B;
     i = (a.Nq + BQ - 1) / BQ - 1 - idx;
   } else {
-    // idx counts the QO tiles of the packed batch, longest sequence first, each sequence's heaviest (last) tile first.
+    // idx counts the QO tiles of the packed batch, each sequence's heaviest (last) tile first.
     // Every warp finds its (sequence, tile) by a cooperative scan of the offsets.  The grid is an upper bound.
     int lt, nts, pb;
-    if (a.B <= kLongestFirst ? !varlen_locate_longest(a.cu_q, a.cu_k, a.B, idx, BQ, 1, 0, &b, &lt, &nts)
-                             : !varlen_locate(a.cu_q, a.B, idx, BQ, 0, &b, &lt, &nts, &pb))
+    if (a.longest_first ? !varlen_locate_longest(a.cu_q, a.cu_k, a.B, idx, BQ, 1, 0, &b, &lt, &nts)
+                        : !varlen_locate(a.cu_q, a.B, idx, BQ, 0, &b, &lt, &nts, &pb))
       return;
     i = nts - 1 - lt;
   }
@@ -442,6 +442,20 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
   a.hkv_global = p->hkv_global > 0 ? p->hkv_global : Hkv;
   a.hkv_offset = p->hkv_offset; a.full_attn = p->full_attn; a.explicit_windows = p->windows != nullptr;
   const long long tiles = VARLEN ? (long long)total_q / BQ + B : (long long)((Nq + BQ - 1) / BQ) * B;
+  const int qn = VARLEN ? std::max(total_q / B, 1) : Nq, kn = VARLEN ? std::max(total_k / B, 1) : Nk;
+  int keys = 0;  // visited by the longest list, tile remainders included
+  for (int h = 0; h < Hkv; ++h) {
+    CowaWin w = hw.w[h];
+    if (VARLEN && p->full_attn) w.n = kn;
+    else if (VARLEN && !p->windows) w = cowa_default_window(kn, a.hkv_global, a.hkv_offset + h, a.sink, a.local);
+    const long long width = (long long)std::min(w.s, kn) + std::min(w.n, kn) + std::min(w.l, kn) + 2 * BQ;
+    keys = std::max(keys, (int)std::min<long long>(width, kn));
+  }
+  // Packed batches: order of the items.  By length where the average sequence has 1024 keys to visit, or where the blocks of
+  // single heads make four waves at most and a long list among the last ones shows (20 prompts of 30 to 1000 tokens, 4 heads:
+  // 33 us, 38 in the batch's order; 7 of 4292 tokens, 16 heads: 46, 54).  Else lists are over so soon that finding an item by
+  // its length costs more than it gives (30 prompts of 100 tokens, 32 heads, D = 64: 24 us, 21 in the batch's order).
+  a.longest_first = VARLEN && B <= kLongestFirst && (keys >= 1024 || tiles * Hq <= 8 * cowa::sm_count());
   if (a.G % 2 == 0) {
     // Which kernel, judged for packed batches by their average sequence, so that equal lengths give what the batched
     // call gives, bit for bit.  At D = 128 (us, one-head / pair kernel):
@@ -459,15 +473,6 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
     //     up to a tenth either way (T 6000, Hq 16, 2.5 items per SM: 0.90; T 2048, Hq 32, 1.7: 1.13).
     // At D = 64 the exponentials bound both and two one-head blocks per SM keep them busier (T 22272, 4 heads, fwd and
     // bwd 1064 / 1138), so that only the shared form is taken there.
-    const int qn = VARLEN ? std::max(total_q / B, 1) : Nq, kn = VARLEN ? std::max(total_k / B, 1) : Nk;
-    int keys = 0;  // visited by the longest list, tile remainders included
-    for (int h = 0; h < Hkv; ++h) {
-      CowaWin w = hw.w[h];
-      if (VARLEN && p->full_attn) w.n = kn;
-      else if (VARLEN && !p->windows) w = cowa_default_window(kn, a.hkv_global, a.hkv_offset + h, a.sink, a.local);
-      const long long width = (long long)std::min(w.s, kn) + std::min(w.n, kn) + std::min(w.l, kn) + 2 * BQ;
-      keys = std::max(keys, (int)std::min<long long>(width, kn));
-    }
     const long long items = tiles * (Hq / 2), judged = (long long)((qn + BQ - 1) / BQ) * B * (Hq / 2);
     if (items > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
     const bool shared = judged <= cowa::resident_clusters(2), even = kn >= 2ll * qn;

@@ -19,6 +19,7 @@ struct FwdArgs {
   int total_q, total_k;
   CowaStrides so;    // of o (batched calls)
   int sink, local, hkv_global, hkv_offset, full_attn, explicit_windows;
+  int longest_first;  // sequences in order of their keys (varlen_locate_longest), else in the batch's
 };
 
 namespace cowa {

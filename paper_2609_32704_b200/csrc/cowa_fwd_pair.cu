@@ -92,8 +92,8 @@ __device__ __forceinline__ bool locate_item(const FwdArgs& a, int idx, PairItem&
     it.Nq = a.Nq; it.Nk = a.Nk; it.qbase = 0; it.kbase = 0; it.bt = it.b;
   } else {
     int lt, nts, pb;
-    if (a.B <= kLongestFirst ? !varlen_locate_longest(a.cu_q, a.cu_k, a.B, idx, BQ, 1, 0, &it.b, &lt, &nts)
-                             : !varlen_locate(a.cu_q, a.B, idx, BQ, 0, &it.b, &lt, &nts, &pb))
+    if (a.longest_first ? !varlen_locate_longest(a.cu_q, a.cu_k, a.B, idx, BQ, 1, 0, &it.b, &lt, &nts)
+                        : !varlen_locate(a.cu_q, a.B, idx, BQ, 0, &it.b, &lt, &nts, &pb))
       return false;
     i = nts - 1 - lt;
     it.qbase = a.cu_q[it.b]; it.Nq = a.cu_q[it.b + 1] - it.qbase;
