@@ -28,9 +28,9 @@ namespace cowa {
 int resident_clusters(int size);
 
 // Pair kernel (cowa_fwd_pair.cu; the tensor maps of the one-head kernel, 64-row boxes of K and V): two QO heads of a
-// group at a time, `items` = tiles x pairs of heads.  split = 1: one persistent block per SM; split = 2, 4, 8: every item
-// shared by a cluster of that many blocks.
+// group at a time, `items` = tiles x pairs of heads.  split = 1: a block per SM at a time, with `rounds` items for its share
+// and others taken over after them; split = 2, 4, 8: every item shared by a cluster of that many blocks.
 template <int D, bool VARLEN>
 int launch_fwd_pair(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mo,
-                    const FwdArgs& a, long long items, int split, cudaStream_t st);
+                    const FwdArgs& a, long long items, int rounds, int split, cudaStream_t st);
 }  // namespace cowa

@@ -1,6 +1,7 @@
 // CoWindow Attention forward (Algorithm 1) for sm_100a: two QO heads of a GQA group per block.
 //
-// One block per SM at a time, each taking over further blocks of the grid (cluster launch control).  A work item is (batch, pair of QO heads that share a KV head, 128-row QO tile);
+// One block per SM at a time, each taking over further blocks of the grid (cluster launch control).  A work item is (batch, pair of QO
+// heads that share a KV head, 128-row QO tile);
 // both heads visit the same KV tiles J_h(i), so one pass over K and V serves 256 query rows.  A step takes two
 // visited 64-key tiles (not necessarily neighbours) as one 128-key operand: S at N = 128 runs at the full tensor
 // rate (512 clocks; as two products of 64 keys 768).  Warps:
@@ -77,7 +78,7 @@ struct PairItem {
 static_assert(sizeof(PairItem) <= 128, "slot of a published item");
 static_assert(4 * PairSmem<128>::kKV >= 2 * BQ * 128 * 4, "fp32 O of both heads fits the K and V slots");
 
-// false: no item of this number (packed batches: the count is an upper bound) or malformed offsets
+// false: no item of this number (packed batches: the count is an upper bound; it.b = -1) or malformed offsets
 template <bool VARLEN>
 __device__ __forceinline__ bool locate_item(const FwdArgs& a, int idx, PairItem& it) {
   const int PG = a.G >> 1;
@@ -93,8 +94,10 @@ __device__ __forceinline__ bool locate_item(const FwdArgs& a, int idx, PairItem&
   } else {
     int lt, nts, pb;
     if (a.longest_first ? !varlen_locate_longest(a.cu_q, a.cu_k, a.B, idx, BQ, 1, 0, &it.b, &lt, &nts)
-                        : !varlen_locate(a.cu_q, a.B, idx, BQ, 0, &it.b, &lt, &nts, &pb))
+                        : !varlen_locate(a.cu_q, a.B, idx, BQ, 0, &it.b, &lt, &nts, &pb)) {
+      it.b = -1;
       return false;
+    }
     i = nts - 1 - lt;
     it.qbase = a.cu_q[it.b]; it.Nq = a.cu_q[it.b + 1] - it.qbase;
     it.kbase = a.cu_k[it.b]; it.Nk = a.cu_k[it.b + 1] - it.kbase;
@@ -130,14 +133,23 @@ __device__ __forceinline__ bool locate_item(const FwdArgs& a, int idx, PairItem&
   return it.nt > 0;
 }
 
-// SPLIT: a cluster of blocks shares one item (few items, long lists): each takes a contiguous part of its steps, and
-// the partial states are merged through distributed shared memory.
-template <int D, bool VARLEN, bool SPLIT>
+// How the items are handed out (FORM).
+//   kTakenOver  an item per number of the grid; a block takes over the numbers whose blocks have not started
+//   kSplit      a cluster of blocks shares one item (few items, long lists): each takes a contiguous part of its steps, and
+//               the partial states are merged through distributed shared memory
+//   kShares     as the first, but the first `starters` numbers stand for `rounds` items each, from alternate ends.  A number
+//               taken over costs a block up to a microsecond between two items, more than short lists hide, and so do the
+//               numbers past a packed batch's last item (us, a fixed share of all / all taken over / three quarters in
+//               shares: 100 prompts of 200 tokens, 16 heads 73 / 78 / 75; 300 of 130, 32 heads 329 / 362 / 316; 48 of 60
+//               to 5000 425 / 430 / 407; 64 of 1000, local 128 496 / 573 / 481)
+constexpr int kTakenOver = 0, kSplit = 1, kShares = 2;
+template <int D, bool VARLEN, int FORM>
 __global__ void __launch_bounds__(kPairThreads, 1)
 cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                      const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
-                     const __grid_constant__ FwdArgs a) {
+                     const __grid_constant__ FwdArgs a, const int starters, const int rounds) {
   using SM = PairSmem<D>;
+  constexpr bool SPLIT = FORM == kSplit, SHARES = FORM == kShares;
   constexpr int NSLAB = D / 64;        // 64-element (128-byte) slabs along D
   constexpr int SLAB = 128 * 128;      // bytes of one slab of a 128-row tile
   constexpr uint32_t TMEM_COLS = 512;  // S/P of head x: [128x, 128x + 128); O of head x: [256 + 128x, ... + D)
@@ -216,9 +228,10 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     if (lead) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); }
     int c = 0;       // steps loaded so far, all items together: step c uses slot c & 1
     uint32_t ni = 0;  // items so far
-    // The grid has a block per item, heaviest items first.  A block starts with its own and, towards the end of an item,
-    // takes over the next one whose block has not started: lists differ in length, and with a fixed share of the items per
-    // block the last SM was busy 20 % longer than the average one (one KV head of 20001 tokens), 25 % for packed prompts.
+    // The grid has a number per item, heaviest items first (SHARES: fewer).  A block starts with its own and, towards the end
+    // of an item, takes over the next one whose block has not started: lists differ in length, and with a fixed share of the
+    // items per block the last SM was busy 20 % longer than the average one (one KV head of 20001 tokens), 25 % for packed
+    // prompts.
     const int csize = SPLIT ? (int)cluster_size() : 1;
     uint32_t asked = 0, answered = 0;  // requests
     auto ask = [&]() {
@@ -237,6 +250,19 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       return x;
     };
     int idx = SPLIT ? blockIdx.x / csize : blockIdx.x;
+    int num = idx, rnd = 0;  // SHARES: this block's number, and how many of its items came before
+    int past = 0x7FFFFFFF;   // ... from this item on there are none
+    if (SHARES && num >= starters) idx += (rounds - 1) * starters;
+    auto more = [&]() { return SHARES && num < starters && rnd + 1 < rounds; };
+    auto next_item_index = [&]() -> int {
+      if (more()) {
+        ++rnd;
+        return rnd * starters + ((rnd & 1) ? starters - 1 - num : num);
+      }
+      const int x = next_index();
+      num = x; rnd = 0;
+      return SHARES && x >= starters ? x + (rounds - 1) * starters : x;
+    };
     while (ok) {
       PairItem& it = *reinterpret_cast<PairItem*>(smem + SM::oItem + (ni & 1) * 128);
       {
@@ -252,11 +278,13 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
           }
         } else if (idx < 0) {
           mine.nt = 0;
-        } else if (!locate_item<VARLEN>(a, idx, mine)) {
-          ask();
-          idx = next_index();
+        } else if ((SHARES && idx >= past) || !locate_item<VARLEN>(a, idx, mine)) {
+          if (SHARES && idx < past && mine.b < 0) past = idx;
+          if (!more()) ask();
+          idx = next_item_index();
           continue;
         }
+        if (SHARES && mine.nt > 0 && mine.nt <= 6 && !more()) ask();  // of up to three steps: no later moment is early enough
         if (ni >= 2) ok = mbar_wait(bar_i_empty + (ni & 1), ((ni >> 1) & 1) ^ 1, a.status);
         if (!ok) break;
         if (lead) {
@@ -282,7 +310,8 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         const uint32_t ph = ((c >> 1) & 1) ^ 1;
         if (c >= 2) ok = mbar_wait(bar_k_empty + sl, ph, a.status);
         if (!ok) break;
-        if (!SPLIT && t == ask_at) ask();  // a microsecond or more before the answer is needed
+        // a microsecond or more before the answer is needed
+        if (!SPLIT && t == ask_at && (!SHARES || (it.nt > 6 && !more()))) ask();
         load_kv(sK + sl * SM::kKV, &tmK, bar_k_full + sl, t);
         if (t == 0) {
           if (ni > 0) ok = mbar_wait(bar_q_empty, (ni - 1) & 1, a.status);
@@ -299,7 +328,7 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         load_kv(sV + sl * SM::kKV, &tmV, bar_v_full + sl, t);
       }
       ++ni;
-      if (!SPLIT && ok) idx = next_index();
+      if (!SPLIT && ok) idx = next_item_index();
     }
     if (asked != answered) mbar_wait(bar_next, (asked - 1) & 1, a.status);  // (a wait ran out) no answer may come later
    } else if (warp == 9) {
@@ -707,7 +736,7 @@ int resident_clusters(int size) {
   if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
     n = cache[dev][i].load(std::memory_order_relaxed);
     if (n > 0) return n;
-    const auto kernel = cowa_fwd_pair_kernel<128, false, true>;
+    const auto kernel = cowa_fwd_pair_kernel<128, false, kSplit>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)size); cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = PairSmem<128>::kBytes;
     cudaLaunchAttribute attr[1];
@@ -726,14 +755,18 @@ int resident_clusters(int size) {
 
 template <int D, bool VARLEN>
 int launch_fwd_pair(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mo,
-                    const FwdArgs& a, long long items, int split, cudaStream_t st) {
-  auto kernel = cowa_fwd_pair_kernel<D, VARLEN, true>;
+                    const FwdArgs& a, long long items, int rounds, int split, cudaStream_t st) {
+  auto kernel = cowa_fwd_pair_kernel<D, VARLEN, kSplit>;
   if constexpr (D == 128) {
-    if (split == 1) kernel = cowa_fwd_pair_kernel<D, VARLEN, false>;
+    if (split == 1) kernel = cowa_fwd_pair_kernel<D, VARLEN, kTakenOver>;
+    if constexpr (VARLEN) {
+      if (split == 1 && rounds > 1) kernel = cowa_fwd_pair_kernel<D, VARLEN, kShares>;
+    }
   }
   COWA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PairSmem<D>::kBytes));
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(items * split));
+  const int starters = (int)std::min<long long>(items, sm_count());
+  cfg.gridDim = dim3((unsigned)(split > 1 ? items * split : items - (rounds - 1ll) * starters));
   cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = PairSmem<D>::kBytes; cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -741,13 +774,13 @@ int launch_fwd_pair(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensor
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = (unsigned)split; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr; cfg.numAttrs = split > 1 ? 2 : 1;
-  COWA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mo, a));
+  COWA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mo, a, starters, rounds));
   return COWA_OK;
 }
 
 #define COWA_INSTANTIATE(D, V)                                                                                          \
   template int launch_fwd_pair<D, V>(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const CUtensorMap&,    \
-                                     const FwdArgs&, long long, int, cudaStream_t);
+                                     const FwdArgs&, long long, int, int, cudaStream_t);
 COWA_INSTANTIATE(128, false)
 COWA_INSTANTIATE(128, true)
 COWA_INSTANTIATE(64, false)
