@@ -71,7 +71,8 @@ def _build_call_module(verbose):
 
 
 def build_library(verbose=False, force=False):
-    """Compiles every .cu under csrc/ and links libcowa.so, beside it _cowa_call.so.  Returns libcowa.so's path."""
+    """Compiles every .cu under csrc/ and links libcowa.so.  Returns its path.  The binding's argument path is built beside it
+    where that can be done (PyTorch, g++, Python headers); without it every call takes the Python path."""
     os.makedirs(OBJ_DIR, exist_ok=True)
     if force:
         for f in os.listdir(OBJ_DIR):
@@ -82,7 +83,6 @@ def build_library(verbose=False, force=False):
     with ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 1)) as ex:
         call = ex.submit(_build_call_module, verbose)
         res = list(ex.map(lambda s: _compile(s, verbose), _sources()))
-        call.result()
     objs = [o for o, _ in res]
     rebuilt = any(ch for _, ch in res)
     if rebuilt or not os.path.exists(LIB_PATH):
@@ -91,6 +91,10 @@ def build_library(verbose=False, force=False):
         if r.returncode != 0:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("link failed")
+    try:
+        call.result()
+    except (ImportError, OSError, RuntimeError) as e:
+        sys.stderr.write(f"{os.path.basename(CALL_SRC)} not built, calls take the Python path: {e}\n")
     return LIB_PATH
 
 
