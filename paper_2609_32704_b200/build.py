@@ -4,6 +4,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -12,7 +13,7 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 OBJ_DIR = os.path.join(HERE, "build")
 LIB_PATH = os.path.join(HERE, "libcowa.so")
 CALL_SRC = os.path.join(HERE, "csrc_py", "cowa_call.cpp")
-CALL_PATH = os.path.join(HERE, "_cowa_call.so")
+CALL_PATH = os.path.join(HERE, "_cowa_call" + sysconfig.get_config_var("EXT_SUFFIX"))  # (another Python does not load it)
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -49,13 +50,26 @@ def _compile(src, verbose):
     return obj, True
 
 
+def _call_stamp():
+    """What the argument path's module was built against, kept beside the objects: PyTorch's headers do not get newer than
+    the module when another version is installed."""
+    return os.path.join(OBJ_DIR, "cowa_call.torch")
+
+
+def _read(path):
+    try:
+        with open(path) as f:
+            return f.read()
+    except OSError:
+        return None
+
+
 def _build_call_module(verbose):
     """The binding's native argument path: a Python extension over torch's headers (no CUDA code)."""
-    if os.path.exists(CALL_PATH) and os.path.getmtime(CALL_PATH) >= max(os.path.getmtime(CALL_SRC), _headers_mtime()):
-        return
-    import sysconfig
-
     import torch
+    if (os.path.exists(CALL_PATH) and os.path.getmtime(CALL_PATH) >= max(os.path.getmtime(CALL_SRC), _headers_mtime())
+            and _read(_call_stamp()) == torch.__version__):
+        return
     root = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(_nvcc())) or "/usr/local/cuda"
     inc = [INCLUDE, os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
@@ -68,6 +82,8 @@ def _build_call_module(verbose):
         sys.stderr.write(r.stdout + r.stderr)
     if r.returncode != 0:
         raise RuntimeError("g++ failed on cowa_call.cpp")
+    with open(_call_stamp(), "w") as f:
+        f.write(torch.__version__)
 
 
 def build_library(verbose=False, force=False):
