@@ -127,7 +127,8 @@ int cowa_prefill(const void* q, const void* k, const void* v, void* o, float* ls
  * evaluated per sequence on the device.  The offsets are read on the device only: a sequence with
  * N_q > N_k, or whose rows leave the tensors, is skipped (N_q < 0 counts as empty) and
  * cowa_check_device_status() then returns COWA_ERR_DEVICE_BAD_SEQLENS.  No workspace; nothing is
- * retained.  Blocks are issued sequence after sequence: passing long sequences first shortens the tail. */
+ * retained.  The order of the sequences does not matter for the results; up to 64 of them are worked on longest first
+ * where that helps.  With more, passing long sequences first shortens the end of the call. */
 int cowa_prefill_varlen(const void* q, const void* k, const void* v, void* o, float* lse,
                         const int32_t* cu_seqlens_q, const int32_t* cu_seqlens_k, int B, int total_q,
                         int total_k, int Hq, int Hkv, int D, const cowa_params_t* p, void* stream);

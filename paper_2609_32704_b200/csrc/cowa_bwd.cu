@@ -45,7 +45,6 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
-#include <type_traits>
 
 #include "cowa_common.h"
 #include "cowa_ptx.cuh"
@@ -452,10 +451,10 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                      dB + (((kk / 4) * SLAB_Q + (kk % 4) * 32) >> 4), ID_ST, kk > 0);
           }
         };
-        auto gemm_acc = [&](uint32_t d_col, uint32_t a_col, uint64_t dB, uint32_t acc_first, int k0_, int k1_) {  // [128 x D] += A(TMEM) B
+        auto gemm_acc = [&](uint32_t d_col, uint32_t a_col, uint64_t dB, uint32_t acc_first) {  // [128 x D] += A(TMEM) B
           if (lead) {
 #pragma unroll
-            for (int kk = k0_; kk < k1_; ++kk)  // 32-query blocks 0, 2 from one warpgroup's columns, 1, 3 from the other's
+            for (int kk = 0; kk < BQT / 16; ++kk)  // 32-query blocks 0, 2 from one warpgroup's columns, 1, 3 from the other's
               mma_ts(tb + d_col, tb + a_col + ((kk >> 1) & 1) * 32 + (kk >> 2) * 16 + (kk & 1) * 8, dB + ((kk * 2048) >> 4), ID_ACC, kk > 0 ? 1u : acc_first);
           }
         };
@@ -514,7 +513,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             ok = mbar_wait(bar_ds_ready, par ^ 1, a.status);
             if (!ok) return;
             tc_fence_after();
-            gemm_acc(cDK, cDS, dQ_mn0 + (st ^ 1) * kQ16, n > 1 ? 1u : 0u, 0, 8);
+            gemm_acc(cDK, cDS, dQ_mn0 + (st ^ 1) * kQ16, n > 1 ? 1u : 0u);
             commit(bar_q_empty + (st ^ 1));
             ok = mbar_wait(bar_s_read, par, a.status);
             if (!ok) return;
@@ -537,7 +536,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           ok = mbar_wait(bar_p_ready, par, a.status);
           if (!ok) return;
           tc_fence_after();
-          gemm_acc(cDV, cS, dO_mn0, n > 0 ? 1u : 0u, 0, 8);
+          gemm_acc(cDV, cS, dO_mn0, n > 0 ? 1u : 0u);
           commit(bar_o_empty);
           if (n + 1 < N) {
             ok = mbar_wait(bar_q_full + (st ^ 1), ((n + 1) >> 1) & 1, a.status);
@@ -558,7 +557,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             tc_fence_after();
             gemm_dq();
             commit(bar_dq_full);
-            gemm_acc(cDK, cDS, dQ_mn0 + ((N - 1) & 1) * kQ16, N > 1 ? 1u : 0u, 0, 8);
+            gemm_acc(cDK, cDS, dQ_mn0 + ((N - 1) & 1) * kQ16, N > 1 ? 1u : 0u);
           }
         }
         commit(bar_done);
@@ -804,25 +803,28 @@ __global__ void cowa_bwd_preprocess_kernel(const __nv_bfloat16* o, const __nv_bf
   if (row >= BH * Tpad) return;
   const long long bh = row / Tpad;
   const int t = (int)(row % Tpad);
-  float4* z = reinterpret_cast<float4*>(acc + (size_t)row * D + part * 8);
-  z[0] = z[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-  float s = 0.f;
+  // All loads ahead of the first store: the compiler does not move them over it.
+  uint4 x = make_uint4(0u, 0u, 0u, 0u), y = x;
+  float l = -INFINITY, s = 0.f;
   if (t < T) {
     const size_t base = (size_t)(bh / H) * so.b + (size_t)(bh % H) * so.h + (size_t)t * so.t + part * 8;
-    const uint4 x = *reinterpret_cast<const uint4*>(o + base);
-    const uint4 y = *reinterpret_cast<const uint4*>(d_o + base);
-    const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+    x = *reinterpret_cast<const uint4*>(o + base);
+    y = *reinterpret_cast<const uint4*>(d_o + base);
+    if (part == 0) l = lse[(size_t)bh * T + t] * -1.4426950408889634f;
+  }
+  float4* z = reinterpret_cast<float4*>(acc + (size_t)row * D + part * 8);
+  z[0] = z[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+  const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      s = fmaf(__uint_as_float(xs[i] << 16), __uint_as_float(ys[i] << 16), s);
-      s = fmaf(__uint_as_float(xs[i] & 0xffff0000u), __uint_as_float(ys[i] & 0xffff0000u), s);
-    }
+  for (int i = 0; i < 4; ++i) {
+    s = fmaf(__uint_as_float(xs[i] << 16), __uint_as_float(ys[i] << 16), s);
+    s = fmaf(__uint_as_float(xs[i] & 0xffff0000u), __uint_as_float(ys[i] & 0xffff0000u), s);
   }
 #pragma unroll
   for (int o_ = TPR / 2; o_ > 0; o_ >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o_);
   if (part == 0) {
     delta[row] = -s;
-    lse2[row] = t < T ? lse[(size_t)bh * T + t] * -1.4426950408889634f : -INFINITY;
+    lse2[row] = l;
   }
 }
 
@@ -972,13 +974,13 @@ cowa_bwd_reduce_dkv_kernel(const __grid_constant__ BwdArgs a, CowaStrides sk, Co
 }
 
 // How the KV tiles are shared among blocks.  A tile whose block takes the whole GQA group keeps dK, dV in TMEM; a shared
-// tile costs every block a prologue and 128 KB of fp32 partial sums (D = 128), about four steps' worth of time, so tiles
-// are shared only where whole ones leave SMs idle:
+// tile costs every block a prologue and 128 KB of fp32 partial sums (D = 128), so tiles are shared only where whole ones
+// leave SMs idle (work and shares are counted in 64-row QO tiles here, half a step of the kernel each):
 //   sink tiles, visited by every query tile, when one is longer than 3/4 of an SM's share of the work: thirds of a share;
-//   all tiles when there are at most two per SM: fifths of a share, four steps at least;
+//   all tiles when there are at most two per SM: fifths of a share, four QO tiles at least;
 //   the last tile per SM when there are at most eight: quarters, so that the last wave ends together.
-// Main kernel, 1000 clocks, whole heads of a group spread / this: 2 x 8K, 16 heads 1147 / 1070; one KV head of 20001 tokens
-// 1021 / 983; 1K, 4 heads 58 / 34.
+// These lines were measured with steps of one QO tile instead of two and have been left where they are; what a body tile's
+// block costs with the longer steps is in choose_run, which takes fewer of the parts reserved here.
 struct BwdPlan {
   int sink_tiles;  // per sequence and head
   int tiles[3], parts[3];  // parts: what the workspace has room for
@@ -1012,7 +1014,7 @@ struct BwdPlan {
   }
 };
 
-// `rest` tiles behind the sink tiles, `avg` steps each; share: an SM's steps
+// `rest` KV tiles behind the sink tiles, `avg` QO tiles each; share: an SM's QO tiles
 void plan_rest(BwdPlan& pl, long long rest, double avg, double share) {
   const int sms = cowa::sm_count();
   pl.tiles[1] = (int)rest; pl.parts[1] = 1;

@@ -636,8 +636,8 @@ __global__ void __launch_bounds__(WPR == 1 ? 128 : WPR * 32) cowa_decode_tile_me
   const int tile = t / a.tpt, row = (t - tile * a.tpt) * a.G + h % a.G;
   const int u = (b * a.Hkv + h / a.G) * a.ntiles + tile;
   Unit x;
-  unit_of(a, u, x);
-  grid_enter();  // the row states are complete and visible
+  unit_of(a, u, x);  // reads the lengths, which the tile kernel does not write: complete before that one began (grid_wait)
+  grid_enter();      // the row states are complete and visible
   const int2 info = x.nt > 0 ? a.ws_unit[u] : make_int2(0, 0);  // no visible key: 0 / 0
   const size_t first = (size_t)(info.x + u) * a.rows + row;  // piece i lies a.rows rows further
   const int S = info.y;

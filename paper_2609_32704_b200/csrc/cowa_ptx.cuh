@@ -97,11 +97,13 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
 }
 
 // ------------------------------------------------------------------ kernels in a row (see cowa::launch_chained)
-// Top of a kernel, ahead of every access to global memory and of its TMEM allocation: the kernel before it in the stream is
+// Top of a kernel, ahead of its TMEM allocation and its accesses to global memory: the kernel before it in the stream is
 // complete and its results are visible.  The next kernel may have its blocks scheduled from here on (not earlier: it would
-// then run beside the kernel before this one).  A kernel's life thus begins while the one before it still writes, so that
-// nothing it reads is read-only for its whole life: no loads through the non-coherent path (ld.global.nc, __ldg, pointers to
-// const declared __restrict__), which the compiler might even move over the wait.
+// then run beside the kernel before this one).  So all that comes before its predecessor is complete when a kernel begins, and
+// what that one does not write may be read before the wait (the tile decode's merge reads the lengths there).  The
+// predecessor itself may still write, so that nothing is read-only for a kernel's whole life: no loads through the
+// non-coherent path (ld.global.nc, __ldg, pointers to const declared __restrict__), which the compiler might even move over
+// the wait.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_enter() {
   grid_wait();
@@ -170,10 +172,6 @@ __device__ __forceinline__ void tma_commit_group() { asm volatile("cp.async.bulk
 template <int N>
 __device__ __forceinline__ void tma_wait_group_read() {
   asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
-}
-template <int N>
-__device__ __forceinline__ void tma_wait_group() {
-  asm volatile("cp.async.bulk.wait_group %0;" ::"n"(N) : "memory");
 }
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
