@@ -783,8 +783,6 @@ int launch_fwd_pair(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensor
                                      const FwdArgs&, long long, int, int, cudaStream_t);
 COWA_INSTANTIATE(128, false)
 COWA_INSTANTIATE(128, true)
-COWA_INSTANTIATE(64, false)
-COWA_INSTANTIATE(64, true)
 #undef COWA_INSTANTIATE
 
 }  // namespace cowa

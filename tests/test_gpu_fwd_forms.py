@@ -1,0 +1,49 @@
+"""The forms of the one-head forward kernel, each at the sizes where its parts are uneven, against the float64 oracle: clusters of 2,
+4 and 8 blocks, four streams in a block, one block per item; lists of as many steps as parts, fewer, and one more; tiles cut by
+the end of the sequence.  Tolerances as in test_gpu_parity."""
+import numpy as np
+import pytest
+import torch
+
+import cowa_inputs
+import paper_2609_32704_b200 as cowa
+from oracle import cowa_oracle as orc
+from test_gpu_parity import DEV, TOL_LSE, check
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("B,Nq,Nk,Hq,Hkv,sink,local", [
+    (1, 1, 64, 1, 1, 0, 7),         # a single step
+    (1, 100, 500, 2, 1, 64, 300),   # few items: as many parts as the list has steps
+    (1, 128, 577, 3, 3, 5, 500),    # odd group: ten steps, the last of one key
+    (1, 129, 1999, 4, 4, 64, 700),  # a second tile of one row
+    (3, 500, 500, 3, 3, 4, 100),    # causal lists from nothing up: tiles with fewer steps than parts
+    (2, 700, 1400, 8, 8, 64, 300),  # 96 items: four streams, or one block each
+    (2, 640, 2500, 10, 5, 100, 900),  # 100 items of long lists: clusters of two at D = 128
+])
+def test_forms_match_the_oracle(D, B, Nq, Nk, Hq, Hkv, sink, local):
+    q = cowa_inputs.make_train_inputs(301, B, Nq, Hq, Hkv, D)[0]
+    _, k, v, _ = cowa_inputs.make_train_inputs(302, B, Nk, Hq, Hkv, D)
+    scale = cowa_inputs.softmax_scale(D)
+    params = cowa.make_params(sink=sink, local=local, softmax_scale=scale)
+    o = torch.full_like(q, float("nan")).to(DEV)
+    lse = torch.full((B, Hq, Nq), float("nan"), dtype=torch.float32, device=DEV)
+    cowa.cowa_prefill(q.to(DEV), k.to(DEV), v.to(DEV), o, lse, params)
+    # the same as a packed batch of equal sequences: bit for bit
+    pack = lambda x: x.permute(1, 0, 2, 3).reshape(x.shape[1], -1, x.shape[3]).contiguous()  # noqa: E731
+    o2 = torch.full_like(pack(o), float("nan"))
+    lse2 = torch.full((Hq, B * Nq), float("nan"), dtype=torch.float32, device=DEV)
+    cu = [torch.from_numpy((np.arange(B + 1) * n).astype(np.int32)).to(DEV) for n in (Nq, Nk)]
+    cowa.cowa_prefill_varlen(pack(q).to(DEV), pack(k).to(DEV), pack(v).to(DEV), o2, lse2, *cu, params)
+    torch.cuda.synchronize()
+    cowa.cowa_check_device_status()
+    assert torch.equal(pack(o), o2)
+    assert torch.equal(lse.permute(1, 0, 2).reshape(Hq, -1), lse2)
+    ws = orc.default_windows(Nk, Hkv, sink, local)
+    f = cowa_inputs.to_f64
+    for b in range(B):
+        o_ref, lse_ref = orc.forward(f(q[b]), f(k[b]), f(v[b]), ws, scale)
+        check(f"lse[b={b}]", lse[b].cpu().numpy(), lse_ref, TOL_LSE, TOL_LSE)
+        check(f"o[b={b}]", o[b].float().cpu().numpy(), o_ref)
