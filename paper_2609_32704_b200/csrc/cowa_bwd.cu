@@ -71,6 +71,8 @@ struct BwdArgs {
   // The KV tiles in launch order: sink tiles, body, tail.  A tile of class c is shared by cls_parts[c] blocks, each with
   // a contiguous part of the tile's steps (QO heads x QO tiles); a shared tile's blocks leave fp32 partial dK, dV.
   int cls_tiles[3], cls_parts[3];
+  // Instead, where `share` is set: a tile has a block for every `share` QO tiles that see it (ShareOut)
+  int share;
   int dq_fixed;        // 1: dQ partial sums travel as 32-bit fixed point (order-independent addition)
   float* dkv_part;     // fp32 partial dK, dV [blocks of shared tiles, 2, BKV, D], summed by a kernel of their own
   // packed (variable-length) batches only: tensors are [H, total, D], sequence b owns rows cu[b] .. cu[b+1]
@@ -99,11 +101,6 @@ __device__ __forceinline__ void bulk_load_1d(void* dst, const void* src, uint32_
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                    smem_u32(dst)),
                "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
-
-__device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes)
                : "memory");
 }
 
@@ -149,7 +146,43 @@ __device__ __forceinline__ bool locate_tile(const BwdArgs& a, int c, int q, Tile
   return true;
 }
 
-// named barrier for one 128-thread warpgroup
+// Batched calls of few tiles, shared out by `share`: the blocks of one batch element are numbered tile after tile, KV tiles
+// ascending, heads within them, batch elements within the numbers.  Warp-cooperative.
+struct ShareOut {
+  __device__ __forceinline__ static int parts_of(const BwdArgs& a, int e) {  // of tile e = KV tile * Hkv + KV head
+    const int k0 = e / a.Hkv * BKV;
+    CowaRange rg[2];
+    cowa_bwd_ranges(a.wins.w[e % a.Hkv], k0, min(k0 + BKV, a.Nk) - 1, a.Nk - a.Nq, a.Nq, BQS, rg);
+    return max(((cowa_range_len(rg[0]) + cowa_range_len(rg[1])) * a.G + a.share - 1) / a.share, 1);
+  }
+  // The tile that holds number i (by_tile: tile i), its first number and parts.
+  __device__ __forceinline__ static void find(const BwdArgs& a, int i, bool by_tile, int* tile, int* first, int* parts) {
+    const int lane = threadIdx.x & 31, n = (a.Nk + BKV - 1) / BKV * a.Hkv;
+    int base = 0;
+    for (int e0 = 0; e0 < n; e0 += 32) {
+      const int e = e0 + lane, p = e < n ? parts_of(a, e) : 0;
+      int incl = p;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const unsigned m = __ballot_sync(0xFFFFFFFFu, by_tile ? i <= e : i < base + incl);
+      if (m) {
+        const int src = __ffs(m) - 1;
+        *tile = e0 + src;
+        *parts = __shfl_sync(0xFFFFFFFFu, p, src);
+        *first = base + __shfl_sync(0xFFFFFFFFu, incl - p, src);
+        return;
+      }
+      base += __shfl_sync(0xFFFFFFFFu, incl, 31);
+    }
+  }
+};
+
+// named barriers: one 128-thread warpgroup; all of the block, where the TMA warp does not wait
+__device__ __forceinline__ void all_arrive() { asm volatile("bar.arrive 3, 512;" ::: "memory"); }
+__device__ __forceinline__ void all_sync() { asm volatile("bar.sync 3, 512;" ::: "memory"); }
 __device__ __forceinline__ void wg_sync(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
 
 template <int D, bool VARLEN>
@@ -170,7 +203,6 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   constexpr uint32_t ID_ACC = idesc_bf16(128, D, 0, 1);    // dV, dK (B = dO / Q, MN-major)
   constexpr uint32_t ID_DQ = idesc_bf16(128, BQT, 1, 1);   // dQ^T (A = K^T, B = dS^T, both MN-major)
 
-  grid_enter();
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* sK = smem + SM::oK;
   uint8_t* sV = smem + SM::oV;
@@ -203,17 +235,45 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform by construction (helps the compiler)
 
-  // ---- work item ----
-  int cls = 0, idx = blockIdx.x, slot = 0;
-  while (cls < 2 && idx >= a.cls_tiles[cls] * a.cls_parts[cls]) {
-    idx -= a.cls_tiles[cls] * a.cls_parts[cls];
-    if (a.cls_parts[cls] > 1) slot += a.cls_tiles[cls] * a.cls_parts[cls];
-    ++cls;
+  // What needs nothing of the kernel before this one is done ahead of the wait for it (not the TMEM allocation, see
+  // cowa_fwd_kernel); the first loads do not wait for TMEM.
+  if (tid == 0) {
+    mbar_init(bar_k, 1); mbar_init(bar_v, 1);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(bar_q_full + s, 1); mbar_init(bar_q_empty + s, 1);
+      mbar_init(bar_dq_free + s, 128);
+    }
+    mbar_init(bar_dq_full, 1); mbar_init(bar_o_full, 1); mbar_init(bar_o_empty, 1);
+    mbar_init(bar_s_full, 1); mbar_init(bar_s_read, 256); mbar_init(bar_p_ready, 256);
+    mbar_init(bar_dp_full, 1); mbar_init(bar_ds_ready, 256);
+    mbar_init(bar_done, 1);
+    fence_mbar_init();
   }
-  const int parts = a.cls_parts[cls], part = idx % parts;
-  slot += idx;  // of this block's partial dK, dV when the tile is shared
+  if (tid == 32) { prefetch_tmap(&tmQ2); prefetch_tmap(&tmdO2); prefetch_tmap(&tmK); prefetch_tmap(&tmV); }
+  __syncthreads();
+  if (VARLEN) grid_enter();
+
+  // ---- work item ----
+  int parts, part, slot = blockIdx.x;  // slot: of this block's partial dK, dV when the tile is shared
   TileAt at;
-  if (!locate_tile<VARLEN>(a, cls, idx / parts, at)) return;
+  if (!VARLEN && a.share > 0) {
+    int e = 0, first = 0;
+    parts = 1;
+    ShareOut::find(a, blockIdx.x / a.B, false, &e, &first, &parts);
+    part = blockIdx.x / a.B - first;
+    at.b = blockIdx.x % a.B; at.hk = e % a.Hkv; at.j = e / a.Hkv; at.pbase = 0;
+  } else {
+    int cls = 0, idx = blockIdx.x;
+    slot = 0;
+    while (cls < 2 && idx >= a.cls_tiles[cls] * a.cls_parts[cls]) {
+      idx -= a.cls_tiles[cls] * a.cls_parts[cls];
+      if (a.cls_parts[cls] > 1) slot += a.cls_tiles[cls] * a.cls_parts[cls];
+      ++cls;
+    }
+    parts = a.cls_parts[cls]; part = idx % parts;
+    slot += idx;
+    if (!locate_tile<VARLEN>(a, cls, idx / parts, at)) return;
+  }
   const int hk = at.hk, b = at.b, j = at.j, pbase = at.pbase;
   // Sequence geometry.  Packed batches: N_q = N_k = the sequence's length, rows start at cu[b]; the fp32
   // dQ accumulator and the LSE / Delta vectors are laid out with every sequence padded to 64 rows (pbase).
@@ -247,25 +307,20 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   if (tid == 0) {
     geo[0] = w.s; geo[1] = w.n; geo[2] = w.g; geo[3] = w.l; geo[4] = off; geo[5] = Nq; geo[6] = Nk; geo[7] = steps;
     *part_out = parts > 1 ? a.dkv_part + (size_t)slot * 2 * (BKV * D) : nullptr;
-    mbar_init(bar_k, 1); mbar_init(bar_v, 1);
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(bar_q_full + s, 1); mbar_init(bar_q_empty + s, 1);
-      mbar_init(bar_dq_free + s, 128);
-    }
-    mbar_init(bar_dq_full, 1); mbar_init(bar_o_full, 1); mbar_init(bar_o_empty, 1);
-    mbar_init(bar_s_full, 1); mbar_init(bar_s_read, 256); mbar_init(bar_p_ready, 256);
-    mbar_init(bar_dp_full, 1); mbar_init(bar_ds_ready, 256);
-    mbar_init(bar_done, 1);
-    fence_mbar_init();
   }
+  if (!VARLEN) grid_enter();
   if (warp == 0) {
     __syncwarp();
-    tmem_alloc(tmem_holder, TMEM_COLS);
-    tmem_relinquish();
+    all_arrive();
+  } else {
+    if (warp == 2) {
+      tmem_alloc(tmem_holder, TMEM_COLS);
+      tmem_relinquish();
+    }
+    tc_fence_before();
+    all_sync();
+    tc_fence_after();
   }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
   constexpr uint32_t tmem_base = 0;  // the allocation is all of TMEM
 
   bool ok = true;
@@ -278,14 +333,12 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
     if (N > 0) ok = (is_dk ? mbar_wait(bar_done, 0, a.status) : mbar_wait(bar_o_empty, (N - 1) & 1, a.status)) && ok;
     tc_fence_after();
-    uint8_t* sOut = is_dk ? sQ : sDO;  // free by then, like V for partial sums
+    uint8_t* sOut = is_dk ? sQ : sDO;  // free by then
     const float mul = is_dk ? a.scale : 1.f;
     if (float* const dst = *part_out) {
-      // A shared tile: this block's part goes out in fp32, one slot per block; a kernel of its own adds the slots in order.
-      // Staged where Q, or V and dO were, rows with their 16-byte chunks permuted (bank conflicts), and
-      // copied as one range: straight from registers a warp's store touches 32 rows (1019 against 983 thousand clocks of
-      // the whole kernel for one KV head of 20001 tokens).
-      uint8_t* sPart = (is_dk ? sQ : r < BKV / 2 ? sV : sDO - SM::kQ) + r * (D * 4);
+      // A shared tile: this block's part goes out in fp32, one slot per block; a kernel of its own adds the slots in order.  A slot
+      // holds 16 bytes of every row after the other, so that a warp's store is one range of 512 bytes.
+      float4* const d4 = reinterpret_cast<float4*>(dst + (is_dk ? 0 : BKV * D)) + r;
 #pragma unroll
       for (int c = 0; c < D / 32; ++c) {
         uint32_t ov[32];
@@ -298,17 +351,8 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         }
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-          *reinterpret_cast<float4*>(sPart + (((c * 8 + q) ^ (r & 7)) << 4)) =
-              make_float4(__uint_as_float(ov[q * 4]) * mul, __uint_as_float(ov[q * 4 + 1]) * mul,
-                          __uint_as_float(ov[q * 4 + 2]) * mul, __uint_as_float(ov[q * 4 + 3]) * mul);
-      }
-      fence_proxy_async_smem();
-      wg_sync(is_dk ? 1 : 2);
-      if (r == 0) {
-        for (int half = 0; half < 2; ++half)
-          bulk_store(dst + (is_dk ? 0 : BKV * D) + half * (BKV * D / 2), is_dk ? sQ + half * SM::kQ : half ? sDO : sV, BKV * D * 2);
-        tma_commit_group();
-        tma_wait_group_read<0>();
+          d4[(c * 8 + q) * BKV] = make_float4(__uint_as_float(ov[q * 4]) * mul, __uint_as_float(ov[q * 4 + 1]) * mul,
+                                              __uint_as_float(ov[q * 4 + 2]) * mul, __uint_as_float(ov[q * 4 + 3]) * mul);
       }
       return;
     }
@@ -378,7 +422,6 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     if (warp == 0) {
       // ================= TMA producer =================
       if (lane == 0 && N > 0) {
-        prefetch_tmap(&tmQ); prefetch_tmap(&tmdO); prefetch_tmap(&tmK); prefetch_tmap(&tmV);
         auto load_kv = [&](uint8_t* tile, const CUtensorMap* tm, uint64_t* bar) {
           mbar_expect_tx(bar, SM::kKV);
           for (int s = 0; s < NSLAB; ++s) tma_load_4d(tile + s * SLAB_KV, tm, bar, s * 64, rbase + k0, hk, bt);
@@ -784,7 +827,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
+  if (warp == 2) {
     __syncwarp();
     tmem_dealloc(tmem_base, TMEM_COLS);
   }
@@ -933,19 +976,28 @@ template <int D, bool VARLEN>
 __global__ void __launch_bounds__(256)
 cowa_bwd_reduce_dkv_kernel(const __grid_constant__ BwdArgs a, CowaStrides sk, CowaStrides sv) {
   grid_enter();
-  constexpr int TPR = D / 8, ROWS = 256 / TPR;  // threads per row (16 bytes of bf16 each), rows per block
-  const int part = threadIdx.x % TPR;
-  int q = blockIdx.x / (BKV / ROWS), c = 0, slot = 0;
-  const int r = blockIdx.x % (BKV / ROWS) * ROWS + threadIdx.x / TPR;
+  constexpr int BLOCKS = BKV * (D / 8) / 256;  // of a tile: a thread takes eight d of a row, a warp 32 rows (see the slots)
+  const int i_ = blockIdx.x % BLOCKS * 256 + threadIdx.x, r = i_ % BKV, part = i_ / BKV;
+  int q = blockIdx.x / BLOCKS, c = 0, slot = 0, parts, step = 1;  // the tile's slots: slot, slot + step, ...
+  TileAt at;
+  if (!VARLEN && a.share > 0) {
+    int e = 0, first = 0;
+    parts = 1;
+    ShareOut::find(a, q / a.B, true, &e, &first, &parts);
+    if (parts == 1) return;
+    at.b = q % a.B; at.hk = e % a.Hkv; at.j = e / a.Hkv;
+    slot = first * a.B + at.b; step = a.B;
+  } else {
   for (; c < 2; ++c) {
     if (a.cls_parts[c] == 1) continue;
     if (q < a.cls_tiles[c]) break;
     q -= a.cls_tiles[c];
     slot += a.cls_tiles[c] * a.cls_parts[c];
   }
-  const int parts = a.cls_parts[c];
-  TileAt at;
+  parts = a.cls_parts[c];
   if (!locate_tile<VARLEN>(a, c, q, at)) return;
+  slot += q * parts;
+  }
   int Nk = a.Nk, rbase = 0;
   if constexpr (VARLEN) {
     rbase = a.cu[at.b];
@@ -955,14 +1007,12 @@ cowa_bwd_reduce_dkv_kernel(const __grid_constant__ BwdArgs a, CowaStrides sk, Co
   const int t = at.j * BKV + r;
   if (t >= Nk) return;
   const int m = blockIdx.y;
-  // the slots hold a row's 16-byte chunks permuted
-  const float* src = a.dkv_part + ((size_t)(slot + q * parts) * 2 + m) * (BKV * D) + (size_t)r * D;
-  const int c0 = ((part * 2) ^ (r & 7)) * 4, c1 = ((part * 2 + 1) ^ (r & 7)) * 4;
+  const float* src = a.dkv_part + ((size_t)slot * 2 + m) * (BKV * D) + ((size_t)part * 2 * BKV + r) * 4;
   float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
 #pragma unroll 4
   for (int i = 0; i < parts; ++i) {
-    const float4 u = *reinterpret_cast<const float4*>(src + (size_t)i * 2 * (BKV * D) + c0);
-    const float4 v = *reinterpret_cast<const float4*>(src + (size_t)i * 2 * (BKV * D) + c1);
+    const float4 u = *reinterpret_cast<const float4*>(src + (size_t)i * step * 2 * (BKV * D));
+    const float4 v = *reinterpret_cast<const float4*>(src + (size_t)i * step * 2 * (BKV * D) + BKV * 4);
     x.x += u.x; x.y += u.y; x.z += u.z; x.w += u.w;
     y.x += v.x; y.y += v.y; y.z += v.z; y.w += v.w;
   }
@@ -985,6 +1035,8 @@ struct BwdPlan {
   int sink_tiles;  // per sequence and head
   int tiles[3], parts[3];  // parts: what the workspace has room for
   int run[3];              // what the blocks take
+  int share = 0;           // ... or, batched calls of few tiles: QO tiles a block
+  long long shared_blocks = 0;
   long long slots() const {
     long long n = 0;
     for (int c = 0; c < 3; ++c)
@@ -992,6 +1044,7 @@ struct BwdPlan {
     return n;
   }
   long long blocks() const {
+    if (share > 0) return shared_blocks;
     long long n = 0;
     for (int c = 0; c < 3; ++c) n += (long long)tiles[c] * run[c];
     return n;
@@ -1010,6 +1063,33 @@ struct BwdPlan {
       const long long n = (long long)tiles[0] * parts[0] + (long long)tiles[1] * p + (long long)tiles[2] * parts[2];
       const double t = (4 + steps / p) * (std::max((double)n / sms, 1.0) + 0.5) + (p > 1 ? 0.02 * tiles[1] * p : 0);
       if (p == 1 || t < best) { best = t; run[1] = p; }
+    }
+  }
+
+  // Few tiles: their blocks by length.  With the same number of parts for every tile the blocks of a causal batch have one to
+  // fourteen steps, and the last SM ends at twice the average (821 tokens x 4, 16 heads: SMs end after 23 to 60 us).
+  // The smallest share with which the blocks make k rounds, for the k that ends first: a block costs about as much as ten QO
+  // tiles besides its own.  cnt: QO tiles of each KV tile of one batch element.
+  void share_out(const int* cnt, int n, int B, long long total, int longest) {
+    const int sms = cowa::sm_count();
+    const long long room = slots();
+    long long best = 0;
+    for (int k = 1; k <= 3; ++k) {
+      const long long most = std::min<long long>((long long)k * sms, room);
+      auto blocks_with = [&](int x) {
+        long long b = 0;
+        for (int i = 0; i < n; ++i) b += std::max((cnt[i] + x - 1) / x, 1);
+        return b * B;
+      };
+      int lo = (int)std::max<long long>((total + most - 1) / std::max<long long>(most, 1), 4), hi = std::max(longest, lo);
+      if (blocks_with(hi) > most) continue;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (blocks_with(mid) <= most) hi = mid;
+        else lo = mid + 1;
+      }
+      const long long t = (long long)k * (10 + hi);
+      if (share == 0 || t < best) { best = t; share = hi; shared_blocks = blocks_with(hi); }
     }
   }
 };
@@ -1034,6 +1114,9 @@ BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& h
   pl.sink_tiles = 0;
   for (int h = 0; h < Hkv; ++h) pl.sink_tiles = std::max(pl.sink_tiles, (std::min(hw.w[h].s, Nk) + BKV - 1) / BKV);
   long long total = 0, sinks = 0, longest = 0, longest_sink = 0;
+  constexpr int kFewTiles = 512;
+  int counts[kFewTiles];  // tile j of head h: [j * Hkv + h]
+  const bool few = (long long)nKV * Hkv * B <= std::min(2 * sms, kFewTiles);
   for (int h = 0; h < Hkv; ++h)
     for (int j = 0; j < nKV; ++j) {
       CowaRange rg[2];
@@ -1041,6 +1124,7 @@ BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& h
       cowa_bwd_ranges(hw.w[h], k0, k1, Nk - Nq, Nq, BQS, rg);
       const long long cnt = (long long)(cowa_range_len(rg[0]) + cowa_range_len(rg[1])) * G;
       total += cnt;
+      if (few) counts[j * Hkv + h] = (int)cnt;
       longest = std::max(longest, cnt);
       if (j < pl.sink_tiles) { sinks += cnt; longest_sink = std::max(longest_sink, cnt); }
     }
@@ -1059,6 +1143,7 @@ BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& h
   const long long budget = heads >= 4 ? room : std::max<long long>(room, 4ll * sms);
   while (pl.slots() > budget) --*std::max_element(pl.parts, pl.parts + 3);
   pl.choose_run(rest > 0 ? (double)(total - sinks) / rest * BQS / BQT : 0.0, reproducible);
+  if (few && !reproducible) pl.share_out(counts, nKV * Hkv, B, total, (int)longest);
   return pl;
 }
 
@@ -1103,7 +1188,8 @@ template <int D, bool VARLEN>
 cudaError_t launch_reduce(const BwdArgs& a, const BwdPlan& pl, const CowaStrides& sk, const CowaStrides& sv, cudaStream_t st) {
   long long shared = 0;
   for (int c = 0; c < 3; ++c)
-    if (pl.run[c] > 1) shared += pl.tiles[c];
+    if (pl.share > 0 || pl.run[c] > 1) shared += pl.tiles[c];
+  if (pl.share > 0 && pl.shared_blocks == shared) return cudaSuccess;  // a block per tile
   if (shared == 0) return cudaSuccess;
   return cowa::launch_chained(cowa_bwd_reduce_dkv_kernel<D, VARLEN>, dim3((unsigned)(shared * (BKV * (D / 8) / 256)), 2), 256, 0, st, a, sk, sv);
 }
@@ -1146,6 +1232,7 @@ int launch_bwd(const void* q, const void* k, const void* v, const void* o, const
   a.wins = hw;
   a.sink_tiles = pl.sink_tiles;
   for (int c = 0; c < 3; ++c) { a.cls_tiles[c] = pl.tiles[c]; a.cls_parts[c] = pl.run[c]; }
+  a.share = pl.share;
   a.dq_fixed = p->deterministic ? 1 : 0;
   a.dkv_part = dkv_part;
   a.cu = nullptr; a.dk = static_cast<__nv_bfloat16*>(dk); a.dv = static_cast<__nv_bfloat16*>(dv); a.total = 0; a.tiles_bound = 0;
@@ -1205,6 +1292,7 @@ int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o
   a.wins = hw;
   a.sink_tiles = pl.sink_tiles;
   for (int c = 0; c < 3; ++c) { a.cls_tiles[c] = pl.tiles[c]; a.cls_parts[c] = pl.run[c]; }
+  a.share = pl.share;
   a.dq_fixed = p->deterministic ? 1 : 0;
   a.dkv_part = delta + (size_t)Hq * Tpad;
   a.cu = cu; a.dk = static_cast<__nv_bfloat16*>(dk); a.dv = static_cast<__nv_bfloat16*>(dv);
