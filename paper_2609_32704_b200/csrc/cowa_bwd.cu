@@ -4,7 +4,7 @@
 //   1. preprocess   -Delta = -rowsum(O * dO) (Algorithm 2 line 13) and -LSE * log2(e), fp32 row vectors
 //                   padded to a multiple of 64 rows (padding: -inf, so that P = 0 there);
 //                   its threads also zero the fp32 dQ accumulator.
-//   2. main kernel  one thread block per (batch, KV head, 128-row KV tile), KV-stationary as in
+//   2. main kernel  a work item per (batch, KV head, 128-row KV tile), KV-stationary as in
 //                   Algorithm 2, looping over the G QO heads of the group and over the 64-row QO
 //                   tiles of I_h(j) (analytic scheduler, ascending).  A step takes two entries of that list, one
 //                   head's after the other's, not necessarily neighbours (with 128-row tiles instead up to a
@@ -30,15 +30,27 @@
 //                   until dQ^T is in registers.  Per step n the MMAs run in the order
 //                     dK(n-1) | dQ^T(n-1) | dP^T(n)   beside the exponentials of step n
 //                     dV(n)   | S^T(n+1)              beside dS^T(n)
-//                   Blocks are ordered sink tiles first (they meet every query tile), then
+//                   At D = 128 S^T(n+1) is issued 1000 clocks later than dV(n) allows, when the second half of dQ^T has
+//                   left its columns, behind the staging of the first (all 128 columns in registers at once: four copies
+//                   of the staging code, 9 to 30 % slower; rotated through one copy: spills).  At D = 64 dQ^T has columns of
+//                   its own, and the lanes that M = 128 leaves over hold it a second time, so that four warps
+//                   drain it instead of two: a step of 3420 clocks waited 500 for dP^T and 450 for S^T(n+1).  us: 35584
+//                   tokens, 32 heads 3433 -> 3190; 3840 x 4, 16 heads, reproducible 347 -> 296; 11120 x 2, 4 heads 252 -> 230.
+//                   Items are ordered sink tiles first (they meet every query tile), then
 //                   head by head with ascending KV tile, so that the blocks in flight sweep the same
 //                   dQ rows at nearly the same time and the reductions hit in L2.
+//                   A block takes over further items (cluster launch control): between two blocks on an SM 2.5 us
+//                   passed, and a block's first product came 1.4 us, its last store 5 us (D = 128) behind them; now Q and
+//                   V of the next item arrive while the last products of this one run, K once dQ^T has read this
+//                   one's, and its first S^T is computed while dK and dV leave through the buffers of dS^T and dO
+//                   (straight from registers, 16 bytes of 32 rows at a time, they hold up the drain).  us, forward and
+//                   backward: 2 x 8K 1004 -> 983, 20001 tokens 797 -> 766, 32K 7345 -> 7250, 24 documents 1564 -> 1546.
 //   3. convert      dQ accumulator (already scaled) -> bf16.
 // Two variations of the main kernel's work split:
-//   - shared tiles: a tile's steps are cut into contiguous parts for several blocks (few tiles, sink tiles that would
-//     be the critical path, the last wave); each block writes fp32 partial dK, dV to its own slot and a
+//   - shared tiles: a tile's steps are cut into contiguous parts, an item each (few tiles, sink tiles that would
+//     be the critical path, the last wave); each item writes fp32 partial dK, dV to its own slot and a
 //     fourth kernel adds the slots in order (BwdPlan).
-//   - VARLEN: packed batch [H, total, D]; a block finds (sequence, KV tile) by a warp scan of the offsets,
+//   - VARLEN: packed batch [H, total, D]; the TMA warp finds (sequence, KV tile) by a warp scan of the offsets,
 //     windows follow from the sequence's own length, the accumulator and the row vectors use a row space
 //     in which every sequence is padded to 64 rows, and a sequence's last, partial KV tile is stored row
 //     by row (cowa_bwd_varlen and its own preprocess / convert kernels).
@@ -73,12 +85,14 @@ struct BwdArgs {
   int cls_tiles[3], cls_parts[3];
   // Instead, where `share` is set: a tile has a block for every `share` QO tiles that see it (ShareOut)
   int share;
+  int single;          // the grid fits the device: a block has one item
   int dq_fixed;        // 1: dQ partial sums travel as 32-bit fixed point (order-independent addition)
   float* dkv_part;     // fp32 partial dK, dV [blocks of shared tiles, 2, BKV, D], summed by a kernel of their own
   // packed (variable-length) batches only: tensors are [H, total, D], sequence b owns rows cu[b] .. cu[b+1]
   const int* cu;       // [B+1] device
-  __nv_bfloat16* dk;   // raw outputs for the last, partial KV tile of a sequence
+  __nv_bfloat16* dk;   // raw outputs for a sequence's last, partial KV tile and for tiles that no query sees
   __nv_bfloat16* dv;
+  CowaStrides sdk, sdv;  // ... (packed batches: contiguous)
   int total, tiles_bound;  // rows of the packed tensors; grid tiles per KV head (upper bound of the real count)
   int sink, local, hkv_global, hkv_offset, full_attn, explicit_windows;
   float scale, scale_log2;
@@ -94,7 +108,9 @@ struct BwdSmem {
   static constexpr int oVec = oDS + 2 * kDS;   // per stage: 128 floats lse2, 128 floats delta
   static constexpr int oDQ = oVec + NST * 1024;  // dQ staging: per drain warp two tiles of 32 query rows x 32 d, fp32
   static constexpr int oBar = oDQ + 8 * 4096;
-  static constexpr int kBytes = oBar + 320;    // 231744 B at D = 128 (limit 232448)
+  static constexpr int oItem = oBar + 320;     // two work items
+  static constexpr int oNext = oItem + 192;    // the next item's number, as the hardware answers
+  static constexpr int kBytes = oNext + 16;    // 231952 B at D = 128 (limit 232448)
 };
 
 __device__ __forceinline__ void bulk_load_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -185,6 +201,17 @@ __device__ __forceinline__ void all_arrive() { asm volatile("bar.arrive 3, 512;"
 __device__ __forceinline__ void all_sync() { asm volatile("bar.sync 3, 512;" ::: "memory"); }
 __device__ __forceinline__ void wg_sync(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
 
+// One work item: a KV tile, or a part of its steps, as the TMA warp publishes it for the other warps.
+struct BwdItem {
+  CowaWin w;
+  int off, Nq, Nk;
+  int steps;     // -1: no more items
+  int k0, hk, b, rbase;
+  float* part;   // where the partial dK, dV of a shared tile go, else nullptr
+};
+static_assert(sizeof(BwdItem) <= 96, "slot of a published item");
+constexpr int kItemReaders = 13;  // warps that read it: MMA 1, compute 8, drain 4
+
 template <int D, bool VARLEN>
 __global__ void __launch_bounds__(512, 1)
 cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -197,8 +224,10 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   constexpr int SLAB_KV = BKV * 128;  // bytes of one 64-wide slab of a 128-row tile
   constexpr int SLAB_Q = BQT * 128;   // ... of a Q or dO tile
   // TMEM columns
-  constexpr uint32_t cS = 0, cDP = 128, cDK = 256, cDV = 384, TMEM_COLS = 512;
-  constexpr uint32_t cDS = cDP + 64, cDQ = cS + 64;  // P^T over the first half of S^T, dS^T over the second of dP^T, dQ^T between
+  constexpr uint32_t cS = 0, cDP = 128, cDK = 256, cDV = cDK + D, TMEM_COLS = 512;
+  // P^T over the first half of S^T, dS^T over the second of dP^T, dQ^T between; at D = 64 there are columns left for it
+  constexpr bool OWN_DQ = D == 64;
+  constexpr uint32_t cDS = cDP + 64, cDQ = OWN_DQ ? 384 : cS + 64;
   constexpr uint32_t ID_ST = idesc_bf16(128, BQT, 0, 0);   // S^T, dP^T
   constexpr uint32_t ID_ACC = idesc_bf16(128, D, 0, 1);    // dV, dK (B = dO / Q, MN-major)
   constexpr uint32_t ID_DQ = idesc_bf16(128, BQT, 1, 1);   // dQ^T (A = K^T, B = dS^T, both MN-major)
@@ -226,94 +255,47 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   uint64_t* bar_dq_free = bars + 13;  // [2] count 128: ... has left the columns of dP^T, of S^T
   uint64_t* bar_done = bars + 15;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 16);
-  float** part_out = reinterpret_cast<float**>(bars + 17);  // this block's partial dK, dV (kept here, not in registers)
   // What the roles would otherwise each hold or compute (registers: nothing spills in the batched form)
   int2* step_info = reinterpret_cast<int2*>(bars + 18);        // [2] by stage: first queries of the step's tiles; bit 0: no pair is masked, bit 1: rows past the sequence's end
   longlong2* dq_at = reinterpret_cast<longlong2*>(bars + 20);  // [4] by step: first elements of its tiles' dQ rows, -1: no second tile
-  int* geo = reinterpret_cast<int*>(bars + 32);                // window, off, Nq, Nk, steps of this block
+  uint64_t* bar_i_full = bars + 29;   // [2] a work item has been published
+  uint64_t* bar_i_empty = bars + 31;  // [2] count kItemReaders: it has been read
+  uint64_t* bar_next = bars + 33;     // the next item's number is here
+  uint64_t* bar_dk_out = bars + 34;   // dK of an item has left the buffer of dS^T
+  uint64_t* bar_dv_out = bars + 35;   // dV ... of dO
+  auto item_at = [&](uint32_t ni) { return reinterpret_cast<BwdItem*>(smem + SM::oItem + (ni & 1) * 96); };
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform by construction (helps the compiler)
 
-  // What needs nothing of the kernel before this one is done ahead of the wait for it (not the TMEM allocation, see
-  // cowa_fwd_kernel); the first loads do not wait for TMEM.
   if (tid == 0) {
     mbar_init(bar_k, 1); mbar_init(bar_v, 1);
     for (int s = 0; s < 2; ++s) {
       mbar_init(bar_q_full + s, 1); mbar_init(bar_q_empty + s, 1);
       mbar_init(bar_dq_free + s, 128);
+      mbar_init(bar_i_full + s, 1); mbar_init(bar_i_empty + s, kItemReaders);
     }
     mbar_init(bar_dq_full, 1); mbar_init(bar_o_full, 1); mbar_init(bar_o_empty, 1);
     mbar_init(bar_s_full, 1); mbar_init(bar_s_read, 256); mbar_init(bar_p_ready, 256);
     mbar_init(bar_dp_full, 1); mbar_init(bar_ds_ready, 256);
-    mbar_init(bar_done, 1);
+    mbar_init(bar_done, 1); mbar_init(bar_next, 1); mbar_init(bar_dk_out, 1); mbar_init(bar_dv_out, 1);
     fence_mbar_init();
   }
   if (tid == 32) { prefetch_tmap(&tmQ2); prefetch_tmap(&tmdO2); prefetch_tmap(&tmK); prefetch_tmap(&tmV); }
   __syncthreads();
-  if (VARLEN) grid_enter();
-
-  // ---- work item ----
-  int parts, part, slot = blockIdx.x;  // slot: of this block's partial dK, dV when the tile is shared
-  TileAt at;
-  if (!VARLEN && a.share > 0) {
-    int e = 0, first = 0;
-    parts = 1;
-    ShareOut::find(a, blockIdx.x / a.B, false, &e, &first, &parts);
-    part = blockIdx.x / a.B - first;
-    at.b = blockIdx.x % a.B; at.hk = e % a.Hkv; at.j = e / a.Hkv; at.pbase = 0;
-  } else {
-    int cls = 0, idx = blockIdx.x;
-    slot = 0;
-    while (cls < 2 && idx >= a.cls_tiles[cls] * a.cls_parts[cls]) {
-      idx -= a.cls_tiles[cls] * a.cls_parts[cls];
-      if (a.cls_parts[cls] > 1) slot += a.cls_tiles[cls] * a.cls_parts[cls];
-      ++cls;
-    }
-    parts = a.cls_parts[cls]; part = idx % parts;
-    slot += idx;
-    if (!locate_tile<VARLEN>(a, cls, idx / parts, at)) return;
-  }
-  const int hk = at.hk, b = at.b, j = at.j, pbase = at.pbase;
-  // Sequence geometry.  Packed batches: N_q = N_k = the sequence's length, rows start at cu[b]; the fp32
-  // dQ accumulator and the LSE / Delta vectors are laid out with every sequence padded to 64 rows (pbase).
-  int Nq = a.Nq, Nk = a.Nk, rbase = 0;
-  CowaWin w = a.wins.w[hk];
-  if constexpr (VARLEN) {
-    rbase = a.cu[b];
-    Nq = Nk = a.cu[b + 1] - rbase;
-    if (rbase < 0 || rbase + Nk > a.total) {  // malformed offsets: report, touch nothing
-      if (threadIdx.x == 0) atomicOr(a.status, (unsigned)COWA_DEV_BAD_SEQLENS);
-      return;
-    }
-    if (a.full_attn) { w.s = 0; w.n = Nk; w.g = 0; w.l = 0; }
-    else if (!a.explicit_windows) w = cowa_default_window(Nk, a.hkv_global, a.hkv_offset + hk, a.sink, a.local);
-  }
-  const int off = Nk - Nq;
-  const int k0 = j * BKV, k1 = min(k0 + BKV, Nk) - 1;
-  CowaRange rg[2];
-  cowa_bwd_ranges(w, k0, k1, off, Nq, BQS, rg);
-  const int cnt = cowa_range_len(rg[0]) + cowa_range_len(rg[1]);  // QO tiles per head
-  const int n0 = cnt * a.G * part / parts;               // (the host checks that these products fit)
-  const int tiles = cnt * a.G * (part + 1) / parts - n0; // this block's QO tiles
-  const int steps = (tiles + 1) >> 1;
-  const int g0 = cnt > 0 ? n0 / cnt : 0, tq0 = n0 - g0 * cnt;  // head of the group and position in I_h(j) of the first
-  const int bt = VARLEN ? 0 : b;                               // batch coordinate of the tensor maps
-  const int hq0 = hk * a.G;                                    // first QO head of the group
-  const int bhq0 = (VARLEN ? 0 : b * a.Hq) + hq0;              // ... as a row of lse2 / delta / dq_acc
-  const size_t vec_stride = (size_t)a.Tpad;                                         // rows per head in lse2 / delta / dq_acc
-  const bool tail_kv = VARLEN && (k0 + BKV > Nk);  // rows after the tile's last valid one belong to the next sequence
-
-  if (tid == 0) {
-    geo[0] = w.s; geo[1] = w.n; geo[2] = w.g; geo[3] = w.l; geo[4] = off; geo[5] = Nq; geo[6] = Nk; geo[7] = steps;
-    *part_out = parts > 1 ? a.dkv_part + (size_t)slot * 2 * (BKV * D) : nullptr;
-  }
-  if (!VARLEN) grid_enter();
+  // What needs nothing of the kernel before this one is done ahead of the wait for it: this, and the first item's geometry, which
+  // the TMA warp works out (not so the TMEM allocation, see cowa_fwd_kernel; the first loads do not wait for that).  A grid that is
+  // not started as a whole cannot let the next kernel in early.
+  auto enter = [&]() {
+    if (a.single) grid_enter();
+    else grid_wait();
+  };
   if (warp == 0) {
-    __syncwarp();
     all_arrive();
   } else {
-    if (warp == 2) {
+    enter();
+    if (warp == 1) {
+      __syncwarp();
       tmem_alloc(tmem_holder, TMEM_COLS);
       tmem_relinquish();
     }
@@ -324,154 +306,183 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   constexpr uint32_t tmem_base = 0;  // the allocation is all of TMEM
 
   bool ok = true;
-  auto step_count = [&]() { return static_cast<const volatile int*>(geo)[7]; };  // (each role reads it for itself)
-
-  // dK (first compute warpgroup) and dV (second, while the last dQ^T and dK are still being computed): TMEM -> bf16 ->
-  // shared -> TMA store.  With dV behind the last dQ^T in the drain warpgroup a block of nine steps took 2000 clocks longer.
-  auto store_grad = [&](bool is_dk) {
-    const int N = step_count(), r = (warp & 3) * 32 + lane;
-    const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-    if (N > 0) ok = (is_dk ? mbar_wait(bar_done, 0, a.status) : mbar_wait(bar_o_empty, (N - 1) & 1, a.status)) && ok;
-    tc_fence_after();
-    uint8_t* sOut = is_dk ? sQ : sDO;  // free by then
-    const float mul = is_dk ? a.scale : 1.f;
-    if (float* const dst = *part_out) {
-      // A shared tile: this block's part goes out in fp32, one slot per block; a kernel of its own adds the slots in order.  A slot
-      // holds 16 bytes of every row after the other, so that a warp's store is one range of 512 bytes.
-      float4* const d4 = reinterpret_cast<float4*>(dst + (is_dk ? 0 : BKV * D)) + r;
-#pragma unroll
-      for (int c = 0; c < D / 32; ++c) {
-        uint32_t ov[32];
-        if (N > 0 && ok) {
-          tmem_ld32(t_lane + (is_dk ? cDK : cDV) + c * 32, ov);
-          tmem_wait_ld();
-        } else {
-#pragma unroll
-          for (int e = 0; e < 32; ++e) ov[e] = 0u;
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          d4[(c * 8 + q) * BKV] = make_float4(__uint_as_float(ov[q * 4]) * mul, __uint_as_float(ov[q * 4 + 1]) * mul,
-                                              __uint_as_float(ov[q * 4 + 2]) * mul, __uint_as_float(ov[q * 4 + 3]) * mul);
-      }
-      return;
-    }
-    if (tail_kv) {
-      // last, partial KV tile of a packed sequence: row by row, straight from registers
-      __nv_bfloat16* dst = (is_dk ? a.dk : a.dv) + ((size_t)hk * a.total + rbase + k0 + r) * D;
-#pragma unroll
-      for (int c = 0; c < D / 32; ++c) {
-        uint32_t ov[32];
-        if (N > 0 && ok) {
-          tmem_ld32(t_lane + (is_dk ? cDK : cDV) + c * 32, ov);
-          tmem_wait_ld();
-        } else {
-#pragma unroll
-          for (int e = 0; e < 32; ++e) ov[e] = 0u;
-        }
-        if (k0 + r < Nk) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            uint4 v;
-            v.x = pack_bf16(__uint_as_float(ov[q * 8 + 0]) * mul, __uint_as_float(ov[q * 8 + 1]) * mul);
-            v.y = pack_bf16(__uint_as_float(ov[q * 8 + 2]) * mul, __uint_as_float(ov[q * 8 + 3]) * mul);
-            v.z = pack_bf16(__uint_as_float(ov[q * 8 + 4]) * mul, __uint_as_float(ov[q * 8 + 5]) * mul);
-            v.w = pack_bf16(__uint_as_float(ov[q * 8 + 6]) * mul, __uint_as_float(ov[q * 8 + 7]) * mul);
-            *reinterpret_cast<uint4*>(dst + c * 32 + q * 8) = v;
-          }
-        }
-      }
-      return;
-    }
-#pragma unroll
-    for (int c = 0; c < D / 32; ++c) {
-      uint32_t ov[32];
-      if (N > 0 && ok) {
-        tmem_ld32(t_lane + (is_dk ? cDK : cDV) + c * 32, ov);
-        tmem_wait_ld();
-      } else {
-#pragma unroll
-        for (int e = 0; e < 32; ++e) ov[e] = 0u;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        uint4 v;
-        v.x = pack_bf16(__uint_as_float(ov[q * 8 + 0]) * mul, __uint_as_float(ov[q * 8 + 1]) * mul);
-        v.y = pack_bf16(__uint_as_float(ov[q * 8 + 2]) * mul, __uint_as_float(ov[q * 8 + 3]) * mul);
-        v.z = pack_bf16(__uint_as_float(ov[q * 8 + 4]) * mul, __uint_as_float(ov[q * 8 + 5]) * mul);
-        v.w = pack_bf16(__uint_as_float(ov[q * 8 + 6]) * mul, __uint_as_float(ov[q * 8 + 7]) * mul);
-        const int d0 = c * 32 + q * 8;
-        const int slab = d0 / 64, chunk = (d0 % 64) / 8;
-        *reinterpret_cast<uint4*>(sOut + slab * SLAB_KV + r * 128 + ((chunk ^ (r & 7)) << 4)) = v;
-      }
-    }
-    fence_proxy_async_smem();
-    wg_sync(is_dk ? 1 : 2);
-    if (r == 0 && ok) {
-      for (int s = 0; s < NSLAB; ++s) tma_store_4d(is_dk ? &tmdK : &tmdV, sOut + s * SLAB_KV, s * 64, rbase + k0, hk, bt);
-      tma_commit_group();
-      tma_wait_group_read<0>();
-    }
+  // Item number ni of this block has been published (its words stay until item_done); its steps, -1 when there are no more items.
+  auto next_item = [&](uint32_t ni) -> int {
+    ok = mbar_wait(bar_i_full + (ni & 1), (ni >> 1) & 1, a.status);
+    return ok ? static_cast<const volatile int*>(&item_at(ni)->steps)[0] : -1;
+  };
+  auto item_done = [&](uint32_t ni) {
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar_i_empty + (ni & 1));
   };
 
   // Register budget per role: 128 per thread at launch (512 threads), 80 + 2 * 152 + 128 = 4 * 128 moved to where the work
   // is.  Each setmaxnreg sits at the top of its own branch so that the code below it is compiled for that budget.
   if (warp < 4) {
     setmaxnreg_dec<80>();
-    const int N = step_count();
     if (warp == 0) {
-      // ================= TMA producer =================
-      if (lane == 0 && N > 0) {
-        auto load_kv = [&](uint8_t* tile, const CUtensorMap* tm, uint64_t* bar) {
-          mbar_expect_tx(bar, SM::kKV);
-          for (int s = 0; s < NSLAB; ++s) tma_load_4d(tile + s * SLAB_KV, tm, bar, s * 64, rbase + k0, hk, bt);
-        };
-        load_kv(sK, &tmK, bar_k);  // S^T(0) waits for K and Q only
-        int g = g0, t_in = tq0;   // head of the group, position in I_h(j): kept incrementally
-        for (int n = 0; n < N && ok; ++n) {
-          const int st = n & 1;
-          const uint32_t ph_e = ((n >> 1) & 1) ^ 1;  // parity of the "stage empty" waits (the first two steps need none)
-          int q0[2], gh[2];
-          q0[0] = cowa_bwd_tile_at(rg, t_in) * BQS; gh[0] = g;
-          if (++t_in == cnt) { t_in = 0; ++g; }
-          const bool two = 2 * n + 1 < tiles;  // else the first tile again, every pair of it masked
-          q0[1] = two ? cowa_bwd_tile_at(rg, t_in) * BQS : q0[0]; gh[1] = two ? g : gh[0];
-          if (two && ++t_in == cnt) { t_in = 0; ++g; }
-          if (n >= 2) ok = mbar_wait(bar_q_empty + st, ph_e, a.status);
-          if (!ok) break;
-          auto info = [&](int x) {
-            return q0[x] + (cowa_tile_full(w, q0[x], BQS, k0, BKV, off, Nq, Nk) ? 1 : 0) + (q0[x] + BQS > Nq ? 2 : 0);
-          };
-          step_info[st] = make_int2(info(0), two ? info(1) : kNoTile);
-          auto rows = [&](int x) -> size_t { return (size_t)(bhq0 + gh[x]) * vec_stride + pbase + q0[x]; };  // in lse2, delta, dq_acc
-          dq_at[n & 3] = make_longlong2((long long)rows(0) * D, two ? (long long)rows(1) * D : -1ll);
-          // neighbours of one head, as nearly always, come in one piece
-          const int pieces = two && gh[1] == gh[0] && q0[1] == q0[0] + BQS ? 1 : 2;
-          auto load_rows = [&](uint8_t* tile, const CUtensorMap* tm, const CUtensorMap* tm2, uint64_t* bar) {
-            for (int x = 0; x < pieces; ++x)
-              for (int s = 0; s < NSLAB; ++s)
-                tma_load_4d(tile + s * SLAB_Q + x * (SLAB_Q / 2), pieces == 1 ? tm2 : tm, bar, s * 64, rbase + q0[x], hq0 + gh[x], bt);
-          };
-          mbar_expect_tx(bar_q_full + st, SM::kQ + 2 * BQT * 4);
-          load_rows(sQ + st * SM::kQ, &tmQ, &tmQ2, bar_q_full + st);
-          for (int x = 0; x < pieces; ++x) {
-            bulk_load_1d(sVec + st * 256 + x * BQS, a.lse2 + rows(x), BQT * 4 / pieces, bar_q_full + st);
-            bulk_load_1d(sVec + st * 256 + 128 + x * BQS, a.delta + rows(x), BQT * 4 / pieces, bar_q_full + st);
-          }
-          if (n == 0) load_kv(sV, &tmV, bar_v);
-          else ok = mbar_wait(bar_o_empty, (n - 1) & 1, a.status);
-          if (!ok) break;
-          mbar_expect_tx(bar_o_full, SM::kQ);
-          load_rows(sDO, &tmdO, &tmdO2, bar_o_full);
+      // ================= TMA producer; works out the items one ahead =================
+      const bool lead = elect_one();
+      int c = 0;        // steps so far, all items together
+      uint32_t ni = 0, kc = 0;  // items so far, those with steps
+      uint32_t asked = 0, answered = 0;
+      auto ask = [&]() {
+        if (lead) {
+          mbar_expect_tx(bar_next, 16);
+          clc_request(smem + SM::oNext, bar_next);
         }
+        ++asked;
+      };
+      int idx = blockIdx.x;
+      if (VARLEN) enter();
+      while (ok) {
+        // ---- work item ----
+        int parts = 1, part = 0, slot = idx;  // slot: of this item's partial dK, dV when the tile is shared
+        TileAt at;
+        bool found = idx >= 0;
+        if (!found) {
+        } else if (!VARLEN && a.share > 0) {
+          int e = 0, first = 0;
+          ShareOut::find(a, idx / a.B, false, &e, &first, &parts);
+          part = idx / a.B - first;
+          at.b = idx % a.B; at.hk = e % a.Hkv; at.j = e / a.Hkv; at.pbase = 0;
+        } else {
+          int cls = 0, q = idx;
+          slot = 0;
+          while (cls < 2 && q >= a.cls_tiles[cls] * a.cls_parts[cls]) {
+            q -= a.cls_tiles[cls] * a.cls_parts[cls];
+            if (a.cls_parts[cls] > 1) slot += a.cls_tiles[cls] * a.cls_parts[cls];
+            ++cls;
+          }
+          parts = a.cls_parts[cls]; part = q % parts;
+          slot += q;
+          found = locate_tile<VARLEN>(a, cls, q / parts, at);
+        }
+        // Sequence geometry.  Packed batches: N_q = N_k = the sequence's length, rows start at cu[b]; the fp32
+        // dQ accumulator and the LSE / Delta vectors are laid out with every sequence padded to 64 rows (pbase).
+        int Nq = a.Nq, Nk = a.Nk, rbase = 0;
+        CowaWin w = a.wins.w[found ? at.hk : 0];
+        if (VARLEN && found) {
+          rbase = a.cu[at.b];
+          Nq = Nk = a.cu[at.b + 1] - rbase;
+          if (rbase < 0 || rbase + Nk > a.total) {  // malformed offsets: report, touch nothing
+            if (lead) atomicOr(a.status, (unsigned)COWA_DEV_BAD_SEQLENS);
+            found = false;
+          }
+          if (a.full_attn) { w.s = 0; w.n = Nk; w.g = 0; w.l = 0; }
+          else if (!a.explicit_windows) w = cowa_default_window(Nk, a.hkv_global, a.hkv_offset + at.hk, a.sink, a.local);
+        }
+        if (!found && idx >= 0) {  // (packed batches: the count of items is an upper bound)
+          if (!a.single) ask();
+        } else {
+          const int hk = at.hk, b = at.b, off = Nk - Nq, k0 = at.j * BKV, k1 = min(k0 + BKV, Nk) - 1;
+          CowaRange rg[2];
+          int cnt = 0, tiles = 0, g = 0, t_in = 0;
+          if (found) {
+            cowa_bwd_ranges(w, k0, k1, off, Nq, BQS, rg);
+            cnt = cowa_range_len(rg[0]) + cowa_range_len(rg[1]);       // QO tiles per head
+            const int n0 = cnt * a.G * part / parts;                   // (the host checks that these products fit)
+            tiles = cnt * a.G * (part + 1) / parts - n0;               // this item's QO tiles
+            g = cnt > 0 ? n0 / cnt : 0; t_in = n0 - g * cnt;           // head of the group and position in I_h(j): kept incrementally
+          }
+          const int N = found ? (tiles + 1) >> 1 : -1;
+          if (!VARLEN && ni == 0) enter();
+          if (ni >= 2) ok = mbar_wait(bar_i_empty + (ni & 1), ((ni >> 1) & 1) ^ 1, a.status);
+          if (!ok) break;
+          if (lead) {
+            BwdItem& it = *item_at(ni);
+            it.w = w; it.off = off; it.Nq = Nq; it.Nk = Nk; it.steps = N; it.k0 = k0; it.hk = hk; it.b = b; it.rbase = rbase;
+            it.part = parts > 1 ? a.dkv_part + (size_t)slot * 2 * (BKV * D) : nullptr;
+            mbar_arrive(bar_i_full + (ni & 1));
+          }
+          __syncwarp();
+          ++ni;
+          if (N < 0) break;
+          const int bt = VARLEN ? 0 : b;                   // batch coordinate of the tensor maps
+          const int hq0 = hk * a.G;                        // first QO head of the group
+          const int bhq0 = (VARLEN ? 0 : b * a.Hq) + hq0;  // ... as a row of lse2 / delta / dq_acc
+          auto load_kv = [&](uint8_t* tile, const CUtensorMap* tm, uint64_t* bar) {
+            if (!lead) return;
+            mbar_expect_tx(bar, SM::kKV);
+            for (int s = 0; s < NSLAB; ++s) tma_load_4d(tile + s * SLAB_KV, tm, bar, s * 64, rbase + k0, hk, bt);
+          };
+          if (c == 0 && N > 0) load_kv(sK, &tmK, bar_k);  // S^T of the first step waits for K and Q only
+          const int ask_at = a.single ? -1 : max(N - 3, 0);  // a microsecond or more before the answer is needed
+          if (N == 0 && !a.single) ask();
+          for (int n = 0; n < N; ++n, ++c) {
+            const int st = c & 1;
+            if (n == ask_at) ask();
+            int q0[2], gh[2];
+            q0[0] = cowa_bwd_tile_at(rg, t_in) * BQS; gh[0] = g;
+            if (++t_in == cnt) { t_in = 0; ++g; }
+            const bool two = 2 * n + 1 < tiles;  // else the first tile again, every pair of it masked
+            q0[1] = two ? cowa_bwd_tile_at(rg, t_in) * BQS : q0[0]; gh[1] = two ? g : gh[0];
+            if (two && ++t_in == cnt) { t_in = 0; ++g; }
+            // neighbours of one head, as nearly always, come in one piece
+            const int pieces = two && gh[1] == gh[0] && q0[1] == q0[0] + BQS ? 1 : 2;
+            auto load_rows = [&](uint8_t* tile, const CUtensorMap* tm, const CUtensorMap* tm2, uint64_t* bar) {
+              for (int x = 0; x < pieces; ++x)
+                for (int s = 0; s < NSLAB; ++s)
+                  tma_load_4d(tile + s * SLAB_Q + x * (SLAB_Q / 2), pieces == 1 ? tm2 : tm, bar, s * 64, rbase + q0[x], hq0 + gh[x], bt);
+            };
+            if (c >= 2) ok = mbar_wait(bar_q_empty + st, ((c >> 1) & 1) ^ 1, a.status);
+            if (!ok) break;
+            if (lead) {
+              auto info = [&](int x) {
+                return q0[x] + (cowa_tile_full(w, q0[x], BQS, k0, BKV, off, Nq, Nk) ? 1 : 0) + (q0[x] + BQS > Nq ? 2 : 0);
+              };
+              step_info[st] = make_int2(info(0), two ? info(1) : kNoTile);
+              auto rows = [&](int x) -> size_t { return (size_t)(bhq0 + gh[x]) * a.Tpad + at.pbase + q0[x]; };  // in lse2, delta, dq_acc
+              dq_at[c & 3] = make_longlong2((long long)rows(0) * D, two ? (long long)rows(1) * D : -1ll);
+              mbar_expect_tx(bar_q_full + st, SM::kQ + 2 * BQT * 4);
+              load_rows(sQ + st * SM::kQ, &tmQ, &tmQ2, bar_q_full + st);
+              for (int x = 0; x < pieces; ++x) {
+                bulk_load_1d(sVec + st * 256 + x * BQS, a.lse2 + rows(x), BQT * 4 / pieces, bar_q_full + st);
+                bulk_load_1d(sVec + st * 256 + 128 + x * BQS, a.delta + rows(x), BQT * 4 / pieces, bar_q_full + st);
+              }
+            }
+            if (n == 0) {  // V over that of the item before once its last dP^T has been computed, K once dQ^T has
+              if (c > 0) ok = mbar_wait(bar_dp_full, (c - 1) & 1, a.status);
+              if (!ok) break;
+              load_kv(sV, &tmV, bar_v);
+            }
+            // (dV of the item before has left the buffer of dO: behind dO's last product)
+            if (n == 0 && c > 0) ok = mbar_wait(bar_dv_out, (kc - 1) & 1, a.status);
+            else if (c > 0) ok = mbar_wait(bar_o_empty, (c - 1) & 1, a.status);
+            if (!ok) break;
+            if (lead) {
+              mbar_expect_tx(bar_o_full, SM::kQ);
+              load_rows(sDO, &tmdO, &tmdO2, bar_o_full);
+            }
+            if (n == 0 && c > 0) {
+              ok = mbar_wait(bar_dq_full, (c - 1) & 1, a.status);
+              if (!ok) break;
+              load_kv(sK, &tmK, bar_k);
+            }
+            __syncwarp();
+          }
+          if (!ok) break;
+          if (N > 0) ++kc;
+        }
+        if (a.single) {
+          idx = -1;
+          continue;
+        }
+        answered = asked;
+        ok = mbar_wait(bar_next, (asked - 1) & 1, a.status);
+        if (!ok) break;
+        idx = __shfl_sync(0xFFFFFFFFu, clc_block(smem + SM::oNext), 0);
+        fence_proxy_async_smem();  // read before the next answer is written
+        __syncwarp();
       }
+      if (asked != answered) mbar_wait(bar_next, (asked - 1) & 1, a.status);  // (a wait ran out) no answer may come later
     } else if (warp == 1) {
       // ================= MMA issuer =================
       // The whole warp runs this loop (uniform control flow, so that descriptors and counters stay in
       // uniform registers); only the elected lane executes the tcgen05 instructions.  Everything that
       // can be computed once is: descriptor of every operand base, stage and parity bookkeeping is
       // incremental.
-      if (N > 0) {
+      {
         const bool lead = elect_one();
         const uint32_t tb = tmem_base;
         // Descriptors: a byte offset o inside a tile is added as o >> 4 to the address field (bits 0-13);
@@ -512,6 +523,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           if (lead) mma_commit(bar);
         };
 
+        const BwdItem* item = nullptr;
         // Packed batches: rows of a tile that lie past the end of the sequence belong to the next one.  Every
         // product they enter is multiplied by an exact zero, but 0 x (Inf or NaN) would still poison this
         // sequence, so they are cleared in shared memory (whole 128-byte rows, by this warp) before use.
@@ -525,7 +537,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           if constexpr (VARLEN) {
             const int2 q0_ = step_info[stage];
             if (!((q0_.x | q0_.y) & 2)) return;
-            const int nq = static_cast<const volatile int*>(geo)[5];
+            const int nq = static_cast<const volatile int*>(&item->Nq)[0];
 #pragma unroll 1
             for (int x = 0; x < 2; ++x) {
               const int q = x && q0_.y != kNoTile ? q0_.y : q0_.x;  // (without a second tile the first lies there again)
@@ -536,39 +548,39 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           }
         };
         auto clear_kv_tail = [&](uint8_t* tile) {
-          if (!tail_kv) return;
-          clear_rows(tile, Nk - k0, BKV, SLAB_KV);
-          fence_proxy_async_smem();
-          __syncwarp();
+          if constexpr (VARLEN) {
+            const int left = static_cast<const volatile int*>(&item->Nk)[0] - static_cast<const volatile int*>(&item->k0)[0];
+            if (left >= BKV) return;
+            clear_rows(tile, left, BKV, SLAB_KV);
+            fence_proxy_async_smem();
+            __syncwarp();
+          }
         };
-        ok = mbar_wait(bar_k, 0, a.status);
-        if (ok) clear_kv_tail(sK);
-        ok = ok && mbar_wait(bar_q_full, 0, a.status);
-        if (ok) {
-          clear_tail(sQ, 0);
-          tc_fence_after();
-          gemm_st(cS, dK_k, dQ_k0);
-          commit(bar_s_full);
-        }
-        auto body = [&](int n, int st) {
-          const uint32_t par = n & 1;
+        int c = 0;        // steps so far: stage, parities
+        uint32_t kc = 0;  // items with steps so far
+        // Step n of an item.  What it waits for of the step before it holds across items, too.
+        auto body = [&](int n, int N) {
+          const int st = c & 1;
+          const uint32_t par = c & 1;
           if (n > 0) {
             ok = mbar_wait(bar_ds_ready, par ^ 1, a.status);
             if (!ok) return;
             tc_fence_after();
             gemm_acc(cDK, cDS, dQ_mn0 + (st ^ 1) * kQ16, n > 1 ? 1u : 0u);
             commit(bar_q_empty + (st ^ 1));
-            ok = mbar_wait(bar_s_read, par, a.status);
+            // dQ^T's columns: S^T of this step is in registers; or those of its own, once the dQ^T before it has left them
+            if (!OWN_DQ) ok = mbar_wait(bar_s_read, par, a.status);
+            else if (c > 1) ok = mbar_wait(bar_dq_free, par, a.status);
             if (!ok) return;
             tc_fence_after();
             gemm_dq();
             commit(bar_dq_full);
           }
           ok = mbar_wait(bar_o_full, par, a.status);
-          if (ok && n > 0) ok = mbar_wait(bar_dq_free, par ^ 1, a.status);
+          if (!OWN_DQ && ok && c > 0) ok = mbar_wait(bar_dq_free, par ^ 1, a.status);
           if (!ok) return;
           if (n == 0) {
-            ok = mbar_wait(bar_v, 0, a.status);
+            ok = mbar_wait(bar_v, kc & 1, a.status);
             if (!ok) return;
             clear_kv_tail(sV);
           }
@@ -582,8 +594,8 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           gemm_acc(cDV, cS, dO_mn0, n > 0 ? 1u : 0u);
           commit(bar_o_empty);
           if (n + 1 < N) {
-            ok = mbar_wait(bar_q_full + (st ^ 1), ((n + 1) >> 1) & 1, a.status);
-            if (ok && n > 0) ok = mbar_wait(bar_dq_free + 1, par ^ 1, a.status);
+            ok = mbar_wait(bar_q_full + (st ^ 1), ((c + 1) >> 1) & 1, a.status);
+            if (!OWN_DQ && ok && c > 0) ok = mbar_wait(bar_dq_free + 1, par ^ 1, a.status);
             if (!ok) return;
             clear_tail(sQ + (st ^ 1) * SM::kQ, st ^ 1);
             tc_fence_after();
@@ -591,25 +603,42 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             commit(bar_s_full);
           }
         };
-#pragma unroll 1
-        for (int n = 0; n < N && ok; ++n) body(n, n & 1);
-        if (ok) {
-          ok = mbar_wait(bar_ds_ready, (N - 1) & 1, a.status);
-          if (ok && N > 1) ok = mbar_wait(bar_dq_free + 1, N & 1, a.status);
-          if (ok) {
+        for (uint32_t ni = 0; ok; ++ni) {
+          const int N = next_item(ni);
+          if (N < 0) break;
+          item = item_at(ni);
+          if (N > 0) {
+            ok = mbar_wait(bar_k, kc & 1, a.status);
+            if (!ok) break;
+            clear_kv_tail(sK);
+            ok = mbar_wait(bar_q_full + (c & 1), (c >> 1) & 1, a.status);
+            if (!OWN_DQ && ok && c > 0) ok = mbar_wait(bar_dq_free + 1, (c - 1) & 1, a.status);
+            if (!ok) break;
+            clear_tail(sQ + (c & 1) * SM::kQ, c & 1);
             tc_fence_after();
-            gemm_dq();
+            gemm_st(cS, dK_k, dQ_k0 + (c & 1) * kQ16);
+            commit(bar_s_full);
+#pragma unroll 1
+            for (int n = 0; n < N && ok; ++n, ++c) body(n, N);
+            if (!ok) break;
+            ok = mbar_wait(bar_ds_ready, (c - 1) & 1, a.status);
+            if (ok && c > 1) ok = mbar_wait(bar_dq_free + (OWN_DQ ? 0 : 1), c & 1, a.status);
+            if (!ok) break;
+            tc_fence_after();
+            gemm_dq();  // K may go now
             commit(bar_dq_full);
-            gemm_acc(cDK, cDS, dQ_mn0 + ((N - 1) & 1) * kQ16, N > 1 ? 1u : 0u);
+            gemm_acc(cDK, cDS, dQ_mn0 + ((c - 1) & 1) * kQ16, N > 1 ? 1u : 0u);
+            commit(bar_q_empty + ((c - 1) & 1));
+            commit(bar_done);
+            ++kc;
           }
+          item_done(ni);
         }
-        commit(bar_done);
       }
     }
   } else if (warp < 12) {
     setmaxnreg_inc<152>();
     {
-      const int N = step_count();
       // ======== two compute warpgroups: P^T and dS^T of two blocks of 32 queries each.  A warpgroup only writes into
       // columns that it has read: P^T (bf16 pairs) into its first block of S^T, dS^T into its second of dP^T.
       const int wg = (warp - 4) >> 2;  // queries [32 wg, 32 wg + 32) of both halves of every step
@@ -620,25 +649,30 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       const uint32_t ds_st = smem_u32(sDS) + ((warp & 3) * 32 + (lane & 15)) * 128;  // this lane's row for stmatrix
       const uint32_t ds_ch = wg * 4 + (lane >> 4);                                   // ... and 16-byte chunk
       const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
+      int c = 0;        // steps so far: stage, parities
+      uint32_t kc = 0;  // items with steps so far
+      for (uint32_t ni = 0; ok; ++ni) {
+      const int N = next_item(ni);
+      if (N < 0) break;
       // queries that see this lane's key: [near_lo, near_hi] and [far_lo, far_hi]
       int near_lo = 0, near_hi = -1, far_lo = 0, far_hi = -1;
       {
-        const volatile int* g_ = geo;
-        const int kcol = k0 + (warp & 3) * 32 + lane;
-        const long long kpos = (long long)kcol - g_[4], qend = g_[5] - 1, far = kpos + g_[1] + g_[2];
-        if (kcol < g_[6]) {
+        const volatile BwdItem* it = item_at(ni);
+        const int kcol = it->k0 + (warp & 3) * 32 + lane;
+        const long long kpos = (long long)kcol - it->off, qend = it->Nq - 1, far = kpos + it->w.n + it->w.g;
+        if (kcol < it->Nk) {
           near_lo = (int)max(min(kpos, qend + 1), 0ll);
-          near_hi = (int)max(kcol < g_[0] ? qend : min(kpos + g_[1] - 1, qend), -1ll);
+          near_hi = (int)max(kcol < it->w.s ? qend : min(kpos + it->w.n - 1, qend), -1ll);
           far_lo = (int)max(min(far, qend + 1), 0ll);
-          far_hi = (int)max(g_[3] > 0 ? min(far + g_[3] - 1, qend) : -1ll, -1ll);
+          far_hi = (int)max(it->w.l > 0 ? min(far + it->w.l - 1, qend) : -1ll, -1ll);
         }
       }
-      for (int n = 0; n < N && ok; ++n) {
-        const int st = n & 1;
-        const uint32_t par = n & 1;
+      for (int n = 0; n < N && ok; ++n, ++c) {
+        const int st = c & 1;
+        const uint32_t par = c & 1;
         const uint32_t sbuf = t_lane + cS + wg * 32, dpbuf = t_lane + cDP + wg * 32;
         const float2* nlse2 = reinterpret_cast<const float2*>(sVec + st * 256 + wg * 32 + pair);  // -LSE log2(e), then -Delta
-        ok = mbar_wait(bar_q_full + st, (n >> 1) & 1, a.status);
+        ok = mbar_wait(bar_q_full + st, (c >> 1) & 1, a.status);
         float2 rc[8];  // row constants, read ahead of the wait for the product: shared memory is busy with its operands
 #pragma unroll
         for (int j = 0; j < 8; ++j) rc[j] = nlse2[(j >> 2) * 32 + (j & 3) * 4];
@@ -665,7 +699,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             tmem_ld_frag(sbuf + cb * 64 + ((uint32_t)(h * 16) << 16), p[cb][h]);
         tmem_wait_ld();
         tc_fence_before();
-        mbar_arrive(bar_s_read);
+        if constexpr (!OWN_DQ) mbar_arrive(bar_s_read);
 #pragma unroll
         for (int cb = 0; cb < 2; ++cb) {
 #pragma unroll
@@ -703,6 +737,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         for (int j = 0; j < 8; ++j) rc[j] = nlse2[64 + (j >> 2) * 32 + (j & 3) * 4];
 
         ok = mbar_wait(bar_dp_full, par, a.status);
+        if (ok && n == 0 && kc > 0) ok = mbar_wait(bar_dk_out, (kc - 1) & 1, a.status);
         if (!ok) break;
         tc_fence_after();
 #pragma unroll
@@ -732,24 +767,112 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         fence_proxy_async_smem();
         mbar_arrive(bar_ds_ready);
       }
-      store_grad(wg == 0);
+      if (!ok) break;
+      // dK (first warpgroup) and dV (second, while the last dQ^T and dK are still being computed).  K, V and Q of the next item
+      // arrive meanwhile.
+      const bool is_dk = wg == 0;
+      const int r = (warp & 3) * 32 + lane;
+      if (N > 0) {
+        ok = is_dk ? mbar_wait(bar_done, kc & 1, a.status) : mbar_wait(bar_o_empty, (c - 1) & 1, a.status);
+        if (!ok) break;
+        ++kc;
+      }
+      tc_fence_after();
+      const uint32_t acc = t_lane + (is_dk ? cDK : cDV);
+      const float mul = is_dk ? a.scale : 1.f;
+      const BwdItem* it = item_at(ni);
+      if (float* const part = it->part) {
+        // A shared tile: this item's part goes out in fp32, one slot per item; a kernel of its own adds the slots in order.  A slot
+        // holds 16 bytes of every row after the other, so that a warp's store is one range of 512 bytes.
+        float4* const d4 = reinterpret_cast<float4*>(part + (is_dk ? 0 : BKV * D)) + r;
+#pragma unroll
+        for (int q = 0; q < D / 32; ++q) {
+          uint32_t ov[32];
+          if (N > 0) {
+            tmem_ld32(acc + q * 32, ov);
+            tmem_wait_ld();
+          } else {
+#pragma unroll
+            for (int e = 0; e < 32; ++e) ov[e] = 0u;
+          }
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            d4[(q * 8 + e) * BKV] = make_float4(__uint_as_float(ov[e * 4]) * mul, __uint_as_float(ov[e * 4 + 1]) * mul,
+                                                __uint_as_float(ov[e * 4 + 2]) * mul, __uint_as_float(ov[e * 4 + 3]) * mul);
+        }
+        __syncwarp();
+        if (N > 0 && r == 0) mbar_arrive(is_dk ? bar_dk_out : bar_dv_out);  // (nothing staged)
+      } else {
+        const int left = it->Nk - it->k0;  // rows of this tile
+        // Through shared memory, but for the last, partial KV tile of a packed sequence, whose other rows belong to the next one, and
+        // for a tile that no query sees: the two barriers count items with steps, as a role that has none could get two ahead.
+        const bool staged = N > 0 && !(VARLEN && left < BKV);
+        const CowaStrides sd = is_dk ? a.sdk : a.sdv;
+        __nv_bfloat16* const dst = (is_dk ? a.dk : a.dv) + (VARLEN ? 0 : (size_t)it->b * sd.b) + (size_t)it->hk * sd.h +
+                                   (size_t)(it->rbase + it->k0 + r) * sd.t;
+        uint8_t* const sOut = (is_dk ? sDS : sDO) + r * 128;
+#pragma unroll
+        for (int q = 0; q < D / 32; ++q) {
+          uint32_t ov[32];
+          if (N > 0) {
+            tmem_ld32(acc + q * 32, ov);
+            tmem_wait_ld();
+          } else {
+#pragma unroll
+            for (int e = 0; e < 32; ++e) ov[e] = 0u;
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            uint4 v;
+            v.x = pack_bf16(__uint_as_float(ov[e * 8 + 0]) * mul, __uint_as_float(ov[e * 8 + 1]) * mul);
+            v.y = pack_bf16(__uint_as_float(ov[e * 8 + 2]) * mul, __uint_as_float(ov[e * 8 + 3]) * mul);
+            v.z = pack_bf16(__uint_as_float(ov[e * 8 + 4]) * mul, __uint_as_float(ov[e * 8 + 5]) * mul);
+            v.w = pack_bf16(__uint_as_float(ov[e * 8 + 6]) * mul, __uint_as_float(ov[e * 8 + 7]) * mul);
+            const int slab = q / 2, chunk = (q & 1) * 4 + e;
+            if (staged) *reinterpret_cast<uint4*>(sOut + slab * SLAB_KV + ((chunk ^ (r & 7)) << 4)) = v;
+            else if (r < left) *reinterpret_cast<uint4*>(dst + q * 32 + e * 8) = v;
+          }
+        }
+        if (staged) {
+          fence_proxy_async_smem();
+          wg_sync(is_dk ? 1 : 2);
+        }
+        if (N > 0 && r == 0) {
+          if (staged) {
+            const int bt = VARLEN ? 0 : it->b;
+            for (int s = 0; s < NSLAB; ++s)
+              tma_store_4d(is_dk ? &tmdK : &tmdV, sOut + s * SLAB_KV, s * 64, it->rbase + it->k0, it->hk, bt);
+            tma_commit_group();
+            tma_wait_group_read<0>();
+          }
+          mbar_arrive(is_dk ? bar_dk_out : bar_dv_out);
+        }
+      }
+      tc_fence_before();
+      item_done(ni);
+      }
     }
   } else {
     {
-      const int N = step_count();
       // ======== dQ drain warpgroup: one d column of dQ^T per thread; TMEM -> shared -> bulk reduce-add ========
       float* sDQ = reinterpret_cast<float*>(smem + SM::oDQ) + (warp & 3) * 2048;
       const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-      const bool mine = (warp & 3) * 32 < D;
-      for (int n = 0; n < N && ok; ++n) {
-        ok = mbar_wait(bar_dq_full, n & 1, a.status);
+      // At D = 64 the lanes 64 to 127 hold the same as the first 64 (K^T is read twice as A): these two warps take half 0.
+      const int d_part = warp & (D / 32 - 1);  // this warp's 32 d
+      int c = 0;  // steps so far
+      for (uint32_t ni = 0; ok; ++ni) {
+      const int N = next_item(ni);
+      if (N < 0) break;
+      item_done(ni);
+      for (int n = 0; n < N && ok; ++n, ++c) {
+        ok = mbar_wait(bar_dq_full, c & 1, a.status);
         if (!ok) break;
         tc_fence_after();
         // 32 query rows of this warp's 32 d: staged in one of two tiles and added to the accumulator as one range
-        const longlong2 at_ = dq_at[n & 3];
+        const longlong2 at_ = dq_at[c & 3];
         auto add_rows = [&](const uint32_t (&v)[32], int half, int odd) {
           const long long at = half ? at_.y : at_.x;
-          if (!mine || at < 0) return;
+          if (at < 0) return;
           float* stage = sDQ + odd * 1024;
           if (lane == 0) tma_wait_group_read<1>();  // the reduction issued from this tile before has read it
           __syncwarp();
@@ -801,7 +924,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
-            float* dst = a.dq_acc + at + (warp & 3) * (BQS * 32) + odd * 1024;
+            float* dst = a.dq_acc + at + d_part * (BQS * 32) + odd * 1024;
             if (a.dq_fixed) bulk_reduce_add_s32(dst, stage, 4096);
             else bulk_reduce_add_f32(dst, stage, 4096);
             tma_commit_group();
@@ -810,16 +933,17 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // First the columns that dP^T waits for, then those of S^T.  One loop body, like the MMA warp's: the roles' loops
         // together outgrow the instruction cache (two and four copies: 32K 7660 us forward and backward, this 7410).
 #pragma unroll 1
-        for (int half = 1; half >= 0; --half) {
+        for (int half = OWN_DQ ? (warp & 3) < 2 : 1, last = OWN_DQ ? half : 0; half >= last; --half) {
           uint32_t v0[32], v1[32];
           tmem_ld32(t_lane + cDQ + half * 64, v0);
           tmem_ld32(t_lane + cDQ + half * 64 + 32, v1);
           tmem_wait_ld();
           tc_fence_before();
-          mbar_arrive(bar_dq_free + (half ^ 1));
+          mbar_arrive(bar_dq_free + (OWN_DQ ? 0 : half ^ 1));
           add_rows(v0, half, 0);
           add_rows(v1, half, 1);
         }
+      }
       }
       if (lane == 0) tma_wait_group_read<0>();
     }
@@ -827,7 +951,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 2) {
+  if (warp == 1) {
     __syncwarp();
     tmem_dealloc(tmem_base, TMEM_COLS);
   }
@@ -1232,10 +1356,11 @@ int launch_bwd(const void* q, const void* k, const void* v, const void* o, const
   a.wins = hw;
   a.sink_tiles = pl.sink_tiles;
   for (int c = 0; c < 3; ++c) { a.cls_tiles[c] = pl.tiles[c]; a.cls_parts[c] = pl.run[c]; }
-  a.share = pl.share;
+  a.share = pl.share; a.single = pl.blocks() <= cowa::sm_count();
   a.dq_fixed = p->deterministic ? 1 : 0;
   a.dkv_part = dkv_part;
   a.cu = nullptr; a.dk = static_cast<__nv_bfloat16*>(dk); a.dv = static_cast<__nv_bfloat16*>(dv); a.total = 0; a.tiles_bound = 0;
+  a.sdk = sk; a.sdv = sv;
   a.sink = 0; a.local = 0; a.hkv_global = 0; a.hkv_offset = 0; a.full_attn = 0; a.explicit_windows = 0;
   if (pl.blocks() > 0x7FFFFFFFll || (long long)Nq / BQS * a.G * 32 > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
   COWA_CUDA_TRY(cudaFuncSetAttribute(cowa_bwd_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1292,11 +1417,12 @@ int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o
   a.wins = hw;
   a.sink_tiles = pl.sink_tiles;
   for (int c = 0; c < 3; ++c) { a.cls_tiles[c] = pl.tiles[c]; a.cls_parts[c] = pl.run[c]; }
-  a.share = pl.share;
+  a.share = pl.share; a.single = pl.blocks() <= cowa::sm_count();
   a.dq_fixed = p->deterministic ? 1 : 0;
   a.dkv_part = delta + (size_t)Hq * Tpad;
   a.cu = cu; a.dk = static_cast<__nv_bfloat16*>(dk); a.dv = static_cast<__nv_bfloat16*>(dv);
   a.total = total; a.tiles_bound = total / BKV + B;
+  a.sdk = a.sdv = sk;
   a.sink = p->sink; a.local = p->local;
   a.hkv_global = p->hkv_global > 0 ? p->hkv_global : Hkv;
   a.hkv_offset = p->hkv_offset; a.full_attn = p->full_attn; a.explicit_windows = p->windows != nullptr;
