@@ -18,7 +18,7 @@
 //                   atomics (Algorithm 2 line 17 needs them only because it gives each QO head its
 //                   own program).  dQ^T is drained by a separate warpgroup through shared memory and
 //                   added to the fp32 accumulator with bulk add-reductions (Algorithm 2 line 15).
-//                   Warp roles: TMA producer / MMA issuer / two compute warpgroups (P, dS; each takes 64
+//                   Warp roles: scheduling / TMA producer / MMA issuer / two compute warpgroups (P, dS; each takes 64
 //                   of the 128 query columns of every step) / dQ drain warpgroup, connected by mbarriers.
 //                   What bounds it: shared memory.  Of a step's ~3920 clocks the products' operands take
 //                   2048 (128 bytes a clock), the Q and dO loads 512, dS^T 256, the dQ staging 1024 written
@@ -50,7 +50,7 @@
 //   - shared tiles: a tile's steps are cut into contiguous parts, an item each (few tiles, sink tiles that would
 //     be the critical path, the last wave); each item writes fp32 partial dK, dV to its own slot and a
 //     fourth kernel adds the slots in order (BwdPlan).
-//   - VARLEN: packed batch [H, total, D]; the TMA warp finds (sequence, KV tile) by a warp scan of the offsets,
+//   - VARLEN: packed batch [H, total, D]; the scheduling warp finds (sequence, KV tile) by a warp scan of the offsets,
 //     windows follow from the sequence's own length, the accumulator and the row vectors use a row space
 //     in which every sequence is padded to 64 rows, and a sequence's last, partial KV tile is stored row
 //     by row (cowa_bwd_varlen and its own preprocess / convert kernels).
@@ -71,6 +71,7 @@ constexpr int BQT = 128;  // QO rows per step (MMA N of S^T / dP^T): two tiles
 constexpr int BQS = 64;   // rows of a QO tile, unit of the padded row space and of the plan's step counts
 constexpr int NST = 2;    // Q stages (Q(n) is read again by dK(n) after S^T(n+1)); dO has one
 constexpr int kNoTile = 0x7FFFFF00;  // in place of a step's second tile: no query of it sees anything
+constexpr int kFewTiles = 296;  // up to so many tiles a batched call's plan is a table
 constexpr float kDqFixedOne = 262144.f;  // 2^18: one unit of dQ in the fixed-point accumulation mode
 
 struct BwdArgs {
@@ -83,8 +84,10 @@ struct BwdArgs {
   // The KV tiles in launch order: sink tiles, body, tail.  A tile of class c is shared by cls_parts[c] blocks, each with
   // a contiguous part of the tile's steps (QO heads x QO tiles); a shared tile's blocks leave fp32 partial dK, dV.
   int cls_tiles[3], cls_parts[3];
-  // Instead, where `share` is set: a tile has a block for every `share` QO tiles that see it (ShareOut)
-  int share;
+  // Instead, where `few` is set: the items of one batch element are numbered tile after tile, KV tiles ascending, heads within
+  // them, batch elements within the numbers; tile e = KV tile * Hkv + KV head has the numbers first[e] .. first[e + 1] - 1.
+  int few;             // tiles of one batch element
+  uint16_t first[kFewTiles + 1], shared[kFewTiles];  // shared: the tiles with several
   int single;          // the grid fits the device: a block has one item
   int dq_fixed;        // 1: dQ partial sums travel as 32-bit fixed point (order-independent addition)
   float* dkv_part;     // fp32 partial dK, dV [blocks of shared tiles, 2, BKV, D], summed by a kernel of their own
@@ -162,55 +165,24 @@ __device__ __forceinline__ bool locate_tile(const BwdArgs& a, int c, int q, Tile
   return true;
 }
 
-// Batched calls of few tiles, shared out by `share`: the blocks of one batch element are numbered tile after tile, KV tiles
-// ascending, heads within them, batch elements within the numbers.  Warp-cooperative.
-struct ShareOut {
-  __device__ __forceinline__ static int parts_of(const BwdArgs& a, int e) {  // of tile e = KV tile * Hkv + KV head
-    const int k0 = e / a.Hkv * BKV;
-    CowaRange rg[2];
-    cowa_bwd_ranges(a.wins.w[e % a.Hkv], k0, min(k0 + BKV, a.Nk) - 1, a.Nk - a.Nq, a.Nq, BQS, rg);
-    return max(((cowa_range_len(rg[0]) + cowa_range_len(rg[1])) * a.G + a.share - 1) / a.share, 1);
-  }
-  // The tile that holds number i (by_tile: tile i), its first number and parts.
-  __device__ __forceinline__ static void find(const BwdArgs& a, int i, bool by_tile, int* tile, int* first, int* parts) {
-    const int lane = threadIdx.x & 31, n = (a.Nk + BKV - 1) / BKV * a.Hkv;
-    int base = 0;
-    for (int e0 = 0; e0 < n; e0 += 32) {
-      const int e = e0 + lane, p = e < n ? parts_of(a, e) : 0;
-      int incl = p;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const unsigned m = __ballot_sync(0xFFFFFFFFu, by_tile ? i <= e : i < base + incl);
-      if (m) {
-        const int src = __ffs(m) - 1;
-        *tile = e0 + src;
-        *parts = __shfl_sync(0xFFFFFFFFu, p, src);
-        *first = base + __shfl_sync(0xFFFFFFFFu, incl - p, src);
-        return;
-      }
-      base += __shfl_sync(0xFFFFFFFFu, incl, 31);
-    }
-  }
-};
-
 // named barriers: one 128-thread warpgroup; all of the block, where the TMA warp does not wait
 __device__ __forceinline__ void all_arrive() { asm volatile("bar.arrive 3, 512;" ::: "memory"); }
 __device__ __forceinline__ void all_sync() { asm volatile("bar.sync 3, 512;" ::: "memory"); }
 __device__ __forceinline__ void wg_sync(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
 
-// One work item: a KV tile, or a part of its steps, as the TMA warp publishes it for the other warps.
+// One work item: a KV tile, or a part of its steps, as the scheduling warp publishes it for the others.
 struct BwdItem {
   CowaWin w;
   int off, Nq, Nk;
   int steps;     // -1: no more items
   int k0, hk, b, rbase;
   float* part;   // where the partial dK, dV of a shared tile go, else nullptr
+  // the TMA warp's: I_h(j), QO tiles per head and of this item, head of the group and position in I_h(j) of the first
+  CowaRange rg[2];
+  int cnt, tiles, g, t_in, pbase;
 };
 static_assert(sizeof(BwdItem) <= 96, "slot of a published item");
-constexpr int kItemReaders = 13;  // warps that read it: MMA 1, compute 8, drain 4
+constexpr int kItemReaders = 14;  // warps that read it: TMA 1, MMA 1, compute 8, drain 4
 
 template <int D, bool VARLEN>
 __global__ void __launch_bounds__(512, 1)
@@ -263,6 +235,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   uint64_t* bar_next = bars + 33;     // the next item's number is here
   uint64_t* bar_dk_out = bars + 34;   // dK of an item has left the buffer of dS^T
   uint64_t* bar_dv_out = bars + 35;   // dV ... of dO
+  uint64_t* bar_ask = bars + 36;      // it is time to ask for the next item
   auto item_at = [&](uint32_t ni) { return reinterpret_cast<BwdItem*>(smem + SM::oItem + (ni & 1) * 96); };
 
   const int tid = threadIdx.x, lane = tid & 31;
@@ -278,20 +251,21 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     mbar_init(bar_dq_full, 1); mbar_init(bar_o_full, 1); mbar_init(bar_o_empty, 1);
     mbar_init(bar_s_full, 1); mbar_init(bar_s_read, 256); mbar_init(bar_p_ready, 256);
     mbar_init(bar_dp_full, 1); mbar_init(bar_ds_ready, 256);
-    mbar_init(bar_done, 1); mbar_init(bar_next, 1); mbar_init(bar_dk_out, 1); mbar_init(bar_dv_out, 1);
+    mbar_init(bar_done, 1); mbar_init(bar_next, 1); mbar_init(bar_dk_out, 1); mbar_init(bar_dv_out, 1); mbar_init(bar_ask, 1);
     fence_mbar_init();
   }
   if (tid == 32) { prefetch_tmap(&tmQ2); prefetch_tmap(&tmdO2); prefetch_tmap(&tmK); prefetch_tmap(&tmV); }
   __syncthreads();
-  // What needs nothing of the kernel before this one is done ahead of the wait for it: this, and the first item's geometry, which
-  // the TMA warp works out (not so the TMEM allocation, see cowa_fwd_kernel; the first loads do not wait for that).  A grid that is
-  // not started as a whole cannot let the next kernel in early.
+  // What needs nothing of the kernel before this one is done ahead of the wait for it: this, and the first item's geometry (not so
+  // the TMEM allocation, see cowa_fwd_kernel; the first loads do not wait for that).  A grid that is not started as a whole cannot
+  // let the next kernel in early.
   auto enter = [&]() {
     if (a.single) grid_enter();
     else grid_wait();
   };
-  if (warp == 0) {
+  if (warp == 0 || warp == 2) {
     all_arrive();
+    if (VARLEN || warp == 0) enter();
   } else {
     enter();
     if (warp == 1) {
@@ -320,162 +294,180 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   // is.  Each setmaxnreg sits at the top of its own branch so that the code below it is compiled for that budget.
   if (warp < 4) {
     setmaxnreg_dec<80>();
-    if (warp == 0) {
-      // ================= TMA producer; works out the items one ahead =================
+    if (warp == 2) {
+      // ================= scheduling: takes over items and works out their geometry, one ahead of the others =================
+      // (In the TMA warp this came between two items' loads: 1.6 us, 3.5 us in packed batches.)
       const bool lead = elect_one();
-      int c = 0;        // steps so far, all items together
-      uint32_t ni = 0, kc = 0;  // items so far, those with steps
-      uint32_t asked = 0, answered = 0;
-      auto ask = [&]() {
+      int idx = blockIdx.x;
+      uint32_t asked = 0;
+      auto next_index = [&]() {
+        if (a.single) return -1;
         if (lead) {
           mbar_expect_tx(bar_next, 16);
           clc_request(smem + SM::oNext, bar_next);
         }
+        ok = mbar_wait(bar_next, asked & 1, a.status);
         ++asked;
-      };
-      int idx = blockIdx.x;
-      if (VARLEN) enter();
-      while (ok) {
-        // ---- work item ----
-        int parts = 1, part = 0, slot = idx;  // slot: of this item's partial dK, dV when the tile is shared
-        TileAt at;
-        bool found = idx >= 0;
-        if (!found) {
-        } else if (!VARLEN && a.share > 0) {
-          int e = 0, first = 0;
-          ShareOut::find(a, idx / a.B, false, &e, &first, &parts);
-          part = idx / a.B - first;
-          at.b = idx % a.B; at.hk = e % a.Hkv; at.j = e / a.Hkv; at.pbase = 0;
-        } else {
-          int cls = 0, q = idx;
-          slot = 0;
-          while (cls < 2 && q >= a.cls_tiles[cls] * a.cls_parts[cls]) {
-            q -= a.cls_tiles[cls] * a.cls_parts[cls];
-            if (a.cls_parts[cls] > 1) slot += a.cls_tiles[cls] * a.cls_parts[cls];
-            ++cls;
-          }
-          parts = a.cls_parts[cls]; part = q % parts;
-          slot += q;
-          found = locate_tile<VARLEN>(a, cls, q / parts, at);
-        }
-        // Sequence geometry.  Packed batches: N_q = N_k = the sequence's length, rows start at cu[b]; the fp32
-        // dQ accumulator and the LSE / Delta vectors are laid out with every sequence padded to 64 rows (pbase).
-        int Nq = a.Nq, Nk = a.Nk, rbase = 0;
-        CowaWin w = a.wins.w[found ? at.hk : 0];
-        if (VARLEN && found) {
-          rbase = a.cu[at.b];
-          Nq = Nk = a.cu[at.b + 1] - rbase;
-          if (rbase < 0 || rbase + Nk > a.total) {  // malformed offsets: report, touch nothing
-            if (lead) atomicOr(a.status, (unsigned)COWA_DEV_BAD_SEQLENS);
-            found = false;
-          }
-          if (a.full_attn) { w.s = 0; w.n = Nk; w.g = 0; w.l = 0; }
-          else if (!a.explicit_windows) w = cowa_default_window(Nk, a.hkv_global, a.hkv_offset + at.hk, a.sink, a.local);
-        }
-        if (!found && idx >= 0) {  // (packed batches: the count of items is an upper bound)
-          if (!a.single) ask();
-        } else {
-          const int hk = at.hk, b = at.b, off = Nk - Nq, k0 = at.j * BKV, k1 = min(k0 + BKV, Nk) - 1;
-          CowaRange rg[2];
-          int cnt = 0, tiles = 0, g = 0, t_in = 0;
-          if (found) {
-            cowa_bwd_ranges(w, k0, k1, off, Nq, BQS, rg);
-            cnt = cowa_range_len(rg[0]) + cowa_range_len(rg[1]);       // QO tiles per head
-            const int n0 = cnt * a.G * part / parts;                   // (the host checks that these products fit)
-            tiles = cnt * a.G * (part + 1) / parts - n0;               // this item's QO tiles
-            g = cnt > 0 ? n0 / cnt : 0; t_in = n0 - g * cnt;           // head of the group and position in I_h(j): kept incrementally
-          }
-          const int N = found ? (tiles + 1) >> 1 : -1;
-          if (!VARLEN && ni == 0) enter();
-          if (ni >= 2) ok = mbar_wait(bar_i_empty + (ni & 1), ((ni >> 1) & 1) ^ 1, a.status);
-          if (!ok) break;
-          if (lead) {
-            BwdItem& it = *item_at(ni);
-            it.w = w; it.off = off; it.Nq = Nq; it.Nk = Nk; it.steps = N; it.k0 = k0; it.hk = hk; it.b = b; it.rbase = rbase;
-            it.part = parts > 1 ? a.dkv_part + (size_t)slot * 2 * (BKV * D) : nullptr;
-            mbar_arrive(bar_i_full + (ni & 1));
-          }
-          __syncwarp();
-          ++ni;
-          if (N < 0) break;
-          const int bt = VARLEN ? 0 : b;                   // batch coordinate of the tensor maps
-          const int hq0 = hk * a.G;                        // first QO head of the group
-          const int bhq0 = (VARLEN ? 0 : b * a.Hq) + hq0;  // ... as a row of lse2 / delta / dq_acc
-          auto load_kv = [&](uint8_t* tile, const CUtensorMap* tm, uint64_t* bar) {
-            if (!lead) return;
-            mbar_expect_tx(bar, SM::kKV);
-            for (int s = 0; s < NSLAB; ++s) tma_load_4d(tile + s * SLAB_KV, tm, bar, s * 64, rbase + k0, hk, bt);
-          };
-          if (c == 0 && N > 0) load_kv(sK, &tmK, bar_k);  // S^T of the first step waits for K and Q only
-          const int ask_at = a.single ? -1 : max(N - 3, 0);  // a microsecond or more before the answer is needed
-          if (N == 0 && !a.single) ask();
-          for (int n = 0; n < N; ++n, ++c) {
-            const int st = c & 1;
-            if (n == ask_at) ask();
-            int q0[2], gh[2];
-            q0[0] = cowa_bwd_tile_at(rg, t_in) * BQS; gh[0] = g;
-            if (++t_in == cnt) { t_in = 0; ++g; }
-            const bool two = 2 * n + 1 < tiles;  // else the first tile again, every pair of it masked
-            q0[1] = two ? cowa_bwd_tile_at(rg, t_in) * BQS : q0[0]; gh[1] = two ? g : gh[0];
-            if (two && ++t_in == cnt) { t_in = 0; ++g; }
-            // neighbours of one head, as nearly always, come in one piece
-            const int pieces = two && gh[1] == gh[0] && q0[1] == q0[0] + BQS ? 1 : 2;
-            auto load_rows = [&](uint8_t* tile, const CUtensorMap* tm, const CUtensorMap* tm2, uint64_t* bar) {
-              for (int x = 0; x < pieces; ++x)
-                for (int s = 0; s < NSLAB; ++s)
-                  tma_load_4d(tile + s * SLAB_Q + x * (SLAB_Q / 2), pieces == 1 ? tm2 : tm, bar, s * 64, rbase + q0[x], hq0 + gh[x], bt);
-            };
-            if (c >= 2) ok = mbar_wait(bar_q_empty + st, ((c >> 1) & 1) ^ 1, a.status);
-            if (!ok) break;
-            if (lead) {
-              auto info = [&](int x) {
-                return q0[x] + (cowa_tile_full(w, q0[x], BQS, k0, BKV, off, Nq, Nk) ? 1 : 0) + (q0[x] + BQS > Nq ? 2 : 0);
-              };
-              step_info[st] = make_int2(info(0), two ? info(1) : kNoTile);
-              auto rows = [&](int x) -> size_t { return (size_t)(bhq0 + gh[x]) * a.Tpad + at.pbase + q0[x]; };  // in lse2, delta, dq_acc
-              dq_at[c & 3] = make_longlong2((long long)rows(0) * D, two ? (long long)rows(1) * D : -1ll);
-              mbar_expect_tx(bar_q_full + st, SM::kQ + 2 * BQT * 4);
-              load_rows(sQ + st * SM::kQ, &tmQ, &tmQ2, bar_q_full + st);
-              for (int x = 0; x < pieces; ++x) {
-                bulk_load_1d(sVec + st * 256 + x * BQS, a.lse2 + rows(x), BQT * 4 / pieces, bar_q_full + st);
-                bulk_load_1d(sVec + st * 256 + 128 + x * BQS, a.delta + rows(x), BQT * 4 / pieces, bar_q_full + st);
-              }
-            }
-            if (n == 0) {  // V over that of the item before once its last dP^T has been computed, K once dQ^T has
-              if (c > 0) ok = mbar_wait(bar_dp_full, (c - 1) & 1, a.status);
-              if (!ok) break;
-              load_kv(sV, &tmV, bar_v);
-            }
-            // (dV of the item before has left the buffer of dO: behind dO's last product)
-            if (n == 0 && c > 0) ok = mbar_wait(bar_dv_out, (kc - 1) & 1, a.status);
-            else if (c > 0) ok = mbar_wait(bar_o_empty, (c - 1) & 1, a.status);
-            if (!ok) break;
-            if (lead) {
-              mbar_expect_tx(bar_o_full, SM::kQ);
-              load_rows(sDO, &tmdO, &tmdO2, bar_o_full);
-            }
-            if (n == 0 && c > 0) {
-              ok = mbar_wait(bar_dq_full, (c - 1) & 1, a.status);
-              if (!ok) break;
-              load_kv(sK, &tmK, bar_k);
-            }
-            __syncwarp();
-          }
-          if (!ok) break;
-          if (N > 0) ++kc;
-        }
-        if (a.single) {
-          idx = -1;
-          continue;
-        }
-        answered = asked;
-        ok = mbar_wait(bar_next, (asked - 1) & 1, a.status);
-        if (!ok) break;
-        idx = __shfl_sync(0xFFFFFFFFu, clc_block(smem + SM::oNext), 0);
+        if (!ok) return -1;
+        const int x = __shfl_sync(0xFFFFFFFFu, clc_block(smem + SM::oNext), 0);
         fence_proxy_async_smem();  // read before the next answer is written
         __syncwarp();
+        return x;
+      };
+      for (uint32_t ni = 0; ok;) {
+        BwdItem it;
+        it.steps = -1;
+        if (idx >= 0) {
+          int parts = 1, part = 0, slot = idx;  // slot: of this item's partial dK, dV when the tile is shared
+          TileAt at;
+          bool found = true;
+          if (!VARLEN && a.few > 0) {
+            const int q = idx / a.B;
+            int e = 0, hi = a.few - 1;  // the last tile with first[e] <= q
+            while (e < hi) {
+              const int mid = (e + hi + 1) >> 1;
+              if (a.first[mid] <= q) e = mid;
+              else hi = mid - 1;
+            }
+            parts = a.first[e + 1] - a.first[e]; part = q - a.first[e];
+            at.b = idx - q * a.B; at.hk = e % a.Hkv; at.j = e / a.Hkv; at.pbase = 0;
+          } else {
+            int cls = 0, q = idx;
+            slot = 0;
+            while (cls < 2 && q >= a.cls_tiles[cls] * a.cls_parts[cls]) {
+              q -= a.cls_tiles[cls] * a.cls_parts[cls];
+              if (a.cls_parts[cls] > 1) slot += a.cls_tiles[cls] * a.cls_parts[cls];
+              ++cls;
+            }
+            parts = a.cls_parts[cls]; part = q % parts;
+            slot += q;
+            found = locate_tile<VARLEN>(a, cls, q / parts, at);
+          }
+          // Sequence geometry.  Packed batches: N_q = N_k = the sequence's length, rows start at cu[b]; the fp32
+          // dQ accumulator and the LSE / Delta vectors are laid out with every sequence padded to 64 rows (pbase).
+          it.Nq = a.Nq; it.Nk = a.Nk; it.rbase = 0;
+          if (found) it.w = a.wins.w[at.hk];
+          if (VARLEN && found) {
+            it.rbase = a.cu[at.b];
+            it.Nq = it.Nk = a.cu[at.b + 1] - it.rbase;
+            if (it.rbase < 0 || it.rbase + it.Nk > a.total) {  // malformed offsets: report, touch nothing
+              if (lead) atomicOr(a.status, (unsigned)COWA_DEV_BAD_SEQLENS);
+              found = false;
+            }
+            if (a.full_attn) { it.w.s = 0; it.w.n = it.Nk; it.w.g = 0; it.w.l = 0; }
+            else if (!a.explicit_windows) it.w = cowa_default_window(it.Nk, a.hkv_global, a.hkv_offset + at.hk, a.sink, a.local);
+          }
+          if (!found) {  // (packed batches: the count of items is an upper bound)
+            idx = next_index();
+            continue;
+          }
+          it.hk = at.hk; it.b = at.b; it.pbase = at.pbase; it.off = it.Nk - it.Nq; it.k0 = at.j * BKV;
+          cowa_bwd_ranges(it.w, it.k0, min(it.k0 + BKV, it.Nk) - 1, it.off, it.Nq, BQS, it.rg);
+          it.cnt = cowa_range_len(it.rg[0]) + cowa_range_len(it.rg[1]);
+          const int n0 = it.cnt * a.G * part / parts;        // (the host checks that these products fit)
+          it.tiles = it.cnt * a.G * (part + 1) / parts - n0;
+          it.steps = (it.tiles + 1) >> 1;
+          it.g = it.cnt > 0 ? n0 / it.cnt : 0; it.t_in = n0 - it.g * it.cnt;
+          it.part = parts > 1 ? a.dkv_part + (size_t)slot * 2 * (BKV * D) : nullptr;
+        }
+        if (ni >= 2) ok = mbar_wait(bar_i_empty + (ni & 1), ((ni >> 1) & 1) ^ 1, a.status);
+        if (!ok) break;
+        if (lead) {
+          *item_at(ni) = it;
+          mbar_arrive(bar_i_full + (ni & 1));
+        }
+        __syncwarp();
+        if (it.steps < 0) break;
+        if (!a.single) ok = mbar_wait(bar_ask, ni & 1, a.status);
+        ++ni;
+        if (ok) idx = next_index();
       }
-      if (asked != answered) mbar_wait(bar_next, (asked - 1) & 1, a.status);  // (a wait ran out) no answer may come later
+    } else if (warp == 0) {
+      // ================= TMA producer =================
+      const bool lead = elect_one();
+      int c = 0;        // steps so far, all items together
+      uint32_t kc = 0;  // items with steps so far
+      for (uint32_t ni = 0; ok; ++ni) {
+        const int N = next_item(ni);
+        if (N < 0) break;
+        const volatile BwdItem* const it = item_at(ni);
+        CowaWin w;
+        w.s = it->w.s; w.n = it->w.n; w.g = it->w.g; w.l = it->w.l;
+        const int off = it->off, Nq = it->Nq, Nk = it->Nk, k0 = it->k0, hk = it->hk, b = it->b, rbase = it->rbase;
+        const int cnt = it->cnt, tiles = it->tiles, pbase = it->pbase;
+        int g = it->g, t_in = it->t_in;  // kept incrementally
+        CowaRange rg[2];
+        rg[0].lo = it->rg[0].lo; rg[0].hi = it->rg[0].hi; rg[1].lo = it->rg[1].lo; rg[1].hi = it->rg[1].hi;
+        item_done(ni);
+        auto ask = [&]() {
+          if (lead && !a.single) mbar_arrive(bar_ask);
+        };
+        const int bt = VARLEN ? 0 : b;                   // batch coordinate of the tensor maps
+        const int hq0 = hk * a.G;                        // first QO head of the group
+        const int bhq0 = (VARLEN ? 0 : b * a.Hq) + hq0;  // ... as a row of lse2 / delta / dq_acc
+        auto load_kv = [&](uint8_t* tile, const CUtensorMap* tm, uint64_t* bar) {
+          if (!lead) return;
+          mbar_expect_tx(bar, SM::kKV);
+          for (int s = 0; s < NSLAB; ++s) tma_load_4d(tile + s * SLAB_KV, tm, bar, s * 64, rbase + k0, hk, bt);
+        };
+        if (c == 0 && N > 0) load_kv(sK, &tmK, bar_k);  // S^T of the first step waits for K and Q only
+        const int ask_at = max(N - 4, 0);               // some microseconds before the next item is needed
+        if (N == 0) ask();
+        for (int n = 0; n < N; ++n, ++c) {
+          const int st = c & 1;
+          if (n == ask_at) ask();
+          int q0[2], gh[2];
+          q0[0] = cowa_bwd_tile_at(rg, t_in) * BQS; gh[0] = g;
+          if (++t_in == cnt) { t_in = 0; ++g; }
+          const bool two = 2 * n + 1 < tiles;  // else the first tile again, every pair of it masked
+          q0[1] = two ? cowa_bwd_tile_at(rg, t_in) * BQS : q0[0]; gh[1] = two ? g : gh[0];
+          if (two && ++t_in == cnt) { t_in = 0; ++g; }
+          // neighbours of one head, as nearly always, come in one piece
+          const int pieces = two && gh[1] == gh[0] && q0[1] == q0[0] + BQS ? 1 : 2;
+          auto load_rows = [&](uint8_t* tile, const CUtensorMap* tm, const CUtensorMap* tm2, uint64_t* bar) {
+            for (int x = 0; x < pieces; ++x)
+              for (int s = 0; s < NSLAB; ++s)
+                tma_load_4d(tile + s * SLAB_Q + x * (SLAB_Q / 2), pieces == 1 ? tm2 : tm, bar, s * 64, rbase + q0[x], hq0 + gh[x], bt);
+          };
+          if (c >= 2) ok = mbar_wait(bar_q_empty + st, ((c >> 1) & 1) ^ 1, a.status);
+          if (!ok) break;
+          if (lead) {
+            auto info = [&](int x) {
+              return q0[x] + (cowa_tile_full(w, q0[x], BQS, k0, BKV, off, Nq, Nk) ? 1 : 0) + (q0[x] + BQS > Nq ? 2 : 0);
+            };
+            step_info[st] = make_int2(info(0), two ? info(1) : kNoTile);
+            auto rows = [&](int x) -> size_t { return (size_t)(bhq0 + gh[x]) * a.Tpad + pbase + q0[x]; };  // in lse2, delta, dq_acc
+            dq_at[c & 3] = make_longlong2((long long)rows(0) * D, two ? (long long)rows(1) * D : -1ll);
+            mbar_expect_tx(bar_q_full + st, SM::kQ + 2 * BQT * 4);
+            load_rows(sQ + st * SM::kQ, &tmQ, &tmQ2, bar_q_full + st);
+            for (int x = 0; x < pieces; ++x) {
+              bulk_load_1d(sVec + st * 256 + x * BQS, a.lse2 + rows(x), BQT * 4 / pieces, bar_q_full + st);
+              bulk_load_1d(sVec + st * 256 + 128 + x * BQS, a.delta + rows(x), BQT * 4 / pieces, bar_q_full + st);
+            }
+          }
+          if (n == 0) {  // V over that of the item before once its last dP^T has been computed, K once dQ^T has
+            if (c > 0) ok = mbar_wait(bar_dp_full, (c - 1) & 1, a.status);
+            if (!ok) break;
+            load_kv(sV, &tmV, bar_v);
+          }
+          // (dV of the item before has left the buffer of dO: behind dO's last product)
+          if (n == 0 && c > 0) ok = mbar_wait(bar_dv_out, (kc - 1) & 1, a.status);
+          else if (c > 0) ok = mbar_wait(bar_o_empty, (c - 1) & 1, a.status);
+          if (!ok) break;
+          if (lead) {
+            mbar_expect_tx(bar_o_full, SM::kQ);
+            load_rows(sDO, &tmdO, &tmdO2, bar_o_full);
+          }
+          if (n == 0 && c > 0) {
+            ok = mbar_wait(bar_dq_full, (c - 1) & 1, a.status);
+            if (!ok) break;
+            load_kv(sK, &tmK, bar_k);
+          }
+          __syncwarp();
+        }
+        if (!ok) break;
+        if (N > 0) ++kc;
+      }
     } else if (warp == 1) {
       // ================= MMA issuer =================
       // The whole warp runs this loop (uniform control flow, so that descriptors and counters stay in
@@ -1053,13 +1045,10 @@ cowa_bwd_preprocess_varlen_kernel(const __nv_bfloat16* o, const __nv_bfloat16* d
 
 // The dQ accumulator to bf16: one 64-row chunk of the row space and one head a block, every row's 16-byte pieces of four
 // rows and one d (see the drain); a thread takes four rows of two d, so that a warp reads 1 KB ranges and writes whole
-// sectors.  (One kernel with the sum of partial dK, dV needs 46 registers and lost occupancy: 137 instead of 112 us at 32K.)
+// sectors.
 template <int D, bool VARLEN>
-__global__ void __launch_bounds__(256)
-cowa_bwd_convert_dq_kernel(const float* acc, __nv_bfloat16* dq, const int* cu, int B, int T, int Tpad, int H, int fixed,
-                           CowaStrides sq, unsigned int* status) {
-  grid_enter();
-  const int nchunk = Tpad / BQS, chunk = VARLEN ? blockIdx.x : blockIdx.x % nchunk, bh = VARLEN ? blockIdx.y : blockIdx.x / nchunk;
+__device__ __forceinline__ void convert_dq(const float* acc, __nv_bfloat16* dq, const int* cu, int B, int T, int Tpad, int fixed,
+                                           const CowaStrides& sq, int H, unsigned int* status, int chunk, int bh) {
   int rows, first;  // rows of this chunk, and the first one's place among the rows of dq
   __nv_bfloat16* out;
   if constexpr (!VARLEN) {
@@ -1095,22 +1084,28 @@ cowa_bwd_convert_dq_kernel(const float* acc, __nv_bfloat16* dq, const int* cu, i
   }
 }
 
-// Partial dK (blockIdx.y = 0) and dV (1) of the shared tiles, added in slot order, to bf16.
 template <int D, bool VARLEN>
 __global__ void __launch_bounds__(256)
-cowa_bwd_reduce_dkv_kernel(const __grid_constant__ BwdArgs a, CowaStrides sk, CowaStrides sv) {
+cowa_bwd_convert_dq_kernel(const float* acc, __nv_bfloat16* dq, const int* cu, int B, int T, int Tpad, int H, int fixed,
+                           CowaStrides sq, unsigned int* status) {
   grid_enter();
-  constexpr int BLOCKS = BKV * (D / 8) / 256;  // of a tile: a thread takes eight d of a row, a warp 32 rows (see the slots)
-  const int i_ = blockIdx.x % BLOCKS * 256 + threadIdx.x, r = i_ % BKV, part = i_ / BKV;
-  int q = blockIdx.x / BLOCKS, c = 0, slot = 0, parts, step = 1;  // the tile's slots: slot, slot + step, ...
+  const int nchunk = Tpad / BQS;
+  convert_dq<D, VARLEN>(acc, dq, cu, B, T, Tpad, fixed, sq, H, status, blockIdx.x % nchunk, blockIdx.x / nchunk);
+}
+
+// Partial dK (m = 0) and dV (1) of the shared tiles, added in slot order, to bf16.
+template <int D>
+constexpr int kReduceBlocks = BKV * (D / 8) / 256;  // of a tile and m: a thread takes eight d of a row, a warp 32 rows (see the slots)
+template <int D, bool VARLEN>
+__device__ __forceinline__ void reduce_dkv(const BwdArgs& a, const CowaStrides& sk, const CowaStrides& sv, int block, int m) {
+  const int i_ = block % kReduceBlocks<D> * 256 + threadIdx.x, r = i_ % BKV, part = i_ / BKV;
+  int q = block / kReduceBlocks<D>, c = 0, slot = 0, parts, step = 1;  // the tile's slots: slot, slot + step, ...
   TileAt at;
-  if (!VARLEN && a.share > 0) {
-    int e = 0, first = 0;
-    parts = 1;
-    ShareOut::find(a, q / a.B, true, &e, &first, &parts);
-    if (parts == 1) return;
+  if (!VARLEN && a.few > 0) {
+    const int e = a.shared[q / a.B];
     at.b = q % a.B; at.hk = e % a.Hkv; at.j = e / a.Hkv;
-    slot = first * a.B + at.b; step = a.B;
+    parts = a.first[e + 1] - a.first[e];
+    slot = a.first[e] * a.B + at.b; step = a.B;
   } else {
   for (; c < 2; ++c) {
     if (a.cls_parts[c] == 1) continue;
@@ -1130,7 +1125,6 @@ cowa_bwd_reduce_dkv_kernel(const __grid_constant__ BwdArgs a, CowaStrides sk, Co
   }
   const int t = at.j * BKV + r;
   if (t >= Nk) return;
-  const int m = blockIdx.y;
   const float* src = a.dkv_part + ((size_t)slot * 2 + m) * (BKV * D) + ((size_t)part * 2 * BKV + r) * 4;
   float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
 #pragma unroll 4
@@ -1147,6 +1141,26 @@ cowa_bwd_reduce_dkv_kernel(const __grid_constant__ BwdArgs a, CowaStrides sk, Co
       make_uint4(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w), pack_bf16(y.x, y.y), pack_bf16(y.z, y.w));
 }
 
+template <int D, bool VARLEN>
+__global__ void __launch_bounds__(256)
+cowa_bwd_reduce_dkv_kernel(const __grid_constant__ BwdArgs a, CowaStrides sk, CowaStrides sv) {
+  grid_enter();
+  reduce_dkv<D, VARLEN>(a, sk, sv, blockIdx.x, blockIdx.y);
+}
+
+// Both in one launch, the sums first, where the accumulator is small: a kernel less in the chain (forward and
+// backward of 1024 tokens, 4 heads, with the table of tiles 25.8 -> 23.0 us).  Long
+// ones keep the conversion's occupancy (with the registers of the sums 137 instead of 112 us at 32K).
+template <int D, bool VARLEN>
+__global__ void __launch_bounds__(256)
+cowa_bwd_finish_kernel(const __grid_constant__ BwdArgs a, CowaStrides sk, CowaStrides sv, int sums, __nv_bfloat16* dq, int T, CowaStrides sq) {
+  grid_enter();
+  const int i = blockIdx.x - sums, nchunk = a.Tpad / BQS;
+  if (i < 0) reduce_dkv<D, VARLEN>(a, sk, sv, blockIdx.x >> 1, blockIdx.x & 1);
+  else convert_dq<D, VARLEN>(a.dq_acc, dq, a.cu, a.B, T, a.Tpad, a.dq_fixed, sq, a.Hq, a.status, i % nchunk, i / nchunk);
+}
+constexpr int kFinishChunks = 2048;  // 64-row chunks of the accumulator, all heads together
+
 // How the KV tiles are shared among blocks.  A tile whose block takes the whole GQA group keeps dK, dV in TMEM; a shared
 // tile costs every block a prologue and 128 KB of fp32 partial sums (D = 128), so tiles are shared only where whole ones
 // leave SMs idle (work and shares are counted in 64-row QO tiles here, half a step of the kernel each):
@@ -1159,8 +1173,10 @@ struct BwdPlan {
   int sink_tiles;  // per sequence and head
   int tiles[3], parts[3];  // parts: what the workspace has room for
   int run[3];              // what the blocks take
-  int share = 0;           // ... or, batched calls of few tiles: QO tiles a block
-  long long shared_blocks = 0;
+  // ... or, batched calls of few tiles (BwdArgs)
+  int few = 0, few_shared = 0;
+  long long few_blocks = 0;
+  uint16_t first[kFewTiles + 1], shared[kFewTiles];
   long long slots() const {
     long long n = 0;
     for (int c = 0; c < 3; ++c)
@@ -1168,7 +1184,7 @@ struct BwdPlan {
     return n;
   }
   long long blocks() const {
-    if (share > 0) return shared_blocks;
+    if (few > 0) return few_blocks;
     long long n = 0;
     for (int c = 0; c < 3; ++c) n += (long long)tiles[c] * run[c];
     return n;
@@ -1192,29 +1208,35 @@ struct BwdPlan {
 
   // Few tiles: their blocks by length.  With the same number of parts for every tile the blocks of a causal batch have one to
   // fourteen steps, and the last SM ends at twice the average (821 tokens x 4, 16 heads: SMs end after 23 to 60 us).
-  // The smallest share with which the blocks make k rounds, for the k that ends first: a block costs about as much as ten QO
-  // tiles besides its own.  cnt: QO tiles of each KV tile of one batch element.
+  // Of shares an eighth apart the one that ends first, as far as can be told: an item costs about as much as five QO
+  // tiles besides its own, a block five more, and its partial sums 0.04; with more items than SMs a part of one is lost at the end.  cnt: QO tiles
+  // of each KV tile of one batch element.
   void share_out(const int* cnt, int n, int B, long long total, int longest) {
     const int sms = cowa::sm_count();
-    const long long room = slots();
-    long long best = 0;
-    for (int k = 1; k <= 3; ++k) {
-      const long long most = std::min<long long>((long long)k * sms, room);
-      auto blocks_with = [&](int x) {
-        long long b = 0;
-        for (int i = 0; i < n; ++i) b += std::max((cnt[i] + x - 1) / x, 1);
-        return b * B;
-      };
-      int lo = (int)std::max<long long>((total + most - 1) / std::max<long long>(most, 1), 4), hi = std::max(longest, lo);
-      if (blocks_with(hi) > most) continue;
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (blocks_with(mid) <= most) hi = mid;
-        else lo = mid + 1;
-      }
-      const long long t = (long long)k * (10 + hi);
-      if (share == 0 || t < best) { best = t; share = hi; shared_blocks = blocks_with(hi); }
+    const long long room = std::min<long long>(slots(), 65535ll * B);
+    double best = 0;
+    int share = 0;
+    for (int x = std::max(longest, 4);; x = std::max(x * 7 / 8, 4)) {
+      long long b = 0;
+      for (int i = 0; i < n; ++i) b += std::max((cnt[i] + x - 1) / x, 1);
+      b *= B;
+      if (b > room) break;
+      double t = 10 + x;
+      if (b > sms) t = std::max(t, 5 + (total + 5. * b) / sms + 0.4 * (5 + x));
+      if (b > (long long)n * B) t += 0.04 * b;
+      if (share == 0 || t < best) { best = t; share = x; few_blocks = b; }
+      if (x == 4) break;
     }
+    if (share == 0) return;
+    few = n;
+    int at = 0;
+    for (int i = 0; i < n; ++i) {
+      const int parts = std::max((cnt[i] + share - 1) / share, 1);
+      first[i] = (uint16_t)at;
+      at += parts;
+      if (parts > 1) shared[few_shared++] = (uint16_t)i;
+    }
+    first[n] = (uint16_t)at;
   }
 };
 
@@ -1238,9 +1260,10 @@ BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& h
   pl.sink_tiles = 0;
   for (int h = 0; h < Hkv; ++h) pl.sink_tiles = std::max(pl.sink_tiles, (std::min(hw.w[h].s, Nk) + BKV - 1) / BKV);
   long long total = 0, sinks = 0, longest = 0, longest_sink = 0;
-  constexpr int kFewTiles = 512;
   int counts[kFewTiles];  // tile j of head h: [j * Hkv + h]
-  const bool few = (long long)nKV * Hkv * B <= std::min(2 * sms, kFewTiles);
+  // (A table's parts do not end with the heads: items side by side no longer sweep the same rows of Q and dQ, which is lost where
+  // these outgrow L2: 31232 tokens, 8 heads 4850 / 4980 us with it.)
+  const bool few = (long long)nKV * Hkv * B <= std::min(2 * sms, kFewTiles) && (long long)B * Hkv * G * Nq <= 131072;
   for (int h = 0; h < Hkv; ++h)
     for (int j = 0; j < nKV; ++j) {
       CowaRange rg[2];
@@ -1308,14 +1331,26 @@ CowaStrides packed_strides(int H, long long T, int D) {
   return st;
 }
 
+// What comes behind the main kernel.
 template <int D, bool VARLEN>
-cudaError_t launch_reduce(const BwdArgs& a, const BwdPlan& pl, const CowaStrides& sk, const CowaStrides& sv, cudaStream_t st) {
+cudaError_t launch_finish(const BwdArgs& a, const BwdPlan& pl, const CowaStrides& sk, const CowaStrides& sv, void* dq_, int T,
+                          const CowaStrides& sq, cudaStream_t st) {
+  __nv_bfloat16* const dq = static_cast<__nv_bfloat16*>(dq_);
+  const long long chunks = (long long)(a.Tpad / BQS) * a.Hq * (VARLEN ? 1 : a.B);
   long long shared = 0;
   for (int c = 0; c < 3; ++c)
-    if (pl.share > 0 || pl.run[c] > 1) shared += pl.tiles[c];
-  if (pl.share > 0 && pl.shared_blocks == shared) return cudaSuccess;  // a block per tile
-  if (shared == 0) return cudaSuccess;
-  return cowa::launch_chained(cowa_bwd_reduce_dkv_kernel<D, VARLEN>, dim3((unsigned)(shared * (BKV * (D / 8) / 256)), 2), 256, 0, st, a, sk, sv);
+    if (pl.run[c] > 1) shared += pl.tiles[c];
+  if (pl.few > 0) shared = (long long)pl.few_shared * a.B;
+  const long long sums = shared * kReduceBlocks<D>;
+  if (sums > 0) {
+    if (chunks <= kFinishChunks)
+      return cowa::launch_chained(cowa_bwd_finish_kernel<D, VARLEN>, dim3((unsigned)(2 * sums + chunks)), 256, 0, st, a, sk, sv,
+                                  (int)(2 * sums), dq, T, sq);
+    cudaError_t e = cowa::launch_chained(cowa_bwd_reduce_dkv_kernel<D, VARLEN>, dim3((unsigned)sums, 2), 256, 0, st, a, sk, sv);
+    if (e != cudaSuccess) return e;
+  }
+  return cowa::launch_chained(cowa_bwd_convert_dq_kernel<D, VARLEN>, dim3((unsigned)chunks), 256, 0, st, a.dq_acc, dq, a.cu, a.B, T,
+                              a.Tpad, a.Hq, a.dq_fixed, sq, a.status);
 }
 
 template <int D>
@@ -1356,7 +1391,10 @@ int launch_bwd(const void* q, const void* k, const void* v, const void* o, const
   a.wins = hw;
   a.sink_tiles = pl.sink_tiles;
   for (int c = 0; c < 3; ++c) { a.cls_tiles[c] = pl.tiles[c]; a.cls_parts[c] = pl.run[c]; }
-  a.share = pl.share; a.single = pl.blocks() <= cowa::sm_count();
+  a.single = pl.blocks() <= cowa::sm_count();
+  a.few = pl.few;
+  std::copy(pl.first, pl.first + pl.few + 1, a.first);
+  std::copy(pl.shared, pl.shared + pl.few_shared, a.shared);
   a.dq_fixed = p->deterministic ? 1 : 0;
   a.dkv_part = dkv_part;
   a.cu = nullptr; a.dk = static_cast<__nv_bfloat16*>(dk); a.dv = static_cast<__nv_bfloat16*>(dv); a.total = 0; a.tiles_bound = 0;
@@ -1374,9 +1412,7 @@ int launch_bwd(const void* q, const void* k, const void* v, const void* o, const
   if (p->bwd_main_start_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_start_event), st));
   COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_kernel<D, false>, dim3((unsigned)pl.blocks()), 512, BwdSmem<D>::kBytes, st, mq, mk, mv, mdo, mdk, mdv, mq2, mdo2, a));
   if (p->bwd_main_stop_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_stop_event), st));
-  COWA_CUDA_TRY((launch_reduce<D, false>(a, pl, sk, sv, st)));
-  COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_convert_dq_kernel<D, false>, dim3((unsigned)(Tpad / BQS * BH)), 256, 0, st, dq_acc,
-                                     static_cast<__nv_bfloat16*>(dq), nullptr, B, T, Tpad, Hq, a.dq_fixed, sq, a.status));
+  COWA_CUDA_TRY((launch_finish<D, false>(a, pl, sk, sv, dq, T, sq, st)));
   return COWA_OK;
 }
 
@@ -1417,7 +1453,8 @@ int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o
   a.wins = hw;
   a.sink_tiles = pl.sink_tiles;
   for (int c = 0; c < 3; ++c) { a.cls_tiles[c] = pl.tiles[c]; a.cls_parts[c] = pl.run[c]; }
-  a.share = pl.share; a.single = pl.blocks() <= cowa::sm_count();
+  a.single = pl.blocks() <= cowa::sm_count();
+  a.few = 0;
   a.dq_fixed = p->deterministic ? 1 : 0;
   a.dkv_part = delta + (size_t)Hq * Tpad;
   a.cu = cu; a.dk = static_cast<__nv_bfloat16*>(dk); a.dv = static_cast<__nv_bfloat16*>(dv);
@@ -1436,9 +1473,7 @@ int launch_bwd_varlen(const void* q, const void* k, const void* v, const void* o
   if (p->bwd_main_start_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_start_event), st));
   COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_kernel<D, true>, dim3((unsigned)pl.blocks()), 512, BwdSmem<D>::kBytes, st, mq, mk, mv, mdo, mdk, mdv, mq2, mdo2, a));
   if (p->bwd_main_stop_event) COWA_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(p->bwd_main_stop_event), st));
-  COWA_CUDA_TRY((launch_reduce<D, true>(a, pl, sk, sk, st)));
-  COWA_CUDA_TRY(cowa::launch_chained(cowa_bwd_convert_dq_kernel<D, true>, chunks, 256, 0, st, dq_acc, static_cast<__nv_bfloat16*>(dq), cu,
-                                     B, total, Tpad, Hq, a.dq_fixed, sq, a.status));
+  COWA_CUDA_TRY((launch_finish<D, true>(a, pl, sk, sk, dq, total, sq, st)));
   return COWA_OK;
 }
 
