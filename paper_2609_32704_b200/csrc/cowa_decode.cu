@@ -50,15 +50,22 @@ void* static_scratch_ptr(cudaError_t* err) {
   return cache[dev];
 }
 
+constexpr int kShareSeqs = 128;  // up to so many sequences every warp looks at all lengths (four a lane)
+constexpr int kMinChunk = 64;    // rows of a split, where there is a choice
+
 struct DecodeArgs {
   const __nv_bfloat16* q;
   const __nv_bfloat16* kc;
   const __nv_bfloat16* vc;
   const int32_t* lens;
-  float* ws_o;  // [B, Hq, S, D]
-  float* ws_m;  // [B, Hq, S]
-  float* ws_l;  // [B, Hq, S]
-  int B, Tmax, Hq, Hkv, S;
+  float* ws_o;  // [splits, G, D]
+  float* ws_m;  // [splits, G]
+  float* ws_l;  // [splits, G]
+  int B, Tmax, Hq, Hkv;
+  int S;        // splits of a (sequence, KV head), on average where they are shared out: the grid is (S, Hkv, B)
+  int shared;   // splits by the sequences' lengths (Shares)
+  float inv_room;       // 1 / (B * S)
+  unsigned head_magic;  // x / hkv_global = (x * head_magic) >> 32 for all lengths up to Tmax; 0: it does not hold
   CowaStrides sk, sv;  // element strides (batch, head, token) of the contiguous-row cache
   int sink, near, hkv_global, hkv_offset, full_attn;
   float scale_log2;
@@ -69,6 +76,100 @@ struct VisMap {
   int lo0, n0, lo1, n1, lo2;
   __device__ __forceinline__ int token(int v) const {
     return v < n0 ? lo0 + v : (v < n0 + n1 ? lo1 + (v - n0) : lo2 + (v - n0 - n1));
+  }
+};
+
+// Rows that a head sees of a sequence of Nk keys (the widest band's head).
+__device__ __forceinline__ int visible_rows(const DecodeArgs& a, int Nk) {
+  const int far = Nk - a.sink - a.near;
+  if (a.full_attn || far <= 0) return max(Nk, 0);
+  const int x = far + a.hkv_global - 1;
+  return a.sink + a.near + (a.head_magic ? (int)__umulhi((unsigned)x, a.head_magic) : x / a.hkv_global);
+}
+
+// How the splits are shared out between sequences of different lengths: the shortest chunk, a multiple of 16 rows, with which
+// all sequences together need no more splits than the grid has blocks.  (With the same number of splits for every sequence a
+// batch waits for its longest: 16 sequences of 3600 to 33800 tokens 48 us, so 40.)  Warp-cooperative.
+struct Shares {
+  static constexpr int kPer = kShareSeqs / 32;
+  int rows[kPer];  // in 16 rows, of sequences lane, lane + 32, ..., -1 past the last one
+  int B, k;        // k: a split's rows / 16
+  unsigned magic;  // x / k = (x * magic) >> 32 for x * k < 2^32
+  __device__ __forceinline__ int splits_of(int i) const {
+    return rows[i] < 0 ? 0 : max((int)__umulhi((unsigned)(rows[i] + k - 1), magic), 1);
+  }
+  __device__ __forceinline__ int count(int k_) {
+    k = k_;
+    magic = 0xFFFFFFFFu / (unsigned)k + 1;
+    int n = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+      if (i * 32 < B) n += splits_of(i);
+    return __reduce_add_sync(0xffffffffu, n);
+  }
+  __device__ __forceinline__ explicit Shares(const DecodeArgs& a) : B(a.B) {
+    const int lane = threadIdx.x & 31;
+    int sum = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      rows[i] = -1;
+      if (i * 32 < B) {
+        if (i * 32 + lane < B) rows[i] = (visible_rows(a, min(a.lens[i * 32 + lane], a.Tmax)) + 15) >> 4;
+        sum += max(rows[i], 0);
+      }
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    const int room = B * a.S, hi = kChunkCap / 16 - 1;  // per KV head; with chunks of hi there is room (splits_for)
+    int at = min(max((int)((float)sum * a.inv_room) + 1, kMinChunk / 16), hi), low = at - 1;  // too short, or nearly: low
+    for (int step = 1; count(at) > room && at < hi; step *= 2) {
+      low = at;
+      at = min(at + step, hi);
+    }
+    while (at - low > 1) {
+      const int mid = (low + at) >> 1;
+      if (count(mid) <= room) at = mid;
+      else low = mid;
+    }
+    if (k != at) count(at);
+  }
+  __device__ __forceinline__ int chunk() const { return k * 16; }
+  // Splits of one KV head of the sequences before b, and of sequence b.
+  __device__ __forceinline__ void of(int b, int* before, int* mine) const {
+    int n = 0, m = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+      if (i * 32 < B) {
+        const int x = splits_of(i);
+        if (i * 32 + (int)(threadIdx.x & 31) < b) n += x;
+        if (i == b >> 5) m = x;
+      }
+    *before = __reduce_add_sync(0xffffffffu, n);
+    *mine = __shfl_sync(0xffffffffu, m, b & 31);
+  }
+  // The sequence of split idx (counted over all heads), -1 past the last one, and the two numbers above.
+  __device__ __forceinline__ int at(int idx, int Hkv, int* before, int* mine) const {
+    const int lane = threadIdx.x & 31;
+    int base = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+      if (i * 32 < B) {
+        const int n = splits_of(i);
+        int incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += y;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, idx < (base + incl) * Hkv);
+        if (m) {
+          const int src = __ffs(m) - 1;
+          *before = base + __shfl_sync(0xffffffffu, incl - n, src);
+          *mine = __shfl_sync(0xffffffffu, n, src);
+          return i * 32 + src;
+        }
+        base += __shfl_sync(0xffffffffu, incl, 31);
+      }
+    return -1;
   }
 };
 
@@ -92,7 +193,8 @@ __device__ __forceinline__ uint4 ldg128(const void* p) {
 // G = columns of the mma n-tile in use: the query heads of the group.
 template <int D, int G>
 // 5 blocks per SM (up to 102 registers, no spills) measured best: fewer, longer splits than at 7 per SM
-__global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const DecodeArgs a) {
+// (D = 64, groups below 8: 7 as before the shares, whose registers cost one otherwise)
+__global__ void __launch_bounds__(kThreads, D == 64 && G < 8 ? 7 : 5) cowa_decode_split_kernel(const DecodeArgs a) {
   static_assert(D == 64 || D == 128, "head dim");
   static_assert(G >= 1 && G <= 8, "group size per mma n-tile");
   constexpr int KC = D / 32;          // 32-wide d chunks (two k16 steps each)
@@ -101,9 +203,17 @@ __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const De
   __shared__ float m_s[G], l_s[G];
 
   cowa_ptx::grid_enter();  // the merge kernel's blocks may be scheduled beside this one's; they wait for its results
-  const int split = blockIdx.x, hk = blockIdx.y;
-  const int b = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  int split = blockIdx.x, hk = blockIdx.y, b = blockIdx.z, S = a.S, chunk = 0;
+  const int slot = (b * a.Hkv + hk) * S + split;  // of this block's state
+  if (a.shared) {
+    const Shares sh(a);
+    int before;
+    b = sh.at(slot, a.Hkv, &before, &S);
+    if (b < 0) return;
+    const int i = slot - before * a.Hkv;
+    hk = (int)__fdividef(i + 0.5f, (float)S); split = i - hk * S; chunk = sh.chunk();  // (i and S are small)
+  }
   const int Nk = a.lens[b];
 
   // visible ranges of this head for the current key length
@@ -112,7 +222,7 @@ __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const De
   else w = cowa_default_window(Nk, a.hkv_global, a.hkv_offset + hk, a.sink, a.near);
   CowaRange rg[3];
   const int nr = cowa_decode_ranges(w, Nk, rg);
-  // index of column c in q, o, lse and the split states ([B, Hq] order)
+  // index of column c in q ([B, Hq] order)
   auto col = [&](int c) -> size_t { return (size_t)b * a.Hq + (size_t)hk * G + c; };
   // address of cache row `tok` of this (sequence, KV head)
   auto row_ptr = [&](const __nv_bfloat16* base, const CowaStrides& cs, int tok) -> const __nv_bfloat16* {
@@ -125,19 +235,31 @@ __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const De
   const int n2 = nr > 2 ? rg[2].hi - rg[2].lo + 1 : 0;
   const int V = vm.n0 + vm.n1 + n2;
 
-  int chunk = (V + a.S - 1) / a.S;
-  chunk = (chunk + 15) & ~15;
+  if (chunk == 0) chunk = ((V + S - 1) / S + 15) & ~15;
   const int c0 = split * chunk;
   const int clen = min(chunk, V - c0);  // <= kChunkCap by the host's choice of S
+  float* const out_o = a.ws_o + (size_t)slot * (G * D);
+  float* const out_m = a.ws_m + (size_t)slot * G;
+  float* const out_l = a.ws_l + (size_t)slot * G;
 
   if (clen <= 0) {  // empty split: neutral partial state
-    for (int i = tid; i < G * D; i += kThreads)
-      a.ws_o[(col(i / D) * a.S + split) * D + (i % D)] = 0.f;
+    for (int i = tid; i < G * D; i += kThreads) out_o[i] = 0.f;
     if (tid < G) {
-      a.ws_m[col(tid) * a.S + split] = -INFINITY;
-      a.ws_l[col(tid) * a.S + split] = 0.f;
+      out_m[tid] = -INFINITY;
+      out_l[tid] = 0.f;
     }
     return;
+  }
+  // Short splits: V is on its way to L2 while K is read and weighed (one row of each thread here; 8K of context, one sequence
+  // 8.8 us, so 7.9).  Long ones have enough in flight, and all of them together would not fit L2.
+  if (chunk <= 2 * kThreads) {
+#pragma unroll
+    for (int r = tid; r < 2 * kThreads; r += kThreads)
+      if (r < clen) {
+        const char* row = reinterpret_cast<const char*>(row_ptr(a.vc, a.sv, vm.token(c0 + r)));
+#pragma unroll
+        for (int i = 0; i < D * 2; i += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + i));
+      }
   }
 
   // ---------------- phase 1: scores ----------------
@@ -261,89 +383,88 @@ __global__ void __launch_bounds__(kThreads, 5) cowa_decode_split_kernel(const De
     float s = 0.f;
 #pragma unroll
     for (int r = 0; r < kThreads / 32; ++r) s += sc[r * G * D + i];
-    a.ws_o[(col(i / D) * a.S + split) * D + (i % D)] = s;
+    out_o[i] = s;
   }
   if (tid < G) {
-    a.ws_m[col(tid) * a.S + split] = m_s[tid];
-    a.ws_l[col(tid) * a.S + split] = l_s[tid];
+    out_m[tid] = m_s[tid];
+    out_l[tid] = l_s[tid];
   }
 }
 
 // Merge of the split states: M = max m_s, L = sum l_s 2^(m_s - M), o = sum o_s 2^(m_s - M) / L,
-// lse = ln2 * (M + log2 L).  One block of 4 warps per (sequence, QO head): every warp reduces M and L
-// with shuffles, takes every fourth split with D/32 columns per lane (several loads in flight), and the
-// four partial sums meet in shared memory.
-template <int D>
-__global__ void __launch_bounds__(128) cowa_decode_combine_kernel(const float* ws_o, const float* ws_m, const float* ws_l,
-                                                                  __nv_bfloat16* o, float* lse, int S) {
-  constexpr int V = D / 32;  // columns per lane
-  __shared__ float part[4][D];
-  const size_t bh = blockIdx.x;
+// lse = ln2 * (M + log2 L).  One block per (sequence, QO head).  A warp takes every W-th group of eight splits, D/32 columns per
+// lane, states and O in one round trip; the running maximum moves between its groups, and the warps' results meet in shared
+// memory.  W: four warps where eight splits a warp are all there are, sixteen for more (one sequence of 57 700 visible rows in
+// 452 splits: with four warps 16 us of 29 were this kernel).
+template <int D, int W>
+__global__ void __launch_bounds__(W * 32) cowa_decode_combine_kernel(const DecodeArgs a, __nv_bfloat16* o, float* lse) {
+  constexpr int V = D / 32, U = 8;  // columns per lane, splits of a group
+  __shared__ float part[W][D], part_m[W], part_l[W];
+  const int bh = blockIdx.x, b = bh / a.Hq, h = bh % a.Hq, G = a.Hq / a.Hkv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  cowa_ptx::grid_enter();  // the split kernel's states are complete and visible
-  const float* m = ws_m + bh * S;
-  const float* l = ws_l + bh * S;
-  const float* po = ws_o + bh * S * D + lane * V;
-  float acc[V];
+  // The lengths are not written by the split kernel and were complete before it began (grid_wait); its states are after the wait.
+  int before = b * a.S, S = a.S;
+  if (a.shared) Shares(a).of(b, &before, &S);
+  cowa_ptx::grid_enter();
+  const size_t first = ((size_t)before * a.Hkv + (size_t)(h / G) * S) * G + h % G;  // split s lies s * G further
+  const float* po = a.ws_o + first * D + lane * V;
+  float mx = -INFINITY, L = 0.f, acc[V];
 #pragma unroll
   for (int i = 0; i < V; ++i) acc[i] = 0.f;
-  float mx = -INFINITY, L = 0.f;
-  constexpr int U = 8;
-  if (S <= 32) {
-    // one round trip: every load is issued before the first use
-    const float ms = lane < S ? m[lane] : -INFINITY;
-    const float ls = lane < S ? l[lane] : 0.f;
+  for (int s0 = warp * U; s0 < S; s0 += W * U) {
+    const bool in = lane < U && s0 + lane < S;
+    const float ms = in ? a.ws_m[first + (size_t)(s0 + lane) * G] : -INFINITY;
+    const float ls = in ? a.ws_l[first + (size_t)(s0 + lane) * G] : 0.f;
     float x[U][V];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int s = warp + 4 * u;
-#pragma unroll
-      for (int i = 0; i < V; ++i) x[u][i] = s < S ? po[(size_t)s * D + i] : 0.f;
+      const float* src = po + (size_t)(s0 + u) * G * D;
+      if constexpr (V == 4) {
+        const float4 y = s0 + u < S ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+        x[u][0] = y.x; x[u][1] = y.y; x[u][2] = y.z; x[u][3] = y.w;
+      } else {
+        const float2 y = s0 + u < S ? *reinterpret_cast<const float2*>(src) : make_float2(0.f, 0.f);
+        x[u][0] = y.x; x[u][1] = y.y;
+      }
     }
-    mx = ms;
+    float m = ms;
 #pragma unroll
-    for (int o_ = 16; o_ > 0; o_ >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o_));
-    const float wl = exp2f(ms - mx);  // empty splits: m = -inf -> weight 0
-    L = ls * wl;
+    for (int k = U / 2; k > 0; k >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, k));
+    m = fmaxf(__shfl_sync(0xffffffffu, m, 0), mx);
+    const float old = mx == -INFINITY ? 0.f : exp2f(mx - m), w = ms == -INFINITY ? 0.f : exp2f(ms - m);
+    mx = m;
+    float l = ls * w;
 #pragma unroll
-    for (int o_ = 16; o_ > 0; o_ >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o_);
+    for (int k = U / 2; k > 0; k >>= 1) l += __shfl_xor_sync(0xffffffffu, l, k);
+    L = L * old + __shfl_sync(0xffffffffu, l, 0);
+#pragma unroll
+    for (int i = 0; i < V; ++i) acc[i] *= old;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const float wgt = __shfl_sync(0xffffffffu, wl, (warp + 4 * u) & 31);
+      const float wu = __shfl_sync(0xffffffffu, w, u);
 #pragma unroll
-      for (int i = 0; i < V; ++i) acc[i] = fmaf(x[u][i], wgt, acc[i]);
-    }
-  } else {
-    for (int s = lane; s < S; s += 32) mx = fmaxf(mx, m[s]);
-#pragma unroll
-    for (int o_ = 16; o_ > 0; o_ >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o_));
-    for (int s = lane; s < S; s += 32) L += l[s] * exp2f(m[s] - mx);
-#pragma unroll
-    for (int o_ = 16; o_ > 0; o_ >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o_);
-    for (int s0 = warp; s0 < S; s0 += 4 * U) {
-      float x[U][V], wgt[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int s = s0 + 4 * u;
-        const bool in = s < S;
-        wgt[u] = in ? exp2f(m[s] - mx) : 0.f;
-#pragma unroll
-        for (int i = 0; i < V; ++i) x[u][i] = in ? po[(size_t)s * D + i] : 0.f;
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int i = 0; i < V; ++i) acc[i] = fmaf(x[u][i], wgt[u], acc[i]);
+      for (int i = 0; i < V; ++i) acc[i] = fmaf(x[u][i], wu, acc[i]);
     }
   }
 #pragma unroll
   for (int i = 0; i < V; ++i) part[warp][lane * V + i] = acc[i];
+  if (lane == 0) { part_m[warp] = mx; part_l[warp] = L; }
   __syncthreads();
   if (tid < D) {
-    const float v = (part[0][tid] + part[1][tid]) + (part[2][tid] + part[3][tid]);
-    o[bh * D + tid] = __float2bfloat16_rn(v / L);
+    mx = part_m[0];
+#pragma unroll
+    for (int k = 1; k < W; ++k) mx = fmaxf(mx, part_m[k]);
+    L = 0.f;
+    float v = 0.f;
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+      const float w = part_m[k] == -INFINITY ? 0.f : exp2f(part_m[k] - mx);
+      L = fmaf(part_l[k], w, L);
+      v = fmaf(part[k][tid], w, v);
+    }
+    o[(size_t)bh * D + tid] = __float2bfloat16_rn(v / L);
+    if (lse && tid == 0) lse[bh] = 0.6931471805599453f * (mx + log2f(L));
   }
-  if (lse && tid == 0) lse[bh] = 0.6931471805599453f * (mx + log2f(L));
 }
 
 // Upper bound of visible rows per head for any key length <= Tmax.
@@ -406,14 +527,16 @@ int pick_splits(int B, int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p)
 }
 
 template <int D>
-cudaError_t launch_combine(unsigned rows, const float* ws_o, const float* ws_m, const float* ws_l, __nv_bfloat16* o,
-                           float* lse, int S, cudaStream_t st) {
-  return cowa::launch_chained(cowa_decode_combine_kernel<D>, dim3(rows), 128, 0, st, ws_o, ws_m, ws_l, o, lse, S);
+cudaError_t launch_combine(const DecodeArgs& a, __nv_bfloat16* o, float* lse, cudaStream_t st) {
+  const dim3 rows((unsigned)(a.B * a.Hq));
+  // (where they are shared out, the longest of a batch may have some times the average)
+  if (a.S > (a.shared ? 16 : 32)) return cowa::launch_chained(cowa_decode_combine_kernel<D, 16>, rows, 512, 0, st, a, o, lse);
+  return cowa::launch_chained(cowa_decode_combine_kernel<D, 4>, rows, 128, 0, st, a, o, lse);
 }
 
 template <int D, int G>
 cudaError_t launch_split(const DecodeArgs& a, cudaStream_t st) {
-  dim3 grid(a.S, a.Hkv, a.B);
+  const dim3 grid(a.S, a.Hkv, a.B);
   return cowa::launch_chained(cowa_decode_split_kernel<D, G>, grid, kThreads, 0, st, a);
 }
 
@@ -474,12 +597,19 @@ int decode_launch(const void* q, const void* kc, const void* vc, const int32_t* 
   a.hkv_global = p->hkv_global > 0 ? p->hkv_global : Hkv;
   a.hkv_offset = p->hkv_offset;
   a.full_attn = p->full_attn;
+  // Sharing out costs a block 0.4 us, more than short splits can gain (up to 128 rows they are as many as there is length for).
+  // Of several waves a longer block is made up for by the blocks that follow, and equal ones keep in step, so that memory idles
+  // while all of them weigh their scores (32 sequences of 1500 to 2600 tokens, 8 groups of one head: 46.9 us, shared out 52).
+  a.shared = B > 1 && B <= kShareSeqs && (long long)S * 128 < max_visible(Tmax, a.hkv_global, p) &&
+             (long long)B * Hkv * S <= resident_blocks(D, Hq / Hkv);
+  a.inv_room = 1.f / ((float)B * S);
+  a.head_magic = a.hkv_global > 1 && ((long long)Tmax + a.hkv_global) * a.hkv_global <= 0xFFFFFFFFll ? 0xFFFFFFFFu / a.hkv_global + 1 : 0;
   a.scale_log2 = p->softmax_scale * 1.4426950408889634f;
   const int G = Hq / Hkv;
   cudaError_t e = (D == 128) ? dispatch_split<128>(G, a, st) : dispatch_split<64>(G, a, st);
   if (e != cudaSuccess) return record_cuda_error(e);
-  e = (D == 128) ? launch_combine<128>((unsigned)(B * Hq), a.ws_o, a.ws_m, a.ws_l, static_cast<__nv_bfloat16*>(o), lse, S, st)
-                 : launch_combine<64>((unsigned)(B * Hq), a.ws_o, a.ws_m, a.ws_l, static_cast<__nv_bfloat16*>(o), lse, S, st);
+  e = (D == 128) ? launch_combine<128>(a, static_cast<__nv_bfloat16*>(o), lse, st)
+                 : launch_combine<64>(a, static_cast<__nv_bfloat16*>(o), lse, st);
   if (e != cudaSuccess) return record_cuda_error(e);
   return COWA_OK;
 }

@@ -30,8 +30,15 @@ COWA_HD int cowa_imax(int a, int b) { return a > b ? a : b; }
 COWA_HD CowaWin cowa_default_window(int Nk, int Hk_global, int h_global, int s, int n) {
   long long L = (long long)Nk - s - n;
   if (L < 0) L = 0;
-  int b0 = (int)(((long long)h_global * L) / Hk_global);
-  int b1 = (int)(((long long)(h_global + 1) * L) / Hk_global);
+  int b0, b1;
+  const unsigned long long end = (unsigned long long)(h_global + 1) * L;
+  if (end <= 0xFFFFFFFFull) {  // as for nearly every call: a 64-bit division is some 100 instructions on the device
+    b0 = (int)(((unsigned)end - (unsigned)L) / (unsigned)Hk_global);
+    b1 = (int)((unsigned)end / (unsigned)Hk_global);
+  } else {
+    b0 = (int)(((long long)h_global * L) / Hk_global);
+    b1 = (int)(((long long)(h_global + 1) * L) / Hk_global);
+  }
   CowaWin w;
   w.s = s; w.n = n; w.g = b0; w.l = b1 - b0;
   return w;

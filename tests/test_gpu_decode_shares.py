@@ -1,0 +1,47 @@
+"""Decode of batches of very different lengths, whose splits are shared out by length, against the float64 oracle: sequences of a few
+rows beside long ones, lengths at the borders of a split, as many sequences as are shared out at most and one more."""
+import numpy as np
+import pytest
+import torch
+
+import cowa_inputs
+import paper_2609_32704_b200 as cowa
+from oracle import cowa_oracle as orc
+from test_gpu_parity import DEV, TOL_LSE, check
+
+pytestmark = pytest.mark.gpu
+
+
+def lengths(B, longest):
+    """From one token up, the longest first or last by turns."""
+    n = [max(1, longest * (i * i + 1) // (B * B)) for i in range(B)]
+    n[-1] = longest
+    return n[::-1] if B % 2 else n
+
+
+@pytest.mark.parametrize("B,longest,Hq,Hkv,D,sink,local", [
+    (2, 33000, 8, 1, 128, 64, 3000),
+    (16, 30000, 16, 2, 128, 64, 3481),
+    (8, 20000, 4, 2, 64, 0, 5000),
+    (33, 9000, 4, 4, 64, 4, 2500),
+    (127, 12000, 2, 1, 64, 16, 4000),
+    (128, 12000, 2, 1, 64, 16, 4000),
+    (129, 12000, 2, 1, 64, 16, 4000),
+    (5, 60000, 2, 1, 128, 128, 151),  # one sequence has nearly all splits
+])
+def test_splits_by_length(B, longest, Hq, Hkv, D, sink, local):
+    lens = lengths(B, longest)
+    q, k, v, _ = cowa_inputs.make_decode_inputs(17, B, longest, Hq, Hkv, D, longest, longest)
+    scale = cowa_inputs.softmax_scale(D)
+    params = cowa.make_params(sink=sink, local=local, softmax_scale=scale)
+    o = torch.full((B, Hq, D), float("nan"), dtype=torch.bfloat16, device=DEV)
+    lse = torch.full((B, Hq), float("nan"), device=DEV)
+    ws = torch.empty(cowa.cowa_decode_workspace_bytes(B, longest, Hq, Hkv, D, params), dtype=torch.uint8, device=DEV)
+    cowa.cowa_decode(q.to(DEV), k.to(DEV), v.to(DEV), torch.tensor(lens, dtype=torch.int32, device=DEV), o, lse, params, ws)
+    torch.cuda.synchronize()
+    f = cowa_inputs.to_f64
+    for b in sorted({0, 1, B // 2, B - 2, B - 1}):
+        n = lens[b]
+        o_ref, lse_ref = orc.decode(f(q[b:b + 1]), f(k[b:b + 1, :, :n]), f(v[b:b + 1, :, :n]), np.array([n]), sink, local, scale)
+        check(f"o[b={b}]", o[b:b + 1].float().cpu().numpy(), o_ref)
+        check(f"lse[b={b}]", lse[b:b + 1].cpu().numpy(), lse_ref, TOL_LSE, TOL_LSE)
