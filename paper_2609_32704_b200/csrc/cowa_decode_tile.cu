@@ -50,11 +50,12 @@ struct Unit {
   int nt;  // visited 64-key tiles
 };
 
-__device__ __forceinline__ void unit_of(const TileArgs& a, int u, Unit& x) {
+__device__ __forceinline__ int length_of(const TileArgs& a, int u) { return a.lens[u / (a.ntiles * a.Hkv)]; }
+__device__ __forceinline__ void unit_of(const TileArgs& a, int u, int Nk, Unit& x) {  // Nk: length_of(a, u)
   const int tile = u % a.ntiles;
   const int bh = u / a.ntiles;
   x.hk = bh % a.Hkv; x.b = bh / a.Hkv;
-  x.Nk = a.lens[x.b];
+  x.Nk = Nk;
   x.off = x.Nk - a.Nq;
   x.tok0 = tile * a.tpt; x.tok1 = min(x.tok0 + a.tpt, a.Nq);
   if (a.full_attn) { x.w.s = 0; x.w.n = x.Nk; x.w.g = 0; x.w.l = 0; }
@@ -179,7 +180,6 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bar_k_full + 6 * NS);
   int* scan = reinterpret_cast<int*>(smem + SM::oScan);  // 6 warp totals; [8], [9] first unit and its list position; [10 ..] per slot: step whose V is not finite
 
-  grid_enter();  // the merge kernel's blocks may be scheduled beside this one's; they wait for its results
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform by construction
   const int nw = (a.rows + 31) >> 5;                       // softmax warps with rows
@@ -193,6 +193,7 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     for (int s = 0; s < NS; ++s) scan[10 + s] = 0;
     fence_mbar_init();
   }
+  grid_enter();  // the merge kernel's blocks may be scheduled beside this one's; they wait for its results
   if (warp == 5) {
     __syncwarp();
     tmem_alloc(tmem_holder, TMEM_COLS);
@@ -200,13 +201,20 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   }
 
   // ---- this block's share of the list of all units' steps ----
+  // Every instruction here delays the first load of K.  A thread works out two units at a time, side by side (their divisions are long
+  // chains), keeps the step counts of the first two, and the block's first unit is handed on as it was worked out.  (One unit
+  // after the other, found and handed on by its number, with 64-bit divisions: 2.9 us for 256 units, so 1.6.)
   const int per = (a.units + kThreads - 1) / kThreads;
   const int u_lo = min(tid * per, a.units), u_hi = min(u_lo + per, a.units);
+  Unit first[2];  // of this thread
   int sum = 0;
-  for (int u = u_lo; u < u_hi; ++u) {
-    Unit x;
-    unit_of(a, u, x);
-    sum += x.nt;
+  for (int u0 = u_lo; u0 < u_hi; u0 += 2) {
+    Unit x[2];
+    const int len0 = length_of(a, u0), len1 = length_of(a, min(u0 + 1, a.units - 1));
+    unit_of(a, u0, len0, x[0]);
+    unit_of(a, min(u0 + 1, a.units - 1), len1, x[1]);
+    sum += x[0].nt + (u0 + 1 < u_hi ? x[1].nt : 0);
+    if (u0 == u_lo) { first[0] = x[0]; first[1] = x[1]; }
   }
   int incl = sum;
 #pragma unroll
@@ -229,12 +237,16 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   const int excl = base + incl - sum;
   if (lo < hi && excl <= lo && lo < excl + sum) {
     int f = excl, u = u_lo;
-    for (; u < u_hi; ++u) {
-      Unit x;
-      unit_of(a, u, x);
-      if (lo < f + x.nt) break;
-      f += x.nt;
+    Unit x = first[0];
+    if (lo >= f + x.nt) {
+      f += x.nt; ++u;
+      x = first[1];
+      while (lo >= f + x.nt) {  // (more than two units a thread)
+        f += x.nt; ++u;
+        unit_of(a, u, length_of(a, u), x);
+      }
     }
+    *reinterpret_cast<Unit*>(smem + SM::oPiece + 128) = x;  // (the slot of the second piece)
     scan[8] = u; scan[9] = f;
   }
   tc_fence_before();
@@ -296,11 +308,19 @@ cowa_decode_tile_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     uint32_t rnd = 0;   // times the slots have been gone through
     uint32_t ni = 0;    // pieces so far
     int pos = lo, u = lo < hi ? scan[8] : 0, f = lo < hi ? scan[9] : 0;
+    Unit unit;  // u
+    if (lo < hi) unit = *reinterpret_cast<const Unit*>(smem + SM::oPiece + 128);
+    __syncwarp();
+    int Nk = 0;  // length of unit u, where `unit` has not been worked out
+    bool have = true;
     while (ok) {
       Piece pc;
       pc.n = 0;
       if (pos < hi) {
-        unit_of(a, u, pc.u);
+        if (have) pc.u = unit;
+        else unit_of(a, u, Nk, pc.u);
+        have = false;
+        Nk = length_of(a, min(u + 1, a.units - 1));  // of the next one, before it is needed
         if (pc.u.nt == 0) { ++u; continue; }
         pc.t0 = pos - f;
         pc.n = min(pc.u.nt, hi - f) - pc.t0;
@@ -636,7 +656,7 @@ __global__ void __launch_bounds__(WPR == 1 ? 128 : WPR * 32) cowa_decode_tile_me
   const int tile = t / a.tpt, row = (t - tile * a.tpt) * a.G + h % a.G;
   const int u = (b * a.Hkv + h / a.G) * a.ntiles + tile;
   Unit x;
-  unit_of(a, u, x);  // reads the lengths, which the tile kernel does not write: complete before that one began (grid_wait)
+  unit_of(a, u, length_of(a, u), x);  // reads the lengths, which the tile kernel does not write: complete before that one began (grid_wait)
   grid_enter();      // the row states are complete and visible
   const int2 info = x.nt > 0 ? a.ws_unit[u] : make_int2(0, 0);  // no visible key: 0 / 0
   const size_t first = (size_t)(info.x + u) * a.rows + row;  // piece i lies a.rows rows further
