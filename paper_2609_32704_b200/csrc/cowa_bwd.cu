@@ -36,6 +36,9 @@
 //                   its own, and the lanes that M = 128 leaves over hold it a second time, so that four warps
 //                   drain it instead of two: a step of 3420 clocks waited 500 for dP^T and 450 for S^T(n+1).  us: 35584
 //                   tokens, 32 heads 3433 -> 3190; 3840 x 4, 16 heads, reproducible 347 -> 296; 11120 x 2, 4 heads 252 -> 230.
+//                   A second buffer for dO, which dP^T waited 250 clocks of the remaining 2835 for: 3280 -> 3155, 298 -> 291,
+//                   234 -> 229.  What is left there is the chain of the compute warps; exponentials on the FMA pipe (one pair
+//                   in eight or four) change nothing.
 //                   Items are ordered sink tiles first (they meet every query tile), then
 //                   head by head with ascending KV tile, so that the blocks in flight sweep the same
 //                   dQ rows at nearly the same time and the reductions hit in L2.
@@ -69,7 +72,9 @@ namespace {
 constexpr int BKV = 128;  // KV rows per block (MMA M)
 constexpr int BQT = 128;  // QO rows per step (MMA N of S^T / dP^T): two tiles
 constexpr int BQS = 64;   // rows of a QO tile, unit of the padded row space and of the plan's step counts
-constexpr int NST = 2;    // Q stages (Q(n) is read again by dK(n) after S^T(n+1)); dO has one
+constexpr int NST = 2;    // Q stages (Q(n) is read again by dK(n) after S^T(n+1))
+template <int D>
+constexpr int NDO = D == 64 ? 2 : 1;  // dO stages: all that there is room for
 constexpr int kNoTile = 0x7FFFFF00;  // in place of a step's second tile: no query of it sees anything
 constexpr int kFewTiles = 296;  // up to so many tiles a batched call's plan is a table
 constexpr float kDqFixedOne = 262144.f;  // 2^18: one unit of dQ in the fixed-point accumulation mode
@@ -107,13 +112,13 @@ struct BwdSmem {
   static constexpr int kKV = BKV * D * 2;      // K or V tile
   static constexpr int kQ = BQT * D * 2;       // Q or dO tile of a step
   static constexpr int kDS = BKV * BQS * 2;    // dS^T of half a step (bf16)
-  static constexpr int oK = 0, oV = kKV, oQ = 2 * kKV, oDO = oQ + NST * kQ, oDS = oDO + kQ;
+  static constexpr int oK = 0, oV = kKV, oQ = 2 * kKV, oDO = oQ + NST * kQ, oDS = oDO + NDO<D> * kQ;
   static constexpr int oVec = oDS + 2 * kDS;   // per stage: 128 floats lse2, 128 floats delta
   static constexpr int oDQ = oVec + NST * 1024;  // dQ staging: per drain warp two tiles of 32 query rows x 32 d, fp32
   static constexpr int oBar = oDQ + 8 * 4096;
-  static constexpr int oItem = oBar + 320;     // two work items
+  static constexpr int oItem = oBar + 352;     // two work items
   static constexpr int oNext = oItem + 192;    // the next item's number, as the hardware answers
-  static constexpr int kBytes = oNext + 16;    // 231952 B at D = 128 (limit 232448)
+  static constexpr int kBytes = oNext + 16;    // 231984 B at D = 128 (limit 232448)
 };
 
 __device__ __forceinline__ void bulk_load_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -216,8 +221,8 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   uint64_t* bar_v = bars + 6;
   uint64_t* bar_q_full = bars + 1;    // [2] Q, LSE, Delta of a step have landed
   uint64_t* bar_q_empty = bars + 3;   // [2] ... are consumed
-  uint64_t* bar_o_full = bars + 5;    // dO ...
-  uint64_t* bar_o_empty = bars + 28;
+  uint64_t* bar_o_full = bars + 37;   // [NDO] dO ...
+  uint64_t* bar_o_empty = bars + 39;  // [NDO]
   uint64_t* bar_s_full = bars + 7;    // S^T is in TMEM
   uint64_t* bar_s_read = bars + 8;    // count 256: S^T is in registers
   uint64_t* bar_p_ready = bars + 9;   // count 256: P^T written over the first half of S^T
@@ -246,9 +251,10 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     for (int s = 0; s < 2; ++s) {
       mbar_init(bar_q_full + s, 1); mbar_init(bar_q_empty + s, 1);
       mbar_init(bar_dq_free + s, 128);
+      mbar_init(bar_o_full + s, 1); mbar_init(bar_o_empty + s, 1);
       mbar_init(bar_i_full + s, 1); mbar_init(bar_i_empty + s, kItemReaders);
     }
-    mbar_init(bar_dq_full, 1); mbar_init(bar_o_full, 1); mbar_init(bar_o_empty, 1);
+    mbar_init(bar_dq_full, 1);
     mbar_init(bar_s_full, 1); mbar_init(bar_s_read, 256); mbar_init(bar_p_ready, 256);
     mbar_init(bar_dp_full, 1); mbar_init(bar_ds_ready, 256);
     mbar_init(bar_done, 1); mbar_init(bar_next, 1); mbar_init(bar_dk_out, 1); mbar_init(bar_dv_out, 1); mbar_init(bar_ask, 1);
@@ -278,6 +284,10 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     tc_fence_after();
   }
   constexpr uint32_t tmem_base = 0;  // the allocation is all of TMEM
+
+  // dO of step c: its stage, and the parity of its turn there
+  auto o_stage = [](int c) { return NDO<D> == 2 ? c & 1 : 0; };
+  auto o_turn = [](int c) { return (uint32_t)(NDO<D> == 2 ? c >> 1 : c) & 1; };
 
   bool ok = true;
   // Item number ni of this block has been published (its words stay until item_done); its steps, -1 when there are no more items.
@@ -452,11 +462,11 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           }
           // (dV of the item before has left the buffer of dO: behind dO's last product)
           if (n == 0 && c > 0) ok = mbar_wait(bar_dv_out, (kc - 1) & 1, a.status);
-          else if (c > 0) ok = mbar_wait(bar_o_empty, (c - 1) & 1, a.status);
+          else if (c >= NDO<D>) ok = mbar_wait(bar_o_empty + o_stage(c), o_turn(c) ^ 1, a.status);
           if (!ok) break;
           if (lead) {
-            mbar_expect_tx(bar_o_full, SM::kQ);
-            load_rows(sDO, &tmdO, &tmdO2, bar_o_full);
+            mbar_expect_tx(bar_o_full + o_stage(c), SM::kQ);
+            load_rows(sDO + o_stage(c) * SM::kQ, &tmdO, &tmdO2, bar_o_full + o_stage(c));
           }
           if (n == 0 && c > 0) {
             ok = mbar_wait(bar_dq_full, (c - 1) & 1, a.status);
@@ -568,7 +578,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             gemm_dq();
             commit(bar_dq_full);
           }
-          ok = mbar_wait(bar_o_full, par, a.status);
+          ok = mbar_wait(bar_o_full + o_stage(c), o_turn(c), a.status);
           if (!OWN_DQ && ok && c > 0) ok = mbar_wait(bar_dq_free, par ^ 1, a.status);
           if (!ok) return;
           if (n == 0) {
@@ -576,15 +586,15 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             if (!ok) return;
             clear_kv_tail(sV);
           }
-          clear_tail(sDO, st);
+          clear_tail(sDO + o_stage(c) * SM::kQ, st);
           tc_fence_after();
-          gemm_st(cDP, dV_k, dO_k0);
+          gemm_st(cDP, dV_k, dO_k0 + o_stage(c) * kQ16);
           commit(bar_dp_full);
           ok = mbar_wait(bar_p_ready, par, a.status);
           if (!ok) return;
           tc_fence_after();
-          gemm_acc(cDV, cS, dO_mn0, n > 0 ? 1u : 0u);
-          commit(bar_o_empty);
+          gemm_acc(cDV, cS, dO_mn0 + o_stage(c) * kQ16, n > 0 ? 1u : 0u);
+          commit(bar_o_empty + o_stage(c));
           if (n + 1 < N) {
             ok = mbar_wait(bar_q_full + (st ^ 1), ((c + 1) >> 1) & 1, a.status);
             if (!OWN_DQ && ok && c > 0) ok = mbar_wait(bar_dq_free + 1, par ^ 1, a.status);
@@ -765,7 +775,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       const bool is_dk = wg == 0;
       const int r = (warp & 3) * 32 + lane;
       if (N > 0) {
-        ok = is_dk ? mbar_wait(bar_done, kc & 1, a.status) : mbar_wait(bar_o_empty, (c - 1) & 1, a.status);
+        ok = is_dk ? mbar_wait(bar_done, kc & 1, a.status) : mbar_wait(bar_o_empty + o_stage(c - 1), o_turn(c - 1), a.status);
         if (!ok) break;
         ++kc;
       }
@@ -802,7 +812,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         const CowaStrides sd = is_dk ? a.sdk : a.sdv;
         __nv_bfloat16* const dst = (is_dk ? a.dk : a.dv) + (VARLEN ? 0 : (size_t)it->b * sd.b) + (size_t)it->hk * sd.h +
                                    (size_t)(it->rbase + it->k0 + r) * sd.t;
-        uint8_t* const sOut = (is_dk ? sDS : sDO) + r * 128;
+        uint8_t* const sOut = (is_dk ? sDS : sDO + o_stage(c - 1) * SM::kQ) + r * 128;
 #pragma unroll
         for (int q = 0; q < D / 32; ++q) {
           uint32_t ov[32];
