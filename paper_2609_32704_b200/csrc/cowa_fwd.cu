@@ -624,9 +624,8 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
   if (D == 128 && split == 1 && a.G % 2 == 0) {
     // Which kernel (us, one-head / pair kernel; at D = 64 the exponentials bound both, and the one-head kernel keeps them
     // busier):
-    //   No more items than clusters of two that the device holds, and a list long enough to pay for the merge: the item is
-    //     shared by a cluster of 2, 4 or 8 blocks, two steps each at least, as long as all clusters are resident.  Hq 32,
-    //     Hkv 8, Nq 128: 1816 keys 37.9 / 25.6, 4941 keys 85 / 36 with clusters of four; of eight, two waves, 54.
+    //   No more items than clusters of two that the device holds, and a list long enough to pay for the merge: two blocks share
+    //     an item.  Hq 32, Hkv 8, Nq 128: 1816 keys 37.9 / 25.6 (fewer items: the clusters above).
     //   Else the pair kernel pays when its larger items still share out evenly (the figures are from a fixed share of the
     //   items per block; now that blocks take items as they come free it has gained up to a fifth where the rule takes it,
     //   and the lines have been left where they are):
@@ -638,16 +637,14 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
     //     up to a tenth either way (T 6000, Hq 16, 2.5 items per SM: 0.90; T 2048, Hq 32, 1.7: 1.13).
     const long long items = tiles * (Hq / 2), judged = (long long)((qn + BQ - 1) / BQ) * B * (Hq / 2);
     if (items > 0x7FFFFFFFll) return COWA_ERR_UNSUPPORTED;
-    const bool shared = judged <= cowa::resident_clusters(2);
-    while (split < 8 && judged <= cowa::resident_clusters(split * 2) && keys >= 512 * split) split *= 2;
+    const bool shared = judged <= cowa::resident_pairs();
     const bool rounds = judged >= 3 * cowa::sm_count() || (alike ? keys >= 1536 : keys >= 1280 && 2 * judged >= 3 * cowa::sm_count());
     // Packed batches whose average sequence has fewer than 1024 keys to visit: three quarters of the items that there are at
     // least in fixed shares, the rest taken over (cowa_fwd_pair.cu).  Half is 2 to 4 % slower for equal lengths, nine tenths
     // 17 % for 24 of 60 to 7000 tokens, local 128; from 1024 keys on lists hide what taking over costs.
     const int share = VARLEN && keys < 1024 ? (int)(0.75 * (total_q / BQ) * (Hq / 2) / cowa::sm_count()) : 1;
     if (shared ? keys >= 1536 : rounds)
-      return cowa::launch_fwd_pair<128, VARLEN>(mq, mk, mv, mo, a, items, std::max(share, 1), split, st);
-    split = 1;
+      return cowa::launch_fwd_pair<128, VARLEN>(mq, mk, mv, mo, a, items, std::max(share, 1), shared ? 2 : 1, st);
   }
   auto launch = [&](auto kernel, int smem) -> int {
     COWA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));

@@ -23,13 +23,13 @@ struct FwdArgs {
 };
 
 namespace cowa {
-// Clusters of `size` (2, 4, 8) blocks of the pair kernel that the current device holds at once: a block takes an SM, and a
-// cluster lies within one GPC, so that large ones leave SMs out (74, 33 and 15 on the B200 measured).
-int resident_clusters(int size);
+// Clusters of two blocks of the pair kernel that the current device holds at once: a block takes an SM, and a cluster lies
+// within one GPC, so that some SMs may be left out (74 on the B200 measured).
+int resident_pairs();
 
 // Pair kernel (cowa_fwd_pair.cu; the tensor maps of the one-head kernel, 64-row boxes of K and V): two QO heads of a
 // group at a time, `items` = tiles x pairs of heads.  split = 1: a block per SM at a time, with `rounds` items for its share
-// and others taken over after them; split = 2, 4, 8: every item shared by a cluster of that many blocks.
+// and others taken over after them; split = 2: every item shared by a cluster of two blocks.
 template <int D, bool VARLEN>
 int launch_fwd_pair(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mo,
                     const FwdArgs& a, long long items, int rounds, int split, cudaStream_t st);

@@ -135,8 +135,8 @@ __device__ __forceinline__ bool locate_item(const FwdArgs& a, int idx, PairItem&
 
 // How the items are handed out (FORM).
 //   kTakenOver  an item per number of the grid; a block takes over the numbers whose blocks have not started
-//   kSplit      a cluster of blocks shares one item (few items, long lists): each takes a contiguous part of its steps, and
-//               the partial states are merged through distributed shared memory
+//   kSplit      two blocks, a cluster, share one item (few items, long lists): each takes half of its steps, and the partial
+//               states are merged through distributed shared memory
 //   kShares     as the first, but the first `starters` numbers stand for `rounds` items each, from alternate ends.  A number
 //               taken over costs a block up to a microsecond between two items, more than short lists hide, and so do the
 //               numbers past a packed batch's last item (us, a fixed share of all / all taken over / three quarters in
@@ -157,8 +157,7 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   constexpr uint32_t IDESC_S2 = idesc_bf16(128, BS, 0, 0), IDESC_S1 = idesc_bf16(128, BK, 0, 0);
   constexpr uint32_t IDESC_O = idesc_bf16(128, D, 0, 1);
 
-  if constexpr (SPLIT) grid_enter();
-  else grid_wait();
+  if constexpr (!SPLIT) grid_wait();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sQ = smem + SM::oQ;      // [2 heads][kQ]
@@ -189,15 +188,36 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       mbar_init(bars + s, (s >= 12 && s < 16) || s == 18 || s == 19 ? 4 : s == 22 || s == 23 ? kItemReaders : 1);
     fence_mbar_init();
   }
-  if (warp == 9) {
+  if (warp == 9 && !SPLIT) {
     __syncwarp();
     tmem_alloc(tmem_holder, TMEM_COLS);
     tmem_relinquish();
   }
-  tc_fence_before();
-  __syncthreads();
+  if constexpr (SPLIT) {
+    // One short item a block: the TMA warp works out a batched call's item ahead of the wait for the kernel before, and does not
+    // wait for TMEM, which is allocated behind it (see cowa_fwd_kernel).  512 tokens behind 32K 54 -> 52.6 us.  (The other forms
+    // lose up to a hundredth so, in registers.)
+    if (tid == 256) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); }
+    __syncthreads();
+    if (warp == 8) {
+      asm volatile("bar.arrive 3, 384;" ::: "memory");
+      if (VARLEN) grid_enter();
+    } else {
+      grid_enter();
+      if (warp == 9) {
+        __syncwarp();
+        tmem_alloc(tmem_holder, TMEM_COLS);
+        tmem_relinquish();
+      }
+      tc_fence_before();
+      asm volatile("bar.sync 3, 384;" ::: "memory");
+    }
+  } else {
+    tc_fence_before();
+    __syncthreads();
+  }
   tc_fence_after();
-  const uint32_t tb = *tmem_holder;
+  const uint32_t tb = SPLIT && warp == 8 ? 0u : *tmem_holder;
 
   bool ok = true;  // false once a bounded wait ran out; every role then falls through to the teardown
   auto warp_arrive = [&](uint64_t* bar) {  // one arrival for the whole warp
@@ -225,14 +245,13 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
    if (warp == 8) {
     // ======================= TMA producer =======================
     const bool lead = elect_one();
-    if (lead) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); }
+    if (!SPLIT && lead) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); }
     int c = 0;       // steps loaded so far, all items together: step c uses slot c & 1
     uint32_t ni = 0;  // items so far
     // The grid has a number per item, heaviest items first (SHARES: fewer).  A block starts with its own and, towards the end
     // of an item, takes over the next one whose block has not started: lists differ in length, and with a fixed share of the
     // items per block the last SM was busy 20 % longer than the average one (one KV head of 20001 tokens), 25 % for packed
     // prompts.
-    const int csize = SPLIT ? (int)cluster_size() : 1;
     uint32_t asked = 0, answered = 0;  // requests
     auto ask = [&]() {
       if (lead) {
@@ -249,7 +268,7 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       __syncwarp();
       return x;
     };
-    int idx = SPLIT ? blockIdx.x / csize : blockIdx.x;
+    int idx = SPLIT ? blockIdx.x / 2 : blockIdx.x;
     int num = idx, rnd = 0;  // SHARES: this block's number, and how many of its items came before
     int past = 0x7FFFFFFF;   // ... from this item on there are none
     if (SHARES && num >= starters) idx += (rounds - 1) * starters;
@@ -271,8 +290,8 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
           if (ni > 0) break;
           if (locate_item<VARLEN>(a, idx, mine)) {
             const int n = (mine.nt + 1) >> 1, rank = (int)cluster_rank();
-            mine.t0 = 2 * (n * rank / csize);
-            mine.nt = max(min(2 * (n * (rank + 1) / csize), mine.nt) - mine.t0, 0);
+            mine.t0 = 2 * (n * rank / 2);
+            mine.nt = max(min(2 * (n * (rank + 1) / 2), mine.nt) - mine.t0, 0);
           } else {
             mine.nt = mine.work = 0;
           }
@@ -284,6 +303,7 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
           idx = next_item_index();
           continue;
         }
+        if (SPLIT && !VARLEN) grid_enter();
         if (SHARES && mine.nt > 0 && mine.nt <= 6 && !more()) ask();  // of up to three steps: no later moment is early enough
         if (ni >= 2) ok = mbar_wait(bar_i_empty + (ni & 1), ((ni >> 1) & 1) ^ 1, a.status);
         if (!ok) break;
@@ -408,6 +428,10 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         }
       }
     }
+   }
+   if constexpr (SPLIT) {  // the softmax warps' merge
+     cluster_sync();
+     cluster_sync();
    }
   } else {
     setmaxnreg_inc<208>();
@@ -639,81 +663,49 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       }
     }
     if (r == 0 && stored) tma_wait_group_read<0>();
-  }
 
-  if constexpr (SPLIT) {
-    // Merge of the cluster's partial states: block `rank` writes every csize-th part of the 256 rows, a warp a row.
-    const PairItem& it = *reinterpret_cast<const PairItem*>(smem + SM::oItem);
-    const int csize = (int)cluster_size(), rank = (int)cluster_rank(), lane = tid & 31;
-    __syncthreads();
-    if (it.nt == 0 && tid < 2 * BQ) reinterpret_cast<float2*>(sQ)[tid] = make_float2(-INFINITY, 0.f);
-    cluster_sync();
-    if (it.work > 0) {
-      const int per = 2 * BQ / csize, first = rank * per;  // this block's rows of the 2 x 128
-      const uint32_t aState = smem_u32(sQ), aO = smem_u32(sK);
-      float* wgt = reinterpret_cast<float*>(sQ + 4096);    // [per][csize]: share of every block's O in a row
-      if (tid < per) {
-        const int xr = first + tid, row = it.q0 + (xr & (BQ - 1)), h = it.h0 + (xr >> 7);
-        float2 ml[8];
-        float M = -INFINITY, L = 0.f;
+    if constexpr (SPLIT) {
+      // Merge of the two blocks' partial states: block `rank` writes head `rank`, a warp 16 rows, all of the other block's O of them in
+      // flight together.  (A row at a time and lane, 32 rows an access: 2 us longer.  Four rows of one block after the other,
+      // the block's own through the cluster's window, too: 61.0 instead of 59.3 us for 512 tokens behind 32K.)
+      const PairItem& item = *reinterpret_cast<const PairItem*>(smem + SM::oItem);
+      const int rank = (int)cluster_rank(), lane = tid & 31;
+      if (item.nt == 0) reinterpret_cast<float2*>(sQ)[tid] = make_float2(-INFINITY, 0.f);
+      cluster_sync();
+      if (item.work > 0) {
+        const int r0 = rank * BQ + warp * 16;  // of the 2 x 128
+        const int steps = (item.work + 1) >> 1, here = rank == 0 ? steps / 2 : steps - steps / 2;
+        const uint32_t other = map_cluster(smem_u32(sK) + r0 * (D * 4), rank ^ 1);
+        const uint8_t* const own = sK + r0 * (D * 4);
+        float4 v[16];
 #pragma unroll
-        for (int p = 0; p < 8; ++p)
-          if (p < csize) {
-            ml[p] = ld_cluster_f2(map_cluster(aState + xr * 8, p));
-            M = fmaxf(M, ml[p].x);
-          }
-#pragma unroll
-        for (int p = 0; p < 8; ++p)
-          if (p < csize) {
-            ml[p].x = ml[p].x == -INFINITY ? 0.f : ex2(ml[p].x - M);
-            L = fmaf(ml[p].y, ml[p].x, L);
-          }
-        const float inv = L == 0.f ? 0.f : 1.f / L;  // a NaN sum has to come out as NaN
-#pragma unroll
-        for (int p = 0; p < 8; ++p)
-          if (p < csize) wgt[tid * csize + p] = ml[p].x * inv;
-        if (row < it.Nq) {
-          const size_t li = VARLEN ? (size_t)h * a.total_q + it.qbase + row : ((size_t)it.b * a.Hq + h) * it.Nq + row;
+        for (int u = 0; u < 16; ++u)  // (a block without a step left no O)
+          v[u] = here < steps ? ld_cluster_f4(other + u * (D * 4) + ((lane ^ (u & 7)) << 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float2 mine = reinterpret_cast<const float2*>(sQ)[r0 + (lane & 15)];
+        const float2 theirs = ld_cluster_f2(map_cluster(smem_u32(sQ) + (r0 + (lane & 15)) * 8, rank ^ 1));
+        const float M = fmaxf(mine.x, theirs.x);
+        float wa = mine.x == -INFINITY ? 0.f : ex2(mine.x - M), wb = theirs.x == -INFINITY ? 0.f : ex2(theirs.x - M);
+        const float L = fmaf(theirs.y, wb, mine.y * wa), inv = L == 0.f ? 0.f : 1.f / L;  // a NaN sum has to come out as NaN
+        wa *= inv; wb *= inv;
+        const int row0 = item.q0 + warp * 16, h = item.h0 + rank;
+        if (lane < 16 && row0 + lane < item.Nq) {
+          const size_t li = VARLEN ? (size_t)h * a.total_q + item.qbase + row0 + lane : ((size_t)item.b * a.Hq + h) * item.Nq + row0 + lane;
           a.lse[li] = 0.6931471805599453f * (M + log2f(L));
         }
-      }
-      __syncthreads();
-      constexpr int LPR = D / 4, RPW = 32 / LPR, U = 4;  // lanes per row (16 bytes of fp32 each), rows a warp takes at
-                                                         // once, such groups of rows in flight
-      const int ch = lane % LPR;
-      for (int i0 = warp * RPW * U + lane / LPR; i0 < per; i0 += (kPairThreads / 32) * RPW * U) {
-        float4 o[U];
+        __nv_bfloat16* const dst = a.o + (VARLEN ? ((size_t)h * a.total_q + item.qbase + row0) * D
+                                                 : (size_t)item.b * a.so.b + (size_t)h * a.so.h + (size_t)row0 * a.so.t) + lane * 4;
+        const long long step = VARLEN ? D : a.so.t;
 #pragma unroll
-        for (int u = 0; u < U; ++u) o[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        const int n = (it.work + 1) >> 1;  // steps of the item, shared out as above
-        for (int p = 0; p < csize; ++p) {
-          if (n * p / csize == n * (p + 1) / csize) continue;  // a block without a step left no O
-          const uint32_t src = map_cluster(aO, p);
-          float4 v[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int xr = first + min(i0 + u * RPW, per - 1);
-            v[u] = ld_cluster_f4(src + xr * (D * 4) + ((ch ^ (xr & 7)) << 4));
-          }
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const float w = wgt[min(i0 + u * RPW, per - 1) * csize + p];
-            o[u].x = fmaf(v[u].x, w, o[u].x); o[u].y = fmaf(v[u].y, w, o[u].y);
-            o[u].z = fmaf(v[u].z, w, o[u].z); o[u].w = fmaf(v[u].w, w, o[u].w);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int i = i0 + u * RPW, xr = first + i, row = it.q0 + (xr & (BQ - 1)), h = it.h0 + (xr >> 7);
-          if (i < per && row < it.Nq) {
-            __nv_bfloat16* dst = a.o + (VARLEN ? ((size_t)h * a.total_q + it.qbase + row) * D
-                                               : (size_t)it.b * a.so.b + (size_t)h * a.so.h + (size_t)row * a.so.t);
-            *reinterpret_cast<uint2*>(dst + ch * 4) = make_uint2(pack_bf16(o[u].x, o[u].y), pack_bf16(o[u].z, o[u].w));
-          }
+        for (int u = 0; u < 16; ++u) {
+          const float4 x = here > 0 ? *reinterpret_cast<const float4*>(own + u * (D * 4) + ((lane ^ (u & 7)) << 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float w0 = __shfl_sync(0xFFFFFFFFu, wa, u), w1 = __shfl_sync(0xFFFFFFFFu, wb, u);
+          if (row0 + u < item.Nq)
+            *reinterpret_cast<uint2*>(dst + u * step) = make_uint2(pack_bf16(fmaf(v[u].x, w1, x.x * w0), fmaf(v[u].y, w1, x.y * w0)),
+                                                                   pack_bf16(fmaf(v[u].z, w1, x.z * w0), fmaf(v[u].w, w1, x.w * w0)));
         }
       }
+      cluster_sync();  // no block leaves while another one reads its shared memory
     }
-    cluster_sync();  // no block leaves while another one reads its shared memory
   }
 
   // ---- teardown ----
@@ -729,28 +721,27 @@ cowa_fwd_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 
 namespace cowa {
 
-int resident_clusters(int size) {
-  static std::atomic<int> cache[64][3];  // per device
-  const int i = size == 2 ? 0 : size == 4 ? 1 : 2;
+int resident_pairs() {
+  static std::atomic<int> cache[64];  // per device
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
-    n = cache[dev][i].load(std::memory_order_relaxed);
+    n = cache[dev].load(std::memory_order_relaxed);
     if (n > 0) return n;
     const auto kernel = cowa_fwd_pair_kernel<128, false, kSplit>;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)size); cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = PairSmem<128>::kBytes;
+    cfg.gridDim = dim3(2); cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = PairSmem<128>::kBytes;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)size; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PairSmem<128>::kBytes) == cudaSuccess &&
         cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0) {
-      cache[dev][i].store(n, std::memory_order_relaxed);
+      cache[dev].store(n, std::memory_order_relaxed);
       return n;
     }
   }
   cudaGetLastError();
-  return size == 2 ? 72 : size == 4 ? 32 : 15;
+  return 72;
 }
 
 template <int D, bool VARLEN>
