@@ -58,12 +58,13 @@ struct DecodeArgs {
   const __nv_bfloat16* kc;
   const __nv_bfloat16* vc;
   const int32_t* lens;
-  float* ws_o;  // [splits, G, D]
-  float* ws_m;  // [splits, G]
-  float* ws_l;  // [splits, G]
+  float* ws_o;  // [B, Hq, S, D]; where the splits are shared out [splits, G, D]
+  float* ws_m;  // [B, Hq, S]; [splits, G]
+  float* ws_l;
   int B, Tmax, Hq, Hkv;
   int S;        // splits of a (sequence, KV head), on average where they are shared out: the grid is (S, Hkv, B)
   int shared;   // splits by the sequences' lengths (Shares)
+  int ahead;    // V is prefetched: splits of at most 2 * kThreads rows
   float inv_room;       // 1 / (B * S)
   unsigned head_magic;  // x / hkv_global = (x * head_magic) >> 32 for all lengths up to Tmax; 0: it does not hold
   CowaStrides sk, sv;  // element strides (batch, head, token) of the contiguous-row cache
@@ -173,6 +174,40 @@ struct Shares {
   }
 };
 
+// The lengths hardly differ: every sequence takes a.S splits, as where nothing is shared out (4 sequences of 57000 to 63000
+// tokens, 8 groups of 4: 26.4 us, shared out 27.7).
+__device__ __forceinline__ bool alike(const DecodeArgs& a) {
+  const int lane = threadIdx.x & 31;
+  int sum = 0, most = 0;
+  for (int i = lane; i < a.B; i += 32) {
+    const int n = visible_rows(a, min(a.lens[i], a.Tmax));
+    sum += n;
+    most = max(most, n);
+  }
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  most = __reduce_max_sync(0xffffffffu, most);
+  return (float)most * a.B <= 1.125f * sum;
+}
+
+struct Share {
+  int b, before, S, chunk;
+};
+__device__ __forceinline__ Share share_at(const DecodeArgs& a, int slot) {
+  const Shares sh(a);
+  Share x;
+  x.b = sh.at(slot, a.Hkv, &x.before, &x.S);
+  x.chunk = sh.chunk();
+  return x;
+}
+__device__ __forceinline__ Share share_of(const DecodeArgs& a, int b) {
+  const Shares sh(a);
+  Share x;
+  x.b = b;
+  sh.of(b, &x.before, &x.S);
+  x.chunk = sh.chunk();
+  return x;
+}
+
 __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                                uint32_t a3, uint32_t b0, uint32_t b1) {
   asm volatile(
@@ -191,9 +226,9 @@ __device__ __forceinline__ uint4 ldg128(const void* p) {
 }
 
 // G = columns of the mma n-tile in use: the query heads of the group.
-template <int D, int G>
+template <int D, int G, bool SHARED>
 // 5 blocks per SM (up to 102 registers, no spills) measured best: fewer, longer splits than at 7 per SM
-// (D = 64, groups below 8: 7 as before the shares, whose registers cost one otherwise)
+// (D = 64, groups below 8: 7, which the shares' registers would make 6)
 __global__ void __launch_bounds__(kThreads, D == 64 && G < 8 ? 7 : 5) cowa_decode_split_kernel(const DecodeArgs a) {
   static_assert(D == 64 || D == 128, "head dim");
   static_assert(G >= 1 && G <= 8, "group size per mma n-tile");
@@ -205,14 +240,17 @@ __global__ void __launch_bounds__(kThreads, D == 64 && G < 8 ? 7 : 5) cowa_decod
   cowa_ptx::grid_enter();  // the merge kernel's blocks may be scheduled beside this one's; they wait for its results
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int split = blockIdx.x, hk = blockIdx.y, b = blockIdx.z, S = a.S, chunk = 0;
-  const int slot = (b * a.Hkv + hk) * S + split;  // of this block's state
-  if (a.shared) {
-    const Shares sh(a);
-    int before;
-    b = sh.at(slot, a.Hkv, &before, &S);
-    if (b < 0) return;
-    const int i = slot - before * a.Hkv;
-    hk = (int)__fdividef(i + 0.5f, (float)S); split = i - hk * S; chunk = sh.chunk();  // (i and S are small)
+  size_t state = ((size_t)(b * a.Hkv + hk) * G) * S + split;  // of the first head, the others' at state + c * apart
+  int apart = S;
+  if (SHARED && !alike(a)) {
+    const int slot = (b * a.Hkv + hk) * S + split;
+    const Share x = share_at(a, slot);
+    if (x.b < 0) return;
+    b = x.b; S = x.S; chunk = x.chunk;
+    const int i = slot - x.before * a.Hkv;
+    hk = (int)__fdividef(i + 0.5f, (float)S); split = i - hk * S;  // (i and S are small)
+    state = (size_t)slot * G;
+    apart = 1;
   }
   const int Nk = a.lens[b];
 
@@ -238,21 +276,18 @@ __global__ void __launch_bounds__(kThreads, D == 64 && G < 8 ? 7 : 5) cowa_decod
   if (chunk == 0) chunk = ((V + S - 1) / S + 15) & ~15;
   const int c0 = split * chunk;
   const int clen = min(chunk, V - c0);  // <= kChunkCap by the host's choice of S
-  float* const out_o = a.ws_o + (size_t)slot * (G * D);
-  float* const out_m = a.ws_m + (size_t)slot * G;
-  float* const out_l = a.ws_l + (size_t)slot * G;
 
   if (clen <= 0) {  // empty split: neutral partial state
-    for (int i = tid; i < G * D; i += kThreads) out_o[i] = 0.f;
+    for (int i = tid; i < G * D; i += kThreads) a.ws_o[(state + (size_t)(i / D) * apart) * D + i % D] = 0.f;
     if (tid < G) {
-      out_m[tid] = -INFINITY;
-      out_l[tid] = 0.f;
+      a.ws_m[state + tid * apart] = -INFINITY;
+      a.ws_l[state + tid * apart] = 0.f;
     }
     return;
   }
-  // Short splits: V is on its way to L2 while K is read and weighed (one row of each thread here; 8K of context, one sequence
-  // 8.8 us, so 7.9).  Long ones have enough in flight, and all of them together would not fit L2.
-  if (chunk <= 2 * kThreads) {
+  // Small calls: V is on its way to L2 while K is read and weighed (8K of context, one sequence 8.8 us, so 8.4).  Where bandwidth
+  // counts, K would wait behind it, and it comes out of L2 a second time (8 sequences, 8 heads of 2000 rows, 65 MB: 16.5 us, so 18.3).
+  if (a.ahead) {
 #pragma unroll
     for (int r = tid; r < 2 * kThreads; r += kThreads)
       if (r < clen) {
@@ -383,84 +418,125 @@ __global__ void __launch_bounds__(kThreads, D == 64 && G < 8 ? 7 : 5) cowa_decod
     float s = 0.f;
 #pragma unroll
     for (int r = 0; r < kThreads / 32; ++r) s += sc[r * G * D + i];
-    out_o[i] = s;
+    a.ws_o[(state + (size_t)(i / D) * apart) * D + i % D] = s;
   }
   if (tid < G) {
-    out_m[tid] = m_s[tid];
-    out_l[tid] = l_s[tid];
+    a.ws_m[state + tid * apart] = m_s[tid];
+    a.ws_l[state + tid * apart] = l_s[tid];
   }
 }
 
 // Merge of the split states: M = max m_s, L = sum l_s 2^(m_s - M), o = sum o_s 2^(m_s - M) / L,
-// lse = ln2 * (M + log2 L).  One block per (sequence, QO head).  A warp takes every W-th group of eight splits, D/32 columns per
-// lane, states and O in one round trip; the running maximum moves between its groups, and the warps' results meet in shared
-// memory.  W: four warps where eight splits a warp are all there are, sixteen for more (one sequence of 57 700 visible rows in
-// 452 splits: with four warps 16 us of 29 were this kernel).
-template <int D, int W>
+// lse = ln2 * (M + log2 L).  One block per (sequence, QO head).  A warp takes every W-th split, eight at a time, D/32 columns per
+// lane, states and O in one round trip, and the running maximum moves between such groups; the warps' results meet in shared memory.
+// W: sixteen warps (one sequence of 57 700 visible rows in 452 splits: with four 16 us of 29 were this kernel), eight where
+// splits are shared out and a sequence has up to 32 on average.  Without sharing four are enough up to 32 splits: a lane reads one
+// split's state and every warp knows M and L.  That form has 32 registers, so that its blocks wait beside five of the split
+// kernel's (with 72: 8 sequences of 8000 tokens 16.6 us, so 17.1; held to 32 with spills 17.9).
+template <int D, int W, bool SHARED>
 __global__ void __launch_bounds__(W * 32) cowa_decode_combine_kernel(const DecodeArgs a, __nv_bfloat16* o, float* lse) {
   constexpr int V = D / 32, U = 8;  // columns per lane, splits of a group
+  constexpr bool kOnce = W * U == 32 && !SHARED;  // S <= 32
   __shared__ float part[W][D], part_m[W], part_l[W];
-  const int bh = blockIdx.x, b = bh / a.Hq, h = bh % a.Hq, G = a.Hq / a.Hkv;
+  const int bh = blockIdx.x;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // The lengths are not written by the split kernel and were complete before it began (grid_wait); its states are after the wait.
-  int before = b * a.S, S = a.S;
-  if (a.shared) Shares(a).of(b, &before, &S);
+  size_t first = (size_t)bh * a.S;  // split s lies s * step further
+  int S = a.S, step = 1;
+  if (SHARED && !alike(a)) {
+    const int b = bh / a.Hq, h = bh % a.Hq, G = a.Hq / a.Hkv;
+    const Share x = share_of(a, b);
+    S = x.S;
+    first = ((size_t)x.before * a.Hkv + (size_t)(h / G) * S) * G + h % G;
+    step = G;
+  }
   cowa_ptx::grid_enter();
-  const size_t first = ((size_t)before * a.Hkv + (size_t)(h / G) * S) * G + h % G;  // split s lies s * G further
+  const float* m = a.ws_m + first;
+  const float* l = a.ws_l + first;
   const float* po = a.ws_o + first * D + lane * V;
   float mx = -INFINITY, L = 0.f, acc[V];
 #pragma unroll
   for (int i = 0; i < V; ++i) acc[i] = 0.f;
-  for (int s0 = warp * U; s0 < S; s0 += W * U) {
-    const bool in = lane < U && s0 + lane < S;
-    const float ms = in ? a.ws_m[first + (size_t)(s0 + lane) * G] : -INFINITY;
-    const float ls = in ? a.ws_l[first + (size_t)(s0 + lane) * G] : 0.f;
+  if constexpr (kOnce) {
+    const float ms = lane < S ? m[lane * step] : -INFINITY;
+    const float ls = lane < S ? l[lane * step] : 0.f;
     float x[U][V];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const float* src = po + (size_t)(s0 + u) * G * D;
-      if constexpr (V == 4) {
-        const float4 y = s0 + u < S ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
-        x[u][0] = y.x; x[u][1] = y.y; x[u][2] = y.z; x[u][3] = y.w;
-      } else {
-        const float2 y = s0 + u < S ? *reinterpret_cast<const float2*>(src) : make_float2(0.f, 0.f);
-        x[u][0] = y.x; x[u][1] = y.y;
-      }
+      const int s = warp + W * u;
+#pragma unroll
+      for (int i = 0; i < V; ++i) x[u][i] = s < S ? po[(size_t)(s * step) * D + i] : 0.f;
     }
-    float m = ms;
+    mx = ms;
 #pragma unroll
-    for (int k = U / 2; k > 0; k >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, k));
-    m = fmaxf(__shfl_sync(0xffffffffu, m, 0), mx);
-    const float old = mx == -INFINITY ? 0.f : exp2f(mx - m), w = ms == -INFINITY ? 0.f : exp2f(ms - m);
-    mx = m;
-    float l = ls * w;
+    for (int k = 16; k > 0; k >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, k));
+    const float w = exp2f(ms - mx);  // empty splits: m = -inf -> weight 0
+    L = ls * w;
 #pragma unroll
-    for (int k = U / 2; k > 0; k >>= 1) l += __shfl_xor_sync(0xffffffffu, l, k);
-    L = L * old + __shfl_sync(0xffffffffu, l, 0);
-#pragma unroll
-    for (int i = 0; i < V; ++i) acc[i] *= old;
+    for (int k = 16; k > 0; k >>= 1) L += __shfl_xor_sync(0xffffffffu, L, k);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const float wu = __shfl_sync(0xffffffffu, w, u);
+      const float wu = __shfl_sync(0xffffffffu, w, (warp + W * u) & 31);
 #pragma unroll
       for (int i = 0; i < V; ++i) acc[i] = fmaf(x[u][i], wu, acc[i]);
     }
+  } else {
+    for (int s0 = warp; s0 < S; s0 += W * U) {
+      const bool in = lane < U && s0 + lane * W < S;
+      const float ms = in ? m[(s0 + lane * W) * step] : -INFINITY;
+      const float ls = in ? l[(s0 + lane * W) * step] : 0.f;
+      float x[U][V];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int s = s0 + u * W;
+        const float* src = po + (size_t)(s * step) * D;
+        if constexpr (V == 4) {
+          const float4 y = s < S ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+          x[u][0] = y.x; x[u][1] = y.y; x[u][2] = y.z; x[u][3] = y.w;
+        } else {
+          const float2 y = s < S ? *reinterpret_cast<const float2*>(src) : make_float2(0.f, 0.f);
+          x[u][0] = y.x; x[u][1] = y.y;
+        }
+      }
+      float top = ms;
+#pragma unroll
+      for (int k = U / 2; k > 0; k >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, k));
+      top = fmaxf(__shfl_sync(0xffffffffu, top, 0), mx);
+      const float old = mx == -INFINITY ? 0.f : exp2f(mx - top), w = ms == -INFINITY ? 0.f : exp2f(ms - top);
+      mx = top;
+      float sum = ls * w;
+#pragma unroll
+      for (int k = U / 2; k > 0; k >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, k);
+      L = L * old + __shfl_sync(0xffffffffu, sum, 0);
+#pragma unroll
+      for (int i = 0; i < V; ++i) acc[i] *= old;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float wu = __shfl_sync(0xffffffffu, w, u);
+#pragma unroll
+        for (int i = 0; i < V; ++i) acc[i] = fmaf(x[u][i], wu, acc[i]);
+      }
+    }
+    if (lane == 0) { part_m[warp] = mx; part_l[warp] = L; }
   }
 #pragma unroll
   for (int i = 0; i < V; ++i) part[warp][lane * V + i] = acc[i];
-  if (lane == 0) { part_m[warp] = mx; part_l[warp] = L; }
   __syncthreads();
   if (tid < D) {
-    mx = part_m[0];
+    float v;
+    if constexpr (kOnce) {
+      v = (part[0][tid] + part[1][tid]) + (part[2][tid] + part[3][tid]);
+    } else {
+      mx = part_m[0];
 #pragma unroll
-    for (int k = 1; k < W; ++k) mx = fmaxf(mx, part_m[k]);
-    L = 0.f;
-    float v = 0.f;
+      for (int k = 1; k < W; ++k) mx = fmaxf(mx, part_m[k]);
+      L = v = 0.f;
 #pragma unroll
-    for (int k = 0; k < W; ++k) {
-      const float w = part_m[k] == -INFINITY ? 0.f : exp2f(part_m[k] - mx);
-      L = fmaf(part_l[k], w, L);
-      v = fmaf(part[k][tid], w, v);
+      for (int k = 0; k < W; ++k) {
+        const float w = part_m[k] == -INFINITY ? 0.f : exp2f(part_m[k] - mx);
+        L = fmaf(part_l[k], w, L);
+        v = fmaf(part[k][tid], w, v);
+      }
     }
     o[(size_t)bh * D + tid] = __float2bfloat16_rn(v / L);
     if (lse && tid == 0) lse[bh] = 0.6931471805599453f * (mx + log2f(L));
@@ -484,7 +560,7 @@ int resident_blocks_of() {
   int dev = 0, sms = 0, occ = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cowa_decode_split_kernel<D, G>, kThreads, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cowa_decode_split_kernel<D, G, false>, kThreads, 0) !=
       cudaSuccess)
     return 0;
   return sms * occ;
@@ -529,15 +605,18 @@ int pick_splits(int B, int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p)
 template <int D>
 cudaError_t launch_combine(const DecodeArgs& a, __nv_bfloat16* o, float* lse, cudaStream_t st) {
   const dim3 rows((unsigned)(a.B * a.Hq));
-  // (where they are shared out, the longest of a batch may have some times the average)
-  if (a.S > (a.shared ? 16 : 32)) return cowa::launch_chained(cowa_decode_combine_kernel<D, 16>, rows, 512, 0, st, a, o, lse);
-  return cowa::launch_chained(cowa_decode_combine_kernel<D, 4>, rows, 128, 0, st, a, o, lse);
+  if (a.shared)
+    return a.S > 32 ? cowa::launch_chained(cowa_decode_combine_kernel<D, 16, true>, rows, 512, 0, st, a, o, lse)
+                    : cowa::launch_chained(cowa_decode_combine_kernel<D, 8, true>, rows, 256, 0, st, a, o, lse);
+  return a.S > 32 ? cowa::launch_chained(cowa_decode_combine_kernel<D, 16, false>, rows, 512, 0, st, a, o, lse)
+                  : cowa::launch_chained(cowa_decode_combine_kernel<D, 4, false>, rows, 128, 0, st, a, o, lse);
 }
 
 template <int D, int G>
 cudaError_t launch_split(const DecodeArgs& a, cudaStream_t st) {
   const dim3 grid(a.S, a.Hkv, a.B);
-  return cowa::launch_chained(cowa_decode_split_kernel<D, G>, grid, kThreads, 0, st, a);
+  return a.shared ? cowa::launch_chained(cowa_decode_split_kernel<D, G, true>, grid, kThreads, 0, st, a)
+                  : cowa::launch_chained(cowa_decode_split_kernel<D, G, false>, grid, kThreads, 0, st, a);
 }
 
 template <int D>
@@ -597,11 +676,15 @@ int decode_launch(const void* q, const void* kc, const void* vc, const int32_t* 
   a.hkv_global = p->hkv_global > 0 ? p->hkv_global : Hkv;
   a.hkv_offset = p->hkv_offset;
   a.full_attn = p->full_attn;
-  // Sharing out costs a block 0.4 us, more than short splits can gain (up to 128 rows they are as many as there is length for).
+  // Sharing out costs 0.6 us, also where the lengths turn out alike (alike() before the first load, a merge kernel that does not
+  // fit beside the split kernel's blocks): too much where the splits are short (8 sequences of 7800 to 8000 tokens, 8 groups, 182
+  // rows a split: 16.6 us, 17.3 with it).
   // Of several waves a longer block is made up for by the blocks that follow, and equal ones keep in step, so that memory idles
   // while all of them weigh their scores (32 sequences of 1500 to 2600 tokens, 8 groups of one head: 46.9 us, shared out 52).
-  a.shared = B > 1 && B <= kShareSeqs && (long long)S * 128 < max_visible(Tmax, a.hkv_global, p) &&
+  a.shared = B > 1 && B <= kShareSeqs && (long long)S * 256 < max_visible(Tmax, a.hkv_global, p) &&
              (long long)B * Hkv * S <= resident_blocks(D, Hq / Hkv);
+  const long long rows = (long long)B * Hkv * max_visible(Tmax, a.hkv_global, p);  // K and V: 4 D bytes each
+  a.ahead = rows * D <= (4ll << 20) && rows <= 2ll * kThreads * S * B * Hkv;
   a.inv_room = 1.f / ((float)B * S);
   a.head_magic = a.hkv_global > 1 && ((long long)Tmax + a.hkv_global) * a.hkv_global <= 0xFFFFFFFFll ? 0xFFFFFFFFu / a.hkv_global + 1 : 0;
   a.scale_log2 = p->softmax_scale * 1.4426950408889634f;

@@ -1,5 +1,6 @@
 """Decode of batches of very different lengths, whose splits are shared out by length, against the float64 oracle: sequences of a few
-rows beside long ones, lengths at the borders of a split, as many sequences as are shared out at most and one more."""
+rows beside long ones, lengths at the borders of a split, as many sequences as are shared out at most and one more; and of batches
+that are alike, which are not, or just not alike."""
 import numpy as np
 import pytest
 import torch
@@ -27,10 +28,28 @@ def lengths(B, longest):
     (127, 12000, 2, 1, 64, 16, 4000),
     (128, 12000, 2, 1, 64, 16, 4000),
     (129, 12000, 2, 1, 64, 16, 4000),
+    (128, 4000, 1, 1, 64, 16, 2000),
+    (129, 4000, 1, 1, 64, 16, 2000),
     (5, 60000, 2, 1, 128, 128, 151),  # one sequence has nearly all splits
 ])
 def test_splits_by_length(B, longest, Hq, Hkv, D, sink, local):
-    lens = lengths(B, longest)
+    compare(lengths(B, longest), longest, Hq, Hkv, D, sink, local)
+
+
+@pytest.mark.parametrize("shortest", [16000, 13000, 11000])  # the longest has 1.0, 1.1 and 1.2 times the average
+@pytest.mark.parametrize("Hq,Hkv,D", [(16, 2, 128), (4, 2, 64)])
+def test_lengths_alike(Hq, Hkv, D, shortest):
+    longest = 16000
+    compare([shortest + (longest - shortest) * i // 7 for i in range(8)], longest, Hq, Hkv, D, 64, 6000)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_one_sequence_in_many_splits(D):
+    compare([40000], 40000, 8, 1, D, 64, 100)
+
+
+def compare(lens, longest, Hq, Hkv, D, sink, local):
+    B = len(lens)
     q, k, v, _ = cowa_inputs.make_decode_inputs(17, B, longest, Hq, Hkv, D, longest, longest)
     scale = cowa_inputs.softmax_scale(D)
     params = cowa.make_params(sink=sink, local=local, softmax_scale=scale)
@@ -40,7 +59,7 @@ def test_splits_by_length(B, longest, Hq, Hkv, D, sink, local):
     cowa.cowa_decode(q.to(DEV), k.to(DEV), v.to(DEV), torch.tensor(lens, dtype=torch.int32, device=DEV), o, lse, params, ws)
     torch.cuda.synchronize()
     f = cowa_inputs.to_f64
-    for b in sorted({0, 1, B // 2, B - 2, B - 1}):
+    for b in sorted({0, min(1, B - 1), B // 2, max(B - 2, 0), B - 1}):
         n = lens[b]
         o_ref, lse_ref = orc.decode(f(q[b:b + 1]), f(k[b:b + 1, :, :n]), f(v[b:b + 1, :, :n]), np.array([n]), sink, local, scale)
         check(f"o[b={b}]", o[b:b + 1].float().cpu().numpy(), o_ref)
