@@ -19,10 +19,11 @@
 // 50 KB, four are resident, and S(t+1) is issued behind O += P V of step t.  An SM then takes a step in 490 clocks (two blocks
 // with two buffers: 800 at the same clock rate); us, before / now: 640 blocks of up to 40 steps 50.9 / 42.6, 1920 of 35
 // 126 / 107, 8896 of 90 (power-limited, 1.3 GHz) 1365 / 1265.
-// Where blocks are too few to fill the chip a list is cut into parts (see the rule in launch_fwd):
+// Where blocks are too few to fill the chip (see the rule in launch_fwd), the last two cutting a list into parts:
+//   NB = 2   two S buffers and two blocks per SM, where two or three are all an SM gets (D = 64);
 //   NS = 4   four streams, each the five warps above with slots and TMEM of its own, in one block (D = 64);
 //   SPLIT    a cluster of 2, 4 or 8 blocks, each with two S buffers, as latency counts and not the number of blocks.
-// Each part keeps its own reference and accumulator; they are merged through (distributed) shared memory.
+// A part keeps its own reference and accumulator; they are merged through (distributed) shared memory.
 // The same kernel serves N_q <= N_k (queries bottom-right aligned) and, with VARLEN, packed batches
 // [H, total, D] whose sequences have their own N_q <= N_k: a block then finds its (sequence, tile) by a
 // warp scan of the offset arrays and stores a sequence's last, partial tile row by row.
@@ -40,12 +41,6 @@ namespace {
 constexpr int BQ = 128, BK = 64;
 constexpr int kFwdThreads = 160;
 
-// D = 64: one S buffer a stream and four streams per SM; D = 128, and clusters: two S buffers, two streams.
-template <int D, bool SPLIT>
-constexpr int kBuffers = D == 128 || SPLIT ? 2 : 1;
-template <int D, bool SPLIT>
-constexpr int kResident = 4 / kBuffers<D, SPLIT>;
-
 template <int D, int NS, bool SPLIT>
 struct FwdSmem {
   static constexpr int kQ = BQ * D * 2;   // Q tile (later the O staging tile)
@@ -54,8 +49,9 @@ struct FwdSmem {
   static constexpr int kBytes = oBar + 32 + NS * 80 + 1024;  // + barriers + alignment slack
 };
 
-template <int D, bool VARLEN, int NS, bool SPLIT>
-__global__ void __launch_bounds__(kFwdThreads * NS, kResident<D, SPLIT> / NS)
+// NB: S/P buffers of a stream (64 columns each, then O of D); an SM holds 4 / NB streams.
+template <int D, bool VARLEN, int NB, int NS, bool SPLIT>
+__global__ void __launch_bounds__(kFwdThreads * NS, 4 / NB / NS)
 cowa_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                 const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
                 const __grid_constant__ FwdArgs a) {
@@ -64,7 +60,6 @@ cowa_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   constexpr int NSLAB = D / 64;          // 64-element (128-byte) slabs along D
   constexpr int SLAB_Q = BQ * 128;       // bytes of one slab of a 128-row tile
   constexpr int SLAB_K = BK * 128;       // ... of a 64-row tile
-  constexpr int NB = kBuffers<D, SPLIT>;  // S/P buffers of 64 columns, then O of D
   constexpr uint32_t cO = 64 * NB, STREAM_COLS = 128 * NB, TMEM_COLS = STREAM_COLS * NS;
   constexpr uint32_t IDESC_S = idesc_bf16(128, BK, 0, 0);
   constexpr uint32_t IDESC_O = idesc_bf16(128, D, 0, 1);
@@ -607,17 +602,24 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
   // Clusters while blocks of half the items do not fill the SMs' two places each: a short list has too little to share for a
   // second block per SM (us, clusters of 1 / 2 / 4 / 8, D = 64: 32 items of 12 steps 13.5 / 10.6 / 8.2 / 9.3, of 164 steps
   // 165 / 71 / 38 / 29; 56 of 28 28 / 17 / 14.3 / 20; 8 of 14 17.7 / 11.6 / 8.7 / 7.0; D = 128: 32 of 12 12.7 / 12.7 / 10.6 /
-  // 12.5, 56 of 28 27 / 20 / 18 / 25, 8 of 14 20 / 15 / 11 / 9).  From a quarter to one item per two places the D = 64 kernel
-  // takes four streams a block (128 items of 42 steps, one block / streams / cluster of two 42 / 23 / 23; 240 of 205
-  // 201 / 152 / 180), above that where long lists leave the last blocks alone on their SMs (696 of up to 95 steps 132 / 112;
-  // 640 of 40 42.6 / 62); at D = 128 clusters of two are better than the pair kernel's, whose items are half as many,
-  // where lists differ in length (128 items of up to 42 steps 26 / 33; 512 tokens behind 32K 59 / 55).
+  // 12.5, 56 of 28 27 / 20 / 18 / 25, 8 of 14 20 / 15 / 11 / 9).  At D = 128 they are also better than the pair kernel's, whose
+  // items are half as many, where lists differ in length (128 items of up to 42 steps 26 / 33; 512 tokens behind 32K 59 / 55).
+  // More items at D = 64, one block of one buffer / four streams / one block of two buffers, us:
+  //   128 items of 20 steps   22 / 15 / 19    192 of 10   21.5 / 21 / 18.5   256 of 12   20 / 25 / 18.5   288 of 9   22 / 29 / 21
+  //   160 of 14               17 / 14 / 15    192 of 19   51 / 28 / 42       256 of 64   54 / 31 / 45     288 of 43  57 / 42 / 48
+  //   320 of up to 12         19 / 26 / 18    352 of 14   46 / 45 / 39       384 of 52   125 / 77 / 105   320 of 40  36 / 33 / 31
+  //   352 of 16, all alike    32 / 38 / 36    448 alike   35 / 47 / 39       576 of 17   28 / 42 / 32     696 of 95  132 / 112
+  // Streams shorten the longest list but leave one block per SM; two buffers shorten a block's step where two or three blocks
+  // are all an SM gets; one buffer wins as soon as four have work to the end: lists alike, or more of them.  (Streams from the
+  // line on also where all lists are alike, 192 of 22 steps 30 / 30 / 27: an average of packed lengths does not tell.)
   const bool alike = kn >= 2ll * qn;  // every tile's list is about as long
   int streams = 1, split = 1;
+  [[maybe_unused]] bool deep = false;  // two S buffers
   if (4 * heads <= 2 * sms) {
     while (split < 8 && 2 * split * heads <= (steps >= 24 ? 2 * sms : sms) && 2 * split <= steps) split *= 2;
   } else if (D == 64) {
-    if (heads <= 2 * sms ? steps >= 8 : heads <= 5 * sms && steps >= 64) streams = kResident<D, false>;
+    if (heads <= 2 * sms ? 12 * steps > heads : heads <= 3 * sms ? 8 * steps > heads : heads <= 5 * sms && steps >= 64) streams = 4;
+    else deep = heads <= (alike && !VARLEN ? 2 : 3) * sms;  // (the same sums in the same order as with one buffer)
   } else if (heads <= sms && steps >= 32 && (!alike || a.G % 2)) {
     split = 2;
   }
@@ -659,11 +661,12 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
     COWA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mo, a));
     return COWA_OK;
   };
-  if (split > 1) return launch(cowa_fwd_kernel<D, VARLEN, 1, true>, FwdSmem<D, 1, true>::kBytes);
+  if (split > 1) return launch(cowa_fwd_kernel<D, VARLEN, 2, 1, true>, FwdSmem<D, 1, true>::kBytes);
   if constexpr (D == 64) {
-    if (streams > 1) return launch(cowa_fwd_kernel<D, VARLEN, kResident<D, false>, false>, FwdSmem<D, kResident<D, false>, false>::kBytes);
+    if (streams > 1) return launch(cowa_fwd_kernel<D, VARLEN, 1, 4, false>, FwdSmem<D, 4, false>::kBytes);
+    if (!deep) return launch(cowa_fwd_kernel<D, VARLEN, 1, 1, false>, FwdSmem<D, 1, false>::kBytes);
   }
-  return launch(cowa_fwd_kernel<D, VARLEN, 1, false>, FwdSmem<D, 1, false>::kBytes);
+  return launch(cowa_fwd_kernel<D, VARLEN, 2, 1, false>, FwdSmem<D, 1, false>::kBytes);
 }
 
 }  // namespace

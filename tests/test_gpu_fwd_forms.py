@@ -1,5 +1,5 @@
 """The forms of the one-head forward kernel, each at the sizes where its parts are uneven, against the float64 oracle: clusters of 2,
-4 and 8 blocks, four streams in a block, one block per item; lists of as many steps as parts, fewer, and one more; tiles cut by
+4 and 8 blocks, four streams in a block, one block per item with one and two buffers; lists of as many steps as parts, fewer, and one more; tiles cut by
 the end of the sequence.  Tolerances as in test_gpu_parity."""
 import numpy as np
 import pytest
@@ -21,6 +21,9 @@ pytestmark = pytest.mark.gpu
     (1, 129, 1999, 4, 4, 64, 700),  # a second tile of one row
     (3, 500, 500, 3, 3, 4, 100),    # causal lists from nothing up: tiles with fewer steps than parts
     (2, 700, 1400, 8, 8, 64, 300),  # 96 items: four streams, or one block each
+    (2, 900, 900, 10, 5, 3, 130),   # 160 items of one to seven steps: two buffers
+    (3, 700, 700, 20, 4, 64, 100),  # 360 items, lists of different lengths: two buffers
+    (3, 520, 1100, 24, 8, 64, 100),  # 360 items, lists alike: one buffer, two in the packed batch
     (2, 640, 2500, 10, 5, 100, 900),  # 100 items of long lists: clusters of two at D = 128
 ])
 def test_forms_match_the_oracle(D, B, Nq, Nk, Hq, Hkv, sink, local):
