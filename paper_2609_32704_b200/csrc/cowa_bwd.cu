@@ -1269,10 +1269,12 @@ BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& h
   const int nKV = (Nk + BKV - 1) / BKV, sms = cowa::sm_count();
   pl.sink_tiles = 0;
   for (int h = 0; h < Hkv; ++h) pl.sink_tiles = std::max(pl.sink_tiles, (std::min(hw.w[h].s, Nk) + BKV - 1) / BKV);
-  long long total = 0, sinks = 0, longest = 0, longest_sink = 0;
+  long long total = 0, sinks = 0, longest = 0, longest_sink = 0, longest_rest = 0;
   int counts[kFewTiles];  // tile j of head h: [j * Hkv + h]
   // (A table's parts do not end with the heads: items side by side no longer sweep the same rows of Q and dQ, which is lost where
-  // these outgrow L2: 31232 tokens, 8 heads 4850 / 4980 us with it.)
+  // these outgrow L2: 31232 tokens, 8 heads 4850 / 4980 us with it.  It costs in long sequences already: us, without / with it,
+  // local 2000: 8192 tokens, 8 heads of one KV head 220 / 277, 4087 tokens x 4 336 / 372.  So with it where sequences are short,
+  // 2000 tokens x 4 154 / 122, 3000 x 3 175 / 147, or a class has a part well above an SM's share, 8000 tokens, 4 heads 152 / 93.)
   const bool few = (long long)nKV * Hkv * B <= std::min(2 * sms, kFewTiles) && (long long)B * Hkv * G * Nq <= 131072;
   for (int h = 0; h < Hkv; ++h)
     for (int j = 0; j < nKV; ++j) {
@@ -1284,6 +1286,7 @@ BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& h
       if (few) counts[j * Hkv + h] = (int)cnt;
       longest = std::max(longest, cnt);
       if (j < pl.sink_tiles) { sinks += cnt; longest_sink = std::max(longest_sink, cnt); }
+      else longest_rest = std::max(longest_rest, cnt);
     }
   total *= B; sinks *= B;
   const double share = (double)total / sms;
@@ -1300,7 +1303,8 @@ BwdPlan bwd_plan(int B, int Nq, int Nk, int Hkv, int G, const CowaHeadWindows& h
   const long long budget = heads >= 4 ? room : std::max<long long>(room, 4ll * sms);
   while (pl.slots() > budget) --*std::max_element(pl.parts, pl.parts + 3);
   pl.choose_run(rest > 0 ? (double)(total - sinks) / rest * BQS / BQT : 0.0, reproducible);
-  if (few && !reproducible) pl.share_out(counts, nKV * Hkv, B, total, (int)longest);
+  const double part = std::max((double)longest_sink / pl.run[0], (double)longest_rest / pl.run[1]);
+  if (few && !reproducible && (part > 1.2 * share || (Nq <= 4096 && (long long)B * Hkv * G * Nq <= 81920))) pl.share_out(counts, nKV * Hkv, B, total, (int)longest);
   return pl;
 }
 
