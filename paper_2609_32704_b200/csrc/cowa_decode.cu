@@ -18,6 +18,8 @@
 // A second kernel merges the splits (log-sum-exp combine with warp shuffles).
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "cowa_common.h"
 #include "cowa_ptx.cuh"
 
@@ -82,9 +84,9 @@ struct VisMap {
 
 // Rows that a head sees of a sequence of Nk keys (the widest band's head).
 __device__ __forceinline__ int visible_rows(const DecodeArgs& a, int Nk) {
-  const int far = Nk - a.sink - a.near;
+  const long long far = (long long)Nk - a.sink - a.near;
   if (a.full_attn || far <= 0) return max(Nk, 0);
-  const int x = far + a.hkv_global - 1;
+  const int x = (int)far + a.hkv_global - 1;
   return a.sink + a.near + (a.head_magic ? (int)__umulhi((unsigned)x, a.head_magic) : x / a.hkv_global);
 }
 
@@ -672,7 +674,8 @@ int decode_launch(const void* q, const void* kc, const void* vc, const int32_t* 
   int rc;
   if ((rc = resolve_strides(p->k_strides, Hkv, Tmax, D, &a.sk))) return rc;
   if ((rc = resolve_strides(p->v_strides, Hkv, Tmax, D, &a.sv))) return rc;
-  a.sink = p->sink; a.near = p->local;
+  // No key lies further than Tmax away: wider windows mean the same as Tmax, and sums of widths stay inside 32 bits.
+  a.sink = std::min(p->sink, Tmax); a.near = std::min(p->local, Tmax);
   a.hkv_global = p->hkv_global > 0 ? p->hkv_global : Hkv;
   a.hkv_offset = p->hkv_offset;
   a.full_attn = p->full_attn;

@@ -43,12 +43,18 @@ def test_lengths_alike(Hq, Hkv, D, shortest):
     compare([shortest + (longest - shortest) * i // 7 for i in range(8)], longest, Hq, Hkv, D, 64, 6000)
 
 
+@pytest.mark.parametrize("sink,local", [(128, 2 ** 31 - 1), (2 ** 31 - 1, 5), (2 ** 31 - 1, 2 ** 31 - 1)])
+@pytest.mark.parametrize("short", [1, 60, 126, 127])
+def test_windows_wider_than_any_sequence(short, sink, local):
+    compare([30000, short] + [30000] * 6, 30000, 16, 2, 128, sink, local, check_at=(0, 1, 2))
+
+
 @pytest.mark.parametrize("D", [64, 128])
 def test_one_sequence_in_many_splits(D):
     compare([40000], 40000, 8, 1, D, 64, 100)
 
 
-def compare(lens, longest, Hq, Hkv, D, sink, local):
+def compare(lens, longest, Hq, Hkv, D, sink, local, check_at=None):
     B = len(lens)
     q, k, v, _ = cowa_inputs.make_decode_inputs(17, B, longest, Hq, Hkv, D, longest, longest)
     scale = cowa_inputs.softmax_scale(D)
@@ -59,7 +65,7 @@ def compare(lens, longest, Hq, Hkv, D, sink, local):
     cowa.cowa_decode(q.to(DEV), k.to(DEV), v.to(DEV), torch.tensor(lens, dtype=torch.int32, device=DEV), o, lse, params, ws)
     torch.cuda.synchronize()
     f = cowa_inputs.to_f64
-    for b in sorted({0, min(1, B - 1), B // 2, max(B - 2, 0), B - 1}):
+    for b in check_at or sorted({0, min(1, B - 1), B // 2, max(B - 2, 0), B - 1}):
         n = lens[b]
         o_ref, lse_ref = orc.decode(f(q[b:b + 1]), f(k[b:b + 1, :, :n]), f(v[b:b + 1, :, :n]), np.array([n]), sink, local, scale)
         check(f"o[b={b}]", o[b:b + 1].float().cpu().numpy(), o_ref)
