@@ -52,23 +52,17 @@ void* static_scratch_ptr(cudaError_t* err) {
   return cache[dev];
 }
 
-constexpr int kShareSeqs = 128;  // up to so many sequences every warp looks at all lengths (four a lane)
-constexpr int kMinChunk = 64;    // rows of a split, where there is a choice
-
 struct DecodeArgs {
   const __nv_bfloat16* q;
   const __nv_bfloat16* kc;
   const __nv_bfloat16* vc;
   const int32_t* lens;
-  float* ws_o;  // [B, Hq, S, D]; where the splits are shared out [splits, G, D]
-  float* ws_m;  // [B, Hq, S]; [splits, G]
+  float* ws_o;  // [B, Hq, S, D]
+  float* ws_m;  // [B, Hq, S]
   float* ws_l;
   int B, Tmax, Hq, Hkv;
-  int S;        // splits of a (sequence, KV head), on average where they are shared out: the grid is (S, Hkv, B)
-  int shared;   // splits by the sequences' lengths (Shares)
-  int ahead;    // V is prefetched: splits of at most 2 * kThreads rows
-  float inv_room;       // 1 / (B * S)
-  unsigned head_magic;  // x / hkv_global = (x * head_magic) >> 32 for all lengths up to Tmax; 0: it does not hold
+  int S;      // splits of a (sequence, KV head)
+  int ahead;  // V is prefetched: splits of at most 2 * kThreads rows
   CowaStrides sk, sv;  // element strides (batch, head, token) of the contiguous-row cache
   int sink, near, hkv_global, hkv_offset, full_attn;
   float scale_log2;
@@ -81,134 +75,6 @@ struct VisMap {
     return v < n0 ? lo0 + v : (v < n0 + n1 ? lo1 + (v - n0) : lo2 + (v - n0 - n1));
   }
 };
-
-// Rows that a head sees of a sequence of Nk keys (the widest band's head).
-__device__ __forceinline__ int visible_rows(const DecodeArgs& a, int Nk) {
-  const long long far = (long long)Nk - a.sink - a.near;
-  if (a.full_attn || far <= 0) return max(Nk, 0);
-  const int x = (int)far + a.hkv_global - 1;
-  return a.sink + a.near + (a.head_magic ? (int)__umulhi((unsigned)x, a.head_magic) : x / a.hkv_global);
-}
-
-// How the splits are shared out between sequences of different lengths: the shortest chunk, a multiple of 16 rows, with which
-// all sequences together need no more splits than the grid has blocks.  (With the same number of splits for every sequence a
-// batch waits for its longest: 16 sequences of 3600 to 33800 tokens 48 us, so 40.)  Warp-cooperative.
-struct Shares {
-  static constexpr int kPer = kShareSeqs / 32;
-  int rows[kPer];  // in 16 rows, of sequences lane, lane + 32, ..., -1 past the last one
-  int B, k;        // k: a split's rows / 16
-  unsigned magic;  // x / k = (x * magic) >> 32 for x * k < 2^32
-  __device__ __forceinline__ int splits_of(int i) const {
-    return rows[i] < 0 ? 0 : max((int)__umulhi((unsigned)(rows[i] + k - 1), magic), 1);
-  }
-  __device__ __forceinline__ int count(int k_) {
-    k = k_;
-    magic = 0xFFFFFFFFu / (unsigned)k + 1;
-    int n = 0;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i)
-      if (i * 32 < B) n += splits_of(i);
-    return __reduce_add_sync(0xffffffffu, n);
-  }
-  __device__ __forceinline__ explicit Shares(const DecodeArgs& a) : B(a.B) {
-    const int lane = threadIdx.x & 31;
-    int sum = 0;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-      rows[i] = -1;
-      if (i * 32 < B) {
-        if (i * 32 + lane < B) rows[i] = (visible_rows(a, min(a.lens[i * 32 + lane], a.Tmax)) + 15) >> 4;
-        sum += max(rows[i], 0);
-      }
-    }
-    sum = __reduce_add_sync(0xffffffffu, sum);
-    const int room = B * a.S, hi = kChunkCap / 16 - 1;  // per KV head; with chunks of hi there is room (splits_for)
-    int at = min(max((int)((float)sum * a.inv_room) + 1, kMinChunk / 16), hi), low = at - 1;  // too short, or nearly: low
-    for (int step = 1; count(at) > room && at < hi; step *= 2) {
-      low = at;
-      at = min(at + step, hi);
-    }
-    while (at - low > 1) {
-      const int mid = (low + at) >> 1;
-      if (count(mid) <= room) at = mid;
-      else low = mid;
-    }
-    if (k != at) count(at);
-  }
-  __device__ __forceinline__ int chunk() const { return k * 16; }
-  // Splits of one KV head of the sequences before b, and of sequence b.
-  __device__ __forceinline__ void of(int b, int* before, int* mine) const {
-    int n = 0, m = 0;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i)
-      if (i * 32 < B) {
-        const int x = splits_of(i);
-        if (i * 32 + (int)(threadIdx.x & 31) < b) n += x;
-        if (i == b >> 5) m = x;
-      }
-    *before = __reduce_add_sync(0xffffffffu, n);
-    *mine = __shfl_sync(0xffffffffu, m, b & 31);
-  }
-  // The sequence of split idx (counted over all heads), -1 past the last one, and the two numbers above.
-  __device__ __forceinline__ int at(int idx, int Hkv, int* before, int* mine) const {
-    const int lane = threadIdx.x & 31;
-    int base = 0;
-#pragma unroll
-    for (int i = 0; i < kPer; ++i)
-      if (i * 32 < B) {
-        const int n = splits_of(i);
-        int incl = n;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += y;
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, idx < (base + incl) * Hkv);
-        if (m) {
-          const int src = __ffs(m) - 1;
-          *before = base + __shfl_sync(0xffffffffu, incl - n, src);
-          *mine = __shfl_sync(0xffffffffu, n, src);
-          return i * 32 + src;
-        }
-        base += __shfl_sync(0xffffffffu, incl, 31);
-      }
-    return -1;
-  }
-};
-
-// The lengths hardly differ: every sequence takes a.S splits, as where nothing is shared out (4 sequences of 57000 to 63000
-// tokens, 8 groups of 4: 26.4 us, shared out 27.7).
-__device__ __forceinline__ bool alike(const DecodeArgs& a) {
-  const int lane = threadIdx.x & 31;
-  int sum = 0, most = 0;
-  for (int i = lane; i < a.B; i += 32) {
-    const int n = visible_rows(a, min(a.lens[i], a.Tmax));
-    sum += n;
-    most = max(most, n);
-  }
-  sum = __reduce_add_sync(0xffffffffu, sum);
-  most = __reduce_max_sync(0xffffffffu, most);
-  return (float)most * a.B <= 1.125f * sum;
-}
-
-struct Share {
-  int b, before, S, chunk;
-};
-__device__ __forceinline__ Share share_at(const DecodeArgs& a, int slot) {
-  const Shares sh(a);
-  Share x;
-  x.b = sh.at(slot, a.Hkv, &x.before, &x.S);
-  x.chunk = sh.chunk();
-  return x;
-}
-__device__ __forceinline__ Share share_of(const DecodeArgs& a, int b) {
-  const Shares sh(a);
-  Share x;
-  x.b = b;
-  sh.of(b, &x.before, &x.S);
-  x.chunk = sh.chunk();
-  return x;
-}
 
 __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                                uint32_t a3, uint32_t b0, uint32_t b1) {
@@ -228,9 +94,9 @@ __device__ __forceinline__ uint4 ldg128(const void* p) {
 }
 
 // G = columns of the mma n-tile in use: the query heads of the group.
-template <int D, int G, bool SHARED>
+template <int D, int G>
 // 5 blocks per SM (up to 102 registers, no spills) measured best: fewer, longer splits than at 7 per SM
-// (D = 64, groups below 8: 7, which the shares' registers would make 6)
+// (D = 64, groups below 8: 7)
 __global__ void __launch_bounds__(kThreads, D == 64 && G < 8 ? 7 : 5) cowa_decode_split_kernel(const DecodeArgs a) {
   static_assert(D == 64 || D == 128, "head dim");
   static_assert(G >= 1 && G <= 8, "group size per mma n-tile");
@@ -241,19 +107,8 @@ __global__ void __launch_bounds__(kThreads, D == 64 && G < 8 ? 7 : 5) cowa_decod
 
   cowa_ptx::grid_enter();  // the merge kernel's blocks may be scheduled beside this one's; they wait for its results
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  int split = blockIdx.x, hk = blockIdx.y, b = blockIdx.z, S = a.S, chunk = 0;
-  size_t state = ((size_t)(b * a.Hkv + hk) * G) * S + split;  // of the first head, the others' at state + c * apart
-  int apart = S;
-  if (SHARED && !alike(a)) {
-    const int slot = (b * a.Hkv + hk) * S + split;
-    const Share x = share_at(a, slot);
-    if (x.b < 0) return;
-    b = x.b; S = x.S; chunk = x.chunk;
-    const int i = slot - x.before * a.Hkv;
-    hk = (int)__fdividef(i + 0.5f, (float)S); split = i - hk * S;  // (i and S are small)
-    state = (size_t)slot * G;
-    apart = 1;
-  }
+  const int split = blockIdx.x, hk = blockIdx.y, b = blockIdx.z, S = a.S;
+  const size_t state = ((size_t)(b * a.Hkv + hk) * G) * S + split;  // of the first head, head c's is at state + c * S
   const int Nk = a.lens[b];
 
   // visible ranges of this head for the current key length
@@ -275,15 +130,16 @@ __global__ void __launch_bounds__(kThreads, D == 64 && G < 8 ? 7 : 5) cowa_decod
   const int n2 = nr > 2 ? rg[2].hi - rg[2].lo + 1 : 0;
   const int V = vm.n0 + vm.n1 + n2;
 
-  if (chunk == 0) chunk = ((V + S - 1) / S + 15) & ~15;
+  // From this sequence's length and the call's sizes alone: its result does not depend on how long the others are.
+  const int chunk = ((V + S - 1) / S + 15) & ~15;
   const int c0 = split * chunk;
   const int clen = min(chunk, V - c0);  // <= kChunkCap by the host's choice of S
 
   if (clen <= 0) {  // empty split: neutral partial state
-    for (int i = tid; i < G * D; i += kThreads) a.ws_o[(state + (size_t)(i / D) * apart) * D + i % D] = 0.f;
+    for (int i = tid; i < G * D; i += kThreads) a.ws_o[(state + (size_t)(i / D) * S) * D + i % D] = 0.f;
     if (tid < G) {
-      a.ws_m[state + tid * apart] = -INFINITY;
-      a.ws_l[state + tid * apart] = 0.f;
+      a.ws_m[state + tid * S] = -INFINITY;
+      a.ws_l[state + tid * S] = 0.f;
     }
     return;
   }
@@ -420,38 +276,30 @@ __global__ void __launch_bounds__(kThreads, D == 64 && G < 8 ? 7 : 5) cowa_decod
     float s = 0.f;
 #pragma unroll
     for (int r = 0; r < kThreads / 32; ++r) s += sc[r * G * D + i];
-    a.ws_o[(state + (size_t)(i / D) * apart) * D + i % D] = s;
+    a.ws_o[(state + (size_t)(i / D) * S) * D + i % D] = s;
   }
   if (tid < G) {
-    a.ws_m[state + tid * apart] = m_s[tid];
-    a.ws_l[state + tid * apart] = l_s[tid];
+    a.ws_m[state + tid * S] = m_s[tid];
+    a.ws_l[state + tid * S] = l_s[tid];
   }
 }
 
 // Merge of the split states: M = max m_s, L = sum l_s 2^(m_s - M), o = sum o_s 2^(m_s - M) / L,
 // lse = ln2 * (M + log2 L).  One block per (sequence, QO head).  A warp takes every W-th split, eight at a time, D/32 columns per
 // lane, states and O in one round trip, and the running maximum moves between such groups; the warps' results meet in shared memory.
-// W: sixteen warps (one sequence of 57 700 visible rows in 452 splits: with four 16 us of 29 were this kernel), eight where
-// splits are shared out and a sequence has up to 32 on average.  Without sharing four are enough up to 32 splits: a lane reads one
-// split's state and every warp knows M and L.  That form has 32 registers, so that its blocks wait beside five of the split
-// kernel's (with 72: 8 sequences of 8000 tokens 16.6 us, so 17.1; held to 32 with spills 17.9).
-template <int D, int W, bool SHARED>
+// W: sixteen warps (one sequence of 57 700 visible rows in 452 splits: with four 16 us of 29 were this kernel); four are enough up
+// to 32 splits, where a lane reads one split's state and every warp knows M and L.  That form has 32 registers, so that its
+// blocks wait beside five of the split kernel's (with 72: 8 sequences of 8000 tokens 16.6 us, so 17.1; held to 32 with spills
+// 17.9).
+template <int D, int W>
 __global__ void __launch_bounds__(W * 32) cowa_decode_combine_kernel(const DecodeArgs a, __nv_bfloat16* o, float* lse) {
   constexpr int V = D / 32, U = 8;  // columns per lane, splits of a group
-  constexpr bool kOnce = W * U == 32 && !SHARED;  // S <= 32
+  constexpr bool kOnce = W * U == 32;  // S <= 32
   __shared__ float part[W][D], part_m[W], part_l[W];
   const int bh = blockIdx.x;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // The lengths are not written by the split kernel and were complete before it began (grid_wait); its states are after the wait.
-  size_t first = (size_t)bh * a.S;  // split s lies s * step further
-  int S = a.S, step = 1;
-  if (SHARED && !alike(a)) {
-    const int b = bh / a.Hq, h = bh % a.Hq, G = a.Hq / a.Hkv;
-    const Share x = share_of(a, b);
-    S = x.S;
-    first = ((size_t)x.before * a.Hkv + (size_t)(h / G) * S) * G + h % G;
-    step = G;
-  }
+  const int S = a.S;
+  const size_t first = (size_t)bh * S;
   cowa_ptx::grid_enter();
   const float* m = a.ws_m + first;
   const float* l = a.ws_l + first;
@@ -460,14 +308,14 @@ __global__ void __launch_bounds__(W * 32) cowa_decode_combine_kernel(const Decod
 #pragma unroll
   for (int i = 0; i < V; ++i) acc[i] = 0.f;
   if constexpr (kOnce) {
-    const float ms = lane < S ? m[lane * step] : -INFINITY;
-    const float ls = lane < S ? l[lane * step] : 0.f;
+    const float ms = lane < S ? m[lane] : -INFINITY;
+    const float ls = lane < S ? l[lane] : 0.f;
     float x[U][V];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int s = warp + W * u;
 #pragma unroll
-      for (int i = 0; i < V; ++i) x[u][i] = s < S ? po[(size_t)(s * step) * D + i] : 0.f;
+      for (int i = 0; i < V; ++i) x[u][i] = s < S ? po[(size_t)s * D + i] : 0.f;
     }
     mx = ms;
 #pragma unroll
@@ -485,13 +333,13 @@ __global__ void __launch_bounds__(W * 32) cowa_decode_combine_kernel(const Decod
   } else {
     for (int s0 = warp; s0 < S; s0 += W * U) {
       const bool in = lane < U && s0 + lane * W < S;
-      const float ms = in ? m[(s0 + lane * W) * step] : -INFINITY;
-      const float ls = in ? l[(s0 + lane * W) * step] : 0.f;
+      const float ms = in ? m[s0 + lane * W] : -INFINITY;
+      const float ls = in ? l[s0 + lane * W] : 0.f;
       float x[U][V];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int s = s0 + u * W;
-        const float* src = po + (size_t)(s * step) * D;
+        const float* src = po + (size_t)s * D;
         if constexpr (V == 4) {
           const float4 y = s < S ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
           x[u][0] = y.x; x[u][1] = y.y; x[u][2] = y.z; x[u][3] = y.w;
@@ -562,7 +410,7 @@ int resident_blocks_of() {
   int dev = 0, sms = 0, occ = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cowa_decode_split_kernel<D, G, false>, kThreads, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cowa_decode_split_kernel<D, G>, kThreads, 0) !=
       cudaSuccess)
     return 0;
   return sms * occ;
@@ -607,18 +455,14 @@ int pick_splits(int B, int Tmax, int Hq, int Hkv, int D, const cowa_params_t* p)
 template <int D>
 cudaError_t launch_combine(const DecodeArgs& a, __nv_bfloat16* o, float* lse, cudaStream_t st) {
   const dim3 rows((unsigned)(a.B * a.Hq));
-  if (a.shared)
-    return a.S > 32 ? cowa::launch_chained(cowa_decode_combine_kernel<D, 16, true>, rows, 512, 0, st, a, o, lse)
-                    : cowa::launch_chained(cowa_decode_combine_kernel<D, 8, true>, rows, 256, 0, st, a, o, lse);
-  return a.S > 32 ? cowa::launch_chained(cowa_decode_combine_kernel<D, 16, false>, rows, 512, 0, st, a, o, lse)
-                  : cowa::launch_chained(cowa_decode_combine_kernel<D, 4, false>, rows, 128, 0, st, a, o, lse);
+  return a.S > 32 ? cowa::launch_chained(cowa_decode_combine_kernel<D, 16>, rows, 512, 0, st, a, o, lse)
+                  : cowa::launch_chained(cowa_decode_combine_kernel<D, 4>, rows, 128, 0, st, a, o, lse);
 }
 
 template <int D, int G>
 cudaError_t launch_split(const DecodeArgs& a, cudaStream_t st) {
   const dim3 grid(a.S, a.Hkv, a.B);
-  return a.shared ? cowa::launch_chained(cowa_decode_split_kernel<D, G, true>, grid, kThreads, 0, st, a)
-                  : cowa::launch_chained(cowa_decode_split_kernel<D, G, false>, grid, kThreads, 0, st, a);
+  return cowa::launch_chained(cowa_decode_split_kernel<D, G>, grid, kThreads, 0, st, a);
 }
 
 template <int D>
@@ -679,17 +523,8 @@ int decode_launch(const void* q, const void* kc, const void* vc, const int32_t* 
   a.hkv_global = p->hkv_global > 0 ? p->hkv_global : Hkv;
   a.hkv_offset = p->hkv_offset;
   a.full_attn = p->full_attn;
-  // Sharing out costs 0.6 us, also where the lengths turn out alike (alike() before the first load, a merge kernel that does not
-  // fit beside the split kernel's blocks): too much where the splits are short (8 sequences of 7800 to 8000 tokens, 8 groups, 182
-  // rows a split: 16.6 us, 17.3 with it).
-  // Of several waves a longer block is made up for by the blocks that follow, and equal ones keep in step, so that memory idles
-  // while all of them weigh their scores (32 sequences of 1500 to 2600 tokens, 8 groups of one head: 46.9 us, shared out 52).
-  a.shared = B > 1 && B <= kShareSeqs && (long long)S * 256 < max_visible(Tmax, a.hkv_global, p) &&
-             (long long)B * Hkv * S <= resident_blocks(D, Hq / Hkv);
   const long long rows = (long long)B * Hkv * max_visible(Tmax, a.hkv_global, p);  // K and V: 4 D bytes each
   a.ahead = rows * D <= (4ll << 20) && rows <= 2ll * kThreads * S * B * Hkv;
-  a.inv_room = 1.f / ((float)B * S);
-  a.head_magic = a.hkv_global > 1 && ((long long)Tmax + a.hkv_global) * a.hkv_global <= 0xFFFFFFFFll ? 0xFFFFFFFFu / a.hkv_global + 1 : 0;
   a.scale_log2 = p->softmax_scale * 1.4426950408889634f;
   const int G = Hq / Hkv;
   cudaError_t e = (D == 128) ? dispatch_split<128>(G, a, st) : dispatch_split<64>(G, a, st);

@@ -1,6 +1,5 @@
-"""Decode of batches of very different lengths, whose splits are shared out by length, against the float64 oracle: sequences of a few
-rows beside long ones, lengths at the borders of a split, as many sequences as are shared out at most and one more; and of batches
-that are alike, which are not, or just not alike."""
+"""Single-token decode of batches of very different lengths against the float64 oracle: sequences of a few rows beside long ones,
+lengths at the borders of a split, hundreds of splits and few; and that a sequence's bits do not depend on how long the others are."""
 import numpy as np
 import pytest
 import torch
@@ -8,6 +7,7 @@ import torch
 import cowa_inputs
 import paper_2609_32704_b200 as cowa
 from oracle import cowa_oracle as orc
+from launched import launched
 from test_gpu_parity import DEV, TOL_LSE, check
 
 pytestmark = pytest.mark.gpu
@@ -36,11 +36,27 @@ def test_splits_by_length(B, longest, Hq, Hkv, D, sink, local):
     compare(lengths(B, longest), longest, Hq, Hkv, D, sink, local)
 
 
-@pytest.mark.parametrize("shortest", [16000, 13000, 11000])  # the longest has 1.0, 1.1 and 1.2 times the average
-@pytest.mark.parametrize("Hq,Hkv,D", [(16, 2, 128), (4, 2, 64)])
-def test_lengths_alike(Hq, Hkv, D, shortest):
-    longest = 16000
-    compare([shortest + (longest - shortest) * i // 7 for i in range(8)], longest, Hq, Hkv, D, 64, 6000)
+@pytest.mark.parametrize("B,longest,Hq,Hkv,D,sink,local,warps", [
+    (8, 30000, 16, 2, 128, 64, 3481, 16),  # more than 32 splits a sequence: sixteen warps merge
+    (8, 30000, 16, 4, 64, 64, 3481, 4),
+    (3, 20000, 8, 8, 128, 0, 1000, 4),
+    (40, 6000, 2, 1, 64, 16, 2000, 4),
+])
+def test_bits_do_not_depend_on_the_other_lengths(B, longest, Hq, Hkv, D, sink, local, warps):
+    q, k, v, _ = cowa_inputs.make_decode_inputs(18, B, longest, Hq, Hkv, D, longest, longest)
+    q, k, v = q.to(DEV), k.to(DEV), v.to(DEV)
+    params = cowa.make_params(sink=sink, local=local, softmax_scale=cowa_inputs.softmax_scale(D))
+    ws = torch.empty(cowa.cowa_decode_workspace_bytes(B, longest, Hq, Hkv, D, params), dtype=torch.uint8, device=DEV)
+    first, results = longest * 5 // 9, []
+    for others in (64, longest // 3, longest):  # the lengths of the sequences behind the first
+        lens = torch.tensor([first] + [max(1, others - 17 * i) for i in range(B - 1)], dtype=torch.int32, device=DEV)
+        o = torch.full((B, Hq, D), float("nan"), dtype=torch.bfloat16, device=DEV)
+        lse = torch.full((B, Hq), float("nan"), device=DEV)
+        kernels = launched(lambda: cowa.cowa_decode(q, k, v, lens, o, lse, params, ws))
+        assert kernels[1] == (f"cowa_decode_combine_kernel<{D},{warps}>", B * Hq)
+        results.append((o[0], lse[0]))
+    for o, lse in results[1:]:
+        assert torch.equal(o, results[0][0]) and torch.equal(lse, results[0][1])
 
 
 @pytest.mark.parametrize("sink,local", [(128, 2 ** 31 - 1), (2 ** 31 - 1, 5), (2 ** 31 - 1, 2 ** 31 - 1)])
