@@ -46,7 +46,14 @@ struct FwdSmem {
   static constexpr int kQ = BQ * D * 2;   // Q tile (later the O staging tile)
   static constexpr int kKV = BK * D * 2;  // one K or V step tile
   static constexpr int oQ = 0, oKV = kQ, oState = kQ + NS * 4 * kKV, oBar = oState + (NS > 1 || SPLIT ? NS * BQ * 8 : 0);
-  static constexpr int kBytes = oBar + 32 + NS * 80 + 1024;  // + barriers + alignment slack
+  static constexpr int kUsed = oBar + 32 + NS * 80 + 1024;  // + barriers + alignment slack
+  // A cluster's blocks hold their TMEM, half of an SM's each, until all of them are through, and neither the allocation nor the
+  // cluster's barrier is a bounded wait.  A third block on an SM would wait for TMEM that two other clusters hold; if their other
+  // blocks waited on other SMs for this cluster's, none would ever end.  So a block takes more than a third of an SM's shared memory
+  // whatever its registers allow (50 KB and 131 registers at D = 64: at 128 three would fit).
+  static constexpr int kSm = 228 * 1024, kReserved = 1024;  // shared memory of an SM, and what each block takes besides its own
+  static constexpr int kBytes = SPLIT ? std::max(kUsed, kSm / 3) : kUsed;
+  static_assert(!SPLIT || (3 * (kBytes + kReserved) > kSm && 2 * (kBytes + kReserved) <= kSm), "two blocks of clusters on an SM");
 };
 
 // NB: S/P buffers of a stream (64 columns each, then O of D); an SM holds 4 / NB streams.

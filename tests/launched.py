@@ -1,4 +1,5 @@
 """Which of the library's kernels a call launches: tests that are about one form of a kernel make sure that it is the one that ran."""
+import collections
 import json
 import os
 import re
@@ -7,9 +8,11 @@ import tempfile
 import torch
 from torch.profiler import ProfilerActivity, profile
 
+Launch = collections.namedtuple("Launch", "kernel blocks shared")  # name with template arguments; blocks; bytes of shared memory of each
+
 
 def launched(call):
-    """[(kernel with its template arguments, blocks)] of the kernels of this library that call() launches, in their order."""
+    """The kernels of this library that call() launches, in their order."""
     call()  # (loading of the kernels, first use of the device)
     torch.cuda.synchronize()
     with profile(activities=[ProfilerActivity.CUDA, ProfilerActivity.CPU]) as p:
@@ -25,6 +28,6 @@ def launched(call):
         m = re.search(r"(cowa_\w+)(<[^>]*>)?", e["name"])
         if m:
             x, y, z = e["args"]["grid"]
-            out.append((m.group(1) + (m.group(2) or "").replace(" ", ""), x * y * z))
+            out.append(Launch(m.group(1) + (m.group(2) or "").replace(" ", ""), x * y * z, e["args"]["shared memory"]))
     assert out, "the profiler saw no kernel of the library"
     return out

@@ -7,6 +7,7 @@ import torch
 
 import cowa_inputs
 import paper_2609_32704_b200 as cowa
+from launched import launched
 from oracle import cowa_oracle as orc
 from test_gpu_parity import DEV, TOL_LSE, check
 
@@ -50,3 +51,20 @@ def test_forms_match_the_oracle(D, B, Nq, Nk, Hq, Hkv, sink, local):
         o_ref, lse_ref = orc.forward(f(q[b]), f(k[b]), f(v[b]), ws, scale)
         check(f"lse[b={b}]", lse[b].cpu().numpy(), lse_ref, TOL_LSE, TOL_LSE)
         check(f"o[b={b}]", o[b].float().cpu().numpy(), o_ref)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("packed", [False, True])
+def test_no_sm_holds_three_blocks_of_clusters(D, packed):
+    """Two hold all TMEM of an SM, and a third one would keep its cluster's other blocks waiting with what they hold: shared memory has
+    to rule it out, as registers depend on the compiler."""
+    q, k, v = (torch.zeros(shape, dtype=torch.bfloat16, device=DEV) for shape in ((4, 128, D), (2, 700, D), (2, 700, D)))
+    o, lse = torch.empty_like(q), torch.empty((4, 128), device=DEV)
+    params = cowa.make_params(sink=4, local=100, softmax_scale=cowa_inputs.softmax_scale(D))
+    if packed:
+        cu = [torch.tensor([0, n], dtype=torch.int32, device=DEV) for n in (128, 700)]
+        kernel, _, shared = launched(lambda: cowa.cowa_prefill_varlen(q, k, v, o, lse, *cu, params))[0]
+    else:
+        kernel, _, shared = launched(lambda: cowa.cowa_prefill(q[None], k[None], v[None], o[None], lse[None], params))[0]
+    assert kernel == f"cowa_fwd_kernel<{D},{str(packed).lower()},2,1,true>"
+    assert 3 * (shared + 1024) > torch.cuda.get_device_properties(0).shared_memory_per_multiprocessor
