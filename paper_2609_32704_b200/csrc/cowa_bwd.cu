@@ -388,7 +388,7 @@ cowa_bwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         }
         __syncwarp();
         if (it.steps < 0) break;
-        if (!a.single) ok = mbar_wait(bar_ask, ni & 1, a.status);
+        if (!a.single) ok = mbar_wait(bar_ask, ni & 1, a.status, cowa_bwd_item_clocks(it.steps));  // nearly all of the item
         ++ni;
         if (ok) idx = next_index();
       }

@@ -160,6 +160,10 @@ COWA_HD void cowa_bwd_ranges(const CowaWin& w, int k0, int k1, int off, int Nq, 
   }
 }
 
+// Limit, in clocks, of a wait that lasts about as long as a work item of `steps` steps (128 queries each, 4000 to 5000 clocks): that
+// of every other wait, about a second, and four times the item.
+COWA_HD long long cowa_bwd_item_clocks(int steps) { return (1ll << 31) + (long long)steps * 16384; }
+
 COWA_HD int cowa_bwd_tile_at(const CowaRange r[2], int t) {
   int n0 = cowa_range_len(r[0]);
   if (t < n0) return r[0].lo + t;
