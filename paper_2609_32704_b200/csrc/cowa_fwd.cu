@@ -368,10 +368,7 @@ cowa_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           }
         }
       };
-      if constexpr (NB == 1) {  // S of this step completed behind the product of the step before
-        l_sum *= alpha;
-        rescale();
-      }
+      if constexpr (NB == 1) rescale();  // S of this step completed behind the product of the step before
 
       // p = 2^(s * scale - m): packed fp32 pairs for the multiply-add and the row sum
       const float2 nsub2 = make_float2(-sub, -sub);
@@ -389,7 +386,7 @@ cowa_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         if constexpr (NB == 1) tmem_st16(t_S + c * 16, pk);  // P over the first 32 columns of S
       }
       const float2 rs2 = add2(add2(rsa[0], rsa[1]), add2(rsa[2], rsa[3]));
-      l_sum = (NB == 2 ? l_sum * alpha : l_sum) + (rs2.x + rs2.y);
+      l_sum = fmaf(l_sum, alpha, rs2.x + rs2.y);  // (all forms alike, whatever the compiler would merge)
 
       // Every step waits for the product of the step before (normally long finished): the accumulator
       // may then be rescaled safely, and no thread ever falls two phases behind on this barrier, which

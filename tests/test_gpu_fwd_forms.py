@@ -53,6 +53,26 @@ def test_forms_match_the_oracle(D, B, Nq, Nk, Hq, Hkv, sink, local):
         check(f"o[b={b}]", o[b].float().cpu().numpy(), o_ref)
 
 
+@pytest.mark.parametrize("step", [6.0, 7.0])
+def test_one_and_two_buffers_add_up_alike_where_the_reference_moves(step):
+    """A batched call with one S buffer and the packed call of the same sequences with two.  From tile to tile the scores rise by
+    more than the 8 (log2) that move a row's reference, by so little more that what was summed before still counts."""
+    B, Nq, Nk, Hq, Hkv, D = 3, 520, 1100, 24, 8, 64
+    gen = torch.Generator().manual_seed(303)
+    q, k, v = (torch.randn(B, H, n, D, generator=gen) for H, n in ((Hq, Nq), (Hkv, Nk), (Hkv, Nk)))
+    q[..., 0], k[..., 0] = 8.0, -step * (torch.arange(Nk) // 64).float()
+    q, k, v = (x.to(torch.bfloat16).to(DEV) for x in (q, k, v))
+    params = cowa.make_params(sink=0, local=Nk, softmax_scale=cowa_inputs.softmax_scale(D))
+    o, lse = torch.empty_like(q), torch.empty((B, Hq, Nq), device=DEV)
+    assert launched(lambda: cowa.cowa_prefill(q, k, v, o, lse, params))[0].kernel == "cowa_fwd_kernel<64,false,1,1,false>"
+    pack = lambda x: x.transpose(0, 1).reshape(x.shape[1], -1, D).contiguous()  # noqa: E731
+    o2, lse2 = torch.empty_like(pack(o)), torch.empty((Hq, B * Nq), device=DEV)
+    cu = [torch.arange(B + 1, dtype=torch.int32, device=DEV) * n for n in (Nq, Nk)]
+    call = lambda: cowa.cowa_prefill_varlen(pack(q), pack(k), pack(v), o2, lse2, *cu, params)  # noqa: E731
+    assert launched(call)[0].kernel == "cowa_fwd_kernel<64,true,2,1,false>"
+    assert torch.equal(pack(o), o2) and torch.equal(lse.transpose(0, 1).reshape(Hq, -1), lse2)
+
+
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("packed", [False, True])
 def test_no_sm_holds_three_blocks_of_clusters(D, packed):
