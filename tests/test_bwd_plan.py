@@ -39,6 +39,49 @@ def bwd_plan(B, Nq, Nk, Hkv, G, windows):
     return cls, {h: steps[h * -(-Nk // 128):(h + 1) * -(-Nk // 128)] for h in range(Hkv)}
 
 
+def blocks_of(B, Nq, Nk, Hkv, G, windows, deterministic=False):
+    """(blocks of the main kernel, table): how the tiles are in fact cut.  table: None, or the parts of every tile of one batch
+    element, KV tiles ascending, heads within them, where few tiles are shared out by their length instead."""
+    (sinks, rest, tail), steps = bwd_plan(B, Nq, Nk, Hkv, G, windows)
+    nkv, run = -(-Nk // 128), [sinks[1], rest[1], tail[1]]
+    per_tile = [[n for _, n in steps[h]] for h in range(Hkv)]
+    nsink = sinks[0] // (B * Hkv)
+    total, n_rest = B * sum(map(sum, per_tile)), B * Hkv * (nkv - nsink)
+    avg = B * sum(sum(x[nsink:]) for x in per_tile) / n_rest if n_rest else 0.0
+    if not deterministic:  # not all parts of body tiles that there is room for
+        best = None
+        for p in range(1, rest[1] + 1):
+            n = sinks[0] * sinks[1] + rest[0] * p + tail[0] * tail[1]
+            t = (4 + avg / 2 / p) * (max(n / SMS, 1.0) + 0.5) + (0.02 * rest[0] * p if p > 1 else 0)
+            if best is None or t < best:
+                best, run[1] = t, p
+    blocks = sinks[0] * run[0] + rest[0] * run[1] + tail[0] * run[2]
+    longest = [max([n for x in per_tile for n in x[a:b]], default=0) for a, b in ((0, nsink), (nsink, nkv))]
+    rows, share = B * Hkv * G * Nq, total / SMS
+    uneven = max(longest[0] / run[0], longest[1] / run[1]) > 1.2 * share
+    if deterministic or nkv * Hkv * B > 2 * SMS or rows > 131072 or not (uneven or Nq <= 4096 and rows <= 81920):
+        return blocks, None
+    cnt = [per_tile[h][j] for j in range(nkv) for h in range(Hkv)]
+    room, best, x = min(slots([sinks, rest, tail]), 65535 * B), None, max(longest + [4])
+    while True:
+        n = B * sum(max(-(-c // x), 1) for c in cnt)
+        if n > room:
+            break
+        t = 10 + x
+        if n > SMS:
+            t = max(t, 5 + (total + 5 * n) / SMS + 0.4 * (5 + x))
+        if n > len(cnt) * B:
+            t += 0.04 * n
+        if best is None or t < best[0]:
+            best = t, x, n
+        if x == 4:
+            break
+        x = max(x * 7 // 8, 4)
+    if best is None:
+        return blocks, None
+    return best[2], [max(-(-c // best[1]), 1) for c in cnt]
+
+
 def slots(cls):
     return sum(t * p for t, p in cls if p > 1)
 
@@ -67,6 +110,19 @@ def test_workspace_holds_the_shared_tiles_and_no_more(B, T, Hq, Hkv, D, sink, lo
     p = cowa.make_params(sink=sink, local=local, softmax_scale=0.1, hkv_global=hg, hkv_offset=off)
     cls, _ = bwd_plan(B, T, T, Hkv, Hq // Hkv, orc.default_windows(T, hg, sink, local)[off:off + Hkv])
     assert slots_asked_for(B, T, Hq, Hkv, D, p) == slots(cls) <= 7 * SMS
+
+
+@pytest.mark.parametrize("B,T,Hq,Hkv,D,sink,local,hg,off", CASES)
+def test_blocks_fit_the_slots(B, T, Hq, Hkv, D, sink, local, hg, off):
+    windows = orc.default_windows(T, hg, sink, local)[off:off + Hkv]
+    cls, steps = bwd_plan(B, T, T, Hkv, Hq // Hkv, windows)
+    for deterministic in (False, True):
+        blocks, table = blocks_of(B, T, T, Hkv, Hq // Hkv, windows, deterministic)
+        if table is None:
+            assert blocks <= sum(t * p for t, p in cls)
+        else:  # a slot per block, whether it needs one or not
+            assert not deterministic and blocks == B * sum(table) <= slots(cls)
+            assert all(p <= max(n, 1) for p, n in zip(table, (steps[h][j][1] for j in range(-(-T // 128)) for h in range(Hkv))))
 
 
 def test_packed_workspace_without_parameters_is_enough_for_all():

@@ -15,7 +15,7 @@ import torch
 import cowa_inputs
 import paper_2609_32704_b200 as cowa
 from oracle import cowa_oracle as orc
-from test_bwd_plan import bwd_plan, slots, slots_asked_for
+from test_bwd_plan import blocks_of, bwd_plan, slots, slots_asked_for
 
 pytestmark = pytest.mark.gpu
 
@@ -274,10 +274,11 @@ def run_fwd_bwd(q, k, v, d_o, params):
     return dq, dk, dv
 
 
-def bwd_case(B, T, Hq, Hkv, D, sink, local, seed=51, windows=None, full_attn=False):
+def bwd_case(B, T, Hq, Hkv, D, sink, local, seed=51, windows=None, full_attn=False, deterministic=False):
     q, k, v, d_o = cowa_inputs.make_train_inputs(seed, B, T, Hq, Hkv, D)
     scale = cowa_inputs.softmax_scale(D)
-    params = cowa.make_params(sink=sink, local=local, softmax_scale=scale, windows=windows, full_attn=full_attn)
+    params = cowa.make_params(sink=sink, local=local, softmax_scale=scale, windows=windows, full_attn=full_attn,
+                              deterministic=deterministic)
     dq, dk, dv = run_fwd_bwd(q.to(DEV), k.to(DEV), v.to(DEV), d_o.to(DEV), params)
     if full_attn:
         ws = [(0, T, 0, 0)] * Hkv
@@ -320,16 +321,20 @@ def test_bwd_full_attn_and_explicit_windows():
     bwd_case(1, 700, 2, 2, 128, 0, 1, windows=[(0, 50, 100, 200), (20, 10, 0, 0)])
 
 
-def test_bwd_tensor_parallel_shard():
+@pytest.mark.parametrize("deterministic", [False, True])
+def test_bwd_tensor_parallel_shard(deterministic):
     # One KV head of eight and its 8 QO heads, as a TP=8 rank holds them: windows of the global head, and (few tiles, a long
-    # sink tile) every tile's steps cut into parts for several blocks.
+    # sink tile) every tile's steps cut into parts for several blocks: by the tiles' lengths, or, reproducible, into the same
+    # number for all sink tiles and for all others.
     T, Hq, D, sink, local = 3000, 8, 128, 40, 200
     scale = cowa_inputs.softmax_scale(D)
     for r in (0, 5):
         q, k, v, d_o = cowa_inputs.make_train_inputs(56 + r, 1, T, Hq, 1, D)
-        params = cowa.make_params(sink=sink, local=local, softmax_scale=scale, hkv_global=8, hkv_offset=r)
+        params = cowa.make_params(sink=sink, local=local, softmax_scale=scale, hkv_global=8, hkv_offset=r, deterministic=deterministic)
         cls, _ = bwd_plan(1, T, T, 1, Hq, orc.default_windows(T, 8, sink, local)[r:r + 1])
         assert slots_asked_for(1, T, Hq, 1, D, params) == slots(cls) and cls[0][1] > 1 and cls[1][1] > 1
+        blocks, table = blocks_of(1, T, T, 1, Hq, orc.default_windows(T, 8, sink, local)[r:r + 1], deterministic)
+        assert (table is None) == deterministic and (blocks == slots(cls) if deterministic else min(table[0], table[1]) > 1)
         dq, dk, dv = run_fwd_bwd(q.to(DEV), k.to(DEV), v.to(DEV), d_o.to(DEV), params)
         ws = orc.default_windows(T, 8, sink, local)[r:r + 1]
         f = cowa_inputs.to_f64
@@ -353,15 +358,22 @@ def test_bwd_group_split_over_some_blocks():
     assert torch.equal(dk1, dk2) and torch.equal(dv1, dv2)
 
 
-def test_bwd_parts_cut_inside_a_head():
-    # Three QO heads per KV head, five parts per tile: a part begins in the middle of a head's steps.
+@pytest.mark.parametrize("deterministic", [False, True])
+def test_bwd_parts_cut_inside_a_head(deterministic):
+    # Three QO heads per KV head, parts that begin in the middle of a head's steps: five per tile, reproducible, or by the
+    # tiles' lengths.
     B, T, Hq, D, local = 2, 700, 3, 128, 64
     ws = orc.default_windows(T, 1, 0, local)
     (_, (_, parts), _), steps = bwd_plan(B, T, T, 1, Hq, ws)
     assert parts == 5 and any(n * i // parts % (n // Hq) for _, n in steps[0] for i in range(1, parts))
     params = cowa.make_params(sink=0, local=local, softmax_scale=cowa_inputs.softmax_scale(D))
     assert slots_asked_for(B, T, Hq, 1, D, params) == 5 * len(steps[0]) * B
-    bwd_case(B, T, Hq, 1, D, 0, local, seed=76)
+    blocks, table = blocks_of(B, T, T, 1, Hq, ws, deterministic)
+    if deterministic:
+        assert table is None and blocks == 5 * len(steps[0]) * B
+    else:
+        assert any(n * i // p % (n // Hq) for p, (_, n) in zip(table, steps[0]) for i in range(1, p))
+    bwd_case(B, T, Hq, 1, D, 0, local, seed=76, deterministic=deterministic)
 
 
 def test_bwd_shared_last_wave():
