@@ -7,7 +7,9 @@ import torch
 
 import cowa_inputs
 import paper_2609_32704_b200 as cowa
+from launched import launched
 from oracle import cowa_oracle as orc
+from test_gpu_fwd_forms import check_form
 from test_gpu_parity import TOL_LSE, check
 
 pytestmark = pytest.mark.gpu
@@ -23,13 +25,28 @@ def _sees(w, rows, off, keys):
     return (d >= 0) & ((d < n) | (k < s) | ((d >= n + g) & (d < n + g + l)))
 
 
-# one shape per forward kernel: (B, Nq, Nk, Hq, Hkv, D, sink, local)
-FORWARD = [
-    (1, 130, 6000, 4, 2, 128, 64, 700),     # an item shared by a cluster of eight blocks
-    (1, 200, 9000, 4, 2, 64, 64, 700),      # the same at D = 64
-    (2, 1100, 4000, 32, 8, 128, 64, 1500),  # two heads per persistent block
-    (1, 300, 700, 4, 2, 128, 16, 100),      # one head per block
+# one shape per form of the forward kernels: (B, Nq, Nk, Hq, Hkv, D, sink, local), and the form as test_gpu_fwd_forms names it
+FORMS = [
+    ((1, 130, 6000, 4, 2, 128, 64, 700), 8),     # an item shared by a cluster of eight blocks
+    ((1, 200, 9000, 4, 2, 64, 64, 700), 8),      # the same at D = 64
+    ((2, 1100, 4000, 32, 8, 128, 64, 1500), "pair"),  # two heads per block, items taken over
+    ((1, 300, 700, 4, 2, 128, 16, 100), 8),      # short lists: some blocks of a cluster have one step, some none
+    ((2, 700, 1400, 4, 4, 64, 64, 300), 2),
+    ((2, 300, 1300, 5, 5, 128, 64, 300), 4),
+    ((2, 600, 2500, 10, 5, 128, 100, 900), "pair, shared item"),
+    ((2, 700, 1400, 8, 8, 128, 64, 300), "plain"),
+    ((2, 900, 1000, 10, 5, 64, 16, 130), "plain"),
+    ((3, 520, 1100, 24, 8, 64, 64, 100), "one buffer"),
+    ((2, 700, 1400, 8, 8, 64, 64, 300), "streams"),
 ]
+FORWARD = [shape for shape, _ in FORMS]
+
+
+@pytest.mark.parametrize("shape,form", FORMS)
+def test_the_shapes_below_reach_every_form(shape, form):
+    B, Nq, Nk, Hq, Hkv, D, sink, local = shape
+    q, k, v = (x.to(DEV) for x in _forward_inputs(B, Nq, Nk, Hq, Hkv, D))
+    check_form(launched(lambda: _forward(q, k, v, sink, local))[0], D, False, form, -(-Nq // 128) * B * Hq)
 
 
 def _forward(q, k, v, sink, local):

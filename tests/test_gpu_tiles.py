@@ -7,6 +7,7 @@ import torch
 
 import cowa_inputs
 import paper_2609_32704_b200 as cowa
+from launched import launched
 from oracle import cowa_oracle as orc
 from test_gpu_parity import TOL_LSE, check, multi_case, _packed_inputs, _run_varlen
 
@@ -39,7 +40,8 @@ def _prefill(B, Nq, Nk, Hq, Hkv, D, sink, local, token_major=False, rows=None, m
     qd = put(q)
     o = torch.full_like(qd, float("nan"))
     lse = torch.full((B, Hq, Nq), float("nan"), dtype=torch.float32, device=DEV)
-    cowa.cowa_prefill(qd, put(k), put(v), o, lse, params)
+    kd, vd = put(k), put(v)
+    kernel = launched(lambda: cowa.cowa_prefill(qd, kd, vd, o, lse, params))[0]
     torch.cuda.synchronize()
     cowa.cowa_check_device_status()
     assert torch.isfinite(o).all() and torch.isfinite(lse).all()
@@ -51,12 +53,13 @@ def _prefill(B, Nq, Nk, Hq, Hkv, D, sink, local, token_major=False, rows=None, m
             o_ref, lse_ref = orc.forward_rows(f(q[b]), f(k[b]), f(v[b]), ws, scale, h, rows)
             check(f"lse[{b},{h}]", lse[b, h].cpu().numpy()[rows], lse_ref, TOL_LSE, TOL_LSE)
             check(f"o[{b},{h}]", o[b, h].float().cpu().numpy()[rows], o_ref)
+    return kernel
 
 
 @pytest.mark.parametrize("B,Nq,Nk,Hq,Hkv,D,sink,local", [
     (1, 130, 6000, 4, 2, 128, 64, 700),    # clusters of 8, last tile of two rows
     (1, 1, 9000, 2, 1, 128, 0, 64),        # one query, one item
-    (2, 128, 3000, 8, 2, 128, 130, 333),   # clusters of 4
+    (2, 128, 3000, 8, 2, 128, 130, 333),   # clusters of 8, whole tiles
     (2, 300, 2999, 32, 8, 128, 5, 1500),   # more than half an item per SM: one block per item
     (1, 257, 7000, 8, 4, 64, 64, 500),     # the shared form at D = 64
 ])
