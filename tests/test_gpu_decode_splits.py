@@ -59,6 +59,43 @@ def test_bits_do_not_depend_on_the_other_lengths(B, longest, Hq, Hkv, D, sink, l
         assert torch.equal(o, results[0][0]) and torch.equal(lse, results[0][1])
 
 
+@pytest.mark.parametrize("call", ["decode", "multi", "paged"])
+def test_lengths_written_by_the_kernel_before(call):
+    """The calls' second kernel starts while the first one runs, and the multi-token merge reads the lengths then: other lengths
+    in every call, each written by a kernel right ahead of it, and the results of calls that had the device to themselves."""
+    B, Tmax, Hq, Hkv, D, page = 6, 30016, 16, 2, 128, 64
+    q, k, v, _ = cowa_inputs.make_decode_inputs(19, B, Tmax, Hq, Hkv, D, Tmax, Tmax)
+    q, k, v = q.to(DEV), k.to(DEV), v.to(DEV)
+    params = cowa.make_params(sink=64, local=3000, softmax_scale=cowa_inputs.softmax_scale(D))
+    ws = [torch.empty(n, dtype=torch.uint8, device=DEV) for n in (cowa.cowa_decode_workspace_bytes(B, Tmax, Hq, Hkv, D, params),
+                                                                  cowa.cowa_decode_multi_workspace_bytes(B, 1, Tmax, Hq, Hkv, D, params))]
+    n = Tmax // page
+    pages = [x.reshape(B, Hkv, n, page, D).transpose(1, 2).reshape(B * n, Hkv, page, D).contiguous() for x in (k, v)]
+    table = torch.arange(B * n, dtype=torch.int32, device=DEV).reshape(B, n)
+    lens = torch.ones(B, dtype=torch.int32, device=DEV)
+
+    def run(o):
+        if call == "decode":
+            cowa.cowa_decode(q, k, v, lens, o, None, params, ws[0])
+        elif call == "multi":
+            cowa.cowa_decode_multi(q[:, None], k, v, lens, o[:, None], None, params, ws[1])
+        else:
+            cowa.cowa_decode_paged(q[:, None], *pages, table, lens, o[:, None], None, params, ws[1])
+
+    steps = torch.tensor([[1 + (i * 7919 + b * 12347) % Tmax for b in range(B)] for i in range(24)], dtype=torch.int32, device=DEV)
+    got, want = ([torch.empty_like(q) for _ in steps] for _ in range(2))
+    for x, o in zip(steps, want):
+        lens.copy_(x)
+        torch.cuda.synchronize()
+        run(o)
+        torch.cuda.synchronize()
+    for x, o in zip(steps, got):
+        torch.add(x, 0, out=lens)
+        run(o)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
 @pytest.mark.parametrize("sink,local", [(128, 2 ** 31 - 1), (2 ** 31 - 1, 5), (2 ** 31 - 1, 2 ** 31 - 1)])
 @pytest.mark.parametrize("short", [1, 60, 126, 127])
 def test_windows_wider_than_any_sequence(short, sink, local):

@@ -46,7 +46,9 @@ FORWARD = [shape for shape, _ in FORMS]
 def test_the_shapes_below_reach_every_form(shape, form):
     B, Nq, Nk, Hq, Hkv, D, sink, local = shape
     q, k, v = (x.to(DEV) for x in _forward_inputs(B, Nq, Nk, Hq, Hkv, D))
-    check_form(launched(lambda: _forward(q, k, v, sink, local))[0], D, False, form, -(-Nq // 128) * B * Hq)
+    o, lse = torch.empty_like(q), torch.empty((B, Hq, Nq), device=DEV)
+    params = cowa.make_params(sink=sink, local=local, softmax_scale=cowa_inputs.softmax_scale(D))
+    check_form(launched(lambda: cowa.cowa_prefill(q, k, v, o, lse, params))[0], D, False, form, -(-Nq // 128) * B * Hq)
 
 
 def _forward(q, k, v, sink, local):
