@@ -27,7 +27,8 @@
  *   - Results do not depend on the contents of other sequences of a batch, but their last bits may depend on its
  *     sizes: the forward calls choose a kernel and a split by B, Nq, Nk, the head counts and, packed, the average
  *     length, the multi-token and paged calls cut a sequence's keys at places that follow from all lengths (the
- *     single-token calls from its own).  The same call on the same sizes and lengths gives the same bits (dq: see cowa_params_t.deterministic).
+ *     single-token calls from its own, B, Tmax and the head counts).  The same call on the same sizes and lengths
+ *     gives the same bits (dq: see cowa_params_t.deterministic).
  *   - Return value: COWA_OK (0) or a negative cowa_status_t.  Arguments are validated
  *     before anything is launched.  There is no CPU fallback.
  *   - Preconditions not checked on the device: near >= 1 for every head (so each
