@@ -618,9 +618,17 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
   // line on also where all lists are alike, 192 of 22 steps 30 / 30 / 27: an average of packed lengths does not tell.)
   const bool alike = kn >= 2ll * qn;  // every tile's list is about as long
   int streams = 1, split = 1;
-  [[maybe_unused]] bool deep = false;  // two S buffers
+  [[maybe_unused]] bool deep = false;  // two S buffers, at D = 64
   if (4 * heads <= 2 * sms) {
     while (split < 8 && 2 * split * heads <= (steps >= 24 ? 2 * sms : sms) && 2 * split <= steps) split *= 2;
+    // A merge is as long as four steps, six at D = 128 (the other blocks' O comes in twice as many pieces), and longer where clusters
+    // of four have to share SMs, as they lie within one GPC each: a list that is cut has to save at least that many.  us, one block / the
+    // clusters above: D = 64, 16 items of 2 steps 4.5 / 6.5, 4 6.0 / 6.3, 5 6.7 / 6.8, 6 7.5 / 6.9, 48 of 6 7.6 / 8.1, 8 9.2 / 9.0;
+    // D = 128, 16 of 2 5.3 / 8.5, 4 6.8 / 7.8, 6 8.3 / 8.5, 8 9.8 / 8.8, 48 of 8 10.0 / 11.4, 12 13.1 / 13.0, 36 of 8 10.0 / 11.1,
+    // 10 11.5 / 12.0, 12 13.0 / 12.3.
+    const bool crowded = split == 4 && 9 * split * heads > 8ll * sms;
+    if (steps - steps / split < (D == 64 ? (crowded ? 6 : 4) : (crowded ? 9 : 6))) split = 1;
+    deep = split == 1;  // (one block on an SM)
   } else if (D == 64) {
     if (heads <= 2 * sms ? 12 * steps > heads : heads <= 3 * sms ? 8 * steps > heads : heads <= 5 * sms && steps >= 64) streams = 4;
     else deep = heads <= (alike && !VARLEN ? 2 : 3) * sms;  // (the same sums in the same order as with one buffer)

@@ -35,11 +35,18 @@ def check_form(launch, D, packed, form, items):
 
 # B, Nq, Nk, Hq, Hkv, sink, local, form at D = 64 and 128 (packed at D = 64 where it is another one)
 FORMS = [
-    (1, 1, 64, 1, 1, 0, 7, "one buffer", "plain"),      # a single step
+    (1, 1, 64, 1, 1, 0, 7, "plain", "plain"),  # a single step
+    (1, 100, 125, 8, 4, 4, 30, "plain", "plain"),  # two steps: nothing to share
+    (2, 128, 250, 4, 4, 4, 500, "plain", "plain"),  # four steps
+    (1, 128, 500, 8, 4, 4, 500, 8, 8),         # eight
+    (3, 300, 380, 6, 2, 4, 380, "plain", "plain"),  # 54 items of six steps ...
+    (3, 300, 620, 6, 2, 4, 620, 2, "plain"),   # ... of ten: half of them is saved, which pays for a merge at D = 64
+    (3, 300, 800, 6, 2, 4, 800, 2, 2),         # ... of thirteen
     (1, 100, 500, 2, 1, 64, 300, 8, 8),        # few items: as many parts as the list has steps
     (1, 128, 577, 3, 3, 5, 500, 8, 8),         # odd group: ten steps, the last of one key
     (1, 129, 1999, 4, 4, 64, 700, 8, 8),       # a second tile of one row
-    (3, 500, 500, 3, 3, 4, 100, 4, 4),         # causal lists from nothing up: tiles with fewer steps than parts
+    (3, 500, 500, 3, 3, 4, 100, 4, "plain"),   # causal lists from nothing up: tiles with fewer steps than parts
+    (2, 500, 500, 3, 3, 4, 100, 4, 4),
     (2, 700, 1400, 8, 8, 64, 300, "streams", "plain"),  # 96 items
     (2, 900, 900, 10, 5, 3, 130, "plain", "plain"),     # 160 items of one to seven steps
     (3, 700, 700, 20, 4, 64, 100, "plain", "plain"),    # 360 items, lists of different lengths
