@@ -624,7 +624,7 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
     // A merge is as long as four steps, six at D = 128 (the other blocks' O comes in twice as many pieces), and longer where clusters
     // of four have to share SMs, as they lie within one GPC each: a list that is cut has to save at least that many.  us, one block / the
     // clusters above: D = 64, 16 items of 2 steps 4.5 / 6.5, 4 6.0 / 6.3, 5 6.7 / 6.8, 6 7.5 / 6.9, 48 of 6 7.6 / 8.1, 8 9.2 / 9.0;
-    // D = 128, 16 of 2 5.3 / 8.5, 4 6.8 / 7.8, 6 8.3 / 8.5, 8 9.8 / 8.8, 48 of 8 10.0 / 11.4, 12 13.1 / 13.0, 36 of 8 10.0 / 11.1,
+    // D = 128, 16 of 2 5.3 / 8.5, 4 6.8 / 7.8, 6 8.3 / 8.5, 8 9.8 / 10.0, 10 11.4 / 10.6, 48 of 8 10.0 / 11.4, 12 13.1 / 13.0, 36 of 8 10.0 / 11.1,
     // 10 11.5 / 12.0, 12 13.0 / 12.3.
     const bool crowded = split == 4 && 9 * split * heads > 8ll * sms;
     if (steps - steps / split < (D == 64 ? (crowded ? 6 : 4) : (crowded ? 9 : 6))) split = 1;
